@@ -31,7 +31,6 @@ namespace {
 
 constexpr int CTRL = 256;      // threads of the single-block control kernels (>= k of GMRES)
 constexpr int KBIG = 1 << 18;  // systems per FP64 BiCGStab call (its control kernels loop over systems)
-constexpr int CHUNK = 1024;    // rows per (system, chunk) reduction item (one warp)
 constexpr int CHUNK_U = 256;   // rows per item of the GMRES update (no per-vector reduction)
 constexpr int TILE = 256;      // rows per SpMV item (one block)
 constexpr int PJ = 16;         // basis vectors per register-tiled projection pass
@@ -93,8 +92,9 @@ __device__ void build_list_block(int k, const int* mask, int* list)
     const int per = (k + nt - 1) / nt;
     const int c0 = tid * per < k ? tid * per : k;
     const int c1 = c0 + per < k ? c0 + per : k;
+    // through L2: other blocks of the running kernel may have written the mask
     int cnt = 0;
-    for (int c = c0; c < c1; ++c) cnt += mask[c] != 0;
+    for (int c = c0; c < c1; ++c) cnt += __ldcg(mask + c) != 0;
     int incl = cnt;
     for (int o = 1; o < 32; o <<= 1) {
         const int v = __shfl_up_sync(SAI_FULL, incl, o);
@@ -114,7 +114,7 @@ __device__ void build_list_block(int k, const int* mask, int* list)
     __syncthreads();
     int pos = wsum[wid] + incl - cnt;
     for (int c = c0; c < c1; ++c)
-        if (mask[c]) list[1 + pos++] = c;
+        if (__ldcg(mask + c)) list[1 + pos++] = c;
     if (tid == nt - 1) list[0] = pos;
     __syncthreads();
 }
@@ -639,39 +639,121 @@ struct Ops {  // A~ (or A~^T) and M (or M^T) with values of type T
 };
 
 // ---------------------------------------------------------------- item kernels
-// An item is (system in list, row chunk of CHUNK rows) handled by one warp.
+// An item of the vector kernels is (system in list, chunk of NS * VROWS rows),
+// one block of VT threads with four rows per thread and piece of VROWS rows,
+// in two 16-byte (FP64) loads per vector. Items run system-major, so the
+// first systems' sums are finished while the others' items still stream. All
+// loads of a piece are issued before its arithmetic: one round trip to memory
+// however few items there are. NS is 1 below LONG_N rows, where the number of
+// items decides, and 4 above: there the FP64 pipe does (an FP64 instruction
+// of a warp takes 64 cycles of its scheduler's pipe), and one chunk's
+// reduction is spread over four times the rows.
+//
+// Inner products: a fixed tree per chunk (its partial), then the block that
+// stores a system's last partial sums them in a fixed order (thread t takes
+// chunks t, t + VT, ..) and runs that system's control step in the same
+// launch; the block that finishes the last system rebuilds the list. The
+// order depends on n alone, so a system gets the same bits whichever systems
+// run with it.
+constexpr int VT = 128;
+constexpr int VROWS = 4 * VT;
+constexpr int LONG_N = 16384;
+
 struct Items {
     int32_t n;
     int64_t ld;
-    int nch;   // CHUNK-row chunks per system
+    int ns;    // pieces of VROWS rows per chunk (the kernels' NS)
+    int nch;   // chunks per system
     int nchu;  // CHUNK_U-row chunks per system (GMRES update)
 };
 
-__host__ __device__ __forceinline__ int nchunks(int64_t n) { return (int)((n + CHUNK - 1) / CHUNK); }
-
-// threads of a single-block control kernel for k systems (it loops over them)
-inline int ctl_threads(int k) { return k <= CTRL ? CTRL : 1024; }
+inline int chunk_pieces(int64_t n) { return n < LONG_N ? 1 : 4; }
+inline int nchunks(int64_t n)
+{
+    const int rows = chunk_pieces(n) * VROWS;
+    return (int)((n + rows - 1) / rows);
+}
+// the instance of a vector kernel for I's chunk size
+#define VK(I, kernel) ((I).ns == 1 ? kernel<1> : kernel<4>)
+#define VKT(I, kernel, T) ((I).ns == 1 ? kernel<T, 1> : kernel<T, 4>)
 
 int item_blocks(int64_t n, int k)
 {
-    int64_t items = (int64_t)nchunks(n) * k;
-    int64_t b = (items + IT_WARPS - 1) / IT_WARPS;
-    const int64_t cap = (int64_t)g_sms * 8;
+    int64_t b = (int64_t)nchunks(n) * k;
+    const int64_t cap = (int64_t)g_sms * 16;
     if (b > cap) b = cap;
     if (b < 1) b = 1;
     return (int)b;
 }
 
-// Loops the calling warp over its items: c = system, q_ = chunk, [r0, r1) = rows.
-#define FOR_ITEMS(I, list, cvar, r0, r1)                                                              \
-    const int cnt_ = (list)[0];                                                                       \
-    const int lane_ = threadIdx.x & 31;                                                               \
-    const int64_t w0_ = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;                        \
-    const int64_t nw_ = ((int64_t)gridDim.x * blockDim.x) >> 5;                                       \
-    for (int64_t it_ = w0_; it_ < (int64_t)cnt_ * (I).nch; it_ += nw_)                                \
-        for (int cvar = (list)[1 + (int)(it_ % cnt_)], q_ = (int)(it_ / cnt_), once_ = 1; once_;      \
-             once_ = 0)                                                                               \
-            for (int64_t r0 = (int64_t)q_ * CHUNK, r1 = min((int64_t)(I).n, r0 + CHUNK); once_; once_ = 0)
+template <class T>
+struct Two;
+template <>
+struct Two<double> {
+    using type = double2;
+};
+template <>
+struct Two<float> {
+    using type = float2;
+};
+
+// The calling thread's four rows of the chunk at row r0: 2t, 2t + 1 and
+// 2 VT + 2t, 2 VT + 2t + 1 (rows past n read as zero and are not stored).
+template <class T>
+struct Row4 {
+    T v[4];
+    __device__ __forceinline__ void load(const T* __restrict__ p, int64_t r0, int64_t n)
+    {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int64_t r = r0 + 2 * VT * h + 2 * (int)threadIdx.x;
+            if (r + 1 < n) {
+                const typename Two<T>::type x = *reinterpret_cast<const typename Two<T>::type*>(p + r);
+                v[2 * h] = x.x;
+                v[2 * h + 1] = x.y;
+            } else {
+                v[2 * h] = r < n ? p[r] : T(0);
+                v[2 * h + 1] = T(0);
+            }
+        }
+    }
+    __device__ __forceinline__ void store(T* __restrict__ p, int64_t r0, int64_t n) const
+    {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int64_t r = r0 + 2 * VT * h + 2 * (int)threadIdx.x;
+            if (r + 1 < n) {
+                typename Two<T>::type x;
+                x.x = v[2 * h];
+                x.y = v[2 * h + 1];
+                *reinterpret_cast<typename Two<T>::type*>(p + r) = x;
+            } else if (r < n) {
+                p[r] = v[2 * h];
+            }
+        }
+    }
+};
+
+// acc + a^T b
+template <class T>
+__device__ __forceinline__ T dot4(const Row4<T>& a, const Row4<T>& b, T acc)
+{
+    return fma(a.v[3], b.v[3], fma(a.v[2], b.v[2], fma(a.v[1], b.v[1], fma(a.v[0], b.v[0], acc))));
+}
+
+// f(c, q, o, r0) for the calling block's items: system c, chunk q, the start
+// o of c's vector and the chunk's first row r0
+template <int NS, class F>
+__device__ __forceinline__ void for_items(const Items& I, const int* __restrict__ list, F f)
+{
+    const int cnt = list[0];
+    for (int64_t it = blockIdx.x; it < (int64_t)cnt * I.nch; it += gridDim.x) {
+        const int ci = (int)(it / I.nch);
+        const int q = (int)(it - (int64_t)ci * I.nch);
+        const int c = list[1 + ci];
+        f(c, q, (int64_t)c * I.ld, (int64_t)q * NS * VROWS);
+    }
+}
 
 // partial index of item (c, q), dot d: [d][c][q]
 __device__ __forceinline__ size_t pidx(int d, int c, int q, int k, int nch)
@@ -684,248 +766,392 @@ struct Sys {
     double *thr, *rho, *rho_old, *alpha, *omega, *beta, *hn;
     int *active, *iters, *status, *mode, *go;
     int *lact, *lgo, *lall;  // lists
+    int* acnt;               // k: items of a system whose partials are stored (zero between launches)
+    int* gcnt;               // systems finished in the running launch (zero between launches)
 };
 
-__device__ __forceinline__ double sum_chunks(const double* part, int d, int c, int k, int nch)
+// Sum of ND values over the block's VT threads in a fixed order, valid in
+// thread 0: warp d adds the threads' values of dot d from shared memory
+// (three additions and five shuffle levels for the block, against five levels
+// in each of its warps).
+template <int ND, class T>
+__device__ __forceinline__ void block_sums(T (&a)[ND], double (&s)[ND])
 {
-    double s = 0.0;
-    for (int q = 0; q < nch; ++q) s += part[pidx(d, c, q, k, nch)];
-    return s;
+    static_assert(VT == 128 && ND <= VT / 32, "a warp per dot, four values per lane");
+    __shared__ T sh[ND][VT];
+    __shared__ double out[ND];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) sh[d][threadIdx.x] = a[d];
+    __syncthreads();
+    if (wid < ND) {
+        const T* x = sh[wid];
+        const T w = warp_sum_t((x[lane] + x[lane + 32]) + (x[lane + 64] + x[lane + 96]));
+        if (lane == 0) out[wid] = (double)w;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int d = 0; d < ND; ++d) s[d] = threadIdx.x == 0 ? out[d] : 0.0;
+}
+
+// (h, l) += x in twice the working precision (Knuth's two-sum)
+__device__ __forceinline__ void two_add(double& h, double& l, double x)
+{
+    const double s = h + x, t = s - h;
+    l += (h - (s - t)) + (x - t);
+    h = s;
+}
+
+// The sums of a system's chunk partials, thread 0 of the block, as block_sums;
+// the dots of COMP (bit d) are added in twice the working precision. BiCGStab's
+// rhat^T r and rhat^T v shrink to the rounding of their partial sums when a
+// system stagnates; summed plainly they are multiples of that rounding and at
+// times exactly zero, which ends the system with a breakdown.
+template <int ND, int COMP>
+__device__ __forceinline__ void chunk_sums(const Items& I, int k, int c, const double* part, double (&s)[ND])
+{
+    __shared__ double hi[ND][VT], lo[ND][VT];
+    __shared__ double out[ND];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        const double* p = part + pidx(d, c, 0, k, I.nch);
+        double h = 0.0, l = 0.0;
+        for (int u = threadIdx.x; u < I.nch; u += VT) {
+            const double x = __ldcg(p + u);
+            if ((COMP >> d) & 1) two_add(h, l, x);
+            else h += x;
+        }
+        hi[d][threadIdx.x] = h;
+        lo[d][threadIdx.x] = l;
+    }
+    __syncthreads();
+    if (wid < ND) {
+        double h = hi[wid][lane], l = lo[wid][lane];
+        if ((COMP >> wid) & 1) {
+#pragma unroll 1
+            for (int u = 1; u < 4; ++u) {
+                two_add(h, l, hi[wid][lane + 32 * u]);
+                l += lo[wid][lane + 32 * u];
+            }
+#pragma unroll 1
+            for (int o = 16; o > 0; o >>= 1) {
+                const double h2 = __shfl_xor_sync(SAI_FULL, h, o), l2 = __shfl_xor_sync(SAI_FULL, l, o);
+                two_add(h, l, h2);
+                l += l2;
+            }
+            h += l;
+        } else {
+            h = warp_sum((h + hi[wid][lane + 32]) + (hi[wid][lane + 64] + hi[wid][lane + 96]));
+        }
+        if (lane == 0) out[wid] = h;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int d = 0; d < ND; ++d) s[d] = threadIdx.x == 0 ? out[d] : 0.0;
+}
+
+// Stores the item's partial sums a (one value per thread). True in the block
+// that stores the system's last ones, with the system's sums s in thread 0;
+// every other block's partials are visible there.
+template <int ND, class T, int COMP = 0>
+__device__ __forceinline__ bool item_sums(const Items& I, int k, int c, int q, T (&a)[ND], double (&s)[ND],
+                                          double* part, int* acnt)
+{
+    __shared__ int last;
+    block_sums<ND, T>(a, s);
+    if (I.nch == 1) {
+        __syncthreads();  // thread 0 has read the sums before the next item's are formed
+        return true;
+    }
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int d = 0; d < ND; ++d) part[pidx(d, c, q, k, I.nch)] = s[d];
+        __threadfence();
+        last = atomicAdd(&acnt[c], 1) == I.nch - 1;
+        if (last) {
+            __threadfence();
+            acnt[c] = 0;
+        }
+    }
+    __syncthreads();
+    const bool mine = last != 0;
+    if (mine) chunk_sums<ND, COMP>(I, k, c, part, s);
+    __syncthreads();  // `last` is read before the next item writes it
+    return mine;
+}
+
+// Called by a block that has finished a system (its control values written by
+// thread 0): the block that finishes the last of the launch's cnt systems
+// rebuilds list from mask. Returns true there.
+__device__ __forceinline__ bool systems_done(const Sys& S, int cnt, int k, const int* mask, int* list)
+{
+    __shared__ int glast;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        glast = atomicAdd(S.gcnt, 1) == cnt - 1;
+        if (glast) {
+            __threadfence();
+            *S.gcnt = 0;
+        }
+    }
+    __syncthreads();
+    const bool mine = glast != 0;
+    if (mine) build_list_block(k, mask, list);
+    __syncthreads();
+    return mine;
 }
 
 // ================================================================== BiCGStab
-__global__ void k_bicg_init(Items I, int k, const double* __restrict__ Bs, double* x, double* r, double* rh,
-                            double* p, double* v, const int* list, double* part)
+// One iteration of the listed systems is nine launches: p; M p; A~ phat;
+// rhat^T v with alpha; s with ||s||; M s; A~ shat; t^T s, t^T t with omega;
+// x, r, ||r||, rhat^T r with the stop test and the next beta. A system that
+// breaks down stays in the iteration's lists with active = 0 (its x and r are
+// not touched again) until the list is rebuilt.
+
+// the next iteration's start: count it, test rho, form beta
+__device__ __forceinline__ void bicg_next(const Sys& S, int c, int maxit)
 {
-    FOR_ITEMS(I, list, c, r0, r1)
-    {
-        double acc = 0.0;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            const double b = Bs[o + i];
-            x[o + i] = 0.0;
-            r[o + i] = b;
-            rh[o + i] = b;
-            p[o + i] = 0.0;
-            v[o + i] = 0.0;
-            acc = fma(b, b, acc);
-        }
-        acc = warp_sum(acc);
-        if (lane_ == 0) part[pidx(0, c, q_, k, I.nch)] = acc;
+    if (S.iters[c] >= maxit) {
+        S.active[c] = 0;
+        S.status[c] = ST_MAXITER;
+        return;
+    }
+    const int it = S.iters[c] + 1;
+    S.iters[c] = it;
+    if (S.rho[c] == 0.0) {
+        S.active[c] = 0;
+        S.status[c] = ST_BREAKDOWN;
+    } else {
+        S.beta[c] = it == 1 ? 0.0 : (S.rho[c] / S.rho_old[c]) * (S.alpha[c] / S.omega[c]);
     }
 }
 
-__global__ void k_bicg_f0(int k, int nch, const double* part, Sys S)
+// r = rhat = b, x = 0, ||b||; the first stop test and iteration start
+template <int NS>
+__global__ void __launch_bounds__(VT) k_bicg_init(Items I, int k, const double* __restrict__ Bs, double* __restrict__ x,
+                                                  double* __restrict__ r, double* __restrict__ rh, Sys S, double* part,
+                                                  int maxit)
 {
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        const double bb = sum_chunks(part, 0, c, k, nch);
-        S.iters[c] = 0;
-        S.rho[c] = bb;  // r^T rhat with r = rhat = b
-        S.alpha[c] = 1.0;
-        S.omega[c] = 1.0;
-        S.mode[c] = 1;
-        S.go[c] = 0;
-        if (sqrt(bb) < S.thr[c]) {
-            S.active[c] = 0;
-            S.status[c] = ST_OK;
-        } else {
-            S.active[c] = 1;
-            S.status[c] = ST_MAXITER;
+    for_items<NS>(I, S.lall, [&](int c, int q, int64_t o, int64_t r0) {
+        double a[1] = {0.0}, s[1];
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> b, z = {{0.0, 0.0, 0.0, 0.0}};
+            b.load(Bs + o, r0, I.n);
+            z.store(x + o, r0, I.n);
+            b.store(r + o, r0, I.n);
+            b.store(rh + o, r0, I.n);
+            a[0] = dot4(b, b, a[0]);
         }
-    }
-    __syncthreads();
-    build_list_block(k, S.active, S.lact);
+        if (item_sums<1, double>(I, k, c, q, a, s, part, S.acnt)) {
+            if (threadIdx.x == 0) {
+                const double bb = s[0];
+                S.iters[c] = 0;
+                S.rho[c] = bb;  // r^T rhat with r = rhat = b
+                S.alpha[c] = 1.0;
+                S.omega[c] = 1.0;
+                S.mode[c] = 1;
+                S.go[c] = 0;
+                if (sqrt(bb) < S.thr[c]) {
+                    S.active[c] = 0;
+                    S.status[c] = ST_OK;
+                } else {
+                    S.active[c] = 1;
+                    S.status[c] = ST_MAXITER;
+                    bicg_next(S, c, maxit);
+                }
+            }
+            systems_done(S, k, k, S.active, S.lact);
+        }
+    });
 }
 
-// iteration start: count it, test rho, form beta
-__global__ void k_bicg_start(int k, int maxit, Sys S)
+template <int NS>
+__global__ void __launch_bounds__(VT) k_bicg_p(Items I, const double* __restrict__ r, double* __restrict__ p,
+                                               const double* __restrict__ v, Sys S)
 {
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        if (!S.active[c]) continue;
-        if (S.iters[c] >= maxit) {
-            S.active[c] = 0;
-            S.status[c] = ST_MAXITER;
-        } else {
-            S.iters[c] += 1;
-            if (S.rho[c] == 0.0) {
+    for_items<NS>(I, S.lact, [&](int c, int, int64_t o, int64_t r0) {
+        const double be = S.beta[c], om = S.omega[c];
+        const bool first = S.iters[c] == 1;
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> rv;
+            rv.load(r + o, r0, I.n);
+            if (!first) {
+                Row4<double> pv, vv;
+                pv.load(p + o, r0, I.n);
+                vv.load(v + o, r0, I.n);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) rv.v[u] = fma(be, fma(-om, vv.v[u], pv.v[u]), rv.v[u]);
+            }
+            rv.store(p + o, r0, I.n);
+        }
+    });
+}
+
+// rhat^T v and alpha
+template <int NS>
+__global__ void __launch_bounds__(VT) k_bicg_alpha(Items I, int k, const double* __restrict__ rh,
+                                                   const double* __restrict__ v, Sys S, double* part, Dims D)
+{
+    const int cnt = S.lact[0];
+    if (blockIdx.x == 0 && threadIdx.x == 0 && cnt > 0) {
+        spmm_work(D, D.nnzM, cnt);
+        spmm_work(D, D.nnzA, cnt);
+        kwork_add(PROF_BICG_VEC, 8.0 * D.n * cnt * (4 + 2), D.n * cnt * (3 + 2));  // p update, rhat^T v
+    }
+    for_items<NS>(I, S.lact, [&](int c, int q, int64_t o, int64_t r0) {
+        double a[1] = {0.0}, s[1];
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> x, y;
+            x.load(rh + o, r0, I.n);
+            y.load(v + o, r0, I.n);
+            a[0] = dot4(x, y, a[0]);
+        }
+        if (item_sums<1, double, 1>(I, k, c, q, a, s, part, S.acnt) && threadIdx.x == 0) {
+            if (s[0] == 0.0) {
                 S.active[c] = 0;
                 S.status[c] = ST_BREAKDOWN;
             } else {
-                S.beta[c] = S.iters[c] == 1 ? 0.0 : (S.rho[c] / S.rho_old[c]) * (S.alpha[c] / S.omega[c]);
+                S.alpha[c] = S.rho[c] / s[0];
             }
         }
-    }
-    __syncthreads();
-    build_list_block(k, S.active, S.lact);
+    });
 }
 
-__global__ void k_bicg_p(Items I, const double* __restrict__ r, double* p, const double* __restrict__ v, Sys S)
+// s = r - alpha v and ||s||: a system whose ||s|| is below its threshold
+// takes the half step, the others go on (list lgo)
+template <int NS>
+__global__ void __launch_bounds__(VT) k_bicg_s(Items I, int k, const double* __restrict__ r,
+                                               const double* __restrict__ v, double* __restrict__ s, Sys S,
+                                               double* part, Dims D)
 {
-    FOR_ITEMS(I, S.lact, c, r0, r1)
-    {
-        const double be = S.beta[c], om = S.omega[c];
-        const bool first = S.iters[c] == 1;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32)
-            p[o + i] = first ? r[o + i] : r[o + i] + be * (p[o + i] - om * v[o + i]);
+    const int cnt = S.lact[0];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (cnt > 0) kwork_add(PROF_BICG_VEC, 8.0 * D.n * cnt * 3, D.n * cnt * 4.0);  // s, ||s||
+        else S.lgo[0] = 0;
     }
-}
-
-// ND inner products (a0,b0), (a1,b1) over the systems of list
-template <int ND>
-__global__ void k_dots(Items I, int k, const double* a0, const double* b0, const double* a1, const double* b1,
-                       const int* list, double* part)
-{
-    FOR_ITEMS(I, list, c, r0, r1)
-    {
-        double s0 = 0.0, s1 = 0.0;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            s0 = fma(a0[o + i], b0[o + i], s0);
-            if (ND > 1) s1 = fma(a1[o + i], b1[o + i], s1);
-        }
-        s0 = warp_sum(s0);
-        if (ND > 1) s1 = warp_sum(s1);
-        if (lane_ == 0) {
-            part[pidx(0, c, q_, k, I.nch)] = s0;
-            if (ND > 1) part[pidx(1, c, q_, k, I.nch)] = s1;
-        }
-    }
-}
-
-__global__ void k_bicg_f1(int k, int nch, const double* part, Sys S, Dims D)
-{
-    const int k1 = S.lact[0];
-    if (threadIdx.x == 0 && k1 > 0) {
-        spmm_work(D, D.nnzM, k1);
-        spmm_work(D, D.nnzA, k1);
-        kwork_add(PROF_BICG_VEC, 8.0 * D.n * k1 * (4 + 2), D.n * k1 * (3 + 2));  // p update, rhat^T v
-    }
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        if (!S.active[c]) continue;
-        const double rv = sum_chunks(part, 0, c, k, nch);
-        if (rv == 0.0) {
-            S.active[c] = 0;
-            S.status[c] = ST_BREAKDOWN;
-        } else {
-            S.alpha[c] = S.rho[c] / rv;
-        }
-    }
-    __syncthreads();
-    build_list_block(k, S.active, S.lact);
-}
-
-__global__ void k_bicg_s(Items I, int k, const double* __restrict__ r, const double* __restrict__ v, double* s,
-                         Sys S, double* part)
-{
-    FOR_ITEMS(I, S.lact, c, r0, r1)
-    {
+    for_items<NS>(I, S.lact, [&](int c, int q, int64_t o, int64_t r0) {
         const double al = S.alpha[c];
-        double acc = 0.0;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            const double sv = r[o + i] - al * v[o + i];
-            s[o + i] = sv;
-            acc = fma(sv, sv, acc);
+        double a[1] = {0.0}, ss[1];
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> x, y;
+            x.load(r + o, r0, I.n);
+            y.load(v + o, r0, I.n);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x.v[u] = fma(-al, y.v[u], x.v[u]);
+            x.store(s + o, r0, I.n);
+            a[0] = dot4(x, x, a[0]);
         }
-        acc = warp_sum(acc);
-        if (lane_ == 0) part[pidx(0, c, q_, k, I.nch)] = acc;
-    }
-}
-
-__global__ void k_bicg_f2(int k, int nch, const double* part, Sys S, Dims D)
-{
-    const int k2 = S.lact[0];
-    if (threadIdx.x == 0 && k2 > 0) kwork_add(PROF_BICG_VEC, 8.0 * D.n * k2 * 3, D.n * k2 * 4.0);  // s, ||s||
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        if (S.active[c]) {
-            const double ss = sum_chunks(part, 0, c, k, nch);
-            S.mode[c] = sqrt(ss) < S.thr[c] ? 2 : 1;
-            S.go[c] = S.mode[c] == 1;
-        } else {
-            S.go[c] = 0;
-        }
-    }
-    __syncthreads();
-    build_list_block(k, S.go, S.lgo);
-}
-
-__global__ void k_bicg_f3(int k, int nch, const double* part, Sys S, Dims D)
-{
-    const int k3 = S.lgo[0];
-    if (threadIdx.x == 0 && k3 > 0) {
-        spmm_work(D, D.nnzM, k3);
-        spmm_work(D, D.nnzA, k3);
-        kwork_add(PROF_BICG_VEC, 8.0 * D.n * k3 * 2, D.n * k3 * 4.0);  // t^T s, t^T t
-    }
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        if (!S.go[c]) continue;
-        const double ts = sum_chunks(part, 0, c, k, nch), tt = sum_chunks(part, 1, c, k, nch);
-        if (tt == 0.0) {
-            S.active[c] = 0;
-            S.go[c] = 0;
-            S.status[c] = ST_BREAKDOWN;
-        } else {
-            S.omega[c] = ts / tt;
-        }
-    }
-    __syncthreads();
-    build_list_block(k, S.active, S.lact);
-}
-
-__global__ void k_bicg_xr(Items I, int k, double* x, double* r, const double* __restrict__ rh,
-                          const double* __restrict__ ph, const double* __restrict__ sh, const double* __restrict__ s,
-                          const double* __restrict__ t, Sys S, double* part)
-{
-    FOR_ITEMS(I, S.lact, c, r0, r1)
-    {
-        const double al = S.alpha[c], om = S.omega[c];
-        const bool half = S.mode[c] == 2;
-        double a0 = 0.0, a1 = 0.0;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            double rv;
-            if (half) {
-                x[o + i] += al * ph[o + i];
-                rv = s[o + i];
-            } else {
-                x[o + i] += al * ph[o + i] + om * sh[o + i];
-                rv = s[o + i] - om * t[o + i];
+        if (item_sums<1, double>(I, k, c, q, a, ss, part, S.acnt)) {
+            if (threadIdx.x == 0) {
+                const int mode = sqrt(ss[0]) < S.thr[c] ? 2 : 1;
+                S.mode[c] = mode;
+                S.go[c] = S.active[c] && mode == 1;
             }
-            r[o + i] = rv;
-            a0 = fma(rv, rv, a0);
-            a1 = fma(rh[o + i], rv, a1);
+            systems_done(S, cnt, k, S.go, S.lgo);
         }
-        a0 = warp_sum(a0);
-        a1 = warp_sum(a1);
-        if (lane_ == 0) {
-            part[pidx(0, c, q_, k, I.nch)] = a0;
-            part[pidx(1, c, q_, k, I.nch)] = a1;
-        }
-    }
+    });
 }
 
-__global__ void k_bicg_f4(int k, int nch, const double* part, Sys S, Dims D, int* any_active)
+// t^T s, t^T t and omega
+template <int NS>
+__global__ void __launch_bounds__(VT) k_bicg_omega(Items I, int k, const double* __restrict__ t,
+                                                   const double* __restrict__ s, Sys S, double* part, Dims D)
 {
-    const int k4 = S.lact[0];
-    if (threadIdx.x == 0 && k4 > 0) kwork_add(PROF_BICG_VEC, 8.0 * D.n * k4 * 8, D.n * k4 * 10.0);  // x, r, two dots
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        if (!S.active[c]) continue;
-        const double rr = sum_chunks(part, 0, c, k, nch), rhr = sum_chunks(part, 1, c, k, nch);
-        if (S.mode[c] == 2 || sqrt(rr) < S.thr[c]) {
-            S.active[c] = 0;
-            S.status[c] = ST_OK;
-        } else if (S.omega[c] == 0.0) {
-            S.active[c] = 0;
-            S.status[c] = ST_BREAKDOWN;
-        } else {
-            S.rho_old[c] = S.rho[c];
-            S.rho[c] = rhr;
-        }
+    const int cnt = S.lgo[0];
+    if (blockIdx.x == 0 && threadIdx.x == 0 && cnt > 0) {
+        spmm_work(D, D.nnzM, cnt);
+        spmm_work(D, D.nnzA, cnt);
+        kwork_add(PROF_BICG_VEC, 8.0 * D.n * cnt * 2, D.n * cnt * 4.0);  // t^T s, t^T t
     }
-    __syncthreads();
-    build_list_block(k, S.active, S.lact);
-    if (threadIdx.x == 0) *any_active = S.lact[0] > 0;
+    for_items<NS>(I, S.lgo, [&](int c, int q, int64_t o, int64_t r0) {
+        double a[2] = {0.0, 0.0}, d[2];
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> x, y;
+            x.load(t + o, r0, I.n);
+            y.load(s + o, r0, I.n);
+            a[0] = dot4(x, y, a[0]);
+            a[1] = dot4(x, x, a[1]);
+        }
+        if (item_sums<2, double>(I, k, c, q, a, d, part, S.acnt) && threadIdx.x == 0) {
+            if (d[1] == 0.0) {
+                S.active[c] = 0;
+                S.status[c] = ST_BREAKDOWN;
+            } else {
+                S.omega[c] = d[0] / d[1];
+            }
+        }
+    });
+}
+
+// x += alpha phat + omega shat, r = s - omega t (the half step: x += alpha
+// phat, r = s), ||r|| and rhat^T r; the stop test and the next iteration's start
+template <int NS>
+__global__ void __launch_bounds__(VT) k_bicg_xr(Items I, int k, double* __restrict__ x, double* __restrict__ r,
+                                                const double* __restrict__ rh, const double* __restrict__ ph,
+                                                const double* __restrict__ sh, const double* __restrict__ s,
+                                                const double* __restrict__ t, Sys S, double* part, Dims D, int maxit,
+                                                int* any_active)
+{
+    const int cnt = S.lact[0];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (cnt > 0) kwork_add(PROF_BICG_VEC, 8.0 * D.n * cnt * 8, D.n * cnt * 10.0);  // x, r, two dots
+        else *any_active = 0;
+    }
+    for_items<NS>(I, S.lact, [&](int c, int q, int64_t o, int64_t r0) {
+        double a[2] = {0.0, 0.0}, d[2];
+        if (S.active[c]) {
+            const double al = S.alpha[c], om = S.omega[c];
+            const bool half = S.mode[c] == 2;
+#pragma unroll
+            for (int e = 0; e < NS; ++e, r0 += VROWS) {
+                Row4<double> xv, pv, rv, hv;
+                xv.load(x + o, r0, I.n);
+                pv.load(ph + o, r0, I.n);
+                rv.load(s + o, r0, I.n);
+                hv.load(rh + o, r0, I.n);
+                if (half) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) xv.v[u] = fma(al, pv.v[u], xv.v[u]);
+                } else {
+                    Row4<double> sv, tv;
+                    sv.load(sh + o, r0, I.n);
+                    tv.load(t + o, r0, I.n);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        xv.v[u] = fma(om, sv.v[u], fma(al, pv.v[u], xv.v[u]));
+                        rv.v[u] = fma(-om, tv.v[u], rv.v[u]);
+                    }
+                }
+                xv.store(x + o, r0, I.n);
+                rv.store(r + o, r0, I.n);
+                a[0] = dot4(rv, rv, a[0]);
+                a[1] = dot4(hv, rv, a[1]);
+            }
+        }
+        if (item_sums<2, double, 2>(I, k, c, q, a, d, part, S.acnt)) {
+            if (threadIdx.x == 0) S.go[c] = 0;  // out of lgo until its next half step
+            if (threadIdx.x == 0 && S.active[c]) {
+                if (S.mode[c] == 2 || sqrt(d[0]) < S.thr[c]) {
+                    S.active[c] = 0;
+                    S.status[c] = ST_OK;
+                } else if (S.omega[c] == 0.0) {
+                    S.active[c] = 0;
+                    S.status[c] = ST_BREAKDOWN;
+                } else {
+                    S.rho_old[c] = S.rho[c];
+                    S.rho[c] = d[1];
+                    bicg_next(S, c, maxit);
+                }
+            }
+            if (systems_done(S, cnt, k, S.active, S.lact) && threadIdx.x == 0) *any_active = S.lact[0] > 0;
+        }
+    });
 }
 
 
@@ -1058,13 +1284,10 @@ sai_status bicgstab_run(const Items& I, int k, const Ops<double>& A, const doubl
     const int64_t ld = I.ld;
     const size_t blk = (size_t)ld * k;
     const int ib = item_blocks(n > 0 ? n : 1, k);
-    const int nch = I.nch;
     const int check_every = 4;
-    const int ct = ctl_threads(k);
     int hflag = 0;
     Buf vecs;
     SAI_TRY(vecs.alloc(sizeof(double) * blk * 8 + 8, st, true));
-    SAI_CUDA(cudaMemsetAsync(vecs.p, 0, sizeof(double) * blk * 8, st));
     double* r = vecs.as<double>();
     double* rh = r + blk;
     double* p = rh + blk;
@@ -1083,61 +1306,46 @@ sai_status bicgstab_run(const Items& I, int k, const Ops<double>& A, const doubl
         P1 = pbuf.as<double>();
         P2 = P1 + pe;
     }
-    k_bicg_init<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, Bsd, Xsd, r, rh, p, v, S.lall, pt);
-    k_bicg_f0<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S);
+    auto apply2 = [&](const double* X, double* Y1, double* Y2, const int* list) {  // Y1 = M X, Y2 = A~ Y1
+        if (pnl) {
+            ProfScope ps(PROF_SPMM, st);
+            pnl_apply2(n, ld, k, A, X, Y1, Y2, list, P1, P2, st);
+        } else {
+            {
+                ProfScope ps(PROF_SPMM, st);
+                spmv<double, 0>(n, ld, A.M, k, X, Y1, nullptr, list, st);
+            }
+            {
+                ProfScope ps(PROF_SPMM, st);
+                spmv<double, 0>(n, ld, A.A, k, Y1, Y2, nullptr, list, st);
+            }
+        }
+    };
+    VK(I, k_bicg_init)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Bsd, Xsd, r, rh, S, pt, maxit);
     SAI_CUDA(cudaGetLastError());
     for (int it = 0; it < maxit; ++it) {
-        k_bicg_start<<<SAI_GRID(1), ct, 0, st>>>(k, maxit, S);
         {
             ProfScope ps(PROF_BICG_VEC, st);
-            k_bicg_p<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, r, p, v, S);
+            VK(I, k_bicg_p)<<<SAI_GRID(ib), VT, 0, st>>>(I, r, p, v, S);
         }
-        if (pnl) {
-            ProfScope ps(PROF_SPMM, st);
-            pnl_apply2(n, ld, k, A, p, ph, v, S.lact, P1, P2, st);
-        } else {
-            {
-                ProfScope ps(PROF_SPMM, st);
-                spmv<double, 0>(n, ld, A.M, k, p, ph, nullptr, S.lact, st);
-            }
-            {
-                ProfScope ps(PROF_SPMM, st);
-                spmv<double, 0>(n, ld, A.A, k, ph, v, nullptr, S.lact, st);
-            }
+        apply2(p, ph, v, S.lact);
+        {
+            ProfScope ps(PROF_BICG_VEC, st);
+            VK(I, k_bicg_alpha)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, rh, v, S, pt, D);
         }
         {
             ProfScope ps(PROF_BICG_VEC, st);
-            k_dots<1><<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, rh, v, nullptr, nullptr, S.lact, pt);
+            VK(I, k_bicg_s)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, r, v, s, S, pt, D);
         }
-        k_bicg_f1<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S, D);
+        apply2(s, sh, t, S.lgo);
         {
             ProfScope ps(PROF_BICG_VEC, st);
-            k_bicg_s<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, r, v, s, S, pt);
-        }
-        k_bicg_f2<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S, D);
-        if (pnl) {
-            ProfScope ps(PROF_SPMM, st);
-            pnl_apply2(n, ld, k, A, s, sh, t, S.lgo, P1, P2, st);
-        } else {
-            {
-                ProfScope ps(PROF_SPMM, st);
-                spmv<double, 0>(n, ld, A.M, k, s, sh, nullptr, S.lgo, st);
-            }
-            {
-                ProfScope ps(PROF_SPMM, st);
-                spmv<double, 0>(n, ld, A.A, k, sh, t, nullptr, S.lgo, st);
-            }
+            VK(I, k_bicg_omega)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, t, s, S, pt, D);
         }
         {
             ProfScope ps(PROF_BICG_VEC, st);
-            k_dots<2><<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, t, s, t, t, S.lgo, pt);
+            VK(I, k_bicg_xr)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Xsd, r, rh, ph, sh, s, t, S, pt, D, maxit, fl);
         }
-        k_bicg_f3<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S, D);
-        {
-            ProfScope ps(PROF_BICG_VEC, st);
-            k_bicg_xr<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, Xsd, r, rh, ph, sh, s, t, S, pt);
-        }
-        k_bicg_f4<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S, D, fl);
         SAI_CUDA(cudaGetLastError());
         if ((it + 1) % check_every == 0 || it + 1 == maxit) {
             SAI_CUDA(cudaMemcpyAsync(&hflag, fl, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1145,9 +1353,6 @@ sai_status bicgstab_run(const Items& I, int k, const Ops<double>& A, const doubl
             if (!hflag) break;
         }
     }
-    // systems still active after maxit passes
-    k_bicg_start<<<SAI_GRID(1), ct, 0, st>>>(k, maxit, S);
-    SAI_CUDA(cudaGetLastError());
     return SAI_OK;
 }
 
@@ -1160,148 +1365,166 @@ sai_status bicgstab_run(const Items& I, int k, const Ops<double>& A, const doubl
 //   alpha = rho / rhat^T v;  q = u - alpha v;  w = M (u + q);  y += alpha w;
 //   r -= alpha A~ w
 // and the recursive residual is tested after the iteration.
-__global__ void k_cgs_init(Items I, int k, const double* __restrict__ Bs, double* x, double* r, double* rh,
-                           double* q, double* p, const int* list, double* part)
-{
-    FOR_ITEMS(I, list, c, r0, r1)
-    {
-        double acc = 0.0;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            const double b = Bs[o + i];
-            x[o + i] = 0.0;
-            r[o + i] = b;
-            rh[o + i] = b;
-            q[o + i] = 0.0;
-            p[o + i] = 0.0;
-            acc = fma(b, b, acc);
-        }
-        acc = warp_sum(acc);
-        if (lane_ == 0) part[pidx(0, c, q_, k, I.nch)] = acc;
-    }
-}
-
 // iteration start: count it, test rho, form beta
-__global__ void k_cgs_start(int k, int maxit, Sys S)
+__device__ __forceinline__ void cgs_next(const Sys& S, int c, int maxit)
 {
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        if (!S.active[c]) continue;
-        if (S.iters[c] >= maxit) {
-            S.active[c] = 0;
-            S.status[c] = ST_MAXITER;
-        } else {
-            S.iters[c] += 1;
-            if (S.rho[c] == 0.0) {
-                S.active[c] = 0;
-                S.status[c] = ST_BREAKDOWN;
-            } else {
-                S.beta[c] = S.iters[c] == 1 ? 0.0 : S.rho[c] / S.rho_old[c];
-            }
-        }
+    if (S.iters[c] >= maxit) {
+        S.active[c] = 0;
+        S.status[c] = ST_MAXITER;
+        return;
     }
-    __syncthreads();
-    build_list_block(k, S.active, S.lact);
+    S.iters[c] += 1;
+    if (S.rho[c] == 0.0) {
+        S.active[c] = 0;
+        S.status[c] = ST_BREAKDOWN;
+    } else {
+        S.beta[c] = S.rho[c] / S.rho_old[c];
+    }
 }
 
-__global__ void k_cgs_up(Items I, const double* __restrict__ r, double* u, double* p, const double* __restrict__ q,
-                         Sys S)
+template <int NS>
+__global__ void __launch_bounds__(VT) k_cgs_up(Items I, const double* __restrict__ r, double* __restrict__ u,
+                                               double* __restrict__ p, const double* __restrict__ q, Sys S)
 {
-    FOR_ITEMS(I, S.lact, c, r0, r1)
-    {
+    for_items<NS>(I, S.lact, [&](int c, int, int64_t o, int64_t r0) {
         const double be = S.beta[c];
         const bool first = S.iters[c] == 1;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            const double uv = first ? r[o + i] : r[o + i] + be * q[o + i];
-            u[o + i] = uv;
-            p[o + i] = first ? uv : uv + be * (q[o + i] + be * p[o + i]);
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> uv;
+            uv.load(r + o, r0, I.n);
+            Row4<double> pn = uv;
+            if (!first) {
+                Row4<double> qv, pv;
+                qv.load(q + o, r0, I.n);
+                pv.load(p + o, r0, I.n);
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    uv.v[w] = fma(be, qv.v[w], uv.v[w]);
+                    pn.v[w] = fma(be, fma(be, pv.v[w], qv.v[w]), uv.v[w]);
+                }
+            }
+            uv.store(u + o, r0, I.n);
+            pn.store(p + o, r0, I.n);
         }
-    }
+    });
 }
 
-__global__ void k_cgs_f1(int k, int nch, const double* part, Sys S, Dims D)
+// a^T b and alpha = rho / a^T b (rhat^T v of CGS, ps^T q of BiCG)
+template <int NS>
+__global__ void __launch_bounds__(VT) k_cgs_alpha(Items I, int k, const double* __restrict__ a,
+                                                  const double* __restrict__ b, Sys S, double* part, Dims D)
 {
-    const int k1 = S.lact[0];
-    if (threadIdx.x == 0 && k1 > 0) {
-        spmm_work(D, D.nnzM, k1);
-        spmm_work(D, D.nnzA, k1);
-        kwork_add(PROF_BICG_VEC, 8.0 * D.n * k1 * (5 + 2), D.n * k1 * (6 + 2));  // u, p updates, rhat^T v
+    const int cnt = S.lact[0];
+    if (blockIdx.x == 0 && threadIdx.x == 0 && cnt > 0) {
+        spmm_work(D, D.nnzM, cnt);
+        spmm_work(D, D.nnzA, cnt);
+        kwork_add(PROF_BICG_VEC, 8.0 * D.n * cnt * (5 + 2), D.n * cnt * (6 + 2));  // u, p updates, rhat^T v
     }
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        if (!S.active[c]) continue;
-        const double sg = sum_chunks(part, 0, c, k, nch);
-        if (sg == 0.0) {
-            S.active[c] = 0;
-            S.status[c] = ST_BREAKDOWN;
-        } else {
-            S.alpha[c] = S.rho[c] / sg;
+    for_items<NS>(I, S.lact, [&](int c, int q, int64_t o, int64_t r0) {
+        double d[1] = {0.0}, s[1];
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> x, y;
+            x.load(a + o, r0, I.n);
+            y.load(b + o, r0, I.n);
+            d[0] = dot4(x, y, d[0]);
         }
-    }
-    __syncthreads();
-    build_list_block(k, S.active, S.lact);
+        if (item_sums<1, double, 1>(I, k, c, q, d, s, part, S.acnt)) {
+            if (threadIdx.x == 0) {
+                if (s[0] == 0.0) {
+                    S.active[c] = 0;
+                    S.status[c] = ST_BREAKDOWN;
+                } else {
+                    S.alpha[c] = S.rho[c] / s[0];
+                }
+            }
+            // the rest of the iteration leaves broken-down systems out
+            systems_done(S, cnt, k, S.active, S.lact);
+        }
+    });
 }
 
-__global__ void k_cgs_q(Items I, const double* __restrict__ u, const double* __restrict__ v, double* q, double* w,
-                        Sys S)
+template <int NS>
+__global__ void __launch_bounds__(VT) k_cgs_q(Items I, const double* __restrict__ u, const double* __restrict__ v,
+                                              double* __restrict__ q, double* __restrict__ w, Sys S)
 {
-    FOR_ITEMS(I, S.lact, c, r0, r1)
-    {
+    for_items<NS>(I, S.lact, [&](int c, int, int64_t o, int64_t r0) {
         const double al = S.alpha[c];
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            const double qv = u[o + i] - al * v[o + i];
-            q[o + i] = qv;
-            w[o + i] = u[o + i] + qv;
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> uv, vv;
+            uv.load(u + o, r0, I.n);
+            vv.load(v + o, r0, I.n);
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                vv.v[h] = fma(-al, vv.v[h], uv.v[h]);
+                uv.v[h] += vv.v[h];
+            }
+            vv.store(q + o, r0, I.n);
+            uv.store(w + o, r0, I.n);
         }
+    });
+}
+
+// the end of a CGS or BiCG iteration for system c: stop test on rr, the next
+// iteration's start with rho = rho_new
+__device__ __forceinline__ void cgs_finish(const Sys& S, int c, double rr, double rho_new, int maxit)
+{
+    if (sqrt(rr) < S.thr[c]) {
+        S.active[c] = 0;
+        S.status[c] = ST_OK;
+    } else {
+        S.rho_old[c] = S.rho[c];
+        S.rho[c] = rho_new;
+        cgs_next(S, c, maxit);
     }
 }
 
-__global__ void k_cgs_xr(Items I, int k, double* x, double* r, const double* __restrict__ rh,
-                         const double* __restrict__ wh, const double* __restrict__ qh, Sys S, double* part)
+__device__ __forceinline__ void cgs_work(const Dims& D, int cnt)
 {
-    FOR_ITEMS(I, S.lact, c, r0, r1)
-    {
+    spmm_work(D, D.nnzM, cnt);
+    spmm_work(D, D.nnzA, cnt);
+    kwork_add(PROF_BICG_VEC, 8.0 * D.n * cnt * (4 + 6), D.n * cnt * (3 + 8));  // q, w; x, r, two dots
+}
+
+template <int NS>
+__global__ void __launch_bounds__(VT) k_cgs_xr(Items I, int k, double* __restrict__ x, double* __restrict__ r,
+                                               const double* __restrict__ rh, const double* __restrict__ wh,
+                                               const double* __restrict__ qh, Sys S, double* part, Dims D, int maxit,
+                                               int* any_active)
+{
+    const int cnt = S.lact[0];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (cnt > 0) cgs_work(D, cnt);
+        else *any_active = 0;
+    }
+    for_items<NS>(I, S.lact, [&](int c, int q, int64_t o, int64_t r0) {
         const double al = S.alpha[c];
-        double a0 = 0.0, a1 = 0.0;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            x[o + i] += al * wh[o + i];
-            const double rv = r[o + i] - al * qh[o + i];
-            r[o + i] = rv;
-            a0 = fma(rv, rv, a0);
-            a1 = fma(rh[o + i], rv, a1);
+        double a[2] = {0.0, 0.0}, d[2];
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> xv, wv, rv, qv, hv;
+            xv.load(x + o, r0, I.n);
+            wv.load(wh + o, r0, I.n);
+            rv.load(r + o, r0, I.n);
+            qv.load(qh + o, r0, I.n);
+            hv.load(rh + o, r0, I.n);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                xv.v[u] = fma(al, wv.v[u], xv.v[u]);
+                rv.v[u] = fma(-al, qv.v[u], rv.v[u]);
+            }
+            xv.store(x + o, r0, I.n);
+            rv.store(r + o, r0, I.n);
+            a[0] = dot4(rv, rv, a[0]);
+            a[1] = dot4(hv, rv, a[1]);
         }
-        a0 = warp_sum(a0);
-        a1 = warp_sum(a1);
-        if (lane_ == 0) {
-            part[pidx(0, c, q_, k, I.nch)] = a0;
-            part[pidx(1, c, q_, k, I.nch)] = a1;
+        if (item_sums<2, double, 2>(I, k, c, q, a, d, part, S.acnt)) {
+            if (threadIdx.x == 0) cgs_finish(S, c, d[0], d[1], maxit);
+            if (systems_done(S, cnt, k, S.active, S.lact) && threadIdx.x == 0) *any_active = S.lact[0] > 0;
         }
-    }
-}
-
-__global__ void k_cgs_f2(int k, int nch, const double* part, Sys S, Dims D, int* any_active)
-{
-    const int k2 = S.lact[0];
-    if (threadIdx.x == 0 && k2 > 0) {
-        spmm_work(D, D.nnzM, k2);
-        spmm_work(D, D.nnzA, k2);
-        kwork_add(PROF_BICG_VEC, 8.0 * D.n * k2 * (4 + 6), D.n * k2 * (3 + 8));  // q, w; x, r, two dots
-    }
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        if (!S.active[c]) continue;
-        const double rr = sum_chunks(part, 0, c, k, nch), rhr = sum_chunks(part, 1, c, k, nch);
-        if (sqrt(rr) < S.thr[c]) {
-            S.active[c] = 0;
-            S.status[c] = ST_OK;
-        } else {
-            S.rho_old[c] = S.rho[c];
-            S.rho[c] = rhr;
-        }
-    }
-    __syncthreads();
-    build_list_block(k, S.active, S.lact);
-    if (threadIdx.x == 0) *any_active = S.lact[0] > 0;
+    });
 }
 
 sai_status cgs_run(const Items& I, int k, const Ops<double>& A, const double* Bsd, double* Xsd, Sys& S, double* pt,
@@ -1311,13 +1534,10 @@ sai_status cgs_run(const Items& I, int k, const Ops<double>& A, const double* Bs
     const int64_t ld = I.ld;
     const size_t blk = (size_t)ld * k;
     const int ib = item_blocks(n > 0 ? n : 1, k);
-    const int nch = I.nch;
     const int check_every = 4;
-    const int ct = ctl_threads(k);
     int hflag = 0;
     Buf vecs;
     SAI_TRY(vecs.alloc(sizeof(double) * blk * 9 + 8, st, true));
-    SAI_CUDA(cudaMemsetAsync(vecs.p, 0, sizeof(double) * blk * 9, st));
     double* r = vecs.as<double>();
     double* rh = r + blk;
     double* u = rh + blk;
@@ -1352,31 +1572,27 @@ sai_status cgs_run(const Items& I, int k, const Ops<double>& A, const double* Bs
             }
         }
     };
-    k_cgs_init<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, Bsd, Xsd, r, rh, q, p, S.lall, pt);
-    k_bicg_f0<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S);  // rho = b^T b, the first test on ||b||
+    VK(I, k_bicg_init)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Bsd, Xsd, r, rh, S, pt, maxit);  // rho = b^T b, the test on ||b||
     SAI_CUDA(cudaGetLastError());
     for (int it = 0; it < maxit; ++it) {
-        k_cgs_start<<<SAI_GRID(1), ct, 0, st>>>(k, maxit, S);
         {
             ProfScope ps(PROF_BICG_VEC, st);
-            k_cgs_up<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, r, u, p, q, S);
+            VK(I, k_cgs_up)<<<SAI_GRID(ib), VT, 0, st>>>(I, r, u, p, q, S);
         }
         apply2(p, ph, v);
         {
             ProfScope ps(PROF_BICG_VEC, st);
-            k_dots<1><<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, rh, v, nullptr, nullptr, S.lact, pt);
+            VK(I, k_cgs_alpha)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, rh, v, S, pt, D);
         }
-        k_cgs_f1<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S, D);
         {
             ProfScope ps(PROF_BICG_VEC, st);
-            k_cgs_q<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, u, v, q, w, S);
+            VK(I, k_cgs_q)<<<SAI_GRID(ib), VT, 0, st>>>(I, u, v, q, w, S);
         }
         apply2(w, wh, qh);
         {
             ProfScope ps(PROF_BICG_VEC, st);
-            k_cgs_xr<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, Xsd, r, rh, wh, qh, S, pt);
+            VK(I, k_cgs_xr)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Xsd, r, rh, wh, qh, S, pt, D, maxit, fl);
         }
-        k_cgs_f2<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S, D, fl);
         SAI_CUDA(cudaGetLastError());
         if ((it + 1) % check_every == 0 || it + 1 == maxit) {
             SAI_CUDA(cudaMemcpyAsync(&hflag, fl, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1384,8 +1600,6 @@ sai_status cgs_run(const Items& I, int k, const Ops<double>& A, const double* Bs
             if (!hflag) break;
         }
     }
-    k_cgs_start<<<SAI_GRID(1), ct, 0, st>>>(k, maxit, S);  // systems still active after maxit
-    SAI_CUDA(cudaGetLastError());
     return SAI_OK;
 }
 
@@ -1398,64 +1612,74 @@ sai_status cgs_run(const Items& I, int k, const Ops<double>& A, const double* Bs
 //   p = r, ps = rs first);  z = M p;  q = A~ z;  qs = K^T ps;
 //   alpha = rho / ps^T q;  y += alpha z;  r -= alpha q;  rs -= alpha qs
 // with the control kernels of CGS (same recurrences for rho, beta, alpha).
-__global__ void k_bicg2_init(Items I, int k, const double* __restrict__ Bs, double* x, double* r, double* rs,
-                             const int* list, double* part)
+template <int NS>
+__global__ void __launch_bounds__(VT) k_bicg2_up(Items I, const double* __restrict__ r, const double* __restrict__ rs,
+                                                 double* __restrict__ p, double* __restrict__ ps, Sys S)
 {
-    FOR_ITEMS(I, list, c, r0, r1)
-    {
-        double acc = 0.0;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            const double b = Bs[o + i];
-            x[o + i] = 0.0;
-            r[o + i] = b;
-            rs[o + i] = b;
-            acc = fma(b, b, acc);
-        }
-        acc = warp_sum(acc);
-        if (lane_ == 0) part[pidx(0, c, q_, k, I.nch)] = acc;
-    }
-}
-
-__global__ void k_bicg2_up(Items I, const double* __restrict__ r, const double* __restrict__ rs, double* p,
-                           double* ps, Sys S)
-{
-    FOR_ITEMS(I, S.lact, c, r0, r1)
-    {
+    for_items<NS>(I, S.lact, [&](int c, int, int64_t o, int64_t r0) {
         const double be = S.beta[c];
         const bool first = S.iters[c] == 1;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            p[o + i] = first ? r[o + i] : r[o + i] + be * p[o + i];
-            ps[o + i] = first ? rs[o + i] : rs[o + i] + be * ps[o + i];
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> rv, sv;
+            rv.load(r + o, r0, I.n);
+            sv.load(rs + o, r0, I.n);
+            if (!first) {
+                Row4<double> pv, qv;
+                pv.load(p + o, r0, I.n);
+                qv.load(ps + o, r0, I.n);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    rv.v[u] = fma(be, pv.v[u], rv.v[u]);
+                    sv.v[u] = fma(be, qv.v[u], sv.v[u]);
+                }
+            }
+            rv.store(p + o, r0, I.n);
+            sv.store(ps + o, r0, I.n);
         }
-    }
+    });
 }
 
-__global__ void k_bicg2_xr(Items I, int k, double* x, double* r, double* rs, const double* __restrict__ z,
-                           const double* __restrict__ q, const double* __restrict__ qs, Sys S, double* part)
+template <int NS>
+__global__ void __launch_bounds__(VT) k_bicg2_xr(Items I, int k, double* __restrict__ x, double* __restrict__ r,
+                                                 double* __restrict__ rs, const double* __restrict__ z,
+                                                 const double* __restrict__ q, const double* __restrict__ qs, Sys S,
+                                                 double* part, Dims D, int maxit, int* any_active)
 {
-    FOR_ITEMS(I, S.lact, c, r0, r1)
-    {
-        const double al = S.alpha[c];
-        double a0 = 0.0, a1 = 0.0;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            x[o + i] += al * z[o + i];
-            const double rv = r[o + i] - al * q[o + i];
-            const double sv = rs[o + i] - al * qs[o + i];
-            r[o + i] = rv;
-            rs[o + i] = sv;
-            a0 = fma(rv, rv, a0);
-            a1 = fma(sv, rv, a1);
-        }
-        a0 = warp_sum(a0);
-        a1 = warp_sum(a1);
-        if (lane_ == 0) {
-            part[pidx(0, c, q_, k, I.nch)] = a0;
-            part[pidx(1, c, q_, k, I.nch)] = a1;
-        }
+    const int cnt = S.lact[0];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (cnt > 0) cgs_work(D, cnt);
+        else *any_active = 0;
     }
+    for_items<NS>(I, S.lact, [&](int c, int ch, int64_t o, int64_t r0) {
+        const double al = S.alpha[c];
+        double a[2] = {0.0, 0.0}, d[2];
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> xv, zv, rv, qv, sv, tv;
+            xv.load(x + o, r0, I.n);
+            zv.load(z + o, r0, I.n);
+            rv.load(r + o, r0, I.n);
+            qv.load(q + o, r0, I.n);
+            sv.load(rs + o, r0, I.n);
+            tv.load(qs + o, r0, I.n);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                xv.v[u] = fma(al, zv.v[u], xv.v[u]);
+                rv.v[u] = fma(-al, qv.v[u], rv.v[u]);
+                sv.v[u] = fma(-al, tv.v[u], sv.v[u]);
+            }
+            xv.store(x + o, r0, I.n);
+            rv.store(r + o, r0, I.n);
+            sv.store(rs + o, r0, I.n);
+            a[0] = dot4(rv, rv, a[0]);
+            a[1] = dot4(sv, rv, a[1]);
+        }
+        if (item_sums<2, double, 2>(I, k, c, ch, a, d, part, S.acnt)) {
+            if (threadIdx.x == 0) cgs_finish(S, c, d[0], d[1], maxit);
+            if (systems_done(S, cnt, k, S.active, S.lact) && threadIdx.x == 0) *any_active = S.lact[0] > 0;
+        }
+    });
 }
 
 // A: the pair of K (M applied first, then A~); T: the pair of K^T (A~^T first, then M^T)
@@ -1466,13 +1690,10 @@ sai_status bicg_run(const Items& I, int k, const Ops<double>& A, const Ops<doubl
     const int64_t ld = I.ld;
     const size_t blk = (size_t)ld * k;
     const int ib = item_blocks(n > 0 ? n : 1, k);
-    const int nch = I.nch;
     const int check_every = 4;
-    const int ct = ctl_threads(k);
     int hflag = 0;
     Buf vecs;
     SAI_TRY(vecs.alloc(sizeof(double) * blk * 8 + 8, st, true));
-    SAI_CUDA(cudaMemsetAsync(vecs.p, 0, sizeof(double) * blk * 8, st));
     double* r = vecs.as<double>();
     double* rs = r + blk;
     double* p = rs + blk;
@@ -1505,27 +1726,23 @@ sai_status bicg_run(const Items& I, int k, const Ops<double>& A, const Ops<doubl
             }
         }
     };
-    k_bicg2_init<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, Bsd, Xsd, r, rs, S.lall, pt);
-    k_bicg_f0<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S);  // rho = b^T b, the first test on ||b||
+    VK(I, k_bicg_init)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Bsd, Xsd, r, rs, S, pt, maxit);  // rho = b^T b, the test on ||b||
     SAI_CUDA(cudaGetLastError());
     for (int it = 0; it < maxit; ++it) {
-        k_cgs_start<<<SAI_GRID(1), ct, 0, st>>>(k, maxit, S);
         {
             ProfScope ps_(PROF_BICG_VEC, st);
-            k_bicg2_up<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, r, rs, p, ps, S);
+            VK(I, k_bicg2_up)<<<SAI_GRID(ib), VT, 0, st>>>(I, r, rs, p, ps, S);
         }
         apply2(A, p, z, q);
         apply2(T, ps, zs, qs);
         {
             ProfScope ps_(PROF_BICG_VEC, st);
-            k_dots<1><<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, ps, q, nullptr, nullptr, S.lact, pt);
+            VK(I, k_cgs_alpha)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, ps, q, S, pt, D);
         }
-        k_cgs_f1<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S, D);
         {
             ProfScope ps_(PROF_BICG_VEC, st);
-            k_bicg2_xr<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, Xsd, r, rs, z, q, qs, S, pt);
+            VK(I, k_bicg2_xr)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Xsd, r, rs, z, q, qs, S, pt, D, maxit, fl);
         }
-        k_cgs_f2<<<SAI_GRID(1), ct, 0, st>>>(k, nch, pt, S, D, fl);
         SAI_CUDA(cudaGetLastError());
         if ((it + 1) % check_every == 0 || it + 1 == maxit) {
             SAI_CUDA(cudaMemcpyAsync(&hflag, fl, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1533,8 +1750,6 @@ sai_status bicg_run(const Items& I, int k, const Ops<double>& A, const Ops<doubl
             if (!hflag) break;
         }
     }
-    k_cgs_start<<<SAI_GRID(1), ct, 0, st>>>(k, maxit, S);  // systems still active after maxit
-    SAI_CUDA(cudaGetLastError());
     return SAI_OK;
 }
 
@@ -1617,40 +1832,47 @@ struct Vec<float> {
     __device__ static float4 scale(float s, const float4& a) { return make_float4(s * a.x, s * a.y, s * a.z, s * a.w); }
 };
 
-template <class T>
-__global__ void k_gm_init(Items I, int k, const T* __restrict__ Bs, T* x, T* r, const int* list, double* part)
+// x = 0, r = b and ||b||^2 of every system into nrm2
+template <class T, int NS>
+__global__ void __launch_bounds__(VT) k_gm_init(Items I, int k, const T* __restrict__ Bs, T* __restrict__ x,
+                                                T* __restrict__ r, const int* list, double* part, int* acnt,
+                                                double* __restrict__ nrm2)
 {
-    FOR_ITEMS(I, list, c, r0, r1)
-    {
-        T acc = 0;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) {
-            const T b = Bs[o + i];
-            x[o + i] = 0;
-            r[o + i] = b;
-            acc = fma(b, b, acc);
+    for_items<NS>(I, list, [&](int c, int q, int64_t o, int64_t r0) {
+        T a[1] = {T(0)};
+        double s[1];
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<T> b, z = {{T(0), T(0), T(0), T(0)}};
+            b.load(Bs + o, r0, I.n);
+            z.store(x + o, r0, I.n);
+            b.store(r + o, r0, I.n);
+            a[0] = dot4(b, b, a[0]);
         }
-        acc = warp_sum_t(acc);
-        if (lane_ == 0) part[pidx(0, c, q_, k, I.nch)] = (double)acc;
-    }
+        if (item_sums<1, T>(I, k, c, q, a, s, part, acnt) && threadIdx.x == 0) nrm2[c] = s[0];
+    });
 }
 
-template <class T>
-__global__ void k_norm2(Items I, int k, const T* __restrict__ r, const int* list, double* part)
+// ||r||^2 of the listed systems into nrm2
+template <class T, int NS>
+__global__ void __launch_bounds__(VT) k_norm2(Items I, int k, const T* __restrict__ r, const int* list, double* part,
+                                              int* acnt, double* __restrict__ nrm2)
 {
-    FOR_ITEMS(I, list, c, r0, r1)
-    {
-        T acc = 0;
-        const int64_t o = (int64_t)c * I.ld;
-        for (int64_t i = r0 + lane_; i < r1; i += 32) acc = fma(r[o + i], r[o + i], acc);
-        acc = warp_sum_t(acc);
-        if (lane_ == 0) part[pidx(0, c, q_, k, I.nch)] = (double)acc;
-    }
+    for_items<NS>(I, list, [&](int c, int q, int64_t o, int64_t r0) {
+        T a[1] = {T(0)};
+        double s[1];
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<T> x;
+            x.load(r + o, r0, I.n);
+            a[0] = dot4(x, x, a[0]);
+        }
+        if (item_sums<1, T>(I, k, c, q, a, s, part, acnt) && threadIdx.x == 0) nrm2[c] = s[0];
+    });
 }
 
 // cycle start: true residual norm, stop tests, g = beta e_1
-__global__ void k_gm_cycle_start(int k, int nch, const double* part, const int* cap, Sys S, Gm G, int first,
-                                 int* any_cyc)
+__global__ void k_gm_cycle_start(int k, const double* nrm2, const int* cap, Sys S, Gm G, int first, int* any_cyc)
 {
     const int c = threadIdx.x;
     if (c < k) {
@@ -1664,7 +1886,7 @@ __global__ void k_gm_cycle_start(int k, int nch, const double* part, const int* 
         G.conv[c] = 0;
         G.jd[c] = 0;
         if (!G.done[c]) {
-            const double beta = sqrt(sum_chunks(part, 0, c, k, nch));
+            const double beta = sqrt(nrm2[c]);
             if (beta < S.thr[c]) {
                 G.done[c] = 1;
                 S.status[c] = ST_OK;
@@ -1723,7 +1945,7 @@ __global__ void k_gm_cycle_start(int k, int nch, const double* part, const int* 
 // shared memory. (Streaming each thread's row vectors through a two-stage
 // cp.async buffer in shared memory instead of registers measured slower:
 // 21.5 against 18.9 ms of the 64^3 step.)
-constexpr int DC_CHUNK = 2 * CHUNK;  // rows per item of the fused dot kernel (one partial per item)
+constexpr int DC_CHUNK = 2048;  // rows per item of the fused dot kernel (one partial per item)
 inline int dc_chunks(int64_t n) { return (int)((n + DC_CHUNK - 1) / DC_CHUNK); }
 
 template <class T>
@@ -2527,13 +2749,13 @@ __global__ void k_cast_f32(int64_t n, const double* __restrict__ a, float* __res
 // beta_c < thr_c (the FP64 stopping test) or when its inner iterations
 // reach maxit; otherwise sets the inner tolerance on the normalised residual
 // thr_in_c = max(tau, 0.3 thr_c / beta_c) and the inner iteration cap.
-__global__ void k_ir_check(int k, int nch, const double* part, const double* thr, double tau, int maxit,
+__global__ void k_ir_check(int k, const double* nrm2, const double* thr, double tau, int maxit,
                            const int* tot, int* done, int* status, double* beta, double* thr_in, int* cap,
                            int* lir, int* any)
 {
     const int c = threadIdx.x;
     if (c < k && !done[c]) {
-        const double b = sqrt(sum_chunks(part, 0, c, k, nch));
+        const double b = sqrt(nrm2[c]);
         beta[c] = b;
         if (b < thr[c]) {
             done[c] = 1;
@@ -2561,27 +2783,42 @@ __global__ void k_ir_check(int k, int nch, const double* part, const double* thr
 }
 
 // r32 = r64 / beta for the refined systems, 0 for the others
-__global__ void k_ir_scale(Items I, int k, const double* __restrict__ r64, const double* beta, const int* done,
-                           float* __restrict__ r32, const int* lall)
+template <int NS>
+__global__ void __launch_bounds__(VT) k_ir_scale(Items I, const double* __restrict__ r64, const double* beta,
+                                                 const int* done, float* __restrict__ r32, const int* lall)
 {
-    FOR_ITEMS(I, lall, c, r0, r1)
-    {
-        const int64_t o = (int64_t)c * I.ld;
+    for_items<NS>(I, lall, [&](int c, int, int64_t o, int64_t r0) {
         const double s = done[c] ? 0.0 : 1.0 / beta[c];
-        for (int64_t i = r0 + lane_; i < r1; i += 32) r32[o + i] = (float)(r64[o + i] * s);
-    }
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> a;
+            Row4<float> b;
+            a.load(r64 + o, r0, I.n);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) b.v[u] = (float)(a.v[u] * s);
+            b.store(r32 + o, r0, I.n);
+        }
+    });
 }
 
 // x64 += beta * d32 for the refined systems; tot += inner iterations
-__global__ void k_ir_update(Items I, double* __restrict__ x64, const float* __restrict__ d32, const double* beta,
-                            const int* lir)
+template <int NS>
+__global__ void __launch_bounds__(VT) k_ir_update(Items I, double* __restrict__ x64, const float* __restrict__ d32,
+                                                  const double* beta, const int* lir)
 {
-    FOR_ITEMS(I, lir, c, r0, r1)
-    {
-        const int64_t o = (int64_t)c * I.ld;
+    for_items<NS>(I, lir, [&](int c, int, int64_t o, int64_t r0) {
         const double b = beta[c];
-        for (int64_t i = r0 + lane_; i < r1; i += 32) x64[o + i] = fma(b, (double)d32[o + i], x64[o + i]);
-    }
+#pragma unroll
+        for (int e = 0; e < NS; ++e, r0 += VROWS) {
+            Row4<double> x;
+            Row4<float> d;
+            x.load(x64 + o, r0, I.n);
+            d.load(d32 + o, r0, I.n);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x.v[u] = fma(b, (double)d.v[u], x.v[u]);
+            x.store(x64 + o, r0, I.n);
+        }
+    });
 }
 
 __global__ void k_ir_total(int k, const int* lir, const int* it_in, int* tot)
@@ -2725,11 +2962,11 @@ sai_status gmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs,
             sai_count_grid_add(-(long long)GM_STEPS_PER_CHECK * GM_LAUNCHES_PER_STEP);
         }
     }
-    k_gm_init<T><<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, Bs, Xs, r, S.lall, pt2);
+    VKT(I, k_gm_init, T)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Bs, Xs, r, S.lall, pt2, S.acnt, S.hn);
     int first = 1;
     sai_status status = SAI_OK;
     for (;;) {
-        k_gm_cycle_start<<<SAI_GRID(1), CTRL, 0, st>>>(k, I.nch, pt2, cap, S, G, first, fl);
+        k_gm_cycle_start<<<SAI_GRID(1), CTRL, 0, st>>>(k, S.hn, cap, S, G, first, fl);
         first = 0;
         SAI_CUDA(cudaMemcpyAsync(&hflag, fl, sizeof(int), cudaMemcpyDeviceToHost, st));
         SAI_CUDA(cudaStreamSynchronize(st));
@@ -2758,7 +2995,7 @@ sai_status gmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs,
         spmv<T, 2>(n, ld, A.M, k, w, Xs, nullptr, G.lcyc, st);  // x += M V y
         k_gm_cycle_end<<<SAI_GRID(1), CTRL, 0, st>>>(k, cap, S, G, fl);
         spmv<T, 1>(n, ld, A.A, k, Xs, r, Bs, G.lcyc, st);
-        k_norm2<T><<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, r, G.lcyc, pt2);
+        VKT(I, k_norm2, T)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, r, G.lcyc, pt2, S.acnt, S.hn);
         SAI_CUDA(cudaGetLastError());
     }
     if (gexec) cudaGraphExecDestroy(gexec);
@@ -3217,8 +3454,7 @@ __global__ void __launch_bounds__(32 * BG_KMAX) k_bg_backsolve(int nt, Bg<T> B)
 // cycle start: true residual norms (partials of the listed systems), stop
 // tests, the active list and its identity list; flags[2] = kb
 template <class T>
-__global__ void k_bg_cycle(int k, int nch, const double* part, const int* __restrict__ cap, int first, Sys S,
-                           Bg<T> B)
+__global__ void k_bg_cycle(int k, const double* nrm2, const int* __restrict__ cap, int first, Sys S, Bg<T> B)
 {
     __shared__ int act[CTRL];
     for (int c = threadIdx.x; c < k; c += blockDim.x) {
@@ -3229,7 +3465,7 @@ __global__ void k_bg_cycle(int k, int nch, const double* part, const int* __rest
         }
         act[c] = 0;
         if (S.active[c]) {
-            const double r = sqrt(sum_chunks(part, 0, c, k, nch));
+            const double r = sqrt(nrm2[c]);
             if (r < S.thr[c]) {
                 S.active[c] = 0;
                 S.status[c] = ST_OK;
@@ -3358,11 +3594,11 @@ sai_status bgmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs
     const int64_t ld = I.ld;
     const int ib = item_blocks(n > 0 ? n : 1, k);
     const unsigned gg = bg_rows_grid(n) * 4;
-    k_gm_init<T><<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, Bs, Xs, R, S.lall, pt2);
+    VKT(I, k_gm_init, T)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Bs, Xs, R, S.lall, pt2, S.acnt, S.hn);
     SAI_CUDA(cudaMemsetAsync(B.flags, 0, sizeof(int) * 4, st));
     int h[3] = {0, 0, 0};
     for (int first = 1;; first = 0) {
-        k_bg_cycle<T><<<SAI_GRID(1), CTRL, 0, st>>>(k, I.nch, pt2, cap, first, S, B);
+        k_bg_cycle<T><<<SAI_GRID(1), CTRL, 0, st>>>(k, S.hn, cap, first, S, B);
         SAI_CUDA(cudaMemcpyAsync(h, B.flags, sizeof(int) * 3, cudaMemcpyDeviceToHost, st));
         SAI_CUDA(cudaStreamSynchronize(st));
         const int kb = h[2];
@@ -3430,7 +3666,7 @@ sai_status bgmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs
         spmv<T, 0>(n, ld, A.M, kb, B.Z, B.T1, nullptr, B.lid, st);
         k_bg_scatter_add<T><<<SAI_GRID(gg), 256, 0, st>>>(n, ld, B.lact, B.T1, Xs);
         spmv<T, 1>(n, ld, A.A, k, Xs, R, Bs, B.lact, st);
-        k_norm2<T><<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, R, B.lact, pt2);
+        VKT(I, k_norm2, T)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, R, B.lact, pt2, S.acnt, S.hn);
         SAI_CUDA(cudaGetLastError());
     }
     return SAI_OK;
@@ -3537,6 +3773,7 @@ sai_status sai_krylov_run(const sai_split_s* h, const sai_precond_s* P, int32_t 
     Items I;
     I.n = n;
     I.ld = ld;
+    I.ns = chunk_pieces(n);
     I.nch = nchunks(n > 0 ? n : 1);
     I.nchu = (int)(((int64_t)(n > 0 ? n : 1) + CHUNK_U - 1) / CHUNK_U);
     const int ib = item_blocks(n > 0 ? n : 1, k);
@@ -3565,9 +3802,10 @@ sai_status sai_krylov_run(const sai_split_s* h, const sai_precond_s* P, int32_t 
 
     Buf sysd, sysi, part, part2, flag, Bs, Xs, capb;
     SAI_TRY(sysd.alloc(sizeof(double) * 7 * k, st, true));
-    SAI_TRY(sysi.alloc(sizeof(int) * (5 * k + 3 * (k + 1)), st, true));
-    const int nslot = prm->method != SAI_GMRES ? 2 : (PS > 2 ? PS : 2);  // partial sums per (system, chunk)
-    SAI_TRY(part.alloc(sizeof(double) * (size_t)k * I.nch * nslot, st, true));
+    SAI_TRY(sysi.alloc(sizeof(int) * (6 * k + 3 * (k + 1) + 1), st, true));
+    // partial sums per (system, chunk): two dots of the vector kernels, PS slots of the GMRES projection
+    const size_t np = prm->method == SAI_GMRES ? (size_t)k * dc_chunks(n > 0 ? n : 1) * PS : (size_t)k * I.nch * 2;
+    SAI_TRY(part.alloc(sizeof(double) * np, st, true));
     SAI_TRY(part2.alloc(sizeof(double) * (size_t)k * I.nch * 2, st, true));
     SAI_TRY(flag.alloc(sizeof(int) * 4, st, true));
     SAI_TRY(Bs.alloc(sizeof(double) * blk + 8, st, true));
@@ -3591,10 +3829,15 @@ sai_status sai_krylov_run(const sai_split_s* h, const sai_precond_s* P, int32_t 
     S.lact = ii + 5 * k;
     S.lgo = S.lact + (k + 1);
     S.lall = S.lgo + (k + 1);
+    S.acnt = S.lall + (k + 1);
+    S.gcnt = S.acnt + k;
     SAI_CUDA(cudaMemcpyAsync(S.thr, thr, sizeof(double) * k, cudaMemcpyHostToDevice, st));
-    SAI_CUDA(cudaMemsetAsync(ii, 0, sizeof(int) * (5 * k + 3 * (k + 1)), st));
-    SAI_CUDA(cudaMemsetAsync(Bs.p, 0, sizeof(double) * blk, st));
-    SAI_CUDA(cudaMemsetAsync(Xs.p, 0, sizeof(double) * blk, st));
+    SAI_CUDA(cudaMemsetAsync(ii, 0, sizeof(int) * (6 * k + 3 * (k + 1) + 1), st));
+    if (prm->method == SAI_GMRES || prm->method == SAI_BGMRES) {
+        // their kernels read whole 16-byte vectors past n: the padding rows are zero
+        SAI_CUDA(cudaMemsetAsync(Bs.p, 0, sizeof(double) * blk, st));
+        SAI_CUDA(cudaMemsetAsync(Xs.p, 0, sizeof(double) * blk, st));
+    }
     int* fl = flag.as<int>();
     int hflag = 0;
     Dims D;
@@ -3715,23 +3958,23 @@ sai_status sai_krylov_run(const sai_split_s* h, const sai_precond_s* P, int32_t 
         D32.site_dots = PROF_GM_DOTS32;
         D32.site_upd = PROF_GM_UPDATE32;
         // r64 = B, x64 = 0 and ||B||^2 partials
-        k_gm_init<double><<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, Bsd, Xsd, r64, S.lall, pt2);
+        VKT(I, k_gm_init, double)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Bsd, Xsd, r64, S.lall, pt2, S.acnt, S.hn);
         const int max_outer = 40;
         for (int outer = 0; outer < max_outer; ++outer) {
-            k_ir_check<<<SAI_GRID(1), CTRL, 0, st>>>(k, I.nch, pt2, thr64, tau, prm->maxit, tot, done, status64, beta,
+            k_ir_check<<<SAI_GRID(1), CTRL, 0, st>>>(k, S.hn, thr64, tau, prm->maxit, tot, done, status64, beta,
                                                      thr_in, cap, lir, fl);
             SAI_CUDA(cudaMemcpyAsync(&hflag, fl, sizeof(int), cudaMemcpyDeviceToHost, st));
             SAI_CUDA(cudaStreamSynchronize(st));
             if (!hflag) break;
-            k_ir_scale<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, r64, beta, done, r32, S.lall);
+            VK(I, k_ir_scale)<<<SAI_GRID(ib), VT, 0, st>>>(I, r64, beta, done, r32, S.lall);
             if (prm->method == SAI_BGMRES)
                 SAI_TRY(bgmres_run<float>(I, k, prm->restart, A32, r32, d32, Bgm.R, Bgm, S, cap, pt2, D32, st));
             else
                 SAI_TRY(gmres_run<float>(I, k, prm->restart, A32, r32, d32, Wk, S, G, cap, pt, pt2, fl, D32, st));
-            k_ir_update<<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, Xsd, d32, beta, lir);
+            VK(I, k_ir_update)<<<SAI_GRID(ib), VT, 0, st>>>(I, Xsd, d32, beta, lir);
             k_ir_total<<<SAI_GRID(1), 32, 0, st>>>(k, lir, S.iters, tot);
             spmv<double, 1>(n, ld, A64.A, k, Xsd, r64, Bsd, lir, st);
-            k_norm2<double><<<SAI_GRID(ib), IT_WARPS * 32, 0, st>>>(I, k, r64, lir, pt2);
+            VKT(I, k_norm2, double)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, r64, lir, pt2, S.acnt, S.hn);
             SAI_CUDA(cudaGetLastError());
         }
         // report the outer status and the total inner iterations
