@@ -1800,6 +1800,7 @@ struct Vec<double> {
     using type = double2;
     static constexpr int W = 2;
     __device__ static double dot(const double2& a, const double2& b) { return fma(a.x, b.x, a.y * b.y); }
+    __device__ static double dot(const double2& a, const double2& b, double c) { return fma(a.x, b.x, fma(a.y, b.y, c)); }
     __device__ static double2 axpy(double a, const double2& x, const double2& y)
     {
         return make_double2(fma(a, x.x, y.x), fma(a, x.y, y.y));
@@ -1819,6 +1820,10 @@ struct Vec<float> {
     __device__ static float dot(const float4& a, const float4& b)
     {
         return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, a.w * b.w)));
+    }
+    __device__ static float dot(const float4& a, const float4& b, float c)
+    {
+        return fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, c))));
     }
     __device__ static float4 axpy(float a, const float4& x, const float4& y)
     {
@@ -3109,24 +3114,27 @@ sai_status gm_work_alloc(size_t blk, int m, Buf& vb, Buf& wb, GmWork<T>& Wk, cud
 // modified Gram-Schmidt and Householder QR.
 
 constexpr int BG_KMAX = 32;  // largest block (systems per block)
-constexpr int BG_CR = 1024;  // rows per chunk of the Gram kernel
-constexpr int BG_GV = 8;     // basis vectors per Gram block (one per warp)
-constexpr int BG_UT = 256;   // threads (rows) per block of the update kernels
-constexpr int BG_HB = 64;    // rows of H staged at a time by the update kernel
+constexpr int BG_CR = 512;   // rows per chunk of the Gram kernel
+constexpr int BG_GV = 8;     // warps per Gram block
+constexpr int BG_UT = 128;   // threads (rows) per block of the triangular solve
+constexpr int BG_UR = 64;    // rows per block of the update kernel
+constexpr int BG_UP = 4;     // its parts: each takes a quarter of the basis vectors
+constexpr int BG_HB = 16;    // rows of H staged at a time and part
+constexpr int BG_LT = 256;   // threads of the least-squares kernel
 
 template <class T>
 struct Bg {
     T *V, *T1, *Z, *R;      // basis ((m+1)*k vectors of ld), work blocks and residuals of k vectors (type T)
     double *Hb;             // Hbar, column-major, ldh = (m+1)*k rows, m*k columns
-    double *hv, *hbeta;     // reflector of column q: hv[q*(k+1) + l], l = 0..kb; its beta
+    double *Q;              // block step i's reflections as one 2 kb x 2 kb matrix, column-major, (2k)^2 apart
+    double *Wn;             // the newest block column's last 2 kb rows, column a at a*2k
     double *G;              // (m+1)*k x k, column-major (ldh)
     double *Ys;             // the cycle's solution coefficients, m*k x k, column-major (ld m*k)
     double *Rt, *Rp;        // k x k column-major: R of the QR (product of passes), one pass's R
-    double *Gm;             // k x k Gram matrix of one QR pass
     double *H1, *H2;        // the two Gram-Schmidt passes' coefficients, nv x kb (ld nv)
     double *part;           // Gram partials [chunk][b][c]
     int *lact, *lid;        // active systems (count + ids); identity list (count + 0..kb-1)
-    int *flags;             // [0] every column converged, [1] error, [2] kb
+    int *flags;             // [0] every column converged, [1] error, [2] kb, [3] arrivals of k_bg_lsq's blocks
     int m, k;
     int64_t ldh;
 };
@@ -3138,43 +3146,71 @@ __host__ __device__ constexpr int bg_vb(int esz, int KB)
     return esz == 4 ? (KB <= 12 ? 4 : (KB <= 16 ? 2 : 1)) : (KB <= 8 ? 2 : 1);
 }
 
+// Sums a[0..31] over the warp: lane l gets the sum of a[l] (31 shuffles, each
+// round halving the values a lane still carries).
+template <class T>
+__device__ __forceinline__ T warp_sum32(T (&a)[32])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < o; ++i) {
+            const T keep = up ? a[i + o] : a[i], send = up ? a[i] : a[i + o];
+            a[i] = keep + __shfl_xor_sync(SAI_FULL, send, o);
+        }
+    }
+    return a[0];
+}
+
+// Gram partials of one chunk of BG_CR rows: a warp per VB basis vectors with
+// VB x KB accumulators, each lane on its own rows in 16-byte pieces (the
+// padding rows of every vector are zero). A chunk is four rounds in FP32:
+// short chunks give the grid enough warps where n is small (27000 rows, 275
+// vectors on average: 53 x 9 blocks; 16 us, chunks of 1024 rows read by scalars 40 us).
 template <class T, int KB>
 __global__ void __launch_bounds__(BG_GV * 32)
 k_bg_gram(int32_t n, int64_t ld, const T* __restrict__ V, int nv, const T* __restrict__ W, int kb,
           double* __restrict__ part)
 {
+    using VT_ = typename Vec<T>::type;
+    constexpr int VW = Vec<T>::W;
     constexpr int VB = bg_vb(sizeof(T), KB);
+    constexpr int NG = (VB * KB + 31) / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b0 = (blockIdx.y * BG_GV + warp) * VB;
     if (b0 >= nv) return;
     const int64_t r0 = (int64_t)blockIdx.x * BG_CR;
     const int64_t r1 = r0 + BG_CR < n ? r0 + BG_CR : n;
-    T acc[VB][KB];
+    T acc[NG][32];
 #pragma unroll
-    for (int u = 0; u < VB; ++u)
+    for (int g = 0; g < NG; ++g)
 #pragma unroll
-        for (int c = 0; c < KB; ++c) acc[u][c] = 0;
-    for (int64_t r = r0 + lane; r < r1; r += 32) {
-        T w[KB];
-#pragma unroll
-        for (int c = 0; c < KB; ++c) w[c] = c < kb ? W[(int64_t)c * ld + r] : T(0);
+        for (int c = 0; c < 32; ++c) acc[g][c] = 0;
+    for (int64_t r = r0 + lane * VW; r < r1; r += 32 * VW) {
+        VT_ x[VB];
 #pragma unroll
         for (int u = 0; u < VB; ++u)
-            if (b0 + u < nv) {
-                const T x = V[(int64_t)(b0 + u) * ld + r];
+            x[u] = b0 + u < nv ? *reinterpret_cast<const VT_*>(V + (int64_t)(b0 + u) * ld + r) : Vec<T>::zero();
 #pragma unroll
-                for (int c = 0; c < KB; ++c) acc[u][c] = fma(x, w[c], acc[u][c]);
+        for (int c = 0; c < KB; ++c)
+            if (c < kb) {
+                const VT_ w = *reinterpret_cast<const VT_*>(W + (int64_t)c * ld + r);
+#pragma unroll
+                for (int u = 0; u < VB; ++u) {
+                    const int i = u * KB + c;
+                    acc[i / 32][i % 32] = Vec<T>::dot(x[u], w, acc[i / 32][i % 32]);
+                }
             }
     }
 #pragma unroll
-    for (int u = 0; u < VB; ++u)
-        if (b0 + u < nv)
-#pragma unroll
-            for (int c = 0; c < KB; ++c)
-                if (c < kb) {
-                    const T sum = warp_sum_t(acc[u][c]);
-                    if (lane == 0) part[((int64_t)blockIdx.x * nv + b0 + u) * kb + c] = (double)sum;
-                }
+    for (int g = 0; g < NG; ++g) {
+        const T sum = warp_sum32(acc[g]);
+        const int i = 32 * g + lane, u = i / KB, c = i % KB;
+        if (u < VB && b0 + u < nv && c < kb)
+            part[((int64_t)blockIdx.x * nv + b0 + u) * kb + c] = (double)sum;
+    }
 }
 
 // H[c*nv + b] = the sum over chunks of part[q][b][c]: a warp per (b, c), lane
@@ -3191,91 +3227,135 @@ __global__ void k_bg_reduce(int nch, int nv, int kb, const double* __restrict__ 
     if (lane == 0) H[(int64_t)c * nv + b] = s;
 }
 
-// W -= V H (overwrite = 0) or W = V H (overwrite = 1); H: nv x kb, ld ldhh
+// W -= V H (overwrite = 0) or W = V H (overwrite = 1); H: nv x kb, ld ldhh.
+// A block takes BG_UR rows; its BG_UP parts each sum a quarter of the basis
+// vectors (eight loads in flight per thread), then add up in a fixed order:
+// four times the warps of a thread per row, which the row count alone cannot
+// give (27000 rows, 275 vectors on average: 23 us, 40 us with one part).
 template <class T, int KB>
-__global__ void __launch_bounds__(BG_UT)
+__global__ void __launch_bounds__(BG_UR * BG_UP)
 k_bg_update(int32_t n, int64_t ld, const T* __restrict__ V, int nv, const double* __restrict__ H, int ldhh,
             int kb, T* __restrict__ W, int overwrite)
 {
-    __shared__ T hs[BG_HB * KB];
-    const T sgn = overwrite ? T(1) : T(-1);
-    for (int64_t base = (int64_t)blockIdx.x * BG_UT; base < n; base += (int64_t)gridDim.x * BG_UT) {
-        const int64_t r = base + threadIdx.x;
+    __shared__ T hs[BG_UP][BG_HB * KB];
+    __shared__ T sums[BG_UR][KB + 1];
+    const int row = threadIdx.x % BG_UR, part = threadIdx.x / BG_UR;
+    const int per = (nv + BG_UP - 1) / BG_UP;  // basis vectors per part
+    const int v0 = part * per, v1 = v0 + per < nv ? v0 + per : nv;
+    for (int64_t base = (int64_t)blockIdx.x * BG_UR; base < n; base += (int64_t)gridDim.x * BG_UR) {
+        const int64_t r = base + row;
         const bool ok = r < n;
         T acc[KB];
 #pragma unroll
-        for (int c = 0; c < KB; ++c) acc[c] = (!overwrite && ok && c < kb) ? W[(int64_t)c * ld + r] : T(0);
-        for (int b0 = 0; b0 < nv; b0 += BG_HB) {
-            const int bl = nv - b0 < BG_HB ? nv - b0 : BG_HB;
+        for (int c = 0; c < KB; ++c) acc[c] = 0;
+        for (int q0 = 0; q0 < per; q0 += BG_HB) {
             __syncthreads();
-            for (int e = threadIdx.x; e < bl * KB; e += BG_UT) {
-                const int t = e / KB, c = e % KB;
-                hs[e] = c < kb ? (T)H[(int64_t)c * ldhh + b0 + t] : T(0);
+            for (int e = threadIdx.x; e < BG_UP * BG_HB * KB; e += BG_UR * BG_UP) {
+                const int p = e / (BG_HB * KB), t = e / KB % BG_HB, c = e % KB;
+                const int b = p * per + q0 + t;
+                hs[p][t * KB + c] = (c < kb && q0 + t < per && b < nv) ? (T)H[(int64_t)c * ldhh + b] : T(0);
             }
             __syncthreads();
-            if (ok)
-                for (int t = 0; t < bl; ++t) {
-                    const T x = sgn * V[(int64_t)(b0 + t) * ld + r];
 #pragma unroll
-                    for (int c = 0; c < KB; ++c) acc[c] = fma(x, hs[t * KB + c], acc[c]);
+            for (int t0 = 0; t0 < BG_HB; t0 += 8) {
+                T x[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    const int b = v0 + q0 + t0 + t;
+                    x[t] = ok && b < v1 ? V[(int64_t)b * ld + r] : T(0);
                 }
+#pragma unroll
+                for (int t = 0; t < 8; ++t)
+#pragma unroll
+                    for (int c = 0; c < KB; ++c) acc[c] = fma(x[t], hs[part][(t0 + t) * KB + c], acc[c]);
+            }
         }
-        if (ok)
+        for (int p = BG_UP - 1; p > 0; --p) {
+            if (part == p)
+#pragma unroll
+                for (int c = 0; c < KB; ++c) sums[row][c] = p == BG_UP - 1 ? acc[c] : acc[c] + sums[row][c];
+            __syncthreads();
+        }
+        if (part == 0 && ok)
 #pragma unroll
             for (int c = 0; c < KB; ++c)
-                if (c < kb) W[(int64_t)c * ld + r] = acc[c];
+                if (c < kb) {
+                    const T v = acc[c] + sums[row][c];
+                    T* w = W + (int64_t)c * ld + r;
+                    *w = overwrite ? v : *w - v;
+                }
     }
 }
 
 // one QR pass's Cholesky factor: Gm (+ shift on the first pass) = Rp^T Rp,
 // Rt = Rp Rt (Rt = Rp on the first pass); a pivot <= 0 sets flags[1]
-__global__ void __launch_bounds__(1024) k_bg_chol(int kb, double leff, double unit, const double* __restrict__ Gm,
-                                                  double* Rp, double* Rt, int first, int* flags)
+__global__ void __launch_bounds__(1024) k_bg_chol(int kb, int nch, double leff, double unit,
+                                                  const double* __restrict__ part, double* Rp, double* Rt, int first,
+                                                  int* flags)
 {
     __shared__ double a[BG_KMAX][BG_KMAX + 1];
     __shared__ double rt[BG_KMAX][BG_KMAX + 1];
     __shared__ double sh;
-    const int t = threadIdx.x;
-    const int i = t / BG_KMAX, q = t % BG_KMAX;
-    if (i < kb && q < kb) a[i][q] = Gm[q * kb + i];
+    const int t = threadIdx.x, lane = t & 31;
+    // the thread's entry (i, q), i <= q, of the triangle, row after row: as few
+    // warps as hold it, since each forms the pivots' square roots on the FP64 pipe
+    int i = 0, q = t;
+    while (i < kb && q >= kb - i) q -= kb - i++;
+    const bool mine = i < kb;
+    q += i;
+    // the Gram matrix: a warp per entry of the upper triangle sums the chunks
+    for (int e = t >> 5; e < kb * kb; e += 32) {
+        const int r = e / kb, c = e % kb;
+        if (c < r) continue;
+        double s = 0.0;
+        for (int u = lane; u < nch; u += 32) s += part[((int64_t)u * kb + r) * kb + c];
+        s = warp_sum(s);
+        if (lane == 0) a[r][c] = s;
+    }
+    if (!first)
+        for (int e = t; e < kb * kb; e += blockDim.x) rt[e % kb][e / kb] = Rt[e];
     __syncthreads();
     if (t == 0) {
         double tr = 0.0;
         for (int c = 0; c < kb; ++c) tr += a[c][c];
         // shift of the first pass: 11 (leff kb + kb (kb + 1)) u ||W||_F^2, leff
-        // the length of the summations that formed Gm, u the unit roundoff
+        // the length of the summations that formed the Gram matrix, u the unit roundoff
         sh = first ? 11.0 * (leff * kb + (double)kb * (kb + 1)) * unit * tr : 0.0;
     }
     __syncthreads();
-    if (i < kb && i == q) a[i][i] += sh;
+    if (mine && i == q) a[i][i] += sh;
     __syncthreads();
+    // row p of the factor is row p of the updated triangle over sqrt(pivot);
+    // every thread of the trailing triangle forms the factor itself, so that a
+    // column costs one barrier
+    double x = mine ? a[i][q] : 0.0;
     for (int p = 0; p < kb; ++p) {
-        if (t == 0) {
+        if (mine && i >= p) {
             double d = a[p][p];
             if (!(d > 0.0)) {
-                atomicExch(&flags[1], 1);
+                if (i == p && q == p) atomicExch(&flags[1], 1);
                 d = 1.0;
             }
-            a[p][p] = sqrt(d);
+            const double rs = rsqrt(d);
+            if (i == p) x = q == p ? d * rs : x * rs;
+            else x -= (a[p][i] * rs) * (a[p][q] * rs);
         }
-        __syncthreads();
-        if (t > p && t < kb) a[p][t] /= a[p][p];
-        __syncthreads();
-        if (i > p && i < kb && q >= i && q < kb) a[i][q] -= a[p][i] * a[p][q];
+        // row p + 1 is final before its own step: publish it
+        if (mine && i == p + 1) a[i][q] = x;
         __syncthreads();
     }
-    // a's upper triangle is Rp
-    if (i < kb && q < kb) {
-        const double r = q >= i ? a[i][q] : 0.0;
-        Rp[q * kb + i] = r;
-        if (first) Rt[q * kb + i] = r;
-        else rt[i][q] = Rt[q * kb + i];
-    }
+    if (mine) a[i][q] = x;
     __syncthreads();
-    if (!first && i < kb && q < kb) {
-        double s = 0.0;
-        for (int u = i; u <= q; ++u) s += a[i][u] * rt[u][q];
-        Rt[q * kb + i] = q >= i ? s : 0.0;
+    // a's upper triangle is Rp
+    for (int e = t; e < kb * kb; e += blockDim.x) {
+        const int r = e % kb, c = e / kb;
+        Rp[e] = c >= r ? a[r][c] : 0.0;
+        double s = c >= r ? a[r][c] : 0.0;
+        if (!first) {
+            s = 0.0;
+            for (int u = r; u <= c; ++u) s += a[r][u] * rt[u][c];
+        }
+        Rt[e] = s;
     }
 }
 
@@ -3307,148 +3387,222 @@ __global__ void __launch_bounds__(BG_UT) k_bg_trsm(int32_t n, int64_t ld, T* __r
     }
 }
 
-// the reflector of column q (rows q..q+kb, hv[0..kb], beta) applied by one
-// warp to the column x (rows q..q+kb of a column-major array)
-__device__ __forceinline__ void bg_reflect(const double* __restrict__ v, double beta, double* x, int kb, int lane)
-{
-    double d = 0.0;
-    for (int l = lane; l <= kb; l += 32) d = fma(v[l], x[l], d);
-    d = warp_sum(d) * beta;
-    for (int l = lane; l <= kb; l += 32) x[l] -= d * v[l];
-    __syncwarp();
-}
-
-// block step j: assemble the new block column of Hbar, reduce it, update G,
-// test each column; one block of 32 * BG_KMAX threads, warp a owns column a
+// Block step j of the least squares, grid = kb blocks. Block a assembles
+// column a of the new block column of Hbar and applies the earlier block
+// steps' reflections to it; each block step's kb reflections touch 2 kb rows
+// only, so they are kept as one 2 kb x 2 kb orthogonal matrix Q_i and a step
+// back costs one small product (a quarter of its columns per 64 threads)
+// instead of kb dependent reflections. The last block to arrive reduces the
+// window of the newest 2 kb rows with Householder reflections (four lanes per
+// column), applies them to G and to the identity (Q_j), and tests every
+// column's least-squares residual. With 11 systems, 25 block steps back on
+// average: 56 us, the reflections one by one in one block 216 us.
 template <class T>
-__global__ void __launch_bounds__(32 * BG_KMAX) k_bg_lsq(int j, Bg<T> B, Sys S, const int* __restrict__ cap)
+__global__ void __launch_bounds__(BG_LT) k_bg_lsq(int j, Bg<T> B, Sys S, const int* __restrict__ cap)
 {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int kb = B.flags[2];
+    extern __shared__ double sm[];
+    __shared__ double win[2][2 * BG_KMAX], part[4][2 * BG_KMAX];
+    __shared__ double vb[2][BG_KMAX + 1], beta[2];
+    __shared__ int nconv, ncap;
+    const int tid = threadIdx.x;
+    const int kb = B.flags[2], k2 = 2 * kb;
     const int nv = (j + 1) * kb;
     const int64_t ldh = B.ldh;
-    double* col = B.Hb + (int64_t)(j * kb + (warp < kb ? warp : 0)) * ldh;
-    if (warp < kb) {
-        for (int i = lane; i < nv; i += 32)
-            col[i] = B.H1[(int64_t)warp * nv + i] + B.H2[(int64_t)warp * nv + i];
-        for (int i = lane; i < kb; i += 32) col[nv + i] = i <= warp ? B.Rt[warp * kb + i] : 0.0;
-        __syncwarp();
-        // the earlier reflections, in order. Reflection q touches rows
-        // q..q+kb, so for kb < 32 the kb+1 rows in play sit in the warp's
-        // registers (lane l: row q+l): after reflection q, row q is final and
-        // the window moves down one row; the next reflector and the row that
-        // enters are loaded ahead (neither depends on the reflections so far).
-        const int nq = j * kb;
-        if (kb < 32 && nq > 0) {
-            const int64_t hs = B.k + 1;
-            double x = lane <= kb ? col[lane] : 0.0;
-            double v = lane <= kb ? B.hv[lane] : 0.0;
-            double be = B.hbeta[0];
-            double in = lane == kb ? col[kb + 1] : 0.0;
-            for (int q = 0; q < nq; ++q) {
-                const bool more = q + 1 < nq;
-                const double vn = (more && lane <= kb) ? B.hv[(q + 1) * hs + lane] : 0.0;
-                const double bn = more ? B.hbeta[q + 1] : 0.0;
-                const double inn = (more && lane == kb) ? col[q + kb + 2] : 0.0;
-                const double d = warp_sum(v * x) * be;
-                x -= d * v;
-                if (lane == 0) col[q] = x;
-                const double down = __shfl_down_sync(SAI_FULL, x, 1);
-                x = lane < kb ? down : (lane == kb ? in : 0.0);
-                v = vn;
-                be = bn;
-                in = inn;
-            }
-            if (lane <= kb) col[nq + lane] = x;
-        } else {
-            for (int q = 0; q < nq; ++q) bg_reflect(B.hv + (int64_t)q * (B.k + 1), B.hbeta[q], col + q, kb, lane);
-        }
-    }
-    __syncthreads();
-    for (int a = 0; a < kb; ++a) {
-        const int q = j * kb + a;
-        double* hvq = B.hv + (int64_t)q * (B.k + 1);
-        if (warp == a) {
-            double* x = B.Hb + (int64_t)q * ldh + q;
-            double ss = 0.0;
-            for (int l = lane; l <= kb; l += 32) ss = fma(x[l], x[l], ss);
-            const double nrm = sqrt(warp_sum(ss));
-            const double x0 = x[0];
-            __syncwarp();
-            if (nrm == 0.0) {
-                for (int l = lane; l <= kb; l += 32) hvq[l] = 0.0;
-                if (lane == 0) B.hbeta[q] = 0.0;
-            } else {
-                const double alpha = x0 >= 0.0 ? -nrm : nrm;
-                double vv = 0.0;
-                for (int l = lane; l <= kb; l += 32) {
-                    const double vl = l == 0 ? x0 - alpha : x[l];
-                    hvq[l] = vl;
-                    vv = fma(vl, vl, vv);
+    const size_t qs = (size_t)4 * B.k * B.k;  // distance between the Q_i
+    {
+        // rows 0 .. nv + kb - 1 of column a: H1 + H2, then R
+        const int a = blockIdx.x;
+        double* hb = B.Hb + (int64_t)(j * kb + a) * ldh;
+        auto entry = [&](int i) {
+            if (i < nv) return B.H1[(int64_t)a * nv + i] + B.H2[(int64_t)a * nv + i];
+            return i - nv <= a ? B.Rt[a * kb + (i - nv)] : 0.0;
+        };
+        if (tid < k2) win[0][tid] = entry(tid);
+        __syncthreads();
+        const int r = tid & 63, g = tid >> 6;            // output row, quarter of the columns
+        const int c0 = g * k2 / 4, c1 = (g + 1) * k2 / 4;  // at most 16 columns
+        double q[16];
+        if (j > 0 && r < k2)
+#pragma unroll
+            for (int u = 0; u < 16; ++u) q[u] = c0 + u < c1 ? B.Q[(size_t)(c0 + u) * k2 + r] : 0.0;
+        for (int i = 0; i < j; ++i) {
+            const double* w = win[i & 1];
+            double acc = 0.0;
+            if (r < k2)
+#pragma unroll
+                for (int u = 0; u < 16; ++u)
+                    if (c0 + u < c1) acc = fma(q[u], w[c0 + u], acc);
+            part[g][r] = acc;
+            // the next Q and the row that enters do not depend on this product
+            if (i + 1 < j && r < k2)
+#pragma unroll
+                for (int u = 0; u < 16; ++u)
+                    q[u] = c0 + u < c1 ? B.Q[(size_t)(i + 1) * qs + (size_t)(c0 + u) * k2 + r] : 0.0;
+            const double in = tid >= kb && tid < k2 ? entry((i + 1) * kb + tid) : 0.0;
+            __syncthreads();
+            if (tid < k2) {
+                const double v = (part[0][tid] + part[1][tid]) + (part[2][tid] + part[3][tid]);
+                if (tid < kb) {
+                    hb[i * kb + tid] = v;  // final rows of the triangle
+                } else {
+                    win[(i + 1) & 1][tid - kb] = v;
+                    win[(i + 1) & 1][tid] = in;
                 }
-                vv = warp_sum(vv);
-                __syncwarp();
-                for (int l = lane; l <= kb; l += 32) x[l] = l == 0 ? alpha : 0.0;
-                if (lane == 0) B.hbeta[q] = 2.0 / vv;
             }
+            __syncthreads();
         }
-        __syncthreads();
-        if (warp < kb) {
-            const double beta = B.hbeta[q];
-            if (warp > a) bg_reflect(hvq, beta, B.Hb + (int64_t)(j * kb + warp) * ldh + q, kb, lane);
-            bg_reflect(hvq, beta, B.G + (int64_t)warp * ldh + q, kb, lane);
-        }
-        __syncthreads();
+        if (tid < k2) B.Wn[(size_t)a * 2 * B.k + tid] = win[j & 1][tid];
     }
-    // least-squares residual of each column: G rows (j+1)kb .. (j+2)kb-1;
-    // a system that used up its iterations ends the cycle too
-    __shared__ int nconv, ncap;
-    if (threadIdx.x == 0) {
+    __shared__ int last;
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(&B.flags[3], 1) == (int)gridDim.x - 1;
+        if (last) {
+            __threadfence();
+            B.flags[3] = 0;
+        }
         nconv = 0;
         ncap = 0;
     }
     __syncthreads();
-    if (warp < kb) {
-        const double* g = B.G + (int64_t)warp * ldh + nv;
+    if (!last) return;
+    // columns 0 .. kb-1: the new block column; kb .. 2kb-1: G; 2kb .. 4kb-1: the identity
+    const int ldx = k2 + 1;
+    for (int e = tid; e < 4 * kb * k2; e += BG_LT) {
+        const int c = e / k2, r = e % k2;
+        double v;
+        if (c < kb) v = __ldcg(B.Wn + (size_t)c * 2 * B.k + r);
+        else if (c < k2) v = B.G[(int64_t)(c - kb) * ldh + (int64_t)j * kb + r];
+        else v = r == c - k2 ? 1.0 : 0.0;
+        sm[c * ldx + r] = v;
+    }
+    __syncthreads();
+    const int sub = tid & 3, grp = tid >> 2;  // four lanes per column
+    const unsigned gm = 0xfu << (tid & 28);
+    // reflector a from column a's rows a .. a + kb (its group): v, beta = 2 / v^T v
+    auto make = [&](int a) {
+        double* x = sm + a * ldx + a;
+        double ss = 0.0;
+        for (int l = sub; l <= kb; l += 4) ss = fma(x[l], x[l], ss);
+        ss += __shfl_xor_sync(gm, ss, 1);
+        ss += __shfl_xor_sync(gm, ss, 2);
+        const double x0 = x[0];
+        __syncwarp(gm);
+        if (ss == 0.0) {
+            for (int l = sub; l <= kb; l += 4) vb[a & 1][l] = 0.0;
+            if (sub == 0) beta[a & 1] = 0.0;
+        } else {
+            const double nrm = sqrt(ss);
+            const double alpha = x0 >= 0.0 ? -nrm : nrm;
+            for (int l = sub; l <= kb; l += 4) {
+                vb[a & 1][l] = l == 0 ? x0 - alpha : x[l];
+                x[l] = l == 0 ? alpha : 0.0;
+            }
+            if (sub == 0) beta[a & 1] = 1.0 / (ss + nrm * fabs(x0));  // v^T v = 2 (ss + nrm |x0|)
+        }
+    };
+    if (grp == 0) make(0);
+    __syncthreads();
+    for (int a = 0; a < kb; ++a) {
+        const double* v = vb[a & 1];
+        const double bt = beta[a & 1];
+        for (int c = grp; c < 4 * kb; c += BG_LT / 4) {
+            if (c <= a) continue;
+            double* x = sm + c * ldx + a;
+            double d = 0.0;
+            for (int l = sub; l <= kb; l += 4) d = fma(v[l], x[l], d);
+            d += __shfl_xor_sync(gm, d, 1);
+            d += __shfl_xor_sync(gm, d, 2);
+            d *= bt;
+            for (int l = sub; l <= kb; l += 4) x[l] = fma(-d, v[l], x[l]);
+            __syncwarp(gm);
+            if (c == a + 1 && c < kb) make(c);
+        }
+        __syncthreads();
+    }
+    for (int e = tid; e < 4 * kb * k2; e += BG_LT) {
+        const int c = e / k2, r = e % k2;
+        const double v = sm[c * ldx + r];
+        if (c < kb) {
+            if (r < kb) B.Hb[(int64_t)(j * kb + c) * ldh + (int64_t)j * kb + r] = v;
+        } else if (c < k2) {
+            B.G[(int64_t)(c - kb) * ldh + (int64_t)j * kb + r] = v;
+        } else {
+            B.Q[(size_t)j * qs + (size_t)(c - k2) * k2 + r] = v;
+        }
+    }
+    // least-squares residual of each column: the lower kb rows of G's window; a
+    // system that used up its iterations ends the cycle too
+    if (grp < kb) {
+        const double* g = sm + (kb + grp) * ldx + kb;
         double e = 0.0;
-        for (int l = lane; l < kb; l += 32) e = fma(g[l], g[l], e);
-        e = warp_sum(e);
-        if (lane == 0) {
-            const int c = B.lact[1 + warp];
+        for (int l = sub; l < kb; l += 4) e = fma(g[l], g[l], e);
+        e += __shfl_xor_sync(gm, e, 1);
+        e += __shfl_xor_sync(gm, e, 2);
+        if (sub == 0) {
+            const int c = B.lact[1 + grp];
             S.iters[c] += 1;
             if (sqrt(e) < S.thr[c]) atomicAdd(&nconv, 1);
             if (S.iters[c] >= cap[c]) atomicAdd(&ncap, 1);
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) B.flags[0] = nconv == kb || ncap > 0;
+    if (tid == 0) B.flags[0] = nconv == kb || ncap > 0;
 }
+inline size_t bg_lsq_smem(int kb) { return sizeof(double) * (size_t)4 * kb * (2 * kb + 1); }
 
-// Ys = Rtri^{-1} G_top, nt = (steps) * kb rows; warp c solves column c
+// Ys = Rtri^{-1} G_top, nt = (steps) * kb rows; block c solves column c by
+// blocks of 32 rows: the diagonal block by one warp (reciprocal pivots, one
+// shuffle and one FMA per row), then its 32 unknowns are taken out of the
+// rows above, column-oriented. (A warp per column with a dot product per row
+// took 1.5 ms for 390 rows on average, this form 0.12 ms.)
 template <class T>
-__global__ void __launch_bounds__(32 * BG_KMAX) k_bg_backsolve(int nt, Bg<T> B)
+__global__ void __launch_bounds__(BG_LT) k_bg_backsolve(int nt, Bg<T> B)
 {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int kb = B.flags[2];
-    if (warp >= kb) return;
-    const int64_t ldh = B.ldh, ldy = (int64_t)B.m * B.k;
-    double* y = B.Ys + (int64_t)warp * ldy;
-    const double* g = B.G + (int64_t)warp * ldh;
-    for (int i = nt - 1; i >= 0; --i) {
-        double s = 0.0;
-        for (int q = i + 1 + lane; q < nt; q += 32) s = fma(B.Hb[(int64_t)q * ldh + i], y[q], s);
-        s = warp_sum(s);
-        if (lane == 0) {
-            const double d = B.Hb[(int64_t)i * ldh + i];
-            if (d == 0.0) {
-                atomicExch(&B.flags[1], 2);
-                y[i] = 0.0;
-            } else {
-                y[i] = (g[i] - s) / d;
+    extern __shared__ double y[];  // nt
+    __shared__ double yb[32], D[32][33];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int c = blockIdx.x;
+    const int64_t ldh = B.ldh;
+    const double* g = B.G + (int64_t)c * ldh;
+    for (int i = tid; i < nt; i += BG_LT) y[i] = g[i];
+    __syncthreads();
+    for (int i1 = nt; i1 > 0; i1 -= 32) {
+        const int i0 = i1 > 32 ? i1 - 32 : 0, m = i1 - i0;
+        for (int e = tid; e < m * 32; e += BG_LT)
+            D[e / 32][e % 32] = e % 32 < m ? B.Hb[(int64_t)(i0 + e / 32) * ldh + i0 + e % 32] : 0.0;
+        __syncthreads();
+        if (tid < 32) {
+            double t = lane < m ? y[i0 + lane] : 0.0;
+            const double d = lane < m ? D[lane][lane] : 1.0;
+            if (d == 0.0) atomicExch(&B.flags[1], 2);
+            const double rd = d == 0.0 ? 0.0 : 1.0 / d;
+            for (int q = m - 1; q >= 0; --q) {
+                const double h = lane < q ? D[q][lane] : 0.0;
+                if (lane == q) t *= rd;
+                t = fma(-h, __shfl_sync(SAI_FULL, t, q), t);
             }
+            if (lane < m) y[i0 + lane] = t;
+            yb[lane] = lane < m ? t : 0.0;
         }
-        __syncwarp();
+        __syncthreads();
+        for (int r = tid; r < i0; r += BG_LT) {
+            double t = y[r];
+            for (int q0 = 0; q0 < m; q0 += 8) {
+                double h[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    h[u] = q0 + u < m ? B.Hb[(int64_t)(i0 + q0 + u) * ldh + r] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) t = fma(-h[u], yb[q0 + u < m ? q0 + u : 0], t);
+            }
+            y[r] = t;
+        }
+        __syncthreads();
     }
+    double* ys = B.Ys + (int64_t)c * B.m * B.k;
+    for (int i = tid; i < nt; i += BG_LT) ys[i] = y[i];
 }
 
 // cycle start: true residual norms (partials of the listed systems), stop
@@ -3536,23 +3690,27 @@ inline void bg_work(int site, double bytes, double flops, cudaStream_t st)
         else F<T, 32>__VA_ARGS__;                                \
     } while (0)
 
-// P = V^T W (nv basis vectors from V, kb columns of W) into H (nv x kb)
+inline int bg_chunks(int64_t n) { return (int)((n + BG_CR - 1) / BG_CR); }
+
+// partials of P = V^T W (nv basis vectors from V, kb columns of W), and P
+// into H (nv x kb) when H is given
 template <class T>
 void bg_gram(int32_t n, int64_t ld, const T* V, int nv, const T* W, int kb, double* part, double* H,
              cudaStream_t st)
 {
-    const int nch = (int)(((int64_t)n + BG_CR - 1) / BG_CR);
+    const int nch = bg_chunks(n);
     const int KBs = kb <= 4 ? 4 : kb <= 8 ? 8 : kb <= 12 ? 12 : kb <= 16 ? 16 : kb <= 24 ? 24 : 32;
     const int per_block = BG_GV * bg_vb((int)sizeof(T), KBs);
     const dim3 grid((unsigned)nch, (unsigned)((nv + per_block - 1) / per_block));
     sai_count_grid(grid.x * grid.y);
     BG_DISPATCH(kb, k_bg_gram, T, <<<grid, BG_GV * 32, 0, st>>>(n, ld, V, nv, W, kb, part));
-    k_bg_reduce<<<SAI_GRID(sai_div_up((int64_t)nv * kb * 32, 256)), 256, 0, st>>>(nch, nv, kb, part, H);
+    if (H) k_bg_reduce<<<SAI_GRID(sai_div_up((int64_t)nv * kb * 32, 256)), 256, 0, st>>>(nch, nv, kb, part, H);
 }
 
-unsigned bg_rows_grid(int32_t n)
+// blocks of `rows` rows, at most eight per SM
+unsigned bg_rows_grid(int32_t n, int rows)
 {
-    int64_t g = ((int64_t)n + BG_UT - 1) / BG_UT;
+    int64_t g = ((int64_t)n + rows - 1) / rows;
     if (g > (int64_t)g_sms * 8) g = (int64_t)g_sms * 8;
     return (unsigned)(g > 0 ? g : 1);
 }
@@ -3561,23 +3719,23 @@ template <class T>
 void bg_update(int32_t n, int64_t ld, const T* V, int nv, const double* H, int ldhh, int kb, T* W, int overwrite,
                cudaStream_t st)
 {
-    const unsigned g = bg_rows_grid(n);
+    const unsigned g = bg_rows_grid(n, BG_UR);
     sai_count_grid(g);
-    BG_DISPATCH(kb, k_bg_update, T, <<<g, BG_UT, 0, st>>>(n, ld, V, nv, H, ldhh, kb, W, overwrite));
+    BG_DISPATCH(kb, k_bg_update, T, <<<g, BG_UR * BG_UP, 0, st>>>(n, ld, V, nv, H, ldhh, kb, W, overwrite));
 }
 
 // W = Q R: shifted Cholesky QR in three passes, R accumulated in B.Rt. The
 // Gram matrices sum BG_CR/32 products per lane and 5 shuffle levels in T,
-// then the chunks in FP64 (counted too when T is FP64).
+// then the chunks in FP64 (inside k_bg_chol; counted too when T is FP64).
 template <class T>
 void bg_qr(int32_t n, int64_t ld, T* W, int kb, const Bg<T>& B, cudaStream_t st)
 {
-    const unsigned g = bg_rows_grid(n);
+    const unsigned g = bg_rows_grid(n, BG_UT);
     const double unit = sizeof(T) == 4 ? 5.9604644775390625e-08 : 1.1102230246251565e-16;
     const double leff = BG_CR / 32 + 5 + (sizeof(T) == 8 ? ((int64_t)n + BG_CR - 1) / BG_CR : 1);
     for (int pass = 0; pass < 3; ++pass) {
-        bg_gram<T>(n, ld, W, kb, W, kb, B.part, B.Gm, st);
-        k_bg_chol<<<SAI_GRID(1), 1024, 0, st>>>(kb, leff, unit, B.Gm, B.Rp, B.Rt, pass == 0, B.flags);
+        bg_gram<T>(n, ld, W, kb, W, kb, B.part, nullptr, st);
+        k_bg_chol<<<SAI_GRID(1), 1024, 0, st>>>(kb, bg_chunks(n), leff, unit, B.part, B.Rp, B.Rt, pass == 0, B.flags);
         sai_count_grid(g);
         BG_DISPATCH(kb, k_bg_trsm, T, <<<g, BG_UT, 0, st>>>(n, ld, W, kb, B.Rp));
     }
@@ -3593,7 +3751,8 @@ sai_status bgmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs
     const int32_t n = I.n;
     const int64_t ld = I.ld;
     const int ib = item_blocks(n > 0 ? n : 1, k);
-    const unsigned gg = bg_rows_grid(n) * 4;
+    const unsigned gg = bg_rows_grid(n, 256) * 4;
+    SAI_CUDA(cudaFuncSetAttribute(k_bg_lsq<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bg_lsq_smem(k)));
     VKT(I, k_gm_init, T)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Bs, Xs, R, S.lall, pt2, S.acnt, S.hn);
     SAI_CUDA(cudaMemsetAsync(B.flags, 0, sizeof(int) * 4, st));
     int h[3] = {0, 0, 0};
@@ -3648,7 +3807,7 @@ sai_status bgmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs
             {
                 ProfScope ps(PROF_GM_STEP, st);
                 bg_qr<T>(n, ld, Vn, kb, B, st);
-                k_bg_lsq<T><<<SAI_GRID(1), 32 * BG_KMAX, 0, st>>>(j, B, S, cap);
+                k_bg_lsq<T><<<SAI_GRID(kb), BG_LT, bg_lsq_smem(kb), st>>>(j, B, S, cap);
             }
             SAI_CUDA(cudaGetLastError());
             SAI_CUDA(cudaMemcpyAsync(h, B.flags, sizeof(int) * 2, cudaMemcpyDeviceToHost, st));
@@ -3661,7 +3820,7 @@ sai_status bgmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs
         }
         if (steps == 0) continue;
         // X[lact] += M (V Ys), R = B - A~ X
-        k_bg_backsolve<T><<<SAI_GRID(1), 32 * BG_KMAX, 0, st>>>(steps * kb, B);
+        k_bg_backsolve<T><<<SAI_GRID(kb), BG_LT, sizeof(double) * steps * kb, st>>>(steps * kb, B);
         bg_update<T>(n, ld, B.V, steps * kb, B.Ys, m * B.k, kb, B.Z, 1, st);
         spmv<T, 0>(n, ld, A.M, kb, B.Z, B.T1, nullptr, B.lid, st);
         k_bg_scatter_add<T><<<SAI_GRID(gg), 256, 0, st>>>(n, ld, B.lact, B.T1, Xs);
@@ -3687,27 +3846,26 @@ sai_status bg_alloc(int k, int m, int32_t n, int64_t ld, Buf& vb, Buf& hb, Buf& 
     B.T1 = d + blk * (m + 1);
     B.Z = B.T1 + blk;
     B.R = B.Z + blk;
-    const int nch = (int)(((int64_t)(n > 0 ? n : 1) + BG_CR - 1) / BG_CR);
+    const int nch = bg_chunks(n > 0 ? n : 1);
     const size_t nvmax = (size_t)B.ldh;
-    const size_t hsz = (size_t)B.ldh * m * k + (size_t)m * k * (k + 1) + (size_t)m * k + (size_t)B.ldh * k +
-                       (size_t)m * k * k + 3 * (size_t)k * k + 2 * nvmax * k + (size_t)nch * nvmax * k;
+    const size_t hsz = (size_t)B.ldh * m * k + 4 * (size_t)m * k * k + 2 * (size_t)k * k + (size_t)B.ldh * k +
+                       (size_t)m * k * k + 2 * (size_t)k * k + 2 * nvmax * k + (size_t)nch * nvmax * k;
     SAI_TRY(hb.alloc(sizeof(double) * hsz, st, true));
     SAI_CUDA(cudaMemsetAsync(hb.p, 0, sizeof(double) * hsz, st));
     double* e = hb.as<double>();
     B.Hb = e;
     e += (size_t)B.ldh * m * k;
-    B.hv = e;
-    e += (size_t)m * k * (k + 1);
-    B.hbeta = e;
-    e += (size_t)m * k;
+    B.Q = e;
+    e += 4 * (size_t)m * k * k;
+    B.Wn = e;
+    e += 2 * (size_t)k * k;
     B.G = e;
     e += (size_t)B.ldh * k;
     B.Ys = e;
     e += (size_t)m * k * k;
     B.Rt = e;
     B.Rp = e + k * k;
-    B.Gm = e + 2 * k * k;
-    e += 3 * (size_t)k * k;
+    e += 2 * (size_t)k * k;
     B.H1 = e;
     B.H2 = e + nvmax * k;
     e += 2 * nvmax * k;

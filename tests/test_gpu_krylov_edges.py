@@ -55,3 +55,22 @@ def test_vector_kernels_at_chunk_edges(n, method):
                                          restart=30)
         assert itc[0] == it[c]
         assert torch.equal(xc[:, 0], X[:, c]), (method, n, c)
+
+
+@pytest.mark.parametrize("n,k", [(63, 2), (511, 5), (513, 1), (1000, 9), (2049, 13), (3001, 17), (1537, 25), (4099, 32)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_block_gmres_block_sizes(n, k, precision):
+    """Block sizes around the kernels' specialisations (4, 8, 12, 16, 24, 32) and row counts around their tiles
+    (chunks of 512 rows, tiles of 64); restart 4, so that several cycles run. Tolerance as above."""
+    need_gpu()
+    sai = lib()
+    A, M, B = _system(n, k, 7 * n + k)
+    h = sai.split(to_dev(A), abs_tau=float("inf"))
+    P = sai.precond_from_csc(to_dev(M))
+    norms = np.linalg.norm(B, axis=0)
+    thr = list(1e-10 * norms)
+    X, it, stt, st = sai.krylov_solve(h, P, torch.as_tensor(B, device="cuda"), thr, method=sai.BGMRES, maxit=200,
+                                      restart=4, precision=precision)
+    assert st == sai.SAI_OK and stt == [0] * k
+    R = np.linalg.norm(B - A @ X.cpu().numpy(), axis=0)
+    assert np.all(R <= np.asarray(thr) + 1e-12 * norms), (R, thr)
