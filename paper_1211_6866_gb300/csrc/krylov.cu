@@ -1947,11 +1947,33 @@ __global__ void k_gm_cycle_start(int k, const double* nrm2, const int* cap, Sys 
 // basis vectors), g fastest so the items of one chunk read its rows of u and
 // z from cache; the block's IT_WARPS warps take interleaved 16-byte row
 // vectors of the chunk and their sums are combined in warp order through
-// shared memory. (Streaming each thread's row vectors through a two-stage
+// shared memory. A warp sums its 2 PD + 2 values together (warp_sum16: 16
+// shuffles and additions against five for each value): with a butterfly per
+// value the reduction was 40% of the kernel's FP64 instructions (50653 rows,
+// 8 systems, FP64: 85 us on average).
+// (Streaming each thread's row vectors through a two-stage
 // cp.async buffer in shared memory instead of registers measured slower:
 // 21.5 against 18.9 ms of the 64^3 step.)
 constexpr int DC_CHUNK = 2048;  // rows per item of the fused dot kernel (one partial per item)
 inline int dc_chunks(int64_t n) { return (int)((n + DC_CHUNK - 1) / DC_CHUNK); }
+
+// Sums a[0..15] over the warp: lanes 2 i and 2 i + 1 get the sum of a[i]
+// (each round halves the values a lane still carries).
+template <class T>
+__device__ __forceinline__ T warp_sum16(T (&a)[16])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 1; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < o / 2; ++i) {
+            const T keep = up ? a[i + o / 2] : a[i], send = up ? a[i] : a[i + o / 2];
+            a[i] = keep + __shfl_xor_sync(SAI_FULL, send, o);
+        }
+    }
+    return a[0] + __shfl_xor_sync(SAI_FULL, a[0], 1);
+}
 
 template <class T>
 __global__ void __launch_bounds__(IT_WARPS * 32) k_dc_dots(Items I, int ndc, const T* __restrict__ u,
@@ -1961,7 +1983,8 @@ __global__ void __launch_bounds__(IT_WARPS * 32) k_dc_dots(Items I, int ndc, con
     using VT = typename Vec<T>::type;
     constexpr int VW = Vec<T>::W;
     constexpr int NR = 2 * PD + 2;
-    __shared__ T red[IT_WARPS][NR];
+    static_assert(NR <= 16, "the values of warp_sum16");
+    __shared__ T red[IT_WARPS][16];
     const int j = *jdev;
     const int ng = j > 0 ? (j + PD - 1) / PD : 1;  // groups of PD basis vectors
     const int cnt = list[0];
@@ -1996,30 +2019,26 @@ __global__ void __launch_bounds__(IT_WARPS * 32) k_dc_dots(Items I, int ndc, con
 #pragma unroll
             for (int i = 0; i < PD; ++i)
                 if (i < ni) {
-                    as[i] += Vec<T>::dot(vv[i], uv);
-                    ac[i] += Vec<T>::dot(vv[i], zv);
+                    as[i] = Vec<T>::dot(vv[i], uv, as[i]);
+                    ac[i] = Vec<T>::dot(vv[i], zv, ac[i]);
                 }
             if (g == 0) {
-                uu += Vec<T>::dot(uv, uv);
-                uz += Vec<T>::dot(uv, zv);
+                uu = Vec<T>::dot(uv, uv, uu);
+                uz = Vec<T>::dot(uv, zv, uz);
             }
         }
+        T sums[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) sums[i] = 0;
 #pragma unroll
         for (int i = 0; i < PD; ++i) {
-            as[i] = warp_sum_t(as[i]);
-            ac[i] = warp_sum_t(ac[i]);
+            sums[2 * i] = as[i];
+            sums[2 * i + 1] = ac[i];
         }
-        uu = warp_sum_t(uu);
-        uz = warp_sum_t(uz);
-        if (lane == 0) {
-#pragma unroll
-            for (int i = 0; i < PD; ++i) {
-                red[wid][2 * i] = as[i];
-                red[wid][2 * i + 1] = ac[i];
-            }
-            red[wid][2 * PD] = uu;
-            red[wid][2 * PD + 1] = uz;
-        }
+        sums[2 * PD] = uu;
+        sums[2 * PD + 1] = uz;
+        const T w = warp_sum16(sums);
+        if ((lane & 1) == 0) red[wid][lane >> 1] = w;
         __syncthreads();
         const int nsl = 2 * ni + (g == 0 ? 2 : 0);
         if ((int)threadIdx.x < nsl) {
@@ -2028,7 +2047,7 @@ __global__ void __launch_bounds__(IT_WARPS * 32) k_dc_dots(Items I, int ndc, con
             const int slot = t < 2 * ni ? 2 * i0 + t : 2 * GM_MAXM + (t - 2 * ni);
             double sum = 0.0;
 #pragma unroll
-            for (int w = 0; w < IT_WARPS; ++w) sum += (double)red[w][widx];
+            for (int v = 0; v < IT_WARPS; ++v) sum += (double)red[v][widx];
             part[((size_t)c * PS + slot) * ndc + q] = sum;
         }
         __syncthreads();
