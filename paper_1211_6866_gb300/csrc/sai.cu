@@ -100,14 +100,13 @@ template <int LCAP_, int SCAP_, int HL_, int HC_, class TQ_ = double>
 struct Tier {
     using TQ = TQ_;  // scalar of the QR factors (double, or float for the refined form)
     static constexpr int LCAP = LCAP_, SCAP = SCAP_, HL = HL_, HC = HC_;
-    static constexpr size_t OFF_Q = 0;
-    static constexpr size_t OFF_CV = OFF_Q + sizeof(TQ) * LCAP * SCAP;
+    static constexpr size_t OFF_CV = 0;
     static constexpr size_t OFF_R = a16(OFF_CV + sizeof(TQ) * LCAP);
     static constexpr size_t OFF_M = OFF_R + 8ull * LCAP;
     static constexpr size_t OFF_G = OFF_M + 8ull * SCAP;
     static constexpr size_t OFF_BETA = OFF_G + 8ull * SCAP;
-    static constexpr size_t OFF_RD = OFF_BETA + sizeof(TQ) * SCAP;
-    static constexpr size_t OFF_LROW = a16(OFF_RD + sizeof(TQ) * SCAP);
+    static constexpr size_t OFF_RI = OFF_BETA + sizeof(TQ) * SCAP;
+    static constexpr size_t OFF_LROW = a16(OFF_RI + 8ull * SCAP);
     static constexpr size_t OFF_HK = OFF_LROW + 4ull * LCAP;
     static constexpr size_t OFF_HV = OFF_HK + 4ull * HL;
     static constexpr size_t OFF_S = OFF_HV + 4ull * HL;
@@ -116,7 +115,9 @@ struct Tier {
     static constexpr size_t OFF_CK = OFF_A1 + 4ull * SCAP;
     static constexpr size_t OFF_CF = OFF_CK + 4ull * HC;
     static constexpr size_t OFF_KP = OFF_CF + (size_t)HC;
-    static constexpr size_t BYTES = a16(OFF_KP + (size_t)SCAP);
+    static constexpr size_t OFF_Q = a16(OFF_KP + (size_t)SCAP);  // the QR factors follow the rest
+    static constexpr size_t Q_BYTES = sizeof(TQ) * LCAP * SCAP;
+    static constexpr size_t BYTES = a16(OFF_Q + Q_BYTES);
     // distance between the workspaces of consecutive groups: a multiple of
     // 128 bytes plus 32, so that the 8-lane groups of one warp start in
     // different shared-memory banks
@@ -125,10 +126,17 @@ struct Tier {
     static_assert(HC >= 2 * SCAP && (HC & (HC - 1)) == 0, "candidate hash");
 };
 
+// Where a tier's workspaces live: in global memory, in shared memory, or the
+// QR factors in global and the rest (hash tables, candidate list, residual,
+// solution) in shared memory. The build of a column is a chain of dependent
+// look-ups in the latter, so a column of the global-memory tiers spent its
+// time waiting for L2: twelve tier-1 columns took 4.2 ms.
+enum { WS_GLOBAL = 0, WS_SHARED = 1, WS_HYBRID = 2 };
+
 using TierS = Tier<32, 8, 64, 128>;         // shared memory, small patterns, ~4.1 KB per group
-using Tier0 = Tier<64, 16, 128, 512>;      // shared memory, ~13.7 KB per warp
-using Tier1 = Tier<256, 64, 512, 2048>;    // global memory, ~150 KB per warp
-using Tier2 = Tier<1024, 128, 2048, 8192>; // global memory, ~1.1 MB per warp
+using Tier0 = Tier<64, 16, 128, 512>;      // shared memory, ~13.8 KB per warp
+using Tier1 = Tier<256, 64, 512, 2048>;    // ~150 KB per warp, 22 KB of it without the factors
+using Tier2 = Tier<1024, 128, 2048, 8192>; // ~1.1 MB per warp, 84 KB of it without the factors
 using Tier3 = Tier<2048, 128, 4096, 65536>; // global memory, ~2.4 MB per warp (up to 32768 candidates)
 using Tier4 = Tier<4096, 2048, 8192, 65536>; // global memory, ~68 MB per warp: the large-pattern tier
 using TierSF = Tier<32, 8, 64, 128, float>;
@@ -182,6 +190,20 @@ struct Grp {
         for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
         return v;
     }
+    // the sums of four values over the group, each with sum()'s additions in
+    // sum()'s order: G/4 consecutive lanes, from u G/4 on, return the sum of
+    // a[u] (G = 32: six shuffles and additions instead of twenty)
+    template <class V>
+    __device__ __forceinline__ V sum4(const V (&a)[4]) const
+    {
+        const bool u2 = (l & (G / 2)) != 0, u1 = (l & (G / 4)) != 0;
+        const V x0 = (u2 ? a[2] : a[0]) + __shfl_xor_sync(mask, u2 ? a[0] : a[2], G / 2);
+        const V x1 = (u2 ? a[3] : a[1]) + __shfl_xor_sync(mask, u2 ? a[1] : a[3], G / 2);
+        V x = (u1 ? x1 : x0) + __shfl_xor_sync(mask, u1 ? x0 : x1, G / 4);
+#pragma unroll
+        for (int o = G / 8; o > 0; o >>= 1) x += __shfl_xor_sync(mask, x, o);
+        return x;
+    }
     __device__ __forceinline__ unsigned long long min_u64(unsigned long long v) const
     {
 #pragma unroll
@@ -195,24 +217,24 @@ struct Grp {
 
 template <class TQ>
 struct WsT {
-    TQ *Q, *cv, *beta, *rd;  // QR factors, Q^T e^, 2/(v^T v), diag(R)
-    double *r, *m, *g;       // FP64 residual, solution, refinement scratch
+    TQ *Q, *cv, *beta;       // QR factors, Q^T e^, 2/(v^T v)
+    double *r, *m, *g, *ri;  // FP64 residual, solution, refinement scratch, 1/diag(R)
     int32_t *Lrow, *hk, *hv, *S, *a0, *a1, *ck;
     uint8_t *cf, *kp;
 };
 
 template <class T>
-__device__ __forceinline__ WsT<typename T::TQ> bind_ws(char* b)
+__device__ __forceinline__ WsT<typename T::TQ> bind_ws(char* b, char* q)
 {
     using TQ = typename T::TQ;
     WsT<TQ> w;
-    w.Q = (TQ*)(b + T::OFF_Q);
+    w.Q = (TQ*)q;
     w.cv = (TQ*)(b + T::OFF_CV);
     w.r = (double*)(b + T::OFF_R);
     w.m = (double*)(b + T::OFF_M);
     w.g = (double*)(b + T::OFF_G);
     w.beta = (TQ*)(b + T::OFF_BETA);
-    w.rd = (TQ*)(b + T::OFF_RD);
+    w.ri = (double*)(b + T::OFF_RI);
     w.Lrow = (int32_t*)(b + T::OFF_LROW);
     w.hk = (int32_t*)(b + T::OFF_HK);
     w.hv = (int32_t*)(b + T::OFF_HV);
@@ -341,8 +363,53 @@ __device__ void col_init(const WsT<typename T::TQ>& w, int32_t k, int& nL, int& 
     nfact = 0;
 }
 
+// The reflector (v, bt) on the rows i0.. of the columns [c0, c1) of A^ (column
+// nS is cv), four at a time: v is read once for the four and their products
+// are summed together. The sums' additions were most of the reflector's FP64
+// instructions, five per column against its one or two products.
+template <class T, int G>
+__device__ __forceinline__ void apply_reflector(const WsT<typename T::TQ>& w, const typename T::TQ* v,
+                                                typename T::TQ bt, int i0, int nL, int c0, int c1, int nS)
+{
+    using TQ = typename T::TQ;
+    constexpr int UR = T::LCAP > 64 ? 4 : 1;  // rows in flight where the factors are in global memory
+    const Grp<G> g;
+#pragma unroll 1
+    for (int c = c0; c < c1; c += 4) {
+        const int nb = c1 - c;  // columns of this pass (at least 4: four)
+        TQ* p[4];
+        TQ d[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            p[u] = c + u == nS ? w.cv : w.Q + (size_t)(c + u) * T::LCAP;
+            d[u] = 0;
+        }
+#pragma unroll UR
+        for (int i = i0 + g.l; i < nL; i += G) {
+            const TQ vi = v[i];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (u < nb) d[u] = fma(vi, p[u][i], d[u]);
+        }
+        const TQ f = bt * g.sum4(d);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) d[u] = g.bcast(f, u * (G / 4));
+#pragma unroll UR
+        for (int i = i0 + g.l; i < nL; i += G) {
+            const TQ vi = v[i];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (u < nb) p[u][i] = fma(-d[u], vi, p[u][i]);
+        }
+        g.sync();
+    }
+}
+
 // Gathers the new columns S[nfact..nS), updates the QR factorisation and
 // solves R m = (Q^T e^)(0:nS). Returns ST_DONE, ST_OVERFLOW or ST_SINGULAR.
+// The reciprocals of R's new diagonal entries are formed side by side, one
+// per lane: a division is about ten dependent FP64 instructions, and one per
+// pivot and triangular solve was half of the refined build's FP64 work.
 template <class T, int G>
 __device__ int ls_update(const WsT<typename T::TQ>& w, const SaiMat& A, int& nL, int nS, int& nfact)
 {
@@ -375,22 +442,8 @@ __device__ int ls_update(const WsT<typename T::TQ>& w, const SaiMat& A, int& nL,
     g.sync();
     // old reflectors on the new columns
 #pragma unroll 1
-    for (int jr = 0; jr < nfact; ++jr) {
-        const TQ* v = w.Q + (size_t)jr * T::LCAP;
-        const TQ bj = w.beta[jr];
-#pragma unroll 1
-        for (int t = nfact; t < nS; ++t) {
-            TQ* col = w.Q + (size_t)t * T::LCAP;
-            TQ d = 0;
-#pragma unroll 1
-            for (int i = jr + g.l; i < nL; i += G) d = fma(v[i], col[i], d);
-            d = g.sum(d);
-            const TQ f = bj * d;
-#pragma unroll 1
-            for (int i = jr + g.l; i < nL; i += G) col[i] = fma(-f, v[i], col[i]);
-            g.sync();
-        }
-    }
+    for (int jr = 0; jr < nfact; ++jr)
+        apply_reflector<T, G>(w, w.Q + (size_t)jr * T::LCAP, w.beta[jr], jr, nL, nfact, nS, nS);
     // factor the trailing block column by column
 #pragma unroll 1
     for (int t = nfact; t < nS; ++t) {
@@ -407,23 +460,14 @@ __device__ int ls_update(const WsT<typename T::TQ>& w, const SaiMat& A, int& nL,
         g.sync();
         if (g.l == 0) {
             col[t] = x0 - alpha;
-            w.rd[t] = alpha;
+            w.ri[t] = (double)alpha;
             w.beta[t] = bt;
         }
         g.sync();
-#pragma unroll 1
-        for (int t2 = t + 1; t2 <= nS; ++t2) {
-            TQ* c2 = t2 < nS ? w.Q + (size_t)t2 * T::LCAP : w.cv;
-            TQ d = 0;
-#pragma unroll 1
-            for (int i = t + g.l; i < nL; i += G) d = fma(col[i], c2[i], d);
-            d = g.sum(d);
-            const TQ f = bt * d;
-#pragma unroll 1
-            for (int i = t + g.l; i < nL; i += G) c2[i] = fma(-f, col[i], c2[i]);
-            g.sync();
-        }
+        apply_reflector<T, G>(w, col, bt, t, nL, t + 1, nS + 1, nS);
     }
+#pragma unroll 1
+    for (int t = nfact + g.l; t < nS; t += G) w.ri[t] = 1.0 / w.ri[t];
     nfact = nS;
     // back substitution (FP64 arithmetic on the stored factors)
 #pragma unroll 1
@@ -431,7 +475,7 @@ __device__ int ls_update(const WsT<typename T::TQ>& w, const SaiMat& A, int& nL,
     g.sync();
 #pragma unroll 1
     for (int t = nS - 1; t >= 0; --t) {
-        const double mt = w.m[t] / (double)w.rd[t];
+        const double mt = w.m[t] * w.ri[t];
         g.sync();
         if (g.l == 0) w.m[t] = mt;
         const TQ* col = w.Q + (size_t)t * T::LCAP;
@@ -443,8 +487,8 @@ __device__ int ls_update(const WsT<typename T::TQ>& w, const SaiMat& A, int& nL,
 }
 
 // r = A~(L,S) m - e^ on L (only the columns with use[t] != 0 when use given);
-// returns ||r||^2.
-template <class T, int G>
+// returns ||r||^2 (NORM).
+template <class T, int G, bool NORM = true>
 __device__ double residual(const WsT<typename T::TQ>& w, const SaiMat& A, int nL, int nS, const uint8_t* use)
 {
     const Grp<G> g;
@@ -463,6 +507,7 @@ __device__ double residual(const WsT<typename T::TQ>& w, const SaiMat& A, int nL
         }
         g.sync();
     }
+    if (!NORM) return 0.0;
     double s = 0.0;
 #pragma unroll 1
     for (int i = g.l; i < nL; i += G) s = fma(w.r[i], w.r[i], s);
@@ -476,7 +521,7 @@ template <class T, int G>
 __device__ void refine(const WsT<typename T::TQ>& w, const SaiMat& A, int nL, int nS)
 {
     const Grp<G> g;
-    residual<T, G>(w, A, nL, nS, nullptr);  // r = A^ m - e^
+    residual<T, G, false>(w, A, nL, nS, nullptr);  // r = A^ m - e^
 #pragma unroll 1
     for (int t = g.l; t < nS; t += G) {
         const int32_t j = w.S[t];
@@ -492,7 +537,7 @@ __device__ void refine(const WsT<typename T::TQ>& w, const SaiMat& A, int nL, in
     // R^T y = g (forward), R(t,i) = Q[i][t] for i > t
 #pragma unroll 1
     for (int t = 0; t < nS; ++t) {
-        const double yt = w.g[t] / (double)w.rd[t];
+        const double yt = w.g[t] * w.ri[t];
         g.sync();
         if (g.l == 0) w.g[t] = yt;
 #pragma unroll 1
@@ -502,7 +547,7 @@ __device__ void refine(const WsT<typename T::TQ>& w, const SaiMat& A, int nL, in
     // R d = y (backward)
 #pragma unroll 1
     for (int t = nS - 1; t >= 0; --t) {
-        const double dt = w.g[t] / (double)w.rd[t];
+        const double dt = w.g[t] * w.ri[t];
         g.sync();
         if (g.l == 0) w.g[t] = dt;
 #pragma unroll 1
@@ -733,8 +778,15 @@ __device__ int psai_column(const WsT<typename T::TQ>& w, const SaiMat& A, int32_
         g.sync();
         if (rn <= a.delta || l >= a.lmax) {
             rn_pre = rn;
-            rn_post = sqrt(residual<T, G>(w, A, nL, nS, w.kp));
-            fl += 2 * sn + 2LL * nL;
+            // with nothing dropped the emitted column's residual is the one just formed
+            bool drop = false;
+#pragma unroll 1
+            for (int t = g.l; t < nS; t += G) drop |= w.kp[t] == 0;
+            rn_post = rn;
+            if (g.any(drop)) {
+                rn_post = sqrt(residual<T, G>(w, A, nL, nS, w.kp));
+                fl += 2 * sn + 2LL * nL;
+            }
             // compact the kept entries to the front of S / m (order preserved)
             int q = 0;
             if (g.l == 0) {
@@ -1614,7 +1666,7 @@ __global__ void __launch_bounds__(64) k_sai_lane(SaiMat A, SpaiArgs sa, PsaiArgs
 // shape run their steps in the same instructions rather than one group after
 // another. SMEM: the workspaces live in dynamic shared memory, one per
 // group; otherwise in gscratch, one per group of the grid.
-template <class T, int G, bool SMEM, bool PSAI>
+template <class T, int G, int WS, bool PSAI>
 __global__ void __launch_bounds__(256) k_sai(SaiMat A, SpaiArgs sa, PsaiArgs pa, const int32_t* __restrict__ work,
                                              int32_t nwork, int* next, char* gscratch, Out out, int32_t* ovf_list,
                                              int* ovf_cnt, int* err, int tier_id)
@@ -1623,11 +1675,11 @@ __global__ void __launch_bounds__(256) k_sai(SaiMat A, SpaiArgs sa, PsaiArgs pa,
     const Grp<G> g;
     constexpr int GPW = 32 / G;  // groups per warp
     const int grp = (int)(threadIdx.x >> 5) * GPW + (g.base / G);  // group index within the block
-    char* base = SMEM ? smem + (size_t)grp * T::STRIDE
-                      : gscratch + ((size_t)blockIdx.x * (blockDim.x / G) + grp) * T::STRIDE;
-    const WsT<typename T::TQ> w = bind_ws<T>(base);
-    double work_bytes = 0.0;
-    long long work_flops = 0, work_flops_q = 0;
+    const size_t gg = (size_t)blockIdx.x * (blockDim.x / G) + grp;  // and within the grid
+    char* base = WS == WS_GLOBAL ? gscratch + gg * T::STRIDE : smem + (size_t)grp * (WS == WS_HYBRID ? T::OFF_Q : T::STRIDE);
+    const WsT<typename T::TQ> w = bind_ws<T>(base, WS == WS_HYBRID ? gscratch + gg * T::Q_BYTES : base + T::OFF_Q);
+    // integers: the FP64 pipe is the kernel's bottleneck
+    long long work_bytes = 0, work_flops = 0, work_flops_q = 0;
 #pragma unroll 1
     for (;;) {
         int first = 0;
@@ -1655,12 +1707,12 @@ __global__ void __launch_bounds__(256) k_sai(SaiMat A, SpaiArgs sa, PsaiArgs pa,
                     oval[t] = w.m[t];
                 }
                 if (big && g.l == 0) out.big_slot[k] = item;
-                double cb = 0.0;
+                int cb = 0;  // in 4-byte words
 #pragma unroll 1
-                for (int t = g.l; t < nS; t += G) cb += 12.0 * (double)(A.cp[w.S[t] + 1] - A.cp[w.S[t]]) + 12.0;
+                for (int t = g.l; t < nS; t += G) cb += 3 * (int)(A.cp[w.S[t] + 1] - A.cp[w.S[t]]) + 3;
 #pragma unroll 1
-                for (int t = g.l; t < nL; t += G) cb += 4.0 * (double)(A.rp[w.Lrow[t] + 1] - A.rp[w.Lrow[t]]);
-                work_bytes += g.sum(cb);
+                for (int t = g.l; t < nL; t += G) cb += (int)(A.rp[w.Lrow[t] + 1] - A.rp[w.Lrow[t]]);
+                work_bytes += 4LL * g.sum(cb);
                 work_flops += cfl;
                 work_flops_q += cfq;
                 if (g.l == 0) {
@@ -1685,9 +1737,9 @@ __global__ void __launch_bounds__(256) k_sai(SaiMat A, SpaiArgs sa, PsaiArgs pa,
         }
         __syncwarp();
     }
-    if (g.l == 0 && work_bytes > 0.0) {
+    if (g.l == 0 && work_bytes > 0) {
         const bool q32 = sizeof(typename T::TQ) < sizeof(double);
-        atomicAdd(&d_swork[2 * PROF_SAI_BUILD], work_bytes);
+        atomicAdd(&d_swork[2 * PROF_SAI_BUILD], (double)work_bytes);
         atomicAdd(&d_swork[2 * PROF_SAI_BUILD + 1], (double)(work_flops + (q32 ? 0 : work_flops_q)));
         if (q32) atomicAdd(&d_swork32, (double)work_flops_q);
     }
@@ -1761,41 +1813,39 @@ __global__ void k_recip(int32_t n, const double* __restrict__ cn2, double* __res
 
 int g_num_sms = 0;
 
-// Launches one tier of the build over a work list: G lanes per column,
-// workspaces in shared memory (SMEM: as many blocks per SM as fit) or in a
-// pool buffer (blocks_per_sm_t12 blocks of 8 warps per SM, no more than the
-// list needs).
-template <class T, int G, bool SMEM, bool PSAI>
+// Launches one tier of the build over a work list: G lanes per column. WS_SHARED
+// (cfg.warps_t0 warps per block, or one where T's workspace is a tier 1's) and
+// WS_HYBRID (one warp per block): as many blocks per SM as fit; WS_GLOBAL:
+// workspaces in a pool buffer, blocks_per_sm_t12 blocks of 8 warps per SM.
+// No more blocks than the list needs.
+template <class T, int G, int WS, bool PSAI>
 sai_status launch_tier(const SaiMat& A, const SpaiArgs& sa, const PsaiArgs& pa, const int32_t* work, int32_t nwork,
                        int* next, const Out& out, int32_t* ovf_list, int* ovf_cnt, int* err, int tier_id,
                        const sai_build_config& cfg, cudaStream_t st)
 {
     if (nwork <= 0) return SAI_OK;
-    const int warps_per_block = SMEM ? cfg.warps_t0 : 8;
+    const int warps_per_block = WS == WS_GLOBAL ? 8 : (WS == WS_SHARED && T::LCAP <= 64 ? cfg.warps_t0 : 1);
     const int threads = 32 * warps_per_block;
     const int groups = threads / G;
-    int blocks;
-    Buf scratch;
-    size_t smem = 0;
-    if (SMEM) {
-        smem = T::STRIDE * groups;
-        SAI_CUDA(cudaFuncSetAttribute(k_sai<T, G, SMEM, PSAI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        int per_sm = 0;
-        SAI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sai<T, G, SMEM, PSAI>, threads, smem));
+    const int need = (nwork + groups - 1) / groups;
+    const size_t smem = WS == WS_GLOBAL ? 0 : (WS == WS_HYBRID ? T::OFF_Q : T::STRIDE) * groups;
+    int per_sm = cfg.blocks_per_sm_t12;
+    if (WS != WS_GLOBAL) {
+        SAI_CUDA(cudaFuncSetAttribute(k_sai<T, G, WS, PSAI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SAI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sai<T, G, WS, PSAI>, threads, smem));
         if (per_sm < 1) per_sm = 1;
-        blocks = g_num_sms * per_sm;
-    } else {
-        blocks = g_num_sms * cfg.blocks_per_sm_t12;
-        const int need = (nwork + groups - 1) / groups;
-        if (blocks > need) blocks = need;
-        SAI_TRY(scratch.alloc(T::STRIDE * (size_t)groups * blocks, st, true));
     }
+    int blocks = g_num_sms * per_sm;
+    if (blocks > need) blocks = need;
+    Buf scratch;
+    if (WS != WS_SHARED)
+        SAI_TRY(scratch.alloc((WS == WS_HYBRID ? T::Q_BYTES : T::STRIDE) * (size_t)groups * blocks, st, true));
     SAI_CUDA(cudaMemsetAsync(next, 0, sizeof(int), st));
     {
         ProfScope ps(PROF_SAI_BUILD, st);
-        k_sai<T, G, SMEM, PSAI><<<SAI_GRID(blocks), threads, smem, st>>>(A, sa, pa, work, nwork, next,
-                                                                        scratch.as<char>(), out, ovf_list, ovf_cnt,
-                                                                        err, tier_id);
+        k_sai<T, G, WS, PSAI><<<SAI_GRID(blocks), threads, smem, st>>>(A, sa, pa, work, nwork, next,
+                                                                      scratch.as<char>(), out, ovf_list, ovf_cnt,
+                                                                      err, tier_id);
     }
     SAI_CUDA(cudaGetLastError());
     return SAI_OK;
@@ -1853,7 +1903,7 @@ sai_status launch_big(const SaiMat& A, const SpaiArgs& sa, const PsaiArgs& pa, c
     SAI_CUDA(cudaMemsetAsync(next, 0, sizeof(int), st));
     {
         ProfScope ps(PROF_SAI_BUILD, st);
-        k_sai<T, 32, false, PSAI><<<SAI_GRID(warps), 32, 0, st>>>(A, sa, pa, work, nwork, next, scratch.as<char>(), out,
+        k_sai<T, 32, WS_GLOBAL, PSAI><<<SAI_GRID(warps), 32, 0, st>>>(A, sa, pa, work, nwork, next, scratch.as<char>(), out,
                                                                   nullptr, nullptr, err, 5);
     }
     SAI_CUDA(cudaGetLastError());
@@ -2023,35 +2073,46 @@ sai_status build_common(const sai_split_s* h, const SpaiArgs& sa, const PsaiArgs
         if (cfg.first_tier == 3)
             SAI_TRY((launch_lane<TQ, PSAI>(A, sa, pa, queue, nq, c + 0, out, ovfs.as<int32_t>(), c + 13, c + 3, st)));
         else if (cfg.first_tier == 1)
-            SAI_TRY((launch_tier<TS, 8, true, PSAI>(A, sa, pa, queue, nq, c + 0, out, ovfs.as<int32_t>(), c + 13,
+            SAI_TRY((launch_tier<TS, 8, WS_SHARED, PSAI>(A, sa, pa, queue, nq, c + 0, out, ovfs.as<int32_t>(), c + 13,
                                                     c + 3, 4, cfg, st)));
         else
-            SAI_TRY((launch_tier<TS, 16, true, PSAI>(A, sa, pa, queue, nq, c + 0, out, ovfs.as<int32_t>(), c + 13,
+            SAI_TRY((launch_tier<TS, 16, WS_SHARED, PSAI>(A, sa, pa, queue, nq, c + 0, out, ovfs.as<int32_t>(), c + 13,
                                                      c + 3, 4, cfg, st)));
         SAI_CUDA(cudaMemcpyAsync(&n0, c + 13, sizeof(int), cudaMemcpyDeviceToHost, st));
         SAI_CUDA(cudaStreamSynchronize(st));
         q0 = ovfs.as<int32_t>();
     }
-    SAI_TRY((launch_tier<T0, 32, true, PSAI>(A, sa, pa, q0, n0, c + 0, out, ovf0.as<int32_t>(), c + 1, c + 3, 0, cfg,
+    SAI_TRY((launch_tier<T0, 32, WS_SHARED, PSAI>(A, sa, pa, q0, n0, c + 0, out, ovf0.as<int32_t>(), c + 1, c + 3, 0, cfg,
                                              st)));
     int hc[4];
     SAI_CUDA(cudaMemcpyAsync(hc, c, sizeof(hc), cudaMemcpyDeviceToHost, st));
     SAI_CUDA(cudaStreamSynchronize(st));
     if (hc[1] > 0) {
-        SAI_TRY((launch_tier<T1, 32, false, PSAI>(A, sa, pa, ovf0.as<int32_t>(), hc[1], c + 0, out,
-                                                     ovf1.as<int32_t>(), c + 2, c + 3, 1, cfg, st)));
+        // Up to two columns per SM a column's latency counts: the workspace in
+        // shared memory (12 columns of the 255^2 anisotropic operator 4.2 -> 3.4
+        // ms); up to 64 per SM the longest columns' latency still does: the
+        // hybrid form, nine columns per SM (tiers 1 and 2 of the Zipf matrix of
+        // order 20000, 7037 and 651 columns: build 48 -> 42 ms). With more, the
+        // number in flight counts: 260095 columns of the 512^2 operator took 461
+        // ms in the hybrid form, 282 ms in the global one (sixteen per SM).
+        const auto tier1 = hc[1] <= 2 * g_num_sms    ? launch_tier<T1, 32, WS_SHARED, PSAI>
+                           : hc[1] <= 64 * g_num_sms ? launch_tier<T1, 32, WS_HYBRID, PSAI>
+                                                     : launch_tier<T1, 32, WS_GLOBAL, PSAI>;
+        SAI_TRY(tier1(A, sa, pa, ovf0.as<int32_t>(), hc[1], c + 0, out, ovf1.as<int32_t>(), c + 2, c + 3, 1, cfg, st));
         SAI_CUDA(cudaMemcpyAsync(hc, c, sizeof(hc), cudaMemcpyDeviceToHost, st));
         SAI_CUDA(cudaStreamSynchronize(st));
         if (hc[2] > 0) {
             // tier 2 queues its overflows in ovf0 (tier 1's input, no longer read)
-            SAI_TRY((launch_tier<T2, 32, false, PSAI>(A, sa, pa, ovf1.as<int32_t>(), hc[2], c + 0, out,
-                                                         ovf0.as<int32_t>(), c + 12, c + 3, 2, cfg, st)));
+            const auto tier2 = hc[2] <= 8 * g_num_sms ? launch_tier<T2, 32, WS_HYBRID, PSAI>
+                                                      : launch_tier<T2, 32, WS_GLOBAL, PSAI>;
+            SAI_TRY(tier2(A, sa, pa, ovf1.as<int32_t>(), hc[2], c + 0, out, ovf0.as<int32_t>(), c + 12, c + 3, 2, cfg,
+                          st));
             int h3 = 0;
             SAI_CUDA(cudaMemcpyAsync(&h3, c + 12, sizeof(int), cudaMemcpyDeviceToHost, st));
             SAI_CUDA(cudaStreamSynchronize(st));
             if (h3 > 0) {
                 // tier 3 queues its overflows in ovf1 (tier 2's input, no longer read)
-                SAI_TRY((launch_tier<T3, 32, false, PSAI>(A, sa, pa, ovf0.as<int32_t>(), h3, c + 0, out,
+                SAI_TRY((launch_tier<T3, 32, WS_GLOBAL, PSAI>(A, sa, pa, ovf0.as<int32_t>(), h3, c + 0, out,
                                                              ovf1.as<int32_t>(), c + 14, c + 3, 3, cfg, st)));
                 int h4 = 0;
                 SAI_CUDA(cudaMemcpyAsync(&h4, c + 14, sizeof(int), cudaMemcpyDeviceToHost, st));
