@@ -68,6 +68,8 @@ __device__ __forceinline__ void spmm_work(const Dims& D, double nnz, int kact)
         kwork_add(D.site_spmm, 8.0 * (D.n + 1) + (4.0 + D.esz) * nnz + 2.0 * D.esz * D.n * kact, 2.0 * nnz * kact);
 }
 
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
 // ---------------------------------------------------------------- lists
 // Rebuild list (count + ascending indices) from mask; called by thread 0 of a
 // single-block kernel after the mask is final.
@@ -1277,6 +1279,13 @@ void pnl_apply2(int32_t n, int64_t ld, int k, const Ops<double>& A, const double
     k_pnl_scatter<<<SAI_GRID(tb), 256, 0, st>>>(n, ld, P1, list, Y2);
 }
 
+// ---------------------------------------------------------------- one cluster per system
+#include "bicg_cluster.cuh"
+
+// Up to this many systems of order CL_MAXN or less run in clusters; with more
+// the multi-kernel form fills the GPU and reads the matrices once for all.
+constexpr int CL_MAXK = CTRL;
+
 sai_status bicgstab_run(const Items& I, int k, const Ops<double>& A, const double* Bsd, double* Xsd, Sys& S,
                         double* pt, int* fl, int maxit, const Dims& D, cudaStream_t st)
 {
@@ -1286,6 +1295,21 @@ sai_status bicgstab_run(const Items& I, int k, const Ops<double>& A, const doubl
     const int ib = item_blocks(n > 0 ? n : 1, k);
     const int check_every = 4;
     int hflag = 0;
+    if (n > 0 && n <= CL_MAXN && k <= CL_MAXK) {
+        const ClMat a = {A.A.rp, A.A.ci, A.A.v, A.A.sp, A.A.sci, A.A.sv}, m = {A.M.rp, A.M.ci, A.M.v, A.M.sp, A.M.sci,
+                                                                              A.M.sv};
+        bool ran;
+        {
+            ProfScope ps(PROF_SPMM, st);
+            ran = cl_launch(a, m, k, n, ld, nullptr, nullptr, nullptr, nullptr, Bsd, Xsd, S.thr, maxit, S.iters,
+                            S.status, st);
+        }
+        if (ran) {
+            if (sai_prof_on()) k_cl_work<<<SAI_GRID(1), 1, 0, st>>>(k, S.iters, D);
+            SAI_CUDA(cudaGetLastError());
+            return SAI_OK;
+        }
+    }
     Buf vecs;
     SAI_TRY(vecs.alloc(sizeof(double) * blk * 8 + 8, st, true));
     double* r = vecs.as<double>();
@@ -1949,8 +1973,11 @@ __global__ void k_gm_cycle_start(int k, const double* nrm2, const int* cap, Sys 
 // vectors of the chunk and their sums are combined in warp order through
 // shared memory. A warp sums its 2 PD + 2 values together (warp_sum16: 16
 // shuffles and additions against five for each value): with a butterfly per
-// value the reduction was 40% of the kernel's FP64 instructions (50653 rows,
-// 8 systems, FP64: 85 us on average).
+// value the reduction was 40% of the kernel's FP64 instructions (FP64, 50653
+// rows, 8 systems: 85 -> 47 us on average; FP32, 262144 rows, 11 systems: 36
+// -> 33.5). Having the block that stores a (system, group)'s last partials
+// add the chunks up cost more than it saves the step kernel: a fence per item
+// took the FP32 pass to 77 us.
 // (Streaming each thread's row vectors through a two-stage
 // cp.async buffer in shared memory instead of registers measured slower:
 // 21.5 against 18.9 ms of the 64^3 step.)
@@ -2418,8 +2445,6 @@ __global__ void __launch_bounds__(IT_WARPS * 32) k_dc_update(Items I, T* __restr
 // stops (the host turns the flag into SAI_CUDA_ERROR).
 __device__ int d_pipe_err;
 constexpr uint32_t PIPE_POLLS = 1u << 21;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count)
 {

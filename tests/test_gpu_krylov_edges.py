@@ -74,3 +74,38 @@ def test_block_gmres_block_sizes(n, k, precision):
     assert st == sai.SAI_OK and stt == [0] * k
     R = np.linalg.norm(B - A @ X.cpu().numpy(), axis=0)
     assert np.all(R <= np.asarray(thr) + 1e-12 * norms), (R, thr)
+
+
+@pytest.mark.parametrize("n", [64, 65, 2560, 2561, 5121, 10303, 20480, 20481])
+@pytest.mark.parametrize("uneven", [False, True])
+def test_bicgstab_in_clusters(n, uneven):
+    """Orders around the cluster form's blocks (2560 rows; one, two, four or eight of them, more for fewer systems)
+    and its limit of 20480; rows of equal length (sliced ELL) and with every 64th row 40 entries longer (CSR). The
+    transposed solve too. Tolerance as above (||A|| grows to 7)."""
+    need_gpu()
+    sai = lib()
+    k = 20
+    A, M, B = _system(n, k, n + 1)
+    if uneven:
+        rng = np.random.default_rng(n)
+        rows = np.repeat(np.arange(0, n, 64), 40)
+        E = sp.coo_matrix((0.01 * rng.standard_normal(rows.size), (rows, rng.integers(0, n, rows.size))), shape=(n, n))
+        A = sp.csc_matrix(A + E)
+        A.sort_indices()
+    h = sai.split(to_dev(A), abs_tau=float("inf"))
+    P = sai.precond_from_csc(to_dev(M))
+    norms = np.linalg.norm(B, axis=0)
+    thr = list(norms * 10.0 ** -np.linspace(2, 10, k))
+    thr[3] = 2.0 * norms[3]
+    Bd = torch.as_tensor(B, device="cuda")
+    for transpose, Aop in ((False, A), (True, A.T)):
+        X, it, stt, st = sai.krylov_solve(h, P, Bd, thr, maxit=60, transpose=transpose)
+        assert st == sai.SAI_OK and stt == [0] * k and it[3] == 0
+        R = np.linalg.norm(B - Aop @ X.cpu().numpy(), axis=0)
+        assert np.all(R <= np.asarray(thr) + 1e-12 * norms), (R, thr)
+        for c in (0, 7, k - 1):
+            xc, itc, _, _ = sai.krylov_solve(h, P, Bd[:, c:c + 1].contiguous(), thr[c:c + 1], maxit=60,
+                                             transpose=transpose)
+            assert itc[0] == it[c] and torch.equal(xc[:, 0], X[:, c]), (n, c)
+    X, it, stt, st = sai.krylov_solve(h, P, Bd, thr, maxit=2)
+    assert st == sai.SAI_MAXITER and max(it) == 2 and stt[3] == sai.SAI_OK and stt[k - 1] == sai.SAI_MAXITER
