@@ -6,13 +6,21 @@
 #include "common.cuh"
 #include "saismw.h"
 
-// Ownership mode of a device buffer: handles returned to the user allocate
-// synchronously (cudaMalloc); buffers that live inside one call use the
-// stream-ordered pool of the call's stream.
+// Ownership mode of a device buffer. CALL: lives inside one call, from the
+// stream-ordered pool, freed on the call's stream. HANDLE: part of a handle
+// returned to the user; up to HANDLE_POOL_MAX bytes from the same pool (a
+// handle has ten to twelve buffers, and cudaMalloc / cudaFree of them took a
+// third of a small split or build), larger ones from cudaMalloc, so that a
+// large handle's memory goes back to the driver when it is destroyed. A
+// handle's creation synchronises its stream before it returns, and its
+// destruction waits for the device (as cudaFree does) before it frees: its
+// buffers may be used on any stream meanwhile.
+constexpr size_t HANDLE_POOL_MAX = size_t(32) << 20;
 struct Buf {
     void* p = nullptr;
     size_t bytes = 0;
     cudaStream_t st = nullptr;
+    int dev = -1;  // device of a HANDLE buffer from the pool (-1: another kind)
     bool async = false;
     Buf() = default;
     Buf(const Buf&) = delete;
@@ -47,7 +55,12 @@ sai_status sai_csc_residual_norms(int32_t n, const int64_t* cp, const int32_t* r
                                   const double* b, const double* x, double* out2_host, cudaStream_t st);
 
 // Handle internals --------------------------------------------------------
+// Waits for the device of a handle's pooled buffer.
+void sai_quiesce(const Buf& b);
+
 struct sai_split_s {
+    sai_split_s() = default;
+    ~sai_split_s() { sai_quiesce(J); }
     int32_t n = 0, s = 0, p = 0, p_keep = 0;
     double tau = 0.0, norm1 = 0.0;
     int64_t nnz_At = 0, nnz_U = 0;
@@ -60,6 +73,8 @@ struct sai_split_s {
 };
 
 struct sai_precond_s {
+    sai_precond_s() = default;
+    ~sai_precond_s() { sai_quiesce(loops); }
     int32_t n = 0;
     int64_t nnz = 0;
     int32_t n_c = 0, l_m = 0;

@@ -11,8 +11,13 @@ sai_status Buf::alloc(size_t nbytes, cudaStream_t s, bool use_async)
     st = s;
     async = use_async;
     bytes = nbytes;
+    dev = -1;
     if (nbytes == 0) return SAI_OK;
-    cudaError_t e = use_async ? cudaMallocAsync(&p, nbytes, s) : cudaMalloc(&p, nbytes);
+    const bool pool = use_async || nbytes <= HANDLE_POOL_MAX;
+    int d = -1;
+    if (pool && !use_async && cudaGetDevice(&d) != cudaSuccess) return SAI_CUDA_ERROR;
+    cudaError_t e = pool ? cudaMallocAsync(&p, nbytes, s) : cudaMalloc(&p, nbytes);
+    if (e == cudaSuccess) dev = d;
     if (e != cudaSuccess) {
         p = nullptr;
         sai_internal_note_cuda_error(e, "device allocation", __FILE__, __LINE__);
@@ -23,12 +28,29 @@ sai_status Buf::alloc(size_t nbytes, cudaStream_t s, bool use_async)
 
 void Buf::release()
 {
-    if (p) {
-        if (async) cudaFreeAsync(p, st);
-        else cudaFree(p);
+    if (p && async) {
+        cudaFreeAsync(p, st);
+    } else if (p && dev >= 0) {
+        // the creating stream may be gone: the device's legacy stream orders the free
+        int cur = -1;
+        const bool other = cudaGetDevice(&cur) == cudaSuccess && cur != dev && cudaSetDevice(dev) == cudaSuccess;
+        cudaFreeAsync(p, nullptr);
+        if (other) cudaSetDevice(cur);
+    } else if (p) {
+        cudaFree(p);
     }
     p = nullptr;
     bytes = 0;
+    dev = -1;
+}
+
+void sai_quiesce(const Buf& b)
+{
+    if (!b.p || b.async || b.dev < 0) return;
+    int cur = -1;
+    const bool other = cudaGetDevice(&cur) == cudaSuccess && cur != b.dev && cudaSetDevice(b.dev) == cudaSuccess;
+    cudaDeviceSynchronize();
+    if (other) cudaSetDevice(cur);
 }
 
 // ------------------------------------------------------------------ scan
