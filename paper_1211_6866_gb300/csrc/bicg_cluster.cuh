@@ -25,13 +25,14 @@ constexpr int CL_VECS = 9;
 constexpr int CL_SLOTS = 6;      // partial sums: rhat^T v; ||s||; t^T s, t^T t; ||r||, rhat^T r
 
 // CSR, or its sliced-ELL copy when sp is given (row0 = 0 then)
+template <class T>
 struct ClMat {
     const int64_t* rp;
     const int32_t* ci;
-    const double* v;
+    const T* v;
     const int64_t* sp;
     const int32_t* sci;
-    const double* sv;
+    const T* sv;
 };
 
 template <bool MULTI>
@@ -52,10 +53,20 @@ __device__ __forceinline__ uint32_t cl_map(uint32_t addr, uint32_t rank)
     return r;
 }
 
-__device__ __forceinline__ double cl_ld(uint32_t addr)
+template <class T>
+__device__ __forceinline__ T cl_ld(uint32_t addr);
+template <>
+__device__ __forceinline__ double cl_ld<double>(uint32_t addr)
 {
     double v;
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+    return v;
+}
+template <>
+__device__ __forceinline__ float cl_ld<float>(uint32_t addr)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
     return v;
 }
 
@@ -76,13 +87,12 @@ struct ClRows {
 
 // y (two rows per lane of the unit at local row lr0) = the rows of A times
 // the vector at shared offset `x` (bytes) of every block of the cluster
-template <bool MULTI>
-__device__ __forceinline__ void cl_spmv(const ClMat& A, const ClRows& W, const double* xs, uint32_t x, int lr0,
-                                        double (&y)[2])
+template <class T, bool MULTI>
+__device__ __forceinline__ void cl_spmv(const ClMat<T>& A, const ClRows& W, const T* xs, uint32_t x, int lr0, T (&y)[2])
 {
     const int lane = threadIdx.x & 31;
     const int32_t* ci[2];
-    const double* va[2];
+    const T* va[2];
     int len[2], stride;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -104,19 +114,19 @@ __device__ __forceinline__ void cl_spmv(const ClMat& A, const ClRows& W, const d
             len[h] = (int)(e - b);
             stride = 1;
         }
-        y[h] = 0.0;
+        y[h] = 0;
     }
     const int most = max(len[0], len[1]);
     for (int k0 = 0; k0 < most; k0 += 4) {
         int col[2][4];
-        double a[2][4], xv[2][4];
+        T a[2][4], xv[2][4];
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const bool in = k0 + u < len[h];
                 col[h][u] = in ? __ldg(ci[h] + (int64_t)(k0 + u) * stride) - W.row0 : 0;
-                a[h][u] = in ? __ldg(va[h] + (int64_t)(k0 + u) * stride) : 0.0;
+                a[h][u] = in ? __ldg(va[h] + (int64_t)(k0 + u) * stride) : T(0);
             }
 #pragma unroll
         for (int h = 0; h < 2; ++h)
@@ -124,7 +134,7 @@ __device__ __forceinline__ void cl_spmv(const ClMat& A, const ClRows& W, const d
             for (int u = 0; u < 4; ++u) {
                 if (MULTI) {
                     const uint32_t rk = __umulhi((uint32_t)col[h][u], W.inv);
-                    xv[h][u] = cl_ld(cl_map(x + 8u * ((uint32_t)col[h][u] - rk * (uint32_t)W.R), rk));
+                    xv[h][u] = cl_ld<T>(cl_map(x + (uint32_t)sizeof(T) * ((uint32_t)col[h][u] - rk * (uint32_t)W.R), rk));
                 } else {
                     xv[h][u] = xs[col[h][u]];
                 }
@@ -188,7 +198,7 @@ __device__ __forceinline__ bool cl_below(double x, double t)
 // system itself). B, X: the system's vectors at off[c] (c * ld without off).
 template <bool MULTI>
 __global__ void __launch_bounds__(CL_T, 1)
-k_bicg_cluster(ClMat A, ClMat M, int n1, int64_t ld, const int64_t* __restrict__ off, const int32_t* __restrict__ lens,
+k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64_t* __restrict__ off, const int32_t* __restrict__ lens,
                const int32_t* __restrict__ row0s, const int32_t* __restrict__ pick, int rmax, int umax,
                const double* __restrict__ B, double* __restrict__ X, const double* __restrict__ thr, int maxit,
                int* __restrict__ iters, int* __restrict__ status)
@@ -271,14 +281,14 @@ k_bicg_cluster(ClMat A, ClMat M, int n1, int64_t ld, const int64_t* __restrict__
         cl_barrier<MULTI>();
         for (int u = wid; u < W.units; u += NW) {
             double y[2];
-            cl_spmv<MULTI>(M, W, p, pa, u * CL_UNIT, y);
+            cl_spmv<double, MULTI>(M, W, p, pa, u * CL_UNIT, y);
             ph[u * CL_UNIT + lane] = y[0];
             ph[u * CL_UNIT + 32 + lane] = y[1];
         }
         cl_barrier<MULTI>();
         for (int u = wid; u < W.units; u += NW) {
             double y[2];
-            cl_spmv<MULTI>(A, W, ph, pha, u * CL_UNIT, y);
+            cl_spmv<double, MULTI>(A, W, ph, pha, u * CL_UNIT, y);
             const int i = u * CL_UNIT + lane;
             v[i] = y[0];
             v[i + 32] = y[1];
@@ -327,14 +337,14 @@ k_bicg_cluster(ClMat A, ClMat M, int n1, int64_t ld, const int64_t* __restrict__
         }
         for (int u = wid; u < W.units; u += NW) {
             double y[2];
-            cl_spmv<MULTI>(M, W, s, sa, u * CL_UNIT, y);
+            cl_spmv<double, MULTI>(M, W, s, sa, u * CL_UNIT, y);
             sh[u * CL_UNIT + lane] = y[0];
             sh[u * CL_UNIT + 32 + lane] = y[1];
         }
         cl_barrier<MULTI>();
         for (int u = wid; u < W.units; u += NW) {
             double y[2];
-            cl_spmv<MULTI>(A, W, sh, sha, u * CL_UNIT, y);
+            cl_spmv<double, MULTI>(A, W, sh, sha, u * CL_UNIT, y);
             const int i = u * CL_UNIT + lane;
             t[i] = y[0];
             t[i + 32] = y[1];
@@ -426,23 +436,17 @@ inline int cl_blocks(int k, int n)
     return C;
 }
 
-// Launches the kernel for k systems; false when the device refuses the shape.
-inline bool cl_launch(const ClMat& A, const ClMat& M, int k, int n, int64_t ld, const int64_t* off, const int32_t* lens,
-                      const int32_t* row0s, const int32_t* pick, const double* B, double* X, const double* thr,
-                      int maxit, int* iters, int* status, cudaStream_t st)
+// Launches kern with k clusters of C blocks; false when the device refuses the shape.
+template <class... Params, class... Args>
+bool cl_run(void (*kern)(Params...), int k, int C, int threads, size_t smem, cudaStream_t st, Args... args)
 {
-    const int C = cl_blocks(k, n);
-    const int rmax = ((n + C - 1) / C + CL_UNIT - 1) / CL_UNIT * CL_UNIT;
-    const int umax = (n + CL_UNIT - 1) / CL_UNIT;
-    const size_t smem = sizeof(double) * ((size_t)CL_VECS * rmax + (size_t)CL_SLOTS * umax);
-    const auto kern = C > 1 ? k_bicg_cluster<true> : k_bicg_cluster<false>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(SAI_GRID(k * C));
-    cfg.blockDim = dim3(CL_T);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at;
@@ -451,11 +455,22 @@ inline bool cl_launch(const ClMat& A, const ClMat& M, int k, int n, int64_t ld, 
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kern, A, M, n, ld, off, lens, row0s, pick, rmax, umax, B, X, thr, maxit, iters,
-                           status) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...) != cudaSuccess) {
         (void)cudaGetLastError();
         sai_count_grid_add(-1);
         return false;
     }
     return true;
+}
+
+inline bool cl_launch(const ClMat<double>& A, const ClMat<double>& M, int k, int n, int64_t ld, const int64_t* off,
+                      const int32_t* lens, const int32_t* row0s, const int32_t* pick, const double* B, double* X,
+                      const double* thr, int maxit, int* iters, int* status, cudaStream_t st)
+{
+    const int C = cl_blocks(k, n);
+    const int rmax = ((n + C - 1) / C + CL_UNIT - 1) / CL_UNIT * CL_UNIT;
+    const int umax = (n + CL_UNIT - 1) / CL_UNIT;
+    const size_t smem = sizeof(double) * ((size_t)CL_VECS * rmax + (size_t)CL_SLOTS * umax);
+    return cl_run(C > 1 ? k_bicg_cluster<true> : k_bicg_cluster<false>, k, C, CL_T, smem, st, A, M, n, ld, off, lens,
+                  row0s, pick, rmax, umax, B, X, thr, maxit, iters, status);
 }

@@ -1,0 +1,496 @@
+// gmres_cluster.cuh -- restarted GMRES of one system in one thread-block
+// cluster (included by krylov.cu inside its namespace).
+//
+// The Arnoldi process with delayed re-orthogonalisation of k_dc_dots /
+// k_dc_step / k_dc_update, restarts included, without leaving the kernel: at
+// small orders a step of the multi-kernel form is five launches that wait for
+// one another (45 us at 35937 rows and 6 systems, most of it latency). Block
+// b of the cluster owns rows [b R, (b + 1) R): the candidate u, t = M u, z =
+// A~ t and x live in its shared memory, its rows of the basis in global
+// memory (read by this block only, so from L1 while they fit). Products
+// gather u, t and x across the cluster; a step has four cluster barriers.
+// Every block keeps the small Hessenberg problem itself and runs the same
+// control arithmetic on the same sums, so no value has to be sent back.
+//
+// Sums: products accumulate in T along 16 rows per lane and component and up
+// a shuffle tree per GC_SUB rows, the rest in FP64 in a fixed order, as in
+// k_dc_dots. The Hessenberg columns are kept in T, the type k_dc_step uses
+// them in (its rotated columns are T values stored as FP64).
+
+constexpr int GC_T = 512;      // threads per block
+constexpr int GC_SUB = 2048;   // rows per partial sum
+constexpr int GC_MAXR = 6144;  // rows per block
+// orders up to which the form is used: FP32 vectors fill the shared memory
+// there; in FP64 the eight SMs' FP64 pipes are slower than all SMs' above
+constexpr int GC_MAXN32 = GC_MAXR * CL_MAXC, GC_MAXN64 = 10240;
+
+// Shared-memory layout of one block (bytes from the start).
+template <class T>
+struct GcLayout {
+    size_t u, t, z, x, hb, r, cs, sn, rc, s, c, parts, red, hp, g, y, bytes;
+    int nsub, ns;  // partial sums per block and slot; slots
+    GcLayout(int R, int m, int C)
+    {
+        nsub = (R + GC_SUB - 1) / GC_SUB;
+        ns = 2 * m + 4;
+        size_t o = 0;
+        auto take = [&](size_t b) {
+            const size_t at = o;
+            o += (b + 15) / 16 * 16;
+            return at;
+        };
+        u = take(sizeof(T) * R);
+        t = take(sizeof(T) * R);
+        z = take(sizeof(T) * R);
+        x = take(sizeof(T) * R);
+        hb = take(sizeof(T) * ((size_t)m * (m + 3) / 2));  // Hbar, column q: q + 2 entries from q (q + 3) / 2
+        r = take(sizeof(T) * ((size_t)m * (m + 1) / 2));   // R, column q: q + 1 entries from q (q + 1) / 2
+        cs = take(sizeof(T) * m);
+        sn = take(sizeof(T) * m);
+        rc = take(sizeof(T) * (m + 2));
+        s = take(sizeof(T) * (m + 1));
+        c = take(sizeof(T) * (m + 1));
+        parts = take(sizeof(double) * (size_t)C * nsub * ns);
+        red = take(sizeof(double) * ns);
+        hp = take(sizeof(double) * (m + 2));
+        g = take(sizeof(double) * (m + 2));
+        y = take(sizeof(T) * (m + 1));
+        bytes = o;
+    }
+};
+
+struct GcArgs {
+    int n, m, R, k;
+    int64_t ld, vs;
+    double tiny;
+    int nsub, ns;
+    uint32_t u, t, z, x, hb, r, cs, sn, rc, s, c, parts, red, hp, g, y;  // offsets of GcLayout
+};
+
+// two sums over the warp at once: lane 0 gets a's, lane 16 b's
+template <class T>
+__device__ __forceinline__ T gc_sum2(T a, T b)
+{
+    const bool up = (threadIdx.x & 16) != 0;
+    T w = (up ? b : a) + __shfl_xor_sync(SAI_FULL, up ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) w += __shfl_xor_sync(SAI_FULL, w, o);
+    return w;
+}
+
+template <class T>
+struct Comp;  // the components of a Vec<T>
+template <>
+struct Comp<float> {
+    __device__ static void fma4(const float4& a, const float4& b, float4& c)
+    {
+        c.x = fmaf(a.x, b.x, c.x);
+        c.y = fmaf(a.y, b.y, c.y);
+        c.z = fmaf(a.z, b.z, c.z);
+        c.w = fmaf(a.w, b.w, c.w);
+    }
+    __device__ static float sum(const float4& a) { return (a.x + a.y) + (a.z + a.w); }
+};
+template <>
+struct Comp<double> {
+    __device__ static void fma4(const double2& a, const double2& b, double2& c)
+    {
+        c.x = fma(a.x, b.x, c.x);
+        c.y = fma(a.y, b.y, c.y);
+    }
+    __device__ static double sum(const double2& a) { return a.x + a.y; }
+};
+
+// v_j = ia (u - V s), u <- ia (z - V c - dd v_j) on the block's rows: a thread
+// per row (W = 1) or per 16-byte piece
+template <class T, int W>
+__device__ __forceinline__ void gc_update(int j, int nrow, const T* V, int64_t vs, T* Vj, T* u, const T* z, const T* sT,
+                                          const T* cT, T ia, T dd)
+{
+    for (int r = (int)threadIdx.x * W; r < nrow; r += GC_T * W) {
+        T a_s[W], a_c[W];
+#pragma unroll
+        for (int e = 0; e < W; ++e) a_s[e] = a_c[e] = 0;
+        for (int i0 = 0; i0 < j; i0 += 8) {
+            T v[8][W];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const bool in = i0 + q < j;
+                const T* p = V + (int64_t)(in ? i0 + q : i0) * vs + r;
+                if (W == 1) {
+                    v[q][0] = in ? *p : T(0);
+                } else {
+                    const typename Vec<T>::type x = *reinterpret_cast<const typename Vec<T>::type*>(p);
+                    const T* xe = reinterpret_cast<const T*>(&x);
+#pragma unroll
+                    for (int e = 0; e < W; ++e) v[q][e] = in ? xe[e] : T(0);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (i0 + q < j) {
+                    const T s = sT[i0 + q], c = cT[i0 + q];
+#pragma unroll
+                    for (int e = 0; e < W; ++e) {
+                        a_s[e] = fma(s, v[q][e], a_s[e]);
+                        a_c[e] = fma(c, v[q][e], a_c[e]);
+                    }
+                }
+        }
+#pragma unroll
+        for (int e = 0; e < W; ++e)
+            if (r + e < nrow) {
+                const T v = ia * (u[r + e] - a_s[e]);
+                Vj[r + e] = v;
+                u[r + e] = ia * fma(-dd, v, z[r + e] - a_c[e]);
+            }
+    }
+}
+
+template <class T, bool MULTI>
+__global__ void __launch_bounds__(GC_T, 1)
+k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restrict__ B, T* __restrict__ X,
+                const double* __restrict__ thr, const int* __restrict__ cap, int* __restrict__ iters,
+                int* __restrict__ status, Dims D)
+{
+    using VT = typename Vec<T>::type;
+    constexpr int VW = Vec<T>::W;
+    constexpr int NW = GC_T / 32;
+    extern __shared__ __align__(16) unsigned char gsm[];
+    __shared__ double sh[3];  // alpha, d, 1 / alpha
+    __shared__ int flag;      // of the last control step: 0 go on, 1 the cycle ends
+    __shared__ int done;      // of the cycle's end: 0 another cycle, 1 stop
+    uint32_t rank = 0, nranks = 1;
+    if (MULTI) {
+        asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+        asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nranks));
+    }
+    const int c = blockIdx.x / nranks;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int m = P.m;
+    ClRows W;
+    W.n = P.n;
+    W.row0 = 0;
+    W.R = P.R;
+    W.base = (int)rank * W.R;
+    W.nrow = max(0, min(W.R, W.n - W.base));
+    W.inv = (uint32_t)((0x100000000ull + (unsigned)W.R - 1) / (unsigned)W.R);
+    W.units = (W.nrow + CL_UNIT - 1) / CL_UNIT;
+    W.unit0 = W.nunits = 0;
+    const int64_t o = (int64_t)c * P.ld + W.base;
+    T* V = Bv.V + o;  // the block's rows of v_0; v_i at V + i vs
+    T *u = (T*)(gsm + P.u), *t = (T*)(gsm + P.t), *z = (T*)(gsm + P.z), *x = (T*)(gsm + P.x);
+    T *hb = (T*)(gsm + P.hb), *Rm = (T*)(gsm + P.r), *cs = (T*)(gsm + P.cs), *sn = (T*)(gsm + P.sn), *rc = (T*)(gsm + P.rc);
+    T *sT = (T*)(gsm + P.s), *cT = (T*)(gsm + P.c), *yT = (T*)(gsm + P.y);
+    double *parts = (double*)(gsm + P.parts), *red = (double*)(gsm + P.red), *hp = (double*)(gsm + P.hp), *g = (double*)(gsm + P.g);
+    const uint32_t ua = smem_u32(u), ta = smem_u32(t), xa = smem_u32(x);
+    const double th = thr[c];
+    const int most = cap[c];
+    int it = 0, stat = ST_OK;         // the same in every thread of the cluster
+    double wsteps = 0.0, wj = 0.0;    // work: steps, and basis vectors over the steps
+    // a partial sum (lane 0: a, lane 16: b, from gc_sum2) to slots sl, sl + 1 of every block
+    auto put2 = [&](T w, int sl, int sub) {
+        const double v = (double)w;
+        double* p = parts + ((size_t)rank * P.nsub + sub) * P.ns + sl;
+        const double a = __shfl_sync(SAI_FULL, v, 0), b = __shfl_sync(SAI_FULL, v, 16);
+        if (MULTI) {
+            // lanes 0..7 send the first value, lanes 16..23 the second
+            const int to = lane & 15;
+            if (to < (int)nranks) cl_st(cl_map(smem_u32(p + (lane >> 4)), (uint32_t)to), lane < 16 ? a : b);
+        } else if (lane == 0) {
+            p[0] = a;
+            p[1] = b;
+        }
+    };
+    // red[t] = the sum of slot t over the blocks and their parts, t < cnt
+    auto total = [&](int cnt) {
+        for (int q = tid; q < cnt; q += GC_T) {
+            double a = 0.0;
+            for (int e = 0; e < (int)nranks * P.nsub; ++e) a += parts[(size_t)e * P.ns + q];
+            red[q] = a;
+        }
+        __syncthreads();
+    };
+    // the block's rows of u = r: ||r||^2 into slot 0 (slot 1: 0)
+    auto norm = [&]() {
+        for (int sub = wid; sub < P.nsub; sub += NW) {
+            VT acc = Vec<T>::zero();
+            const int r1 = min(W.nrow, (sub + 1) * GC_SUB);
+            for (int r = sub * GC_SUB + lane * VW; r < r1; r += 32 * VW) {
+                const VT a = *reinterpret_cast<const VT*>(u + r);
+                Comp<T>::fma4(a, a, acc);
+            }
+            put2(gc_sum2(Comp<T>::sum(acc), T(0)), 0, sub);
+        }
+    };
+    for (int i = tid; i < P.R; i += GC_T) {
+        u[i] = i < W.nrow ? B[o + i] : T(0);
+        t[i] = z[i] = x[i] = 0;
+    }
+    __syncthreads();
+    cl_barrier<MULTI>();  // every block of the cluster runs before its memory is written
+    norm();
+    cl_barrier<MULTI>();
+    for (;;) {
+        // cycle start: true residual norm, stop tests
+        total(1);
+        const double beta = sqrt(red[0]);
+        if (beta < th) {
+            stat = ST_OK;
+            break;
+        }
+        if (it >= most) {
+            stat = ST_MAXITER;
+            break;
+        }
+        int jd = 0;
+        bool conv = false;
+        for (int j = 0; j <= m; ++j) {
+            if (j < m) {  // the last step of a cycle needs no operator application
+                for (int q = wid; q < W.units; q += NW) {
+                    T y[2];
+                    cl_spmv<T, MULTI>(M, W, u, ua, q * CL_UNIT, y);
+                    t[q * CL_UNIT + lane] = y[0];
+                    t[q * CL_UNIT + 32 + lane] = y[1];
+                }
+                cl_barrier<MULTI>();
+                for (int q = wid; q < W.units; q += NW) {
+                    T y[2];
+                    cl_spmv<T, MULTI>(A, W, t, ta, q * CL_UNIT, y);
+                    z[q * CL_UNIT + lane] = y[0];
+                    z[q * CL_UNIT + 32 + lane] = y[1];
+                }
+                __syncthreads();
+            }
+            // s = V^T u, c = V^T z (slots 2 i, 2 i + 1), u^T u, u^T z (2 j, 2 j + 1)
+            for (int q = wid; q < (j + 1) * P.nsub; q += NW) {
+                const int i = q / P.nsub, sub = q - i * P.nsub;
+                const int r1 = min(W.nrow, (sub + 1) * GC_SUB);
+                VT as = Vec<T>::zero(), ac = Vec<T>::zero();
+                const T* v = i < j ? V + (int64_t)i * P.vs : u;
+#pragma unroll 4
+                for (int r = sub * GC_SUB + lane * VW; r < r1; r += 32 * VW) {
+                    const VT vv = *reinterpret_cast<const VT*>(v + r);
+                    Comp<T>::fma4(vv, *reinterpret_cast<const VT*>(u + r), as);
+                    Comp<T>::fma4(vv, *reinterpret_cast<const VT*>(z + r), ac);
+                }
+                put2(gc_sum2(Comp<T>::sum(as), Comp<T>::sum(ac)), 2 * i, sub);
+            }
+            cl_barrier<MULTI>();
+            total(2 * j + 2);
+            wsteps += 1.0;
+            wj += j;
+            // alpha, d = v_j^T z
+            if (wid == 0) {
+                double ss = 0.0, sc = 0.0;
+                for (int i = lane; i < j; i += 32) {
+                    ss = fma(red[2 * i], red[2 * i], ss);
+                    sc = fma(red[2 * i], red[2 * i + 1], sc);
+                }
+                const double w = gc_sum2(ss, sc);
+                ss = __shfl_sync(SAI_FULL, w, 0);
+                sc = __shfl_sync(SAI_FULL, w, 16);
+                const double uu = red[2 * j], a2 = uu - ss;
+                const bool ok = a2 > P.tiny * uu;
+                const double ial = ok ? rsqrt(a2) : 0.0;
+                if (lane == 0) {
+                    sh[0] = ok ? a2 * ial : 0.0;
+                    sh[1] = (red[2 * j + 1] - sc) * ial;
+                    sh[2] = ial;
+                }
+            }
+            for (int i = tid; i < j; i += GC_T) {
+                sT[i] = (T)red[2 * i];
+                cT[i] = (T)red[2 * i + 1];
+            }
+            __syncthreads();
+            const double al = sh[0], d = sh[1], ial = sh[2];
+            if (j >= 1) {
+                // column j - 1: first-pass coefficients + s, subdiagonal alpha
+                T* hc = hb + (size_t)(j - 1) * (j + 2) / 2;
+                for (int i = tid; i <= j; i += GC_T) hc[i] = rc[i] = (T)(i < j ? hp[i] + red[2 * i] : al);
+                __syncthreads();
+                if (tid == 0) {
+                    T ri = rc[0];
+                    for (int i = 0; i < j - 1; ++i) {
+                        const T b = rc[i + 1];
+                        rc[i] = cs[i] * ri + sn[i] * b;
+                        ri = -sn[i] * ri + cs[i] * b;
+                    }
+                    const T a = ri, b = rc[j];
+                    const T den = sqrt(a * a + b * b);
+                    const T cn = den == (T)0 ? (T)1 : a / den, s_ = den == (T)0 ? (T)0 : b / den;
+                    cs[j - 1] = cn;
+                    sn[j - 1] = s_;
+                    rc[j - 1] = cn * a + s_ * b;
+                    const T gj1 = (T)g[j - 1];
+                    const double gj = (double)(-s_ * gj1);
+                    g[j] = gj;
+                    g[j - 1] = (double)(cn * gj1);
+                    // bit 0: the cycle ends; bit 1: converged
+                    flag = fabs(gj) < th ? 3 : (al == 0.0 || it + 1 >= most || j >= m ? 1 : 0);
+                }
+                __syncthreads();
+                T* rr = Rm + (size_t)(j - 1) * j / 2;
+                for (int i = tid; i < j; i += GC_T) rr[i] = rc[i];
+                ++it;
+                jd = j;
+            } else {
+                if (tid == 0) {
+                    g[0] = al;  // v_0 = r0 / alpha
+                    flag = al == 0.0 ? 3 : 0;
+                }
+                __syncthreads();
+            }
+            const int f = flag;
+            if (f) {
+                conv = (f & 2) != 0;
+                break;
+            }
+            // first-pass coefficients of column j: ([c; d] - Hbar s) / alpha
+            for (int i = tid; i <= j; i += GC_T) {
+                T hs = 0;
+                for (int q = i > 0 ? i - 1 : 0; q < j; ++q) hs = fma(hb[(size_t)q * (q + 3) / 2 + i], sT[q], hs);
+                const double cz = i < j ? red[2 * i + 1] : d;
+                hp[i] = (cz - (double)hs) * ial;
+            }
+            if (W.nrow >= GC_T * 2)
+                gc_update<T, VW>(j, W.nrow, V, P.vs, V + (int64_t)j * P.vs, u, z, sT, cT, (T)ial, (T)d);
+            else
+                gc_update<T, 1>(j, W.nrow, V, P.vs, V + (int64_t)j * P.vs, u, z, sT, cT, (T)ial, (T)d);
+            cl_barrier<MULTI>();  // u is gathered next; red, hp, flag are rewritten after it
+        }
+        __syncthreads();
+        // y = R^{-1} g by one warp, column by column, with the pivots' reciprocals
+        if (wid == 0) {
+            constexpr int RPL = GM_MAXM / 32;
+            double w[RPL], rd[RPL];
+            bool bad = false;
+#pragma unroll
+            for (int q = 0; q < RPL; ++q) {
+                const int i = lane + 32 * q;
+                w[q] = i < jd ? g[i] : 0.0;
+                const double dg = i < jd ? (double)Rm[(size_t)i * (i + 1) / 2 + i] : 1.0;
+                bad |= dg == 0.0;
+                rd[q] = 1.0 / dg;
+            }
+            bad = __any_sync(SAI_FULL, bad);
+            for (int q = jd - 1; q >= 0; --q) {
+                double yq = 0.0;
+#pragma unroll
+                for (int e = 0; e < RPL; ++e)
+                    if (q / 32 == e) {
+                        if (lane == q % 32) w[e] *= rd[e];
+                        yq = __shfl_sync(SAI_FULL, w[e], q % 32);
+                    }
+#pragma unroll
+                for (int e = 0; e < RPL; ++e) {
+                    const int i = lane + 32 * e;
+                    if (32 * e < q && i < q) w[e] = fma(-(double)Rm[(size_t)q * (q + 1) / 2 + i], yq, w[e]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < RPL; ++q)
+                if (lane + 32 * q < jd) yT[lane + 32 * q] = (T)w[q];
+            if (lane == 0) done = bad;
+        }
+        __syncthreads();
+        if (done) {
+            stat = ST_BREAKDOWN;
+            break;
+        }
+        // u = V y, x += M u
+        for (int r = tid; r < W.nrow; r += GC_T) {
+            T a = 0;
+#pragma unroll 8
+            for (int i = 0; i < jd; ++i) a = fma(yT[i], V[(int64_t)i * P.vs + r], a);
+            u[r] = a;
+        }
+        cl_barrier<MULTI>();
+        for (int q = wid; q < W.units; q += NW) {
+            T y[2];
+            cl_spmv<T, MULTI>(M, W, u, ua, q * CL_UNIT, y);
+            x[q * CL_UNIT + lane] += y[0];
+            x[q * CL_UNIT + 32 + lane] += y[1];
+        }
+        if (conv) {
+            stat = ST_OK;
+            break;
+        }
+        if (it >= most) {
+            stat = ST_MAXITER;
+            break;
+        }
+        cl_barrier<MULTI>();
+        // u = r = b - A~ x
+        for (int q = wid; q < W.units; q += NW) {
+            T y[2];
+            cl_spmv<T, MULTI>(A, W, x, xa, q * CL_UNIT, y);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = q * CL_UNIT + 32 * h + lane;
+                u[r] = r < W.nrow ? B[o + r] - y[h] : T(0);
+            }
+        }
+        __syncthreads();
+        norm();
+        cl_barrier<MULTI>();
+    }
+    __syncthreads();
+    for (int i = tid; i < W.nrow; i += GC_T) X[o + i] = x[i];
+    if (rank == 0 && tid == 0) {
+        iters[c] = it;
+        status[c] = stat;
+        const double nz = D.nnzA + D.nnzM;
+        kwork_add(D.site_spmm, wsteps * (((4.0 + D.esz) * nz + 16.0 * (D.n + 1)) / P.k + 4.0 * D.esz * D.n),
+                  wsteps * 2.0 * nz);
+        kwork_add(D.site_dots, D.esz * D.n * (wj + 2.0 * wsteps), D.n * 4.0 * (wj + wsteps));
+        kwork_add(D.site_upd, D.esz * D.n * (wj + 4.0 * wsteps), D.n * (4.0 * wj + 6.0 * wsteps));
+    }
+    cl_barrier<MULTI>();  // no block leaves while another may read its memory
+}
+
+// Runs the k systems in clusters when they fit; false otherwise.
+template <class T>
+bool gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* Bs, T* Xs, const GmWork<T>& Wk, Sys& S,
+               const int* cap, const Dims& D, double tiny, cudaStream_t st)
+{
+    if (n < 1 || n > (sizeof(T) == 4 ? GC_MAXN32 : GC_MAXN64)) return false;
+    int C = 1;
+    while (C < CL_MAXC && (int64_t)C * GC_MAXR < n) C *= 2;
+    if ((int64_t)k * C > 4 * (int64_t)g_sms) return false;  // more systems: the multi-kernel form fills the GPU
+    while (C < CL_MAXC && (int64_t)2 * C * k <= (int64_t)g_sms * 7 / 8 && n / (2 * C) >= 2 * CL_UNIT) C *= 2;
+    const int R = ((n + C - 1) / C + CL_UNIT - 1) / CL_UNIT * CL_UNIT;
+    const GcLayout<T> L(R, m, C);
+    if (L.bytes > 220 * 1024) return false;
+    GcArgs P;
+    P.n = n;
+    P.m = m;
+    P.R = R;
+    P.k = k;
+    P.ld = ld;
+    P.vs = Wk.B.vs;
+    P.tiny = tiny;
+    P.nsub = L.nsub;
+    P.ns = L.ns;
+    P.u = (uint32_t)L.u;
+    P.t = (uint32_t)L.t;
+    P.z = (uint32_t)L.z;
+    P.x = (uint32_t)L.x;
+    P.hb = (uint32_t)L.hb;
+    P.r = (uint32_t)L.r;
+    P.cs = (uint32_t)L.cs;
+    P.sn = (uint32_t)L.sn;
+    P.rc = (uint32_t)L.rc;
+    P.s = (uint32_t)L.s;
+    P.c = (uint32_t)L.c;
+    P.parts = (uint32_t)L.parts;
+    P.red = (uint32_t)L.red;
+    P.hp = (uint32_t)L.hp;
+    P.g = (uint32_t)L.g;
+    P.y = (uint32_t)L.y;
+    const ClMat<T> a = {A.A.rp, A.A.ci, A.A.v, A.A.sp, A.A.sci, A.A.sv},
+                   mm = {A.M.rp, A.M.ci, A.M.v, A.M.sp, A.M.sci, A.M.sv};
+    const auto kern = C > 1 ? k_gmres_cluster<T, true> : k_gmres_cluster<T, false>;
+    return cl_run(kern, k, C, GC_T, L.bytes, st, a, mm, P, Wk.B, Bs, Xs, (const double*)S.thr, cap, S.iters, S.status, D);
+}

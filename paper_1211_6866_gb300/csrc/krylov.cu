@@ -1296,8 +1296,8 @@ sai_status bicgstab_run(const Items& I, int k, const Ops<double>& A, const doubl
     const int check_every = 4;
     int hflag = 0;
     if (n > 0 && n <= CL_MAXN && k <= CL_MAXK) {
-        const ClMat a = {A.A.rp, A.A.ci, A.A.v, A.A.sp, A.A.sci, A.A.sv}, m = {A.M.rp, A.M.ci, A.M.v, A.M.sp, A.M.sci,
-                                                                              A.M.sv};
+        const ClMat<double> a = {A.A.rp, A.A.ci, A.A.v, A.A.sp, A.A.sci, A.A.sv},
+                            m = {A.M.rp, A.M.ci, A.M.v, A.M.sp, A.M.sci, A.M.sv};
         bool ran;
         {
             ProfScope ps(PROF_SPMM, st);
@@ -2951,6 +2951,8 @@ void arnoldi_step(const Items& I, int k, const Ops<T>& A, const GmWork<T>& Wk, S
     }
 }
 
+#include "gmres_cluster.cuh"
+
 constexpr int GM_STEPS_PER_CHECK = 4;  // Arnoldi steps between host checks (one graph)
 constexpr int GM_LAUNCHES_PER_STEP = 5;
 
@@ -2969,6 +2971,10 @@ sai_status gmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs,
     if (cb > (int64_t)g_sms * 8) cb = (int64_t)g_sms * 8;
     // alpha^2 below 64 unit roundoffs of u^T u: u lies in span(V) to working accuracy
     const double tiny = 64.0 * (sizeof(T) == 4 ? 5.96e-8 : 1.11e-16);
+    {
+        ProfScope ps(D.site_dots, st);
+        if (gc_launch<T>(n, ld, k, m, A, Bs, Xs, Wk, S, cap, D, tiny, st)) return SAI_OK;
+    }
     // dynamic shared memory of the two kernels that stage Hbar / R (their
     // static shared memory counts against the same per-block limit)
     const size_t tri_smem = sizeof(double) * ((size_t)m * (m + 1) + m);

@@ -109,3 +109,42 @@ def test_bicgstab_in_clusters(n, uneven):
             assert itc[0] == it[c] and torch.equal(xc[:, 0], X[:, c]), (n, c)
     X, it, stt, st = sai.krylov_solve(h, P, Bd, thr, maxit=2)
     assert st == sai.SAI_MAXITER and max(it) == 2 and stt[3] == sai.SAI_OK and stt[k - 1] == sai.SAI_MAXITER
+
+
+@pytest.mark.parametrize("n,k,m,precision", [
+    (64, 1, 1, 0), (65, 3, 7, 1), (129, 40, 127, 0), (1000, 2, 127, 1), (2049, 5, 3, 0), (2304, 200, 20, 1),
+    (10240, 4, 30, 0), (10241, 4, 30, 0), (16385, 20, 12, 1), (33333, 3, 30, 1), (49152, 2, 8, 1), (49153, 2, 8, 1)])
+@pytest.mark.parametrize("uneven", [False, True])
+def test_gmres_in_clusters(n, k, m, precision, uneven):
+    """GMRES(m) around the limits of the cluster form (10240 rows in FP64, 49152 in FP32), with restart lengths from 1
+    to the largest, one to eight blocks per cluster and more systems than clusters at once; rows of equal length and
+    with every 64th row 40 entries longer. Tolerance as above; a system solved alone agrees within the two residuals."""
+    need_gpu()
+    sai = lib()
+    A, M, B = _system(n, k, 3 * n + m)
+    if uneven:
+        rng = np.random.default_rng(n)
+        rows = np.repeat(np.arange(0, n, 64), 40)
+        E = sp.coo_matrix((0.01 * rng.standard_normal(rows.size), (rows, rng.integers(0, n, rows.size))), shape=(n, n))
+        A = sp.csc_matrix(A + E)
+        A.sort_indices()
+    h = sai.split(to_dev(A), abs_tau=float("inf"))
+    P = sai.precond_from_csc(to_dev(M))
+    norms = np.linalg.norm(B, axis=0)
+    thr = list(norms * 10.0 ** -np.linspace(3, 10, k))
+    thr[0] = 2.0 * norms[0]
+    Bd = torch.as_tensor(B, device="cuda")
+    kw = dict(method=sai.GMRES, restart=m, maxit=400, precision=precision)
+    X, it, stt, st = sai.krylov_solve(h, P, Bd, thr, **kw)
+    assert st == sai.SAI_OK and stt == [0] * k and it[0] == 0
+    R = np.linalg.norm(B - A @ X.cpu().numpy(), axis=0)
+    assert np.all(R <= np.asarray(thr) + 1e-12 * norms), (R, thr)
+    c = k - 1
+    xc, itc, _, _ = sai.krylov_solve(h, P, Bd[:, c:c + 1].contiguous(), thr[c:c + 1], **kw)
+    # the blocks per cluster, and so the order of the sums, depend on k: the two solutions differ by A^-1 times their
+    # residuals, ||A^-1|| <= 1/2
+    dx = np.linalg.norm((xc[:, 0] - X[:, c]).cpu().numpy())
+    assert abs(itc[0] - it[c]) <= 1 and dx <= thr[c] + 1e-12 * norms[c]
+    if k > 1:
+        X, it, stt, st = sai.krylov_solve(h, P, Bd, thr, **dict(kw, maxit=2))
+        assert st == sai.SAI_MAXITER and stt[c] == sai.SAI_MAXITER and it[c] == 2 and stt[0] == sai.SAI_OK
