@@ -18,7 +18,7 @@
 
 constexpr int CL_T = 512;        // threads per block
 constexpr int CL_MAXR = 2560;    // rows per block: nine vectors of 20 KB
-constexpr int CL_MAXC = 8;       // blocks per cluster (the portable limit)
+constexpr int CL_MAXC = 8;       // blocks per cluster (the portable limit; 16 where all systems run at once)
 constexpr int CL_MAXN = CL_MAXR * CL_MAXC;
 constexpr int CL_UNIT = 64;      // rows per reduction unit
 constexpr int CL_VECS = 9;
@@ -116,33 +116,47 @@ __device__ __forceinline__ void cl_spmv(const ClMat<T>& A, const ClRows& W, cons
         }
         y[h] = 0;
     }
-    const int most = max(len[0], len[1]);
-    for (int k0 = 0; k0 < most; k0 += 4) {
-        int col[2][4];
-        T a[2][4], xv[2][4];
+    // BT entries of both rows at a time: their indices and values, then their
+    // gathers (from this block's shared memory when all of the warp's columns
+    // are its own, as most are on a grid: 30 cycles against 250 across the
+    // cluster), then their products in order
+    constexpr int BT = sizeof(T) == 4 ? 8 : 4;
+    // the warp's longest row: its votes below need every lane in every round
+    const int most = __reduce_max_sync(SAI_FULL, max(len[0], len[1]));
+    for (int k0 = 0; k0 < most; k0 += BT) {
+        int col[2][BT];
+        T a[2][BT], xv[2][BT];
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < BT; ++u) {
                 const bool in = k0 + u < len[h];
-                col[h][u] = in ? __ldg(ci[h] + (int64_t)(k0 + u) * stride) - W.row0 : 0;
+                col[h][u] = in ? __ldg(ci[h] + (int64_t)(k0 + u) * stride) - W.row0 : W.base;
                 a[h][u] = in ? __ldg(va[h] + (int64_t)(k0 + u) * stride) : T(0);
             }
+        bool own = true;
+        if (MULTI) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int u = 0; u < BT; ++u) own &= (unsigned)(col[h][u] - W.base) < (unsigned)W.R;
+            own = __all_sync(SAI_FULL, own);
+        }
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (MULTI) {
+            for (int u = 0; u < BT; ++u) {
+                if (!MULTI || own) {
+                    xv[h][u] = xs[col[h][u] - W.base];
+                } else {
                     const uint32_t rk = __umulhi((uint32_t)col[h][u], W.inv);
                     xv[h][u] = cl_ld<T>(cl_map(x + (uint32_t)sizeof(T) * ((uint32_t)col[h][u] - rk * (uint32_t)W.R), rk));
-                } else {
-                    xv[h][u] = xs[col[h][u]];
                 }
             }
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < BT; ++u)
                 if (k0 + u < len[h]) y[h] = fma(a[h][u], xv[h][u], y[h]);
     }
 }
@@ -172,17 +186,20 @@ __device__ __forceinline__ double cl_total(const double* parts, int slot, int ps
         return warp_sum(h);
     }
     for (int u = lane; u < nunits; u += 32) two_add(h, l, p[u]);
-#pragma unroll 1
-    for (int o = 16; o > 0; o >>= 1) {
-        const double h2 = __shfl_xor_sync(SAI_FULL, h, o), l2 = __shfl_xor_sync(SAI_FULL, l, o);
-        // the partner adds the same pair the other way round: take the lower lane's order in both
+    // up the tree the sums alone wait for one another; a node's rounding error
+    // is known to all 2^(level + 1) lanes below it and enters with that weight,
+    // so that the lanes' errors add up to the tree's (exact scalings)
+    double w = 0.5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1, w *= 0.5) {
+        const double h2 = __shfl_xor_sync(SAI_FULL, h, o);
         const bool lo = (lane & o) == 0;
-        double a = lo ? h : h2, b = lo ? l : l2;
-        two_add(a, b, lo ? h2 : h);
+        double a = lo ? h : h2, e = 0.0;  // the same operands in the same order in both lanes
+        two_add(a, e, lo ? h2 : h);
         h = a;
-        l = b + (lo ? l2 : l);
+        l = fma(w, e, l);
     }
-    return h + l;
+    return h + warp_sum(l);
 }
 
 // sqrt(x) < t, with the root taken only where the squares are too close to tell
@@ -204,7 +221,7 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64
                int* __restrict__ iters, int* __restrict__ status)
 {
     extern __shared__ __align__(16) double sm[];
-    __shared__ double sc[4];  // alpha, omega, beta of the running iteration
+    __shared__ double sc[5];  // alpha, omega, beta, alpha / (omega rho), rho of the running iteration
     __shared__ int flag;      // 0 go on (first iteration), 1 half step, then stop, 2 stop, 3 go on
     uint32_t rank = 0, nranks = 1;
     if (MULTI) {
@@ -245,7 +262,7 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64
     }
     cl_barrier<MULTI>();
     // control values live in warp 0, lane by lane the same
-    double rho = 0.0, rho_old = 0.0, alpha = 1.0, omega = 1.0;
+    double rho = 0.0, omega = 1.0;
     int it = 0, stat = ST_OK;
     // the next iteration's start: count it, test rho, form beta
     auto next = [&]() {
@@ -258,7 +275,8 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64
             stat = ST_BREAKDOWN;
             return 2;
         }
-        if (lane == 0) sc[2] = it == 1 ? 0.0 : (rho / rho_old) * (alpha / omega);
+        // beta = (rho / rho_old) (alpha / omega), the quotient without rho formed earlier
+        if (lane == 0) sc[2] = it == 1 ? 0.0 : rho * sc[3];
         return 0;
     };
     if (wid == 0) {
@@ -302,8 +320,11 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64
                 stat = ST_BREAKDOWN;
                 f = 2;
             } else {
-                alpha = rho / rv;
-                if (lane == 0) sc[0] = alpha;
+                const double alpha = rho / rv;
+                if (lane == 0) {
+                    sc[0] = alpha;
+                    sc[4] = rho;
+                }
             }
             if (lane == 0) flag = f;
         }
@@ -369,6 +390,8 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64
         if (flag == 2) break;
         {
             const double al = sc[0], om = sc[1];
+            // beside the update, in the warp that has the fewest units
+            if (wid == NW - 1 && lane == 0) sc[3] = al / (om * sc[4]);
             for (int u = wid; u < W.units; u += NW) {
                 const int i = u * CL_UNIT + lane;
                 double rv[2];
@@ -393,7 +416,6 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64
             } else if (omega == 0.0) {
                 stat = ST_BREAKDOWN;
             } else {
-                rho_old = rho;
                 rho = rhr;
                 f = next();
                 if (f == 0) f = 3;  // p is formed with beta from here on
@@ -436,6 +458,29 @@ inline int cl_blocks(int k, int n)
     return C;
 }
 
+// true when the GPU holds k clusters of 16 blocks of kern at once
+template <class... Params>
+bool cl_fits16(void (*kern)(Params...), int k, int threads, size_t smem)
+{
+    if (16 * (int64_t)k > g_sms) return false;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16u * (unsigned)k);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 16;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int most = 0;
+    const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&most, kern, &cfg) == cudaSuccess;
+    if (!ok) (void)cudaGetLastError();
+    return ok && most >= k;
+}
+
 // Launches kern with k clusters of C blocks; false when the device refuses the shape.
 template <class... Params, class... Args>
 bool cl_run(void (*kern)(Params...), int k, int C, int threads, size_t smem, cudaStream_t st, Args... args)
@@ -467,10 +512,21 @@ inline bool cl_launch(const ClMat<double>& A, const ClMat<double>& M, int k, int
                       const int32_t* lens, const int32_t* row0s, const int32_t* pick, const double* B, double* X,
                       const double* thr, int maxit, int* iters, int* status, cudaStream_t st)
 {
-    const int C = cl_blocks(k, n);
-    const int rmax = ((n + C - 1) / C + CL_UNIT - 1) / CL_UNIT * CL_UNIT;
+    int C = cl_blocks(k, n);
     const int umax = (n + CL_UNIT - 1) / CL_UNIT;
-    const size_t smem = sizeof(double) * ((size_t)CL_VECS * rmax + (size_t)CL_SLOTS * umax);
+    int rmax = 0;
+    size_t smem = 0;
+    auto shape = [&](int blocks) {
+        C = blocks;
+        rmax = ((n + C - 1) / C + CL_UNIT - 1) / CL_UNIT * CL_UNIT;
+        smem = sizeof(double) * ((size_t)CL_VECS * rmax + (size_t)CL_SLOTS * umax);
+    };
+    shape(C);
+    // from 512 rows per block on the FP64 pipe outweighs the barriers
+    if (C == CL_MAXC && rmax >= 512) {
+        shape(16);
+        if (!cl_fits16(k_bicg_cluster<true>, k, CL_T, smem)) shape(CL_MAXC);
+    }
     return cl_run(C > 1 ? k_bicg_cluster<true> : k_bicg_cluster<false>, k, C, CL_T, smem, st, A, M, n, ld, off, lens,
                   row0s, pick, rmax, umax, B, X, thr, maxit, iters, status);
 }

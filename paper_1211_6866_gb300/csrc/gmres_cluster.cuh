@@ -18,6 +18,7 @@
 // them in (its rotated columns are T values stored as FP64).
 
 constexpr int GC_T = 512;      // threads per block
+constexpr int GC_UT = GC_T - 32;  // of them in the update; the last warp runs the Givens rotations meanwhile
 constexpr int GC_SUB = 2048;   // rows per partial sum
 constexpr int GC_MAXR = 6144;  // rows per block
 // orders up to which the form is used: FP32 vectors fill the shared memory
@@ -107,7 +108,7 @@ template <class T, int W>
 __device__ __forceinline__ void gc_update(int j, int nrow, const T* V, int64_t vs, T* Vj, T* u, const T* z, const T* sT,
                                           const T* cT, T ia, T dd)
 {
-    for (int r = (int)threadIdx.x * W; r < nrow; r += GC_T * W) {
+    for (int r = (int)threadIdx.x * W; r < nrow; r += GC_UT * W) {
         T a_s[W], a_c[W];
 #pragma unroll
         for (int e = 0; e < W; ++e) a_s[e] = a_c[e] = 0;
@@ -309,56 +310,58 @@ k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restri
                 // column j - 1: first-pass coefficients + s, subdiagonal alpha
                 T* hc = hb + (size_t)(j - 1) * (j + 2) / 2;
                 for (int i = tid; i <= j; i += GC_T) hc[i] = rc[i] = (T)(i < j ? hp[i] + red[2 * i] : al);
-                __syncthreads();
-                if (tid == 0) {
+                ++it;
+                jd = j;
+            }
+            __syncthreads();
+            // column j - 1 rotated, the residual estimate and the stop tests by
+            // the last warp, whose result the others need only after the update
+            // (a stopping step's update is not used)
+            if (tid == GC_UT) {
+                if (j >= 1) {
+                    T* rr = Rm + (size_t)(j - 1) * j / 2;
                     T ri = rc[0];
                     for (int i = 0; i < j - 1; ++i) {
-                        const T b = rc[i + 1];
-                        rc[i] = cs[i] * ri + sn[i] * b;
-                        ri = -sn[i] * ri + cs[i] * b;
+                        const T b = rc[i + 1], ci = cs[i], si = sn[i];
+                        rr[i] = ci * ri + si * b;
+                        ri = -si * ri + ci * b;
                     }
                     const T a = ri, b = rc[j];
                     const T den = sqrt(a * a + b * b);
                     const T cn = den == (T)0 ? (T)1 : a / den, s_ = den == (T)0 ? (T)0 : b / den;
                     cs[j - 1] = cn;
                     sn[j - 1] = s_;
-                    rc[j - 1] = cn * a + s_ * b;
+                    rr[j - 1] = cn * a + s_ * b;
                     const T gj1 = (T)g[j - 1];
                     const double gj = (double)(-s_ * gj1);
                     g[j] = gj;
                     g[j - 1] = (double)(cn * gj1);
                     // bit 0: the cycle ends; bit 1: converged
-                    flag = fabs(gj) < th ? 3 : (al == 0.0 || it + 1 >= most || j >= m ? 1 : 0);
-                }
-                __syncthreads();
-                T* rr = Rm + (size_t)(j - 1) * j / 2;
-                for (int i = tid; i < j; i += GC_T) rr[i] = rc[i];
-                ++it;
-                jd = j;
-            } else {
-                if (tid == 0) {
+                    flag = fabs(gj) < th ? 3 : (al == 0.0 || it >= most || j >= m ? 1 : 0);
+                } else {
                     g[0] = al;  // v_0 = r0 / alpha
                     flag = al == 0.0 ? 3 : 0;
                 }
-                __syncthreads();
-            }
-            const int f = flag;
-            if (f) {
-                conv = (f & 2) != 0;
-                break;
             }
             // first-pass coefficients of column j: ([c; d] - Hbar s) / alpha
-            for (int i = tid; i <= j; i += GC_T) {
+            for (int i = tid; i <= j && tid < GC_UT; i += GC_UT) {
                 T hs = 0;
                 for (int q = i > 0 ? i - 1 : 0; q < j; ++q) hs = fma(hb[(size_t)q * (q + 3) / 2 + i], sT[q], hs);
                 const double cz = i < j ? red[2 * i + 1] : d;
                 hp[i] = (cz - (double)hs) * ial;
             }
-            if (W.nrow >= GC_T * 2)
-                gc_update<T, VW>(j, W.nrow, V, P.vs, V + (int64_t)j * P.vs, u, z, sT, cT, (T)ial, (T)d);
-            else
-                gc_update<T, 1>(j, W.nrow, V, P.vs, V + (int64_t)j * P.vs, u, z, sT, cT, (T)ial, (T)d);
+            if (tid < GC_UT) {
+                if (W.nrow >= GC_T * 2)
+                    gc_update<T, VW>(j, W.nrow, V, P.vs, V + (int64_t)j * P.vs, u, z, sT, cT, (T)ial, (T)d);
+                else
+                    gc_update<T, 1>(j, W.nrow, V, P.vs, V + (int64_t)j * P.vs, u, z, sT, cT, (T)ial, (T)d);
+            }
             cl_barrier<MULTI>();  // u is gathered next; red, hp, flag are rewritten after it
+            const int f = flag;
+            if (f) {
+                conv = (f & 2) != 0;
+                break;
+            }
         }
         __syncthreads();
         // y = R^{-1} g by one warp, column by column, with the pivots' reciprocals
@@ -460,7 +463,12 @@ bool gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* Bs, T*
     while (C < CL_MAXC && (int64_t)C * GC_MAXR < n) C *= 2;
     if ((int64_t)k * C > 4 * (int64_t)g_sms) return false;  // more systems: the multi-kernel form fills the GPU
     while (C < CL_MAXC && (int64_t)2 * C * k <= (int64_t)g_sms * 7 / 8 && n / (2 * C) >= 2 * CL_UNIT) C *= 2;
-    const int R = ((n + C - 1) / C + CL_UNIT - 1) / CL_UNIT * CL_UNIT;
+    auto rows = [&](int blocks) { return ((n + blocks - 1) / blocks + CL_UNIT - 1) / CL_UNIT * CL_UNIT; };
+    // from 512 rows per block on the work outweighs the barriers
+    if (C == CL_MAXC && rows(C) >= 512 &&
+        cl_fits16(k_gmres_cluster<T, true>, k, GC_T, GcLayout<T>(rows(16), m, 16).bytes))
+        C = 16;
+    const int R = rows(C);
     const GcLayout<T> L(R, m, C);
     if (L.bytes > 220 * 1024) return false;
     GcArgs P;
