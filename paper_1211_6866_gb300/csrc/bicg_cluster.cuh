@@ -24,15 +24,18 @@ constexpr int CL_UNIT = 64;      // rows per reduction unit
 constexpr int CL_VECS = 9;
 constexpr int CL_SLOTS = 6;      // partial sums: rhat^T v; ||s||; t^T s, t^T t; ||r||, rhat^T r
 
-// CSR, or its sliced-ELL copy when sp is given (row0 = 0 then)
+// A matrix in slices of 32 rows, entries column-major within a slice (slice q
+// at sp[q] .. sp[q + 1]). With ord, the rows of each block are sorted by
+// length and position i holds row ord[i] of its block (-1: none): slices of
+// unsorted rows of unequal length would be mostly padding, and a CSR row per
+// lane takes a memory transaction per lane and entry (a 2000-row power-law
+// system forward and backward, build included: 15.6 ms with CSR rows, 12.1 ms sorted).
 template <class T>
 struct ClMat {
-    const int64_t* rp;
-    const int32_t* ci;
-    const T* v;
     const int64_t* sp;
     const int32_t* sci;
     const T* sv;
+    const int32_t* ord;
 };
 
 template <bool MULTI>
@@ -78,92 +81,206 @@ __device__ __forceinline__ void cl_st(uint32_t addr, double v)
 // The block's part of the system.
 struct ClRows {
     int n, R, base, nrow;  // order, rows per block, first row, rows of this block
-    int row0;              // the system's first row in the matrices
     uint32_t inv;          // ceil(2^32 / R): row / R = umulhi(row, inv) for rows below 2^32 / R
     int units;             // units of this block
     int unit0;             // index of its first unit in the system
     int nunits;            // units of the system
 };
 
-// y (two rows per lane of the unit at local row lr0) = the rows of A times
-// the vector at shared offset `x` (bytes) of every block of the cluster
-template <class T, bool MULTI>
-__device__ __forceinline__ void cl_spmv(const ClMat<T>& A, const ClRows& W, const T* xs, uint32_t x, int lr0, T (&y)[2])
+__device__ __forceinline__ ClRows cl_rows(int n, int R, int rank)
 {
+    ClRows W;
+    W.n = n;
+    W.R = R;
+    W.base = rank * R;
+    W.nrow = max(0, min(R, n - W.base));
+    W.inv = (uint32_t)((0x100000000ull + (unsigned)R - 1) / (unsigned)R);
+    W.units = (W.nrow + CL_UNIT - 1) / CL_UNIT;
+    W.unit0 = W.base / CL_UNIT;
+    W.nunits = (n + CL_UNIT - 1) / CL_UNIT;
+    return W;
+}
+
+// dst = A src (MODE 0), dst += A src (1) or dst = b - A src (2) on the block's
+// rows, src spread over the cluster. A warp takes 64 positions, two per lane.
+// Not inlined: the kernels are one long pass per iteration, and its copies
+// would push that pass out of the instruction cache. Ends without a barrier.
+template <class T, bool MULTI, int MODE>
+__device__ __noinline__ void cl_apply(const ClMat<T>* Am, const ClRows* Wp, const T* src, T* dst, const T* b)
+{
+    const ClMat<T> A = *Am;
+    const ClRows W = *Wp;
     const int lane = threadIdx.x & 31;
-    const int32_t* ci[2];
-    const T* va[2];
-    int len[2], stride;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int lr = lr0 + 32 * h + lane;  // local row
-        if (A.sp) {
-            const int sl = (W.base + lr0) / 32 + h;
-            const bool in = lr0 + 32 * h < W.nrow;
-            const int64_t b = in ? A.sp[sl] : 0, e = in ? A.sp[sl + 1] : 0;
-            ci[h] = A.sci + b + lane;
-            va[h] = A.sv + b + lane;
-            len[h] = (int)(e - b) / 32;
-            stride = 32;
-        } else {
-            const bool in = lr < W.nrow;
-            const int64_t g = (int64_t)W.row0 + W.base + lr;
-            const int64_t b = in ? A.rp[g] : 0, e = in ? A.rp[g + 1] : 0;
-            ci[h] = A.ci + b;
-            va[h] = A.v + b;
-            len[h] = (int)(e - b);
-            stride = 1;
-        }
-        y[h] = 0;
-    }
+    const uint32_t sa = smem_u32(src);
+    __builtin_assume(__isShared(src));
+    __builtin_assume(__isShared(dst));
     // BT entries of both rows at a time: their indices and values, then their
     // gathers (from this block's shared memory when all of the warp's columns
     // are its own, as most are on a grid: 30 cycles against 250 across the
     // cluster), then their products in order
     constexpr int BT = sizeof(T) == 4 ? 8 : 4;
-    // the warp's longest row: its votes below need every lane in every round
-    const int most = __reduce_max_sync(SAI_FULL, max(len[0], len[1]));
-    for (int k0 = 0; k0 < most; k0 += BT) {
-        int col[2][BT];
-        T a[2][BT], xv[2][BT];
+#pragma unroll 1
+    for (int q = threadIdx.x >> 5; q < W.units; q += blockDim.x >> 5) {
+        const int32_t* ci[2];
+        const T* va[2];
+        int len[2], row[2];
+        T y[2];
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int u = 0; u < BT; ++u) {
-                const bool in = k0 + u < len[h];
-                col[h][u] = in ? __ldg(ci[h] + (int64_t)(k0 + u) * stride) - W.row0 : W.base;
-                a[h][u] = in ? __ldg(va[h] + (int64_t)(k0 + u) * stride) : T(0);
-            }
-        bool own = true;
-        if (MULTI) {
+        for (int h = 0; h < 2; ++h) {
+            const int at = q * CL_UNIT + 32 * h;
+            const bool in = at < W.nrow;
+            const int64_t sl = (W.base + at) / 32;
+            const int64_t e0 = in ? A.sp[sl] : 0, e1 = in ? A.sp[sl + 1] : 0;
+            row[h] = !in ? -1 : A.ord ? A.ord[W.base + at + lane] : (at + lane < W.nrow ? at + lane : -1);
+            ci[h] = A.sci + e0 + lane;
+            va[h] = A.sv + e0 + lane;
+            len[h] = (int)(e1 - e0) / 32;
+            y[h] = 0;
+        }
+        const int most = max(len[0], len[1]);  // the same in every lane: the votes below need all of them
+#pragma unroll 1
+        for (int k0 = 0; k0 < most; k0 += BT) {
+            int col[2][BT];
+            T a[2][BT], xv[2][BT];
 #pragma unroll
             for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int u = 0; u < BT; ++u) own &= (unsigned)(col[h][u] - W.base) < (unsigned)W.R;
-            own = __all_sync(SAI_FULL, own);
+                for (int u = 0; u < BT; ++u) {
+                    const bool in = k0 + u < len[h];
+                    col[h][u] = in ? __ldg(ci[h] + (k0 + u) * 32) : -1;
+                    a[h][u] = in ? __ldg(va[h] + (k0 + u) * 32) : T(0);
+                }
+            bool own = true;
+            if (MULTI) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int u = 0; u < BT; ++u) own &= col[h][u] < 0 || (unsigned)(col[h][u] - W.base) < (unsigned)W.R;
+                own = __all_sync(SAI_FULL, own);
+            }
+            if (!MULTI || own) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int u = 0; u < BT; ++u) xv[h][u] = src[max(col[h][u], W.base) - W.base];
+            } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int u = 0; u < BT; ++u) {
+                        const uint32_t j = (uint32_t)max(col[h][u], 0), rk = __umulhi(j, W.inv);
+                        xv[h][u] = cl_ld<T>(cl_map(sa + (uint32_t)sizeof(T) * (j - rk * (uint32_t)W.R), rk));
+                    }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int u = 0; u < BT; ++u)
+                    if (col[h][u] >= 0) y[h] = fma(a[h][u], xv[h][u], y[h]);
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int u = 0; u < BT; ++u) {
-                if (!MULTI || own) {
-                    xv[h][u] = xs[col[h][u] - W.base];
-                } else {
-                    const uint32_t rk = __umulhi((uint32_t)col[h][u], W.inv);
-                    xv[h][u] = cl_ld<T>(cl_map(x + (uint32_t)sizeof(T) * ((uint32_t)col[h][u] - rk * (uint32_t)W.R), rk));
-                }
+            if (row[h] >= 0) {
+                if (MODE == 0) dst[row[h]] = y[h];
+                else if (MODE == 1) dst[row[h]] += y[h];
+                else dst[row[h]] = b[row[h]] - y[h];
             }
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int u = 0; u < BT; ++u)
-                if (k0 + u < len[h]) y[h] = fma(a[h][u], xv[h][u], y[h]);
     }
+}
+
+// ---- the sorted form of a CSR matrix for blocks of R rows (grid: a block per block of rows)
+__global__ void __launch_bounds__(512) k_cl_sort(int n, int R, const int64_t* __restrict__ rp, int32_t* __restrict__ ord,
+                                                 int64_t* __restrict__ cnt)
+{
+    constexpr int NB = 1024;  // bins by length, the longest first
+    __shared__ int off[NB];
+    __shared__ int ws[16];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int base = blockIdx.x * R, nrow = max(0, min(R, n - base));
+    auto bin = [&](int r) {  // steps of 96 from 512 entries on: an order of 49152 fits
+        const int len = (int)(rp[base + r + 1] - rp[base + r]);
+        return NB - 1 - min(NB - 1, len < 512 ? len : 512 + (len - 512) / 96);
+    };
+    for (int i = tid; i < NB; i += 512) off[i] = 0;
+    for (int i = tid; i < R; i += 512) ord[base + i] = -1;
+    __syncthreads();
+    for (int r = tid; r < nrow; r += 512) atomicAdd(&off[bin(r)], 1);
+    __syncthreads();
+    // exclusive prefix over the bins, two per thread
+    const int c0 = off[2 * tid], c1 = off[2 * tid + 1];
+    int incl = c0 + c1;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(SAI_FULL, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) ws[wid] = incl;
+    __syncthreads();
+    int before = incl - c0 - c1;
+    for (int w = 0; w < wid; ++w) before += ws[w];
+    off[2 * tid] = before;
+    off[2 * tid + 1] = before + c0;
+    __syncthreads();
+    // rows of equal length land in any order: a row's product does not depend on its place
+    for (int r = tid; r < nrow; r += 512) ord[base + atomicAdd(&off[bin(r)], 1)] = r;
+    __syncthreads();
+    for (int s = wid; s < R / 32; s += 16) {
+        const int r = ord[base + 32 * s + lane];
+        const unsigned len = r >= 0 ? (unsigned)(rp[base + r + 1] - rp[base + r]) : 0u;
+        const unsigned w = __reduce_max_sync(SAI_FULL, len);
+        if (lane == 0) cnt[base / 32 + s] = (int64_t)w * 32;
+    }
+}
+
+template <class T>
+__global__ void k_cl_fill(int nsl, int R, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                          const T* __restrict__ v, const int32_t* __restrict__ ord, const int64_t* __restrict__ sp,
+                          int32_t* __restrict__ sci, T* __restrict__ sv)
+{
+    const int sl = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
+    if (sl >= nsl) return;
+    const int base = sl * 32 / R * R;
+    const int r = ord[(int64_t)sl * 32 + lane];
+    const int64_t b = sp[sl], w = (sp[sl + 1] - b) / 32;
+    const int64_t r0 = r >= 0 ? rp[base + r] : 0, len = r >= 0 ? rp[base + r + 1] - r0 : 0;
+    for (int64_t k = 0; k < w; ++k) {
+        const int64_t q = b + k * 32 + lane;
+        sci[q] = k < len ? ci[r0 + k] : -1;  // not multiplied: its factor may be infinite
+        sv[q] = k < len ? v[r0 + k] : T(0);
+    }
+}
+
+// The matrix of a cluster kernel: its sliced-ELL copy, or the sorted form of
+// its CSR arrays for C blocks of R rows in buf (live until the kernel has run).
+template <class T>
+sai_status cl_matrix(const Mat<T>& X, int n, int R, int C, Buf (&buf)[4], ClMat<T>& out, cudaStream_t st)
+{
+    if (X.sp) {
+        out = {X.sp, X.sci, X.sv, nullptr};
+        return SAI_OK;
+    }
+    const int nsl = C * (R / 32);
+    Buf cnt;
+    SAI_TRY(cnt.alloc(sizeof(int64_t) * (size_t)nsl, st, true));
+    SAI_TRY(buf[0].alloc(sizeof(int32_t) * (size_t)C * R, st, true));
+    SAI_TRY(buf[1].alloc(sizeof(int64_t) * ((size_t)nsl + 1), st, true));
+    k_cl_sort<<<SAI_GRID(C), 512, 0, st>>>(n, R, X.rp, buf[0].as<int32_t>(), cnt.as<int64_t>());
+    SAI_TRY(sai_scan_counts_i64(cnt.as<int64_t>(), buf[1].as<int64_t>(), nsl, st));
+    int64_t total = 0;
+    SAI_CUDA(cudaMemcpyAsync(&total, buf[1].as<int64_t>() + nsl, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    SAI_CUDA(cudaStreamSynchronize(st));
+    SAI_TRY(buf[2].alloc(sizeof(int32_t) * (size_t)(total > 0 ? total : 1), st, true));
+    SAI_TRY(buf[3].alloc(sizeof(T) * (size_t)(total > 0 ? total : 1), st, true));
+    k_cl_fill<T><<<SAI_GRID(sai_div_up((int64_t)nsl * 32, 256)), 256, 0, st>>>(
+        nsl, R, X.rp, X.ci, X.v, buf[0].as<int32_t>(), buf[1].as<int64_t>(), buf[2].as<int32_t>(), buf[3].as<T>());
+    SAI_CUDA(cudaGetLastError());
+    out = {buf[1].as<int64_t>(), buf[2].as<int32_t>(), buf[3].as<T>(), buf[0].as<int32_t>()};
+    return SAI_OK;
 }
 
 // Stores a unit's partial sum in slot `slot` of every block of the cluster.
 template <bool MULTI>
-__device__ __forceinline__ void cl_put(double v, int slot, int unit, double* parts, int pstride, int nranks)
+__device__ __noinline__ void cl_put(double v, int slot, int unit, double* parts, int pstride, int nranks)
 {
     v = warp_sum(v);
     const int lane = threadIdx.x & 31;
@@ -176,7 +293,7 @@ __device__ __forceinline__ void cl_put(double v, int slot, int unit, double* par
 }
 
 // The sum of a slot's units (one warp; the same bits in every block).
-__device__ __forceinline__ double cl_total(const double* parts, int slot, int pstride, int nunits, bool comp)
+__device__ __noinline__ double cl_total(const double* parts, int slot, int pstride, int nunits, bool comp)
 {
     const int lane = threadIdx.x & 31;
     const double* p = parts + slot * pstride;
@@ -211,12 +328,10 @@ __device__ __forceinline__ bool cl_below(double x, double t)
     return sqrt(x) < t;
 }
 
-// One cluster per system (blockIdx.x / cluster size = index in `pick`, or the
-// system itself). B, X: the system's vectors at off[c] (c * ld without off).
+// One cluster per system (blockIdx.x / cluster size). B, X: the system's vectors at c * ld.
 template <bool MULTI>
 __global__ void __launch_bounds__(CL_T, 1)
-k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64_t* __restrict__ off, const int32_t* __restrict__ lens,
-               const int32_t* __restrict__ row0s, const int32_t* __restrict__ pick, int rmax, int umax,
+k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n, int64_t ld, int rmax, int umax,
                const double* __restrict__ B, double* __restrict__ X, const double* __restrict__ thr, int maxit,
                int* __restrict__ iters, int* __restrict__ status)
 {
@@ -228,25 +343,21 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64
         asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
         asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nranks));
     }
-    const int q = blockIdx.x / nranks;
-    const int c = pick ? pick[q] : q;
+    const int c = blockIdx.x / nranks;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     constexpr int NW = CL_T / 32;
-    ClRows W;
-    W.n = lens ? lens[c] : n1;
-    W.row0 = row0s ? row0s[c] : 0;
-    W.R = ((W.n + (int)nranks - 1) / (int)nranks + CL_UNIT - 1) / CL_UNIT * CL_UNIT;
-    W.base = (int)rank * W.R;
-    W.nrow = max(0, min(W.R, W.n - W.base));
-    W.inv = (uint32_t)((0x100000000ull + (unsigned)W.R - 1) / (unsigned)W.R);
-    W.units = (W.nrow + CL_UNIT - 1) / CL_UNIT;
-    W.unit0 = W.base / CL_UNIT;
-    W.nunits = (W.n + CL_UNIT - 1) / CL_UNIT;
-    const int64_t o = (off ? off[c] : (int64_t)c * ld) + W.base;
+    __shared__ ClRows W;
+    __shared__ ClMat<double> As, Ms;
+    if (threadIdx.x == 0) {
+        W = cl_rows(n, rmax, (int)rank);
+        As = A;
+        Ms = M;
+    }
+    __syncthreads();
+    const int64_t o = (int64_t)c * ld + W.base;
     double *p = sm, *ph = p + rmax, *s = ph + rmax, *sh = s + rmax;  // gathered by the cluster
     double *r = sh + rmax, *rh = r + rmax, *v = rh + rmax, *t = v + rmax, *x = t + rmax;
     double* parts = x + rmax;  // [slot][unit]
-    const uint32_t pa = smem_u32(p), pha = smem_u32(ph), sa = smem_u32(s), sha = smem_u32(sh);
     const double th = thr[c];
     // r = rhat = p = b (the rows past the end are zero and stay so), x = 0
     for (int i = threadIdx.x; i < rmax; i += CL_T) {
@@ -297,20 +408,13 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64
                 }
         }
         cl_barrier<MULTI>();
-        for (int u = wid; u < W.units; u += NW) {
-            double y[2];
-            cl_spmv<double, MULTI>(M, W, p, pa, u * CL_UNIT, y);
-            ph[u * CL_UNIT + lane] = y[0];
-            ph[u * CL_UNIT + 32 + lane] = y[1];
-        }
+        cl_apply<double, MULTI, 0>(&Ms, &W, p, ph, nullptr);
         cl_barrier<MULTI>();
+        cl_apply<double, MULTI, 0>(&As, &W, ph, v, nullptr);
+        __syncthreads();
         for (int u = wid; u < W.units; u += NW) {
-            double y[2];
-            cl_spmv<double, MULTI>(A, W, ph, pha, u * CL_UNIT, y);
             const int i = u * CL_UNIT + lane;
-            v[i] = y[0];
-            v[i + 32] = y[1];
-            cl_put<MULTI>(fma(rh[i + 32], y[1], rh[i] * y[0]), 0, W.unit0 + u, parts, umax, (int)nranks);
+            cl_put<MULTI>(fma(rh[i + 32], v[i + 32], rh[i] * v[i]), 0, W.unit0 + u, parts, umax, (int)nranks);
         }
         cl_barrier<MULTI>();
         if (wid == 0) {
@@ -356,21 +460,14 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n1, int64_t ld, const int64
             stat = ST_OK;
             break;
         }
-        for (int u = wid; u < W.units; u += NW) {
-            double y[2];
-            cl_spmv<double, MULTI>(M, W, s, sa, u * CL_UNIT, y);
-            sh[u * CL_UNIT + lane] = y[0];
-            sh[u * CL_UNIT + 32 + lane] = y[1];
-        }
+        cl_apply<double, MULTI, 0>(&Ms, &W, s, sh, nullptr);
         cl_barrier<MULTI>();
+        cl_apply<double, MULTI, 0>(&As, &W, sh, t, nullptr);
+        __syncthreads();
         for (int u = wid; u < W.units; u += NW) {
-            double y[2];
-            cl_spmv<double, MULTI>(A, W, sh, sha, u * CL_UNIT, y);
             const int i = u * CL_UNIT + lane;
-            t[i] = y[0];
-            t[i + 32] = y[1];
-            cl_put<MULTI>(fma(y[1], s[i + 32], y[0] * s[i]), 2, W.unit0 + u, parts, umax, (int)nranks);
-            cl_put<MULTI>(fma(y[1], y[1], y[0] * y[0]), 3, W.unit0 + u, parts, umax, (int)nranks);
+            cl_put<MULTI>(fma(t[i + 32], s[i + 32], t[i] * s[i]), 2, W.unit0 + u, parts, umax, (int)nranks);
+            cl_put<MULTI>(fma(t[i + 32], t[i + 32], t[i] * t[i]), 3, W.unit0 + u, parts, umax, (int)nranks);
         }
         cl_barrier<MULTI>();
         if (wid == 0) {
@@ -508,9 +605,9 @@ bool cl_run(void (*kern)(Params...), int k, int C, int threads, size_t smem, cud
     return true;
 }
 
-inline bool cl_launch(const ClMat<double>& A, const ClMat<double>& M, int k, int n, int64_t ld, const int64_t* off,
-                      const int32_t* lens, const int32_t* row0s, const int32_t* pick, const double* B, double* X,
-                      const double* thr, int maxit, int* iters, int* status, cudaStream_t st)
+// BiCGStab of k systems in clusters; *ran is false when the device refuses the shape.
+inline sai_status cl_bicgstab(const Ops<double>& A, int k, int n, int64_t ld, const double* B, double* X,
+                              const double* thr, int maxit, int* iters, int* status, cudaStream_t st, bool* ran)
 {
     int C = cl_blocks(k, n);
     const int umax = (n + CL_UNIT - 1) / CL_UNIT;
@@ -527,6 +624,12 @@ inline bool cl_launch(const ClMat<double>& A, const ClMat<double>& M, int k, int
         shape(16);
         if (!cl_fits16(k_bicg_cluster<true>, k, CL_T, smem)) shape(CL_MAXC);
     }
-    return cl_run(C > 1 ? k_bicg_cluster<true> : k_bicg_cluster<false>, k, C, CL_T, smem, st, A, M, n, ld, off, lens,
-                  row0s, pick, rmax, umax, B, X, thr, maxit, iters, status);
+    ClMat<double> a, m;
+    Buf ab[4], mb[4];
+    *ran = false;
+    if (cl_matrix(A.A, n, rmax, C, ab, a, st) != SAI_OK || cl_matrix(A.M, n, rmax, C, mb, m, st) != SAI_OK)
+        return SAI_OK;  // no memory for the sorted forms: the kernels below need none
+    *ran = cl_run(C > 1 ? k_bicg_cluster<true> : k_bicg_cluster<false>, k, C, CL_T, smem, st, a, m, n, ld, rmax, umax,
+                  B, X, thr, maxit, iters, status);
+    return SAI_OK;
 }

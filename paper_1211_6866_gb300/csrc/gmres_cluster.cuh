@@ -169,22 +169,20 @@ k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restri
     const int c = blockIdx.x / nranks;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int m = P.m;
-    ClRows W;
-    W.n = P.n;
-    W.row0 = 0;
-    W.R = P.R;
-    W.base = (int)rank * W.R;
-    W.nrow = max(0, min(W.R, W.n - W.base));
-    W.inv = (uint32_t)((0x100000000ull + (unsigned)W.R - 1) / (unsigned)W.R);
-    W.units = (W.nrow + CL_UNIT - 1) / CL_UNIT;
-    W.unit0 = W.nunits = 0;
+    __shared__ ClRows W;
+    __shared__ ClMat<T> As, Ms;
+    if (tid == 0) {
+        W = cl_rows(P.n, P.R, (int)rank);
+        As = A;
+        Ms = M;
+    }
+    __syncthreads();
     const int64_t o = (int64_t)c * P.ld + W.base;
     T* V = Bv.V + o;  // the block's rows of v_0; v_i at V + i vs
     T *u = (T*)(gsm + P.u), *t = (T*)(gsm + P.t), *z = (T*)(gsm + P.z), *x = (T*)(gsm + P.x);
     T *hb = (T*)(gsm + P.hb), *Rm = (T*)(gsm + P.r), *cs = (T*)(gsm + P.cs), *sn = (T*)(gsm + P.sn), *rc = (T*)(gsm + P.rc);
     T *sT = (T*)(gsm + P.s), *cT = (T*)(gsm + P.c), *yT = (T*)(gsm + P.y);
     double *parts = (double*)(gsm + P.parts), *red = (double*)(gsm + P.red), *hp = (double*)(gsm + P.hp), *g = (double*)(gsm + P.g);
-    const uint32_t ua = smem_u32(u), ta = smem_u32(t), xa = smem_u32(x);
     const double th = thr[c];
     const int most = cap[c];
     int it = 0, stat = ST_OK;         // the same in every thread of the cluster
@@ -248,19 +246,9 @@ k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restri
         bool conv = false;
         for (int j = 0; j <= m; ++j) {
             if (j < m) {  // the last step of a cycle needs no operator application
-                for (int q = wid; q < W.units; q += NW) {
-                    T y[2];
-                    cl_spmv<T, MULTI>(M, W, u, ua, q * CL_UNIT, y);
-                    t[q * CL_UNIT + lane] = y[0];
-                    t[q * CL_UNIT + 32 + lane] = y[1];
-                }
+                cl_apply<T, MULTI, 0>(&Ms, &W, u, t, nullptr);
                 cl_barrier<MULTI>();
-                for (int q = wid; q < W.units; q += NW) {
-                    T y[2];
-                    cl_spmv<T, MULTI>(A, W, t, ta, q * CL_UNIT, y);
-                    z[q * CL_UNIT + lane] = y[0];
-                    z[q * CL_UNIT + 32 + lane] = y[1];
-                }
+                cl_apply<T, MULTI, 0>(&As, &W, t, z, nullptr);
                 __syncthreads();
             }
             // s = V^T u, c = V^T z (slots 2 i, 2 i + 1), u^T u, u^T z (2 j, 2 j + 1)
@@ -410,12 +398,7 @@ k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restri
             u[r] = a;
         }
         cl_barrier<MULTI>();
-        for (int q = wid; q < W.units; q += NW) {
-            T y[2];
-            cl_spmv<T, MULTI>(M, W, u, ua, q * CL_UNIT, y);
-            x[q * CL_UNIT + lane] += y[0];
-            x[q * CL_UNIT + 32 + lane] += y[1];
-        }
+        cl_apply<T, MULTI, 1>(&Ms, &W, u, x, nullptr);
         if (conv) {
             stat = ST_OK;
             break;
@@ -425,16 +408,7 @@ k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restri
             break;
         }
         cl_barrier<MULTI>();
-        // u = r = b - A~ x
-        for (int q = wid; q < W.units; q += NW) {
-            T y[2];
-            cl_spmv<T, MULTI>(A, W, x, xa, q * CL_UNIT, y);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r = q * CL_UNIT + 32 * h + lane;
-                u[r] = r < W.nrow ? B[o + r] - y[h] : T(0);
-            }
-        }
+        cl_apply<T, MULTI, 2>(&As, &W, x, u, B + o);  // r = b - A~ x
         __syncthreads();
         norm();
         cl_barrier<MULTI>();
@@ -453,15 +427,16 @@ k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restri
     cl_barrier<MULTI>();  // no block leaves while another may read its memory
 }
 
-// Runs the k systems in clusters when they fit; false otherwise.
+// Runs the k systems in clusters when they fit (*ran).
 template <class T>
-bool gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* Bs, T* Xs, const GmWork<T>& Wk, Sys& S,
-               const int* cap, const Dims& D, double tiny, cudaStream_t st)
+sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* Bs, T* Xs, const GmWork<T>& Wk, Sys& S,
+               const int* cap, const Dims& D, double tiny, cudaStream_t st, bool* ran)
 {
-    if (n < 1 || n > (sizeof(T) == 4 ? GC_MAXN32 : GC_MAXN64)) return false;
+    *ran = false;
+    if (n < 1 || n > (sizeof(T) == 4 ? GC_MAXN32 : GC_MAXN64)) return SAI_OK;
     int C = 1;
     while (C < CL_MAXC && (int64_t)C * GC_MAXR < n) C *= 2;
-    if ((int64_t)k * C > 4 * (int64_t)g_sms) return false;  // more systems: the multi-kernel form fills the GPU
+    if ((int64_t)k * C > 4 * (int64_t)g_sms) return SAI_OK;  // more systems: the multi-kernel form fills the GPU
     while (C < CL_MAXC && (int64_t)2 * C * k <= (int64_t)g_sms * 7 / 8 && n / (2 * C) >= 2 * CL_UNIT) C *= 2;
     auto rows = [&](int blocks) { return ((n + blocks - 1) / blocks + CL_UNIT - 1) / CL_UNIT * CL_UNIT; };
     // from 512 rows per block on the work outweighs the barriers
@@ -470,7 +445,7 @@ bool gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* Bs, T*
         C = 16;
     const int R = rows(C);
     const GcLayout<T> L(R, m, C);
-    if (L.bytes > 220 * 1024) return false;
+    if (L.bytes > 220 * 1024) return SAI_OK;
     GcArgs P;
     P.n = n;
     P.m = m;
@@ -497,8 +472,10 @@ bool gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* Bs, T*
     P.hp = (uint32_t)L.hp;
     P.g = (uint32_t)L.g;
     P.y = (uint32_t)L.y;
-    const ClMat<T> a = {A.A.rp, A.A.ci, A.A.v, A.A.sp, A.A.sci, A.A.sv},
-                   mm = {A.M.rp, A.M.ci, A.M.v, A.M.sp, A.M.sci, A.M.sv};
-    const auto kern = C > 1 ? k_gmres_cluster<T, true> : k_gmres_cluster<T, false>;
-    return cl_run(kern, k, C, GC_T, L.bytes, st, a, mm, P, Wk.B, Bs, Xs, (const double*)S.thr, cap, S.iters, S.status, D);
+    ClMat<T> a, mm;
+    Buf ab[4], mb[4];
+    if (cl_matrix(A.A, n, R, C, ab, a, st) != SAI_OK || cl_matrix(A.M, n, R, C, mb, mm, st) != SAI_OK) return SAI_OK;
+    *ran = cl_run(C > 1 ? k_gmres_cluster<T, true> : k_gmres_cluster<T, false>, k, C, GC_T, L.bytes, st, a, mm, P, Wk.B, Bs,
+                  Xs, (const double*)S.thr, cap, S.iters, S.status, D);
+    return SAI_OK;
 }

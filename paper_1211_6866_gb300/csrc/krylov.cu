@@ -1296,13 +1296,10 @@ sai_status bicgstab_run(const Items& I, int k, const Ops<double>& A, const doubl
     const int check_every = 4;
     int hflag = 0;
     if (n > 0 && n <= CL_MAXN && k <= CL_MAXK) {
-        const ClMat<double> a = {A.A.rp, A.A.ci, A.A.v, A.A.sp, A.A.sci, A.A.sv},
-                            m = {A.M.rp, A.M.ci, A.M.v, A.M.sp, A.M.sci, A.M.sv};
         bool ran;
         {
             ProfScope ps(PROF_SPMM, st);
-            ran = cl_launch(a, m, k, n, ld, nullptr, nullptr, nullptr, nullptr, Bsd, Xsd, S.thr, maxit, S.iters,
-                            S.status, st);
+            SAI_TRY(cl_bicgstab(A, k, n, ld, Bsd, Xsd, S.thr, maxit, S.iters, S.status, st, &ran));
         }
         if (ran) {
             if (sai_prof_on()) k_cl_work<<<SAI_GRID(1), 1, 0, st>>>(k, S.iters, D);
@@ -2972,8 +2969,10 @@ sai_status gmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs,
     // alpha^2 below 64 unit roundoffs of u^T u: u lies in span(V) to working accuracy
     const double tiny = 64.0 * (sizeof(T) == 4 ? 5.96e-8 : 1.11e-16);
     {
+        bool ran;
         ProfScope ps(D.site_dots, st);
-        if (gc_launch<T>(n, ld, k, m, A, Bs, Xs, Wk, S, cap, D, tiny, st)) return SAI_OK;
+        SAI_TRY(gc_launch<T>(n, ld, k, m, A, Bs, Xs, Wk, S, cap, D, tiny, st, &ran));
+        if (ran) return SAI_OK;
     }
     // dynamic shared memory of the two kernels that stage Hbar / R (their
     // static shared memory counts against the same per-block limit)

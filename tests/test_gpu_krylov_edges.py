@@ -148,3 +148,32 @@ def test_gmres_in_clusters(n, k, m, precision, uneven):
     if k > 1:
         X, it, stt, st = sai.krylov_solve(h, P, Bd, thr, **dict(kw, maxit=2))
         assert st == sai.SAI_MAXITER and stt[c] == sai.SAI_MAXITER and it[c] == 2 and stt[0] == sai.SAI_OK
+
+
+@pytest.mark.parametrize("n,k", [(700, 150), (4999, 20), (20480, 3)])
+@pytest.mark.parametrize("method", ["bicgstab", "gmres", "gmres32"])
+def test_cluster_rows_sorted_by_length(n, k, method):
+    """A few rows far longer than the rest (around the steps of the sort by length: 511, 512, 607, 608 entries, and n),
+    in the first, a middle and the last block. Their off-diagonal sums stay below 0.3, so the tolerance above holds."""
+    need_gpu()
+    sai = lib()
+    A, M, B = _system(n, k, n)
+    rng = np.random.default_rng(n)
+    rows, cols = [], []
+    for i, length in zip((0, 1, n // 2, n // 2 + 1, n - 1), (511, 512, 607, 608, n)):
+        cols.append(rng.permutation(n)[:length])
+        rows.append(np.full(length, i))
+    val = np.concatenate([0.3 / r.size * rng.uniform(-1, 1, r.size) for r in rows])
+    A = sp.csc_matrix(A + sp.coo_matrix((val, (np.concatenate(rows), np.concatenate(cols))), shape=(n, n)))
+    A.sort_indices()
+    h = sai.split(to_dev(A), abs_tau=float("inf"))
+    P = sai.precond_from_csc(to_dev(M))
+    norms = np.linalg.norm(B, axis=0)
+    kw = {"bicgstab": {}, "gmres": dict(method=sai.GMRES, restart=20),
+          "gmres32": dict(method=sai.GMRES, restart=20, precision=1)}[method]
+    for transpose, Aop in ((False, A), (True, A.T)):
+        X, it, stt, st = sai.krylov_solve(h, P, torch.as_tensor(B, device="cuda"), list(1e-9 * norms), maxit=100,
+                                          transpose=transpose, **kw)
+        assert st == sai.SAI_OK and stt == [0] * k
+        R = np.linalg.norm(B - Aop @ X.cpu().numpy(), axis=0)
+        assert np.all(R <= 1e-9 * norms + 1e-12 * norms), R / norms
