@@ -9,13 +9,13 @@
 //   one its matrix alone would give.
 // Solve: the sum(s_i + 1) right-hand sides [b_i, u_i1 .. u_is_i] are Krylov
 //   systems of different lengths, stored one after another. Work items are
-//   (system, chunk of BR rows), listed once for the whole batch: one block
-//   each in the SpMV (a thread per row), one warp each in the vector kernels;
+//   (system, chunk of rows), listed once for the whole batch: a block per
+//   chunk of SB rows in the SpMV, a warp per chunk of BR in the vector kernels;
 //   a stopped system's items return at once. Inner products are summed per
-//   item in a fixed order and per system over its items in order. The
-//   control kernels run one warp (or thread) per system. Groups of 8
-//   iterations are captured once as a CUDA graph and replayed, with one host
-//   check of the "any system still running" flag per group.
+//   BR rows in a fixed order and per system over those in order. alpha and
+//   omega are formed by the last SpMV block of a system, the other control
+//   values by a warp per system: 9 launches per iteration. The loop is one
+//   CUDA graph (or groups of 8 iterations with a host check after each).
 // SMW: one block per matrix solves its s_i x s_i system (partial pivoting);
 //   then x_i = yhat_i - What_i z_i, and rr per matrix.
 #include <math.h>
@@ -31,6 +31,9 @@ namespace {
 
 constexpr int BR = 256;  // rows per work item (one block, one thread per row)
 
+constexpr int SB = 2048;     // rows per SpMV item
+constexpr int SB_CAP = 24576;  // doubles of the staged vector: 192 KB beside the item's results
+
 enum { B_OK = 0, B_MAXITER = 5, B_BREAKDOWN = 6 };  // same values as sai_status
 
 // System table of the batch (device arrays).
@@ -44,6 +47,23 @@ struct BSys {
     const int32_t* it_r0;   // first local row of item q
     const int32_t* nsm;     // systems of c's matrix (s + 1)
     int32_t nitems;
+    // SpMV items: SB rows of a system, as a block of the matrices' sorted rows
+    const int32_t* sp_sys;
+    const int32_t* sp_blk;
+    const int4* blk;  // (first row, rows, row0 of the matrix, first local row) per block
+    int32_t nsp;
+    int32_t ncap;  // longest vector that is staged in shared memory
+};
+
+#include "sorted_rows.cuh"
+
+// A~ or M of the batch, its rows sorted by length within blocks of SB
+struct BMat {
+    const int64_t* sp;
+    const int32_t* sci;
+    const double* sv;
+    const int32_t* ord;
+    int stage;  // gathers from shared memory where the vector fits
 };
 
 // Algorithmic work of the batched BiCGStab, added per system by the control
@@ -87,34 +107,147 @@ __device__ __forceinline__ double sys_sum(const BSys& Y, const double* part, int
     return warp_sum(a);
 }
 
-// y_c = A~ x_c (mode 0) for the systems with flag set, over their own block;
-// A~ in CSR with global row / column indices (block diagonal).
-__global__ void __launch_bounds__(BR) k_b_spmv(BSys Y, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                               const double* __restrict__ v, const double* __restrict__ X,
-                                               double* __restrict__ Yv, const int* flags)
+// alpha = rho / rhat^T v of system c (one warp)
+__device__ void b_alpha(const BSys& Y, const double* part, const BState& S, const BWork& Wk, int c)
 {
-    for (int32_t q = blockIdx.x; q < Y.nitems; q += gridDim.x) {
-        const int c = Y.it_sys[q];
-        if (!flags[c]) continue;
-        const int64_t i = Y.it_r0[q] + threadIdx.x;
-        if (i >= Y.len[c]) continue;
-        const int64_t o = Y.off[c];
-        const int32_t r0 = Y.row0[c];
-        const int64_t b = rp[r0 + i], e = rp[r0 + i + 1];
-        double acc = 0.0;
-        for (int64_t q0 = b; q0 < e; q0 += 8) {
-            int32_t col[8];
-            double a[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                col[u] = q0 + u < e ? ci[q0 + u] - r0 : 0;
-                a[u] = q0 + u < e ? v[q0 + u] : 0.0;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) acc = fma(a[u], X[o + col[u]], acc);
+    const double rv = sys_sum(Y, part, c);
+    if ((threadIdx.x & 31) == 0) {
+        bwork_pair(Y, Wk, c);
+        bwork_add(PROF_BICG_VEC, 8.0 * Y.len[c] * (4 + 2), (double)Y.len[c] * (3 + 2));  // p update, rhat^T v
+        if (rv == 0.0) {
+            S.active[c] = 0;
+            S.status[c] = B_BREAKDOWN;
+        } else {
+            S.alpha[c] = S.rho[c] / rv;
         }
-        Yv[o + i] = acc;
     }
+}
+
+// omega = t^T s / t^T t of system c (one warp)
+__device__ void b_omega(const BSys& Y, const double* part, const BState& S, const BWork& Wk, int c)
+{
+    const double ts = sys_sum(Y, part, c);
+    const double tt = sys_sum(Y, part + Y.nitems, c);
+    if ((threadIdx.x & 31) == 0) {
+        bwork_pair(Y, Wk, c);
+        bwork_add(PROF_BICG_VEC, 8.0 * Y.len[c] * 2, 4.0 * Y.len[c]);  // t^T s, t^T t
+        if (tt == 0.0) {
+            S.active[c] = 0;
+            S.go[c] = 0;
+            S.status[c] = B_BREAKDOWN;
+        } else {
+            S.omega[c] = ts / tt;
+        }
+    }
+}
+
+// y_c = A~ x_c on the rows of an item, with ND inner products of the new rows
+// per vector item of BR rows: ND = 1: a^T y, ND = 2: y^T a, y^T y (the sums in
+// the order of the vector kernels). The last block of a system forms alpha or
+// omega of them.
+//
+// The matrices are unstructured: a warp's gathers touch up to 32 lines, and its
+// FMAs run to its longest row. With CSR rows and batches of 8 entries that took
+// 70 us for A~ and 25 for M (267 systems of 2.3k to 10k rows, 9.4 and 2.1
+// entries per row; the FMAs of the entries alone are 25 and 6). The block
+// copies the whole vector to shared memory (stage; coalesced, 3.4 loads per row
+// instead of 9 scattered ones), its rows are sorted by length, and entries go
+// two at a time, so that few FMAs are spent on padding and two blocks of 1024
+// threads fit. The batch's solve: 12.8 ms before; 11.5 with four entries at a
+// time, 11.1 with 512 threads, 10.3 like this. M's few gathers stay in L2.
+template <int ND>
+__global__ void __launch_bounds__(1024) k_b_spmv(BSys Y, BMat A, const double* __restrict__ X, double* __restrict__ Yv,
+                                                 const int* flags, const double* __restrict__ a, double* part, BState S,
+                                                 BWork Wk, int* arrived)
+{
+    extern __shared__ __align__(16) double bsm[];
+    __shared__ int last;
+    double *ys = bsm, *xs = bsm + SB;
+    const int c = Y.sp_sys[blockIdx.x];
+    if (!flags[c]) return;
+    const int b = Y.sp_blk[blockIdx.x], nt = blockDim.x;
+    const int4 bl = Y.blk[b];
+    const int n = Y.len[c];
+    const double* x = X + Y.off[c];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = nt >> 5;
+    const bool stage = A.stage && n <= Y.ncap;
+    if (stage) {
+        int i = threadIdx.x;
+        for (; i + 7 * nt < n; i += 8 * nt) {
+            double t[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) t[u] = x[i + u * nt];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) xs[i + u * nt] = t[u];
+        }
+        for (; i < n; i += nt) xs[i] = x[i];
+        __syncthreads();
+    }
+    for (int s = wid; s < (bl.y + 31) / 32; s += nw) {
+        const int64_t sl = (int64_t)b * (SB / 32) + s;
+        const int64_t e0 = A.sp[sl];
+        const int w = (int)(A.sp[sl + 1] - e0) / 32;
+        const int row = A.ord[sl * 32 + lane];
+        const int32_t* ci = A.sci + e0 + lane;
+        const double* va = A.sv + e0 + lane;
+        double acc = 0.0;
+        auto row_sum = [&](auto get) {
+#pragma unroll 1
+            for (int k = 0; k < w; k += 2) {
+                int32_t col[2];
+                double m[2], xv[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    col[u] = k + u < w ? __ldg(ci + (k + u) * 32) : -1;
+                    m[u] = k + u < w ? __ldg(va + (k + u) * 32) : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) xv[u] = get(max(col[u], 0));
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (col[u] >= 0) acc = fma(m[u], xv[u], acc);
+            }
+        };
+        if (stage) row_sum([&](int j) { return xs[j]; });
+        else row_sum([&](int j) { return x[j]; });
+        if (row >= 0) ys[row] = acc;
+    }
+    __syncthreads();
+    for (int q = wid; q < (bl.y + BR - 1) / BR; q += nw) {
+        const int64_t o = Y.off[c] + bl.w;
+        double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int t = 0; t < BR / 32; ++t) {
+            const int i = q * BR + lane + 32 * t;
+            if (i < bl.y) {
+                const double y = ys[i];
+                Yv[o + i] = y;
+                if (ND > 0) s0 = fma(a[o + i], y, s0);
+                if (ND > 1) s1 = fma(y, y, s1);
+            }
+        }
+        if (ND > 0) {
+            const int at = Y.first[c] + bl.w / BR + q;
+            s0 = warp_sum(s0);
+            if (ND > 1) s1 = warp_sum(s1);
+            if (lane == 0) {
+                part[at] = s0;
+                if (ND > 1) part[Y.nitems + at] = s1;
+            }
+        }
+    }
+    if (ND == 0) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&arrived[c], 1) == (n + SB - 1) / SB - 1;
+    }
+    __syncthreads();
+    if (!last || wid > 0) return;
+    __threadfence();
+    if (lane == 0) arrived[c] = 0;
+    if (ND == 1) b_alpha(Y, part, S, Wk, c);
+    else b_omega(Y, part, S, Wk, c);
 }
 
 // The vector kernels take one warp per item (system, BR rows): lane l holds
@@ -152,8 +285,25 @@ __global__ void __launch_bounds__(BR) k_b_init(BSys Y, const double* __restrict_
     }
 }
 
+// the start of system c's next iteration (one thread)
+__device__ __forceinline__ void b_start(const BState& S, int maxit, int c)
+{
+    if (S.iters[c] >= maxit) {
+        S.active[c] = 0;
+        S.status[c] = B_MAXITER;
+    } else {
+        S.iters[c] += 1;
+        if (S.rho[c] == 0.0) {
+            S.active[c] = 0;
+            S.status[c] = B_BREAKDOWN;
+        } else {
+            S.beta[c] = S.iters[c] == 1 ? 0.0 : (S.rho[c] / S.rho_old[c]) * (S.alpha[c] / S.omega[c]);
+        }
+    }
+}
+
 // one warp per system
-__global__ void k_b_f0(BSys Y, const double* part, BState S)
+__global__ void k_b_f0(BSys Y, const double* part, int maxit, BState S)
 {
     const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (c >= Y.nsys) return;
@@ -171,24 +321,7 @@ __global__ void k_b_f0(BSys Y, const double* part, BState S)
         } else {
             S.active[c] = 1;
             S.status[c] = B_MAXITER;
-        }
-    }
-}
-
-__global__ void k_b_start(int32_t nsys, int maxit, BState S)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= nsys || !S.active[c]) return;
-    if (S.iters[c] >= maxit) {
-        S.active[c] = 0;
-        S.status[c] = B_MAXITER;
-    } else {
-        S.iters[c] += 1;
-        if (S.rho[c] == 0.0) {
-            S.active[c] = 0;
-            S.status[c] = B_BREAKDOWN;
-        } else {
-            S.beta[c] = S.iters[c] == 1 ? 0.0 : (S.rho[c] / S.rho_old[c]) * (S.alpha[c] / S.omega[c]);
+            b_start(S, maxit, c);
         }
     }
 }
@@ -208,51 +341,6 @@ __global__ void __launch_bounds__(BR) k_b_p(BSys Y, const double* __restrict__ r
         for (int t = 0; t < RPL; ++t) {
             const int64_t i = r0 + lane + 32 * t;
             if (i < n) p[o + i] = first ? r[o + i] : r[o + i] + be * (p[o + i] - om * v[o + i]);
-        }
-    }
-}
-
-template <int ND>
-__global__ void __launch_bounds__(BR) k_b_dots(BSys Y, const double* a0, const double* b0, const double* a1,
-                                               const double* b1, const int* flags, double* part)
-{
-    const int lane = threadIdx.x & 31;
-    FOR_WARP_ITEMS(Y, q)
-    {
-        const int c = Y.it_sys[q];
-        if (!flags[c]) continue;
-        const int64_t o = Y.off[c], r0 = Y.it_r0[q], n = Y.len[c];
-        double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-        for (int t = 0; t < RPL; ++t) {
-            const int64_t i = r0 + lane + 32 * t;
-            if (i < n) {
-                s0 = fma(a0[o + i], b0[o + i], s0);
-                if (ND > 1) s1 = fma(a1[o + i], b1[o + i], s1);
-            }
-        }
-        s0 = warp_sum(s0);
-        if (ND > 1) s1 = warp_sum(s1);
-        if (lane == 0) {
-            part[q] = s0;
-            if (ND > 1) part[Y.nitems + q] = s1;
-        }
-    }
-}
-
-__global__ void k_b_f1(BSys Y, const double* part, BState S, BWork Wk)
-{
-    const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (c >= Y.nsys || !S.active[c]) return;
-    const double rv = sys_sum(Y, part, c);
-    if ((threadIdx.x & 31) == 0) {
-        bwork_pair(Y, Wk, c);
-        bwork_add(PROF_BICG_VEC, 8.0 * Y.len[c] * (4 + 2), (double)Y.len[c] * (3 + 2));  // p update, rhat^T v
-        if (rv == 0.0) {
-            S.active[c] = 0;
-            S.status[c] = B_BREAKDOWN;
-        } else {
-            S.alpha[c] = S.rho[c] / rv;
         }
     }
 }
@@ -298,25 +386,6 @@ __global__ void k_b_f2(BSys Y, const double* part, BState S)
     }
 }
 
-__global__ void k_b_f3(BSys Y, const double* part, BState S, BWork Wk)
-{
-    const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (c >= Y.nsys || !S.go[c]) return;
-    const double ts = sys_sum(Y, part, c);
-    const double tt = sys_sum(Y, part + Y.nitems, c);
-    if ((threadIdx.x & 31) == 0) {
-        bwork_pair(Y, Wk, c);
-        bwork_add(PROF_BICG_VEC, 8.0 * Y.len[c] * 2, 4.0 * Y.len[c]);  // t^T s, t^T t
-        if (tt == 0.0) {
-            S.active[c] = 0;
-            S.go[c] = 0;
-            S.status[c] = B_BREAKDOWN;
-        } else {
-            S.omega[c] = ts / tt;
-        }
-    }
-}
-
 __global__ void __launch_bounds__(BR) k_b_xr(BSys Y, double* x, double* r, const double* __restrict__ rh,
                                              const double* __restrict__ ph, const double* __restrict__ sh_,
                                              const double* __restrict__ s, const double* __restrict__ t, BState S,
@@ -357,7 +426,7 @@ __global__ void __launch_bounds__(BR) k_b_xr(BSys Y, double* x, double* r, const
     }
 }
 
-__global__ void k_b_f4(BSys Y, const double* part, BState S)
+__global__ void k_b_f4(BSys Y, const double* part, int maxit, BState S)
 {
     const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (c >= Y.nsys || !S.active[c]) return;
@@ -374,6 +443,7 @@ __global__ void k_b_f4(BSys Y, const double* part, BState S)
         } else {
             S.rho_old[c] = S.rho[c];
             S.rho[c] = rhr;
+            b_start(S, maxit, c);
         }
     }
 }
@@ -770,8 +840,25 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
             it_sys[q] = c;
             it_r0[q] = (q - first[c]) * BR;
         }
+    // blocks of SB rows of each matrix, and the SpMV items over them
+    std::vector<int4> blk;
+    std::vector<int32_t> sp_sys, sp_blk;
+    int32_t nmax = 0;
+    for (int32_t m = 0; m < nmat; ++m) {
+        const int32_t b0 = (int32_t)blk.size(), n = hs[m]->n;
+        nmax = n > nmax ? n : nmax;
+        for (int32_t r = 0; r < n; r += SB)
+            blk.push_back(make_int4((int32_t)R0[m] + r, n - r < SB ? n - r : SB, (int32_t)R0[m], r));
+        for (int32_t c = sys0[m]; c < sys0[m + 1]; ++c)
+            for (int32_t q = b0; q < (int32_t)blk.size(); ++q) {
+                sp_sys.push_back(c);
+                sp_blk.push_back(q);
+            }
+    }
+    const int32_t nsp = (int32_t)sp_sys.size(), nblk = (int32_t)blk.size();
     Buf tab, vecs, bst, bsi, part, misc;
-    const size_t tab_bytes = sizeof(int64_t) * (nsys + nmat + nmat + 1) +
+    const size_t tab_bytes = sizeof(int4) * (size_t)nblk + sizeof(int32_t) * 2 * ((size_t)nsp + 1) +
+                             sizeof(int64_t) * (nsys + nmat + nmat + 1) +
                              sizeof(int32_t) * (4 * (size_t)nsys + 1 + 2 * (size_t)nit + 2 * (size_t)nmat + joff[nmat] + 1);
     SAI_TRY(tab.alloc(tab_bytes + 64, st, true));
     char* tp = tab.as<char>();
@@ -782,6 +869,11 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
         return at;
     };
     BSys Y;
+    Y.blk = (const int4*)put(blk.data(), sizeof(int4) * nblk);
+    Y.sp_sys = (const int32_t*)put(sp_sys.data(), sizeof(int32_t) * nsp);
+    Y.sp_blk = (const int32_t*)put(sp_blk.data(), sizeof(int32_t) * nsp);
+    Y.nsp = nsp;
+    Y.ncap = nmax < SB_CAP ? nmax : SB_CAP;
     Y.nsys = nsys;
     Y.nitems = nit;
     Y.off = (const int64_t*)put(off.data(), sizeof(int64_t) * nsys);
@@ -818,7 +910,7 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     double* sh = s + NV;
     double* t = sh + NV;
     SAI_TRY(bst.alloc(sizeof(double) * 6 * (size_t)nsys, st, true));
-    SAI_TRY(bsi.alloc(sizeof(int) * (5 * (size_t)nsys + 2), st, true));
+    SAI_TRY(bsi.alloc(sizeof(int) * (6 * (size_t)nsys + 2), st, true));
     SAI_TRY(part.alloc(sizeof(double) * 2 * (size_t)(nit > 0 ? nit : 1), st, true));
     SAI_TRY(misc.alloc(sizeof(double) * ((size_t)joff[nmat] + 2 * (size_t)nmat + 4), st, true));
     BState S;
@@ -836,7 +928,8 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     S.mode = ip + 3 * nsys;
     S.go = ip + 4 * nsys;
     int* any = ip + 5 * nsys;
-    SAI_CUDA(cudaMemsetAsync(ip, 0, sizeof(int) * (5 * (size_t)nsys + 2), st));
+    int* arrived = any + 2;  // SpMV blocks done per system, 0 between launches
+    SAI_CUDA(cudaMemsetAsync(ip, 0, sizeof(int) * (6 * (size_t)nsys + 2), st));
 
     // right-hand sides and the Theorem 2 thresholds of each matrix
     std::vector<double> thr(nsys);
@@ -870,37 +963,45 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
 
     // ---- batched BiCGStab (right preconditioning: A~ M z = rhs, y = M z)
     const int64_t *Ar = bd.Atr_rp.as<int64_t>(), *Mr = P.Mr_rp.as<int64_t>();
-    const int32_t *Ac = bd.Atr_ci.as<int32_t>(), *Mc = P.Mr_ci.as<int32_t>();
-    const double *Av = bd.Atr_v.as<double>(), *Mv = P.Mr_v.as<double>();
-    const unsigned gi = grid_for(nit, cap);                   // SpMV: one block per item
+    Buf sa[4], smb[4];
+    const RowBlocks rb{(int)N, SB, Y.blk};
+    SAI_TRY(sorted_rows<double>(rb, nblk, Ar, bd.Atr_ci.as<int32_t>(), bd.Atr_v.as<double>(), sa, st));
+    SAI_TRY(sorted_rows<double>(rb, nblk, Mr, P.Mr_ci.as<int32_t>(), P.Mr_v.as<double>(), smb, st));
+    // staging pays where a row has more entries than the copy has loads per row
+    auto bmat = [&](const Buf (&b)[4], int64_t nnz) {
+        return BMat{b[1].as<int64_t>(), b[2].as<int32_t>(), b[3].as<double>(), b[0].as<int32_t>(), nnz > 4 * N};
+    };
+    const BMat Am = bmat(sa, bd.nnz_At), Mm = bmat(smb, P.nnz);
+    const size_t sm0 = sizeof(double) * SB, sm1 = sm0 + sizeof(double) * (size_t)Y.ncap;
+    for (auto kern : {k_b_spmv<0>, k_b_spmv<1>, k_b_spmv<2>})
+        SAI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
     const unsigned gw = grid_for(sai_div_up(nit, BR / 32), cap);  // vector kernels: one warp per item
-    const unsigned gs = sai_div_up((int64_t)nsys * 32, 256), gt = sai_div_up(nsys, 256);
+    const unsigned gs = sai_div_up((int64_t)nsys * 32, 256);
     double* pt = part.as<double>();
     const int maxit = prm->krylov.maxit;
     BWork Wk;
     Wk.Arp = Ar;
     Wk.Mrp = Mr;
     double* Xd = X;  // the iterates of the current pass
+    auto spmv = [&](decltype(&k_b_spmv<0>) kern, const BMat& Mt, const double* xin, double* yout, const int* flags,
+                    const double* dot, cudaStream_t q) {
+        const bool stg = Mt.stage;
+        kern<<<SAI_GRID(nsp), stg ? 1024 : 256, stg ? sm1 : sm0, q>>>(Y, Mt, xin, yout, flags, dot, pt, S, Wk, arrived);
+    };
     // profile scopes act only while a profile is open, when no graph is captured
     auto iteration = [&](cudaStream_t q) {
-        k_b_start<<<SAI_GRID(gt), 256, 0, q>>>(nsys, maxit, S);
         {
             ProfScope ps(PROF_BICG_VEC, q);
             k_b_p<<<SAI_GRID(gw), BR, 0, q>>>(Y, r, p, v, S);
         }
         {
             ProfScope ps(PROF_SPMM, q);
-            k_b_spmv<<<SAI_GRID(gi), BR, 0, q>>>(Y, Mr, Mc, Mv, p, ph, S.active);
+            spmv(k_b_spmv<0>, Mm, p, ph, S.active, nullptr, q);
         }
         {
             ProfScope ps(PROF_SPMM, q);
-            k_b_spmv<<<SAI_GRID(gi), BR, 0, q>>>(Y, Ar, Ac, Av, ph, v, S.active);
+            spmv(k_b_spmv<1>, Am, ph, v, S.active, rh, q);
         }
-        {
-            ProfScope ps(PROF_BICG_VEC, q);
-            k_b_dots<1><<<SAI_GRID(gw), BR, 0, q>>>(Y, rh, v, nullptr, nullptr, S.active, pt);
-        }
-        k_b_f1<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, S, Wk);
         {
             ProfScope ps(PROF_BICG_VEC, q);
             k_b_s<<<SAI_GRID(gw), BR, 0, q>>>(Y, r, v, s, S, pt);
@@ -908,24 +1009,19 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
         k_b_f2<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, S);
         {
             ProfScope ps(PROF_SPMM, q);
-            k_b_spmv<<<SAI_GRID(gi), BR, 0, q>>>(Y, Mr, Mc, Mv, s, sh, S.go);
+            spmv(k_b_spmv<0>, Mm, s, sh, S.go, nullptr, q);
         }
         {
             ProfScope ps(PROF_SPMM, q);
-            k_b_spmv<<<SAI_GRID(gi), BR, 0, q>>>(Y, Ar, Ac, Av, sh, t, S.go);
+            spmv(k_b_spmv<2>, Am, sh, t, S.go, s, q);
         }
-        {
-            ProfScope ps(PROF_BICG_VEC, q);
-            k_b_dots<2><<<SAI_GRID(gw), BR, 0, q>>>(Y, t, s, t, t, S.go, pt);
-        }
-        k_b_f3<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, S, Wk);
         {
             ProfScope ps(PROF_BICG_VEC, q);
             k_b_xr<<<SAI_GRID(gw), BR, 0, q>>>(Y, Xd, r, rh, ph, sh, s, t, S, pt);
         }
-        k_b_f4<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, S);
+        k_b_f4<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, maxit, S);
     };
-    constexpr int ITERS_PER_CHECK = 8, LAUNCHES = ITERS_PER_CHECK * 14 + 1;
+    constexpr int ITERS_PER_CHECK = 8, LAUNCHES = ITERS_PER_CHECK * 9 + 1;
     int* nbody = any + 1;  // body runs of the while graph
     // One pass of the batched BiCGStab from x = 0 on the right-hand sides
     // Bsrc (thresholds in S.thr), iterates into Xdst. Without an open
@@ -936,11 +1032,11 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     // ITERS_PER_CHECK iterations run as a captured graph with one host check
     // of the "any system active" flag per group. Both run on a library
     // stream ordered after the caller's; iterations past maxit change nothing
-    // (k_b_start retires those systems).
+    // (k_b_f4 retires those systems).
     auto run_pass = [&](const double* Bsrc, double* Xdst) -> sai_status {
         Xd = Xdst;
         k_b_init<<<SAI_GRID(gw), BR, 0, st>>>(Y, Bsrc, Xdst, r, rh, p, v, pt);
-        k_b_f0<<<SAI_GRID(gs), 256, 0, st>>>(Y, pt, S);
+        k_b_f0<<<SAI_GRID(gs), 256, 0, st>>>(Y, pt, maxit, S);
         SAI_CUDA(cudaMemsetAsync(any, 0, sizeof(int) * 2, st));
         SAI_CUDA(cudaGetLastError());
         cudaStream_t q = st;
@@ -1032,7 +1128,6 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
             }
         }
         if (gexec) cudaGraphExecDestroy(gexec);
-        k_b_start<<<SAI_GRID(gt), 256, 0, q>>>(nsys, maxit, S);  // systems still running after maxit
         if (ev_in) {
             cudaEventRecord(ev_out, q);
             cudaStreamWaitEvent(st, ev_out, 0);
@@ -1094,7 +1189,7 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
             int* dsel = (int*)(D + NV);  // the continued systems
             SAI_CUDA(cudaMemcpyAsync(dsel, sel.data(), sizeof(int) * nsys, cudaMemcpyHostToDevice, st));
             SAI_CUDA(cudaMemsetAsync(R, 0, sizeof(double) * (size_t)NV, st));
-            k_b_spmv<<<SAI_GRID(gi), BR, 0, st>>>(Y, Ar, Ac, Av, X, R, dsel);
+            spmv(k_b_spmv<0>, Am, X, R, dsel, nullptr, st);
             k_b_resid<<<SAI_GRID(gw), BR, 0, st>>>(Y, Bv, dsel, R);
             SAI_CUDA(cudaGetLastError());
             SAI_CUDA(cudaMemcpyAsync(S.thr, thr2.data(), sizeof(double) * nsys, cudaMemcpyHostToDevice, st));

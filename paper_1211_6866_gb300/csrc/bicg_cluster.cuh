@@ -188,68 +188,6 @@ __device__ __noinline__ void cl_apply(const ClMat<T>* Am, const ClRows* Wp, cons
     }
 }
 
-// ---- the sorted form of a CSR matrix for blocks of R rows (grid: a block per block of rows)
-__global__ void __launch_bounds__(512) k_cl_sort(int n, int R, const int64_t* __restrict__ rp, int32_t* __restrict__ ord,
-                                                 int64_t* __restrict__ cnt)
-{
-    constexpr int NB = 1024;  // bins by length, the longest first
-    __shared__ int off[NB];
-    __shared__ int ws[16];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int base = blockIdx.x * R, nrow = max(0, min(R, n - base));
-    auto bin = [&](int r) {  // steps of 96 from 512 entries on: an order of 49152 fits
-        const int len = (int)(rp[base + r + 1] - rp[base + r]);
-        return NB - 1 - min(NB - 1, len < 512 ? len : 512 + (len - 512) / 96);
-    };
-    for (int i = tid; i < NB; i += 512) off[i] = 0;
-    for (int i = tid; i < R; i += 512) ord[base + i] = -1;
-    __syncthreads();
-    for (int r = tid; r < nrow; r += 512) atomicAdd(&off[bin(r)], 1);
-    __syncthreads();
-    // exclusive prefix over the bins, two per thread
-    const int c0 = off[2 * tid], c1 = off[2 * tid + 1];
-    int incl = c0 + c1;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(SAI_FULL, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) ws[wid] = incl;
-    __syncthreads();
-    int before = incl - c0 - c1;
-    for (int w = 0; w < wid; ++w) before += ws[w];
-    off[2 * tid] = before;
-    off[2 * tid + 1] = before + c0;
-    __syncthreads();
-    // rows of equal length land in any order: a row's product does not depend on its place
-    for (int r = tid; r < nrow; r += 512) ord[base + atomicAdd(&off[bin(r)], 1)] = r;
-    __syncthreads();
-    for (int s = wid; s < R / 32; s += 16) {
-        const int r = ord[base + 32 * s + lane];
-        const unsigned len = r >= 0 ? (unsigned)(rp[base + r + 1] - rp[base + r]) : 0u;
-        const unsigned w = __reduce_max_sync(SAI_FULL, len);
-        if (lane == 0) cnt[base / 32 + s] = (int64_t)w * 32;
-    }
-}
-
-template <class T>
-__global__ void k_cl_fill(int nsl, int R, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                          const T* __restrict__ v, const int32_t* __restrict__ ord, const int64_t* __restrict__ sp,
-                          int32_t* __restrict__ sci, T* __restrict__ sv)
-{
-    const int sl = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (sl >= nsl) return;
-    const int base = sl * 32 / R * R;
-    const int r = ord[(int64_t)sl * 32 + lane];
-    const int64_t b = sp[sl], w = (sp[sl + 1] - b) / 32;
-    const int64_t r0 = r >= 0 ? rp[base + r] : 0, len = r >= 0 ? rp[base + r + 1] - r0 : 0;
-    for (int64_t k = 0; k < w; ++k) {
-        const int64_t q = b + k * 32 + lane;
-        sci[q] = k < len ? ci[r0 + k] : -1;  // not multiplied: its factor may be infinite
-        sv[q] = k < len ? v[r0 + k] : T(0);
-    }
-}
-
 // The matrix of a cluster kernel: its sliced-ELL copy, or the sorted form of
 // its CSR arrays for C blocks of R rows in buf (live until the kernel has run).
 template <class T>
@@ -259,21 +197,7 @@ sai_status cl_matrix(const Mat<T>& X, int n, int R, int C, Buf (&buf)[4], ClMat<
         out = {X.sp, X.sci, X.sv, nullptr};
         return SAI_OK;
     }
-    const int nsl = C * (R / 32);
-    Buf cnt;
-    SAI_TRY(cnt.alloc(sizeof(int64_t) * (size_t)nsl, st, true));
-    SAI_TRY(buf[0].alloc(sizeof(int32_t) * (size_t)C * R, st, true));
-    SAI_TRY(buf[1].alloc(sizeof(int64_t) * ((size_t)nsl + 1), st, true));
-    k_cl_sort<<<SAI_GRID(C), 512, 0, st>>>(n, R, X.rp, buf[0].as<int32_t>(), cnt.as<int64_t>());
-    SAI_TRY(sai_scan_counts_i64(cnt.as<int64_t>(), buf[1].as<int64_t>(), nsl, st));
-    int64_t total = 0;
-    SAI_CUDA(cudaMemcpyAsync(&total, buf[1].as<int64_t>() + nsl, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    SAI_CUDA(cudaStreamSynchronize(st));
-    SAI_TRY(buf[2].alloc(sizeof(int32_t) * (size_t)(total > 0 ? total : 1), st, true));
-    SAI_TRY(buf[3].alloc(sizeof(T) * (size_t)(total > 0 ? total : 1), st, true));
-    k_cl_fill<T><<<SAI_GRID(sai_div_up((int64_t)nsl * 32, 256)), 256, 0, st>>>(
-        nsl, R, X.rp, X.ci, X.v, buf[0].as<int32_t>(), buf[1].as<int64_t>(), buf[2].as<int32_t>(), buf[3].as<T>());
-    SAI_CUDA(cudaGetLastError());
+    SAI_TRY(sorted_rows<T>(RowBlocks{n, R, nullptr}, C, X.rp, X.ci, X.v, buf, st));
     out = {buf[1].as<int64_t>(), buf[2].as<int32_t>(), buf[3].as<T>(), buf[0].as<int32_t>()};
     return SAI_OK;
 }

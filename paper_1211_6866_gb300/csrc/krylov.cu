@@ -1280,6 +1280,7 @@ void pnl_apply2(int32_t n, int64_t ld, int k, const Ops<double>& A, const double
 }
 
 // ---------------------------------------------------------------- one cluster per system
+#include "sorted_rows.cuh"
 #include "bicg_cluster.cuh"
 
 // Up to this many systems of order CL_MAXN or less run in clusters; with more
