@@ -12,9 +12,8 @@
 //   (system, chunk of rows), listed once for the whole batch: a block per
 //   chunk of SB rows in the SpMV, a warp per chunk of BR in the vector kernels;
 //   a stopped system's items return at once. Inner products are summed per
-//   BR rows in a fixed order and per system over those in order. alpha and
-//   omega are formed by the last SpMV block of a system, the other control
-//   values by a warp per system: 9 launches per iteration. The loop is one
+//   BR rows in a fixed order and per system over those in order. The control
+//   kernels run a warp per system: 11 launches per iteration. The loop is one
 //   CUDA graph (or groups of 8 iterations with a host check after each).
 // SMW: one block per matrix solves its s_i x s_i system (partial pivoting);
 //   then x_i = yhat_i - What_i z_i, and rr per matrix.
@@ -107,44 +106,9 @@ __device__ __forceinline__ double sys_sum(const BSys& Y, const double* part, int
     return warp_sum(a);
 }
 
-// alpha = rho / rhat^T v of system c (one warp)
-__device__ void b_alpha(const BSys& Y, const double* part, const BState& S, const BWork& Wk, int c)
-{
-    const double rv = sys_sum(Y, part, c);
-    if ((threadIdx.x & 31) == 0) {
-        bwork_pair(Y, Wk, c);
-        bwork_add(PROF_BICG_VEC, 8.0 * Y.len[c] * (4 + 2), (double)Y.len[c] * (3 + 2));  // p update, rhat^T v
-        if (rv == 0.0) {
-            S.active[c] = 0;
-            S.status[c] = B_BREAKDOWN;
-        } else {
-            S.alpha[c] = S.rho[c] / rv;
-        }
-    }
-}
-
-// omega = t^T s / t^T t of system c (one warp)
-__device__ void b_omega(const BSys& Y, const double* part, const BState& S, const BWork& Wk, int c)
-{
-    const double ts = sys_sum(Y, part, c);
-    const double tt = sys_sum(Y, part + Y.nitems, c);
-    if ((threadIdx.x & 31) == 0) {
-        bwork_pair(Y, Wk, c);
-        bwork_add(PROF_BICG_VEC, 8.0 * Y.len[c] * 2, 4.0 * Y.len[c]);  // t^T s, t^T t
-        if (tt == 0.0) {
-            S.active[c] = 0;
-            S.go[c] = 0;
-            S.status[c] = B_BREAKDOWN;
-        } else {
-            S.omega[c] = ts / tt;
-        }
-    }
-}
-
 // y_c = A~ x_c on the rows of an item, with ND inner products of the new rows
 // per vector item of BR rows: ND = 1: a^T y, ND = 2: y^T a, y^T y (the sums in
-// the order of the vector kernels). The last block of a system forms alpha or
-// omega of them.
+// the order of the vector kernels).
 //
 // The matrices are unstructured: a warp's gathers touch up to 32 lines, and its
 // FMAs run to its longest row. With CSR rows and batches of 8 entries that took
@@ -154,14 +118,14 @@ __device__ void b_omega(const BSys& Y, const double* part, const BState& S, cons
 // instead of 9 scattered ones), its rows are sorted by length, and entries go
 // two at a time, so that few FMAs are spent on padding and two blocks of 1024
 // threads fit. The batch's solve: 12.8 ms before; 11.5 with four entries at a
-// time, 11.1 with 512 threads, 10.3 like this. M's few gathers stay in L2.
+// time, 11.2 with 512 threads, 10.2 like this (11.1 with alpha and omega formed
+// by the last block of a system: each block then ends in a fence and an atomic).
+// M's few gathers stay in L2.
 template <int ND>
 __global__ void __launch_bounds__(1024) k_b_spmv(BSys Y, BMat A, const double* __restrict__ X, double* __restrict__ Yv,
-                                                 const int* flags, const double* __restrict__ a, double* part, BState S,
-                                                 BWork Wk, int* arrived)
+                                                 const int* flags, const double* __restrict__ a, double* part)
 {
     extern __shared__ __align__(16) double bsm[];
-    __shared__ int last;
     double *ys = bsm, *xs = bsm + SB;
     const int c = Y.sp_sys[blockIdx.x];
     if (!flags[c]) return;
@@ -236,18 +200,6 @@ __global__ void __launch_bounds__(1024) k_b_spmv(BSys Y, BMat A, const double* _
             }
         }
     }
-    if (ND == 0) return;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(&arrived[c], 1) == (n + SB - 1) / SB - 1;
-    }
-    __syncthreads();
-    if (!last || wid > 0) return;
-    __threadfence();
-    if (lane == 0) arrived[c] = 0;
-    if (ND == 1) b_alpha(Y, part, S, Wk, c);
-    else b_omega(Y, part, S, Wk, c);
 }
 
 // The vector kernels take one warp per item (system, BR rows): lane l holds
@@ -345,6 +297,24 @@ __global__ void __launch_bounds__(BR) k_b_p(BSys Y, const double* __restrict__ r
     }
 }
 
+// alpha = rho / rhat^T v (one warp per system)
+__global__ void k_b_alpha(BSys Y, const double* part, BState S, BWork Wk)
+{
+    const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (c >= Y.nsys || !S.active[c]) return;
+    const double rv = sys_sum(Y, part, c);
+    if ((threadIdx.x & 31) == 0) {
+        bwork_pair(Y, Wk, c);
+        bwork_add(PROF_BICG_VEC, 8.0 * Y.len[c] * (4 + 2), (double)Y.len[c] * (3 + 2));  // p update, rhat^T v
+        if (rv == 0.0) {
+            S.active[c] = 0;
+            S.status[c] = B_BREAKDOWN;
+        } else {
+            S.alpha[c] = S.rho[c] / rv;
+        }
+    }
+}
+
 __global__ void __launch_bounds__(BR) k_b_s(BSys Y, const double* __restrict__ r, const double* __restrict__ v, double* s,
                                             BState S, double* part)
 {
@@ -383,6 +353,26 @@ __global__ void k_b_f2(BSys Y, const double* part, BState S)
         bwork_add(PROF_BICG_VEC, 8.0 * Y.len[c] * 3, 4.0 * Y.len[c]);  // s, ||s||
         S.mode[c] = sqrt(ss) < S.thr[c] ? 2 : 1;
         S.go[c] = S.mode[c] == 1;
+    }
+}
+
+// omega = t^T s / t^T t (one warp per system)
+__global__ void k_b_omega(BSys Y, const double* part, BState S, BWork Wk)
+{
+    const int c = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (c >= Y.nsys || !S.go[c]) return;
+    const double ts = sys_sum(Y, part, c);
+    const double tt = sys_sum(Y, part + Y.nitems, c);
+    if ((threadIdx.x & 31) == 0) {
+        bwork_pair(Y, Wk, c);
+        bwork_add(PROF_BICG_VEC, 8.0 * Y.len[c] * 2, 4.0 * Y.len[c]);  // t^T s, t^T t
+        if (tt == 0.0) {
+            S.active[c] = 0;
+            S.go[c] = 0;
+            S.status[c] = B_BREAKDOWN;
+        } else {
+            S.omega[c] = ts / tt;
+        }
     }
 }
 
@@ -910,7 +900,7 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     double* sh = s + NV;
     double* t = sh + NV;
     SAI_TRY(bst.alloc(sizeof(double) * 6 * (size_t)nsys, st, true));
-    SAI_TRY(bsi.alloc(sizeof(int) * (6 * (size_t)nsys + 2), st, true));
+    SAI_TRY(bsi.alloc(sizeof(int) * (5 * (size_t)nsys + 2), st, true));
     SAI_TRY(part.alloc(sizeof(double) * 2 * (size_t)(nit > 0 ? nit : 1), st, true));
     SAI_TRY(misc.alloc(sizeof(double) * ((size_t)joff[nmat] + 2 * (size_t)nmat + 4), st, true));
     BState S;
@@ -928,8 +918,7 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     S.mode = ip + 3 * nsys;
     S.go = ip + 4 * nsys;
     int* any = ip + 5 * nsys;
-    int* arrived = any + 2;  // SpMV blocks done per system, 0 between launches
-    SAI_CUDA(cudaMemsetAsync(ip, 0, sizeof(int) * (6 * (size_t)nsys + 2), st));
+    SAI_CUDA(cudaMemsetAsync(ip, 0, sizeof(int) * (5 * (size_t)nsys + 2), st));
 
     // right-hand sides and the Theorem 2 thresholds of each matrix
     std::vector<double> thr(nsys);
@@ -986,7 +975,7 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     auto spmv = [&](decltype(&k_b_spmv<0>) kern, const BMat& Mt, const double* xin, double* yout, const int* flags,
                     const double* dot, cudaStream_t q) {
         const bool stg = Mt.stage;
-        kern<<<SAI_GRID(nsp), stg ? 1024 : 256, stg ? sm1 : sm0, q>>>(Y, Mt, xin, yout, flags, dot, pt, S, Wk, arrived);
+        kern<<<SAI_GRID(nsp), stg ? 1024 : 256, stg ? sm1 : sm0, q>>>(Y, Mt, xin, yout, flags, dot, pt);
     };
     // profile scopes act only while a profile is open, when no graph is captured
     auto iteration = [&](cudaStream_t q) {
@@ -1002,6 +991,7 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
             ProfScope ps(PROF_SPMM, q);
             spmv(k_b_spmv<1>, Am, ph, v, S.active, rh, q);
         }
+        k_b_alpha<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, S, Wk);
         {
             ProfScope ps(PROF_BICG_VEC, q);
             k_b_s<<<SAI_GRID(gw), BR, 0, q>>>(Y, r, v, s, S, pt);
@@ -1015,13 +1005,14 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
             ProfScope ps(PROF_SPMM, q);
             spmv(k_b_spmv<2>, Am, sh, t, S.go, s, q);
         }
+        k_b_omega<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, S, Wk);
         {
             ProfScope ps(PROF_BICG_VEC, q);
             k_b_xr<<<SAI_GRID(gw), BR, 0, q>>>(Y, Xd, r, rh, ph, sh, s, t, S, pt);
         }
         k_b_f4<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, maxit, S);
     };
-    constexpr int ITERS_PER_CHECK = 8, LAUNCHES = ITERS_PER_CHECK * 9 + 1;
+    constexpr int ITERS_PER_CHECK = 8, LAUNCHES = ITERS_PER_CHECK * 11 + 1;
     int* nbody = any + 1;  // body runs of the while graph
     // One pass of the batched BiCGStab from x = 0 on the right-hand sides
     // Bsrc (thresholds in S.thr), iterates into Xdst. Without an open
