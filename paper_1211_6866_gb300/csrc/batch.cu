@@ -22,6 +22,7 @@
 #include <memory>
 #include <new>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -31,7 +32,8 @@ namespace {
 constexpr int BR = 256;  // rows per work item (one block, one thread per row)
 
 constexpr int SB = 2048;     // rows per SpMV item
-constexpr int SB_CAP = 24576;  // doubles of the staged vector: 192 KB beside the item's results
+constexpr int SB_CAP = 12288;  // rows of the longest staged vector: 96 KB, two blocks per SM
+constexpr int SB_ROW = 4;      // entries per row from which a matrix's products are staged
 
 enum { B_OK = 0, B_MAXITER = 5, B_BREAKDOWN = 6 };  // same values as sai_status
 
@@ -46,12 +48,10 @@ struct BSys {
     const int32_t* it_r0;   // first local row of item q
     const int32_t* nsm;     // systems of c's matrix (s + 1)
     int32_t nitems;
-    // SpMV items: SB rows of a system, as a block of the matrices' sorted rows
-    const int32_t* sp_sys;
-    const int32_t* sp_blk;
-    const int4* blk;  // (first row, rows, row0 of the matrix, first local row) per block
-    int32_t nsp;
-    int32_t ncap;  // longest vector that is staged in shared memory
+    const int4* blk;  // blocks of SB sorted rows: (first row, rows, row0 of the matrix, first local row)
+    // SpMV items (system, block), the systems of more than SB_CAP rows first
+    const int2* item;
+    int32_t nitem, nlong;
 };
 
 #include "sorted_rows.cuh"
@@ -62,7 +62,6 @@ struct BMat {
     const int32_t* sci;
     const double* sv;
     const int32_t* ord;
-    int stage;  // gathers from shared memory where the vector fits
 };
 
 // Algorithmic work of the batched BiCGStab, added per system by the control
@@ -113,29 +112,31 @@ __device__ __forceinline__ double sys_sum(const BSys& Y, const double* part, int
 // The matrices are unstructured: a warp's gathers touch up to 32 lines, and its
 // FMAs run to its longest row. With CSR rows and batches of 8 entries that took
 // 70 us for A~ and 25 for M (267 systems of 2.3k to 10k rows, 9.4 and 2.1
-// entries per row; the FMAs of the entries alone are 25 and 6). The block
-// copies the whole vector to shared memory (stage; coalesced, 3.4 loads per row
-// instead of 9 scattered ones), its rows are sorted by length, and entries go
-// two at a time, so that few FMAs are spent on padding and two blocks of 1024
-// threads fit. The batch's solve: 12.8 ms before; 11.5 with four entries at a
-// time, 11.2 with 512 threads, 10.2 like this (11.1 with alpha and omega formed
-// by the last block of a system: each block then ends in a fence and an atomic).
-// M's few gathers stay in L2.
-template <int ND>
-__global__ void __launch_bounds__(1024) k_b_spmv(BSys Y, BMat A, const double* __restrict__ X, double* __restrict__ Yv,
-                                                 const int* flags, const double* __restrict__ a, double* part)
+// entries per row; the FMAs of the entries alone are 25 and 6). Rows are now
+// sorted by length, and entries go two at a time, so that few FMAs are spent
+// on padding and every warp slot is filled; and with STAGE the block copies the
+// whole vector to shared memory (coalesced, at most 6 loads per row instead of
+// 9 scattered ones). The solve of the 267 systems: 12.8 ms before, 12.2 sorted
+// only, 10.5 staged as well (11.5 with four entries at a time, 11.2 with 512
+// threads per staged block). 2736 systems of up to 50000 rows: 336 ms before, 207 sorted
+// only, 208 with the vectors up to SB_CAP staged, 216 up to twice that (one block per SM),
+// 369 with everything in one launch of staged blocks' size. A matrix of few
+// entries per row, M here, is not staged: the copy would cost more loads than its gathers.
+template <int ND, bool STAGE>
+__global__ void __launch_bounds__(STAGE ? 1024 : 256)
+    k_b_spmv(BSys Y, BMat A, const double* __restrict__ X, double* __restrict__ Yv, const int* flags,
+             const double* __restrict__ a, double* part)
 {
     extern __shared__ __align__(16) double bsm[];
     double *ys = bsm, *xs = bsm + SB;
-    const int c = Y.sp_sys[blockIdx.x];
+    const int2 item = Y.item[(STAGE ? Y.nlong : 0) + blockIdx.x];
+    const int c = item.x, b = item.y;
     if (!flags[c]) return;
-    const int b = Y.sp_blk[blockIdx.x], nt = blockDim.x;
+    const int nt = blockDim.x, n = Y.len[c];
     const int4 bl = Y.blk[b];
-    const int n = Y.len[c];
     const double* x = X + Y.off[c];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = nt >> 5;
-    const bool stage = A.stage && n <= Y.ncap;
-    if (stage) {
+    if (STAGE) {
         int i = threadIdx.x;
         for (; i + 7 * nt < n; i += 8 * nt) {
             double t[8];
@@ -155,25 +156,21 @@ __global__ void __launch_bounds__(1024) k_b_spmv(BSys Y, BMat A, const double* _
         const int32_t* ci = A.sci + e0 + lane;
         const double* va = A.sv + e0 + lane;
         double acc = 0.0;
-        auto row_sum = [&](auto get) {
 #pragma unroll 1
-            for (int k = 0; k < w; k += 2) {
-                int32_t col[2];
-                double m[2], xv[2];
+        for (int k = 0; k < w; k += 2) {
+            int32_t col[2];
+            double m[2], xv[2];
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    col[u] = k + u < w ? __ldg(ci + (k + u) * 32) : -1;
-                    m[u] = k + u < w ? __ldg(va + (k + u) * 32) : 0.0;
-                }
-#pragma unroll
-                for (int u = 0; u < 2; ++u) xv[u] = get(max(col[u], 0));
-#pragma unroll
-                for (int u = 0; u < 2; ++u)
-                    if (col[u] >= 0) acc = fma(m[u], xv[u], acc);
+            for (int u = 0; u < 2; ++u) {
+                col[u] = k + u < w ? __ldg(ci + (k + u) * 32) : -1;
+                m[u] = k + u < w ? __ldg(va + (k + u) * 32) : 0.0;
             }
-        };
-        if (stage) row_sum([&](int j) { return xs[j]; });
-        else row_sum([&](int j) { return x[j]; });
+#pragma unroll
+            for (int u = 0; u < 2; ++u) xv[u] = STAGE ? xs[max(col[u], 0)] : x[max(col[u], 0)];
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (col[u] >= 0) acc = fma(m[u], xv[u], acc);
+        }
         if (row >= 0) ys[row] = acc;
     }
     __syncthreads();
@@ -832,22 +829,20 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
         }
     // blocks of SB rows of each matrix, and the SpMV items over them
     std::vector<int4> blk;
-    std::vector<int32_t> sp_sys, sp_blk;
-    int32_t nmax = 0;
+    std::vector<int2> item, shorter;
+    int32_t nst = 0;  // longest staged vector
     for (int32_t m = 0; m < nmat; ++m) {
         const int32_t b0 = (int32_t)blk.size(), n = hs[m]->n;
-        nmax = n > nmax ? n : nmax;
         for (int32_t r = 0; r < n; r += SB)
             blk.push_back(make_int4((int32_t)R0[m] + r, n - r < SB ? n - r : SB, (int32_t)R0[m], r));
+        if (n <= SB_CAP && n > nst) nst = n;
         for (int32_t c = sys0[m]; c < sys0[m + 1]; ++c)
-            for (int32_t q = b0; q < (int32_t)blk.size(); ++q) {
-                sp_sys.push_back(c);
-                sp_blk.push_back(q);
-            }
+            for (int32_t q = b0; q < (int32_t)blk.size(); ++q) (n > SB_CAP ? item : shorter).push_back(make_int2(c, q));
     }
-    const int32_t nsp = (int32_t)sp_sys.size(), nblk = (int32_t)blk.size();
+    const int32_t nlong = (int32_t)item.size(), nblk = (int32_t)blk.size();
+    item.insert(item.end(), shorter.begin(), shorter.end());
     Buf tab, vecs, bst, bsi, part, misc;
-    const size_t tab_bytes = sizeof(int4) * (size_t)nblk + sizeof(int32_t) * 2 * ((size_t)nsp + 1) +
+    const size_t tab_bytes = sizeof(int4) * (size_t)nblk + sizeof(int2) * item.size() +
                              sizeof(int64_t) * (nsys + nmat + nmat + 1) +
                              sizeof(int32_t) * (4 * (size_t)nsys + 1 + 2 * (size_t)nit + 2 * (size_t)nmat + joff[nmat] + 1);
     SAI_TRY(tab.alloc(tab_bytes + 64, st, true));
@@ -860,10 +855,9 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     };
     BSys Y;
     Y.blk = (const int4*)put(blk.data(), sizeof(int4) * nblk);
-    Y.sp_sys = (const int32_t*)put(sp_sys.data(), sizeof(int32_t) * nsp);
-    Y.sp_blk = (const int32_t*)put(sp_blk.data(), sizeof(int32_t) * nsp);
-    Y.nsp = nsp;
-    Y.ncap = nmax < SB_CAP ? nmax : SB_CAP;
+    Y.item = (const int2*)put(item.data(), sizeof(int2) * item.size());
+    Y.nitem = (int32_t)item.size();
+    Y.nlong = nlong;
     Y.nsys = nsys;
     Y.nitems = nit;
     Y.off = (const int64_t*)put(off.data(), sizeof(int64_t) * nsys);
@@ -956,13 +950,14 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     const RowBlocks rb{(int)N, SB, Y.blk};
     SAI_TRY(sorted_rows<double>(rb, nblk, Ar, bd.Atr_ci.as<int32_t>(), bd.Atr_v.as<double>(), sa, st));
     SAI_TRY(sorted_rows<double>(rb, nblk, Mr, P.Mr_ci.as<int32_t>(), P.Mr_v.as<double>(), smb, st));
-    // staging pays where a row has more entries than the copy has loads per row
-    auto bmat = [&](const Buf (&b)[4], int64_t nnz) {
-        return BMat{b[1].as<int64_t>(), b[2].as<int32_t>(), b[3].as<double>(), b[0].as<int32_t>(), nnz > 4 * N};
+    auto bmat = [](const Buf (&b)[4]) {
+        return BMat{b[1].as<int64_t>(), b[2].as<int32_t>(), b[3].as<double>(), b[0].as<int32_t>()};
     };
-    const BMat Am = bmat(sa, bd.nnz_At), Mm = bmat(smb, P.nnz);
-    const size_t sm0 = sizeof(double) * SB, sm1 = sm0 + sizeof(double) * (size_t)Y.ncap;
-    for (auto kern : {k_b_spmv<0>, k_b_spmv<1>, k_b_spmv<2>})
+    const BMat Am = bmat(sa), Mm = bmat(smb);
+    const bool some = nlong < Y.nitem;
+    const bool stA = some && bd.nnz_At > SB_ROW * N, stM = some && P.nnz > SB_ROW * N;
+    const size_t sm0 = sizeof(double) * SB, sm1 = sm0 + sizeof(double) * (size_t)nst;
+    for (auto kern : {k_b_spmv<0, true>, k_b_spmv<1, true>, k_b_spmv<2, true>})
         SAI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
     const unsigned gw = grid_for(sai_div_up(nit, BR / 32), cap);  // vector kernels: one warp per item
     const unsigned gs = sai_div_up((int64_t)nsys * 32, 256);
@@ -972,11 +967,18 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     Wk.Arp = Ar;
     Wk.Mrp = Mr;
     double* Xd = X;  // the iterates of the current pass
-    auto spmv = [&](decltype(&k_b_spmv<0>) kern, const BMat& Mt, const double* xin, double* yout, const int* flags,
+    // one launch, or one for the staged systems and one for the long ones
+    auto spmv = [&](auto nd, bool stage, const BMat& Mt, const double* xin, double* yout, const int* flags,
                     const double* dot, cudaStream_t q) {
-        const bool stg = Mt.stage;
-        kern<<<SAI_GRID(nsp), stg ? 1024 : 256, stg ? sm1 : sm0, q>>>(Y, Mt, xin, yout, flags, dot, pt);
+        constexpr int ND = decltype(nd)::value;
+        const int32_t nshort = stage ? Y.nitem - Y.nlong : 0;
+        if (nshort > 0) k_b_spmv<ND, true><<<SAI_GRID(nshort), 1024, sm1, q>>>(Y, Mt, xin, yout, flags, dot, pt);
+        if (Y.nitem > nshort)
+            k_b_spmv<ND, false><<<SAI_GRID(Y.nitem - nshort), 256, sm0, q>>>(Y, Mt, xin, yout, flags, dot, pt);
     };
+    using I0 = std::integral_constant<int, 0>;
+    using I1 = std::integral_constant<int, 1>;
+    using I2 = std::integral_constant<int, 2>;
     // profile scopes act only while a profile is open, when no graph is captured
     auto iteration = [&](cudaStream_t q) {
         {
@@ -985,11 +987,11 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
         }
         {
             ProfScope ps(PROF_SPMM, q);
-            spmv(k_b_spmv<0>, Mm, p, ph, S.active, nullptr, q);
+            spmv(I0(), stM, Mm, p, ph, S.active, nullptr, q);
         }
         {
             ProfScope ps(PROF_SPMM, q);
-            spmv(k_b_spmv<1>, Am, ph, v, S.active, rh, q);
+            spmv(I1(), stA, Am, ph, v, S.active, rh, q);
         }
         k_b_alpha<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, S, Wk);
         {
@@ -999,11 +1001,11 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
         k_b_f2<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, S);
         {
             ProfScope ps(PROF_SPMM, q);
-            spmv(k_b_spmv<0>, Mm, s, sh, S.go, nullptr, q);
+            spmv(I0(), stM, Mm, s, sh, S.go, nullptr, q);
         }
         {
             ProfScope ps(PROF_SPMM, q);
-            spmv(k_b_spmv<2>, Am, sh, t, S.go, s, q);
+            spmv(I2(), stA, Am, sh, t, S.go, s, q);
         }
         k_b_omega<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, S, Wk);
         {
@@ -1012,7 +1014,8 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
         }
         k_b_f4<<<SAI_GRID(gs), 256, 0, q>>>(Y, pt, maxit, S);
     };
-    constexpr int ITERS_PER_CHECK = 8, LAUNCHES = ITERS_PER_CHECK * 11 + 1;
+    constexpr int ITERS_PER_CHECK = 8;
+    const int LAUNCHES = ITERS_PER_CHECK * (11 + (nlong > 0 ? 2 * stA + 2 * stM : 0)) + 1;
     int* nbody = any + 1;  // body runs of the while graph
     // One pass of the batched BiCGStab from x = 0 on the right-hand sides
     // Bsrc (thresholds in S.thr), iterates into Xdst. Without an open
@@ -1180,7 +1183,7 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
             int* dsel = (int*)(D + NV);  // the continued systems
             SAI_CUDA(cudaMemcpyAsync(dsel, sel.data(), sizeof(int) * nsys, cudaMemcpyHostToDevice, st));
             SAI_CUDA(cudaMemsetAsync(R, 0, sizeof(double) * (size_t)NV, st));
-            spmv(k_b_spmv<0>, Am, X, R, dsel, nullptr, st);
+            spmv(I0(), stA, Am, X, R, dsel, nullptr, st);
             k_b_resid<<<SAI_GRID(gw), BR, 0, st>>>(Y, Bv, dsel, R);
             SAI_CUDA(cudaGetLastError());
             SAI_CUDA(cudaMemcpyAsync(S.thr, thr2.data(), sizeof(double) * nsys, cudaMemcpyHostToDevice, st));

@@ -1,8 +1,8 @@
 """The batched products at the edges of their blocks: 2048 rows per block, rows sorted by length within it, vectors of up
-to 24576 rows staged in shared memory. One batch holds orders on both sides of each limit, with rows of up to 700
-entries among rows of three.
+to 12288 rows staged in shared memory. One batch holds orders on both sides of each limit, with rows of up to 700
+entries among rows of three or seven.
 
-Tolerance: A is diagonally dominant by 2 with ||A|| <= 7, and the solver stops on the recursive residual; in at most 60
+Tolerance: A is diagonally dominant by 2 with ||A|| <= 9, and the solver stops on the recursive residual; in at most 60
 iterations the true one differs from it by less than 60 * 8 u * ||A|| ||x|| <= 1e-12 ||b||."""
 import numpy as np
 import pytest
@@ -13,9 +13,11 @@ from gpu_helpers import lib, need_gpu, to_dev, torch
 pytestmark = pytest.mark.gpu
 
 
-def _matrix(n, rng):
-    A = sp.diags([-1.0 - 0.5 * rng.random(max(n - 1, 0)), np.full(n, 4.5), -1.0 * np.ones(max(n - 1, 0))], (-1, 0, 1),
-                 shape=(n, n))
+def _matrix(n, rng, bands):
+    A = sp.diags([-1.0 - 0.5 * rng.random(n), np.full(n, 5.5), -np.ones(n)], (-1, 0, 1), shape=(n, n))
+    for o in (-7, -3, 3, 7) if bands else ():  # rows long enough for staging
+        if abs(o) < n:
+            A = A + sp.diags([np.full(n - abs(o), 0.1)], (o,), shape=(n, n))
     rows, cols = [], []
     for i in {0, n // 2, n - 1}:
         length = min(n, int(rng.integers(1, 701)))
@@ -28,14 +30,16 @@ def _matrix(n, rng):
     return A
 
 
-@pytest.mark.parametrize("orders", [(1, 2, 31, 33), (255, 257, 2047, 2048, 2049, 6145), (24575, 24576, 24577, 700, 40001)])
+@pytest.mark.parametrize("bands", [False, True])
+@pytest.mark.parametrize("orders", [(1, 2, 31, 33), (255, 257, 2047, 2048, 2049, 6145), (24575, 24576, 24577, 700, 40001), (12287, 12288),
+                                    (12289, 14337), (12288, 12289, 64)])
 @pytest.mark.parametrize("kw", [dict(sai="spai", delta=0.4, mn=2, max_aug=5), dict(sai="psai", delta=0.4, tol=1e-3,
                                                                                   tol_mode=1, lmax=3)])
-def test_batch_at_block_edges(orders, kw):
+def test_batch_at_block_edges(orders, kw, bands):
     need_gpu()
     sai = lib()
     rng = np.random.default_rng(sum(orders))
-    As = [_matrix(n, rng) for n in orders]
+    As = [_matrix(n, rng, bands) for n in orders]
     bs = [rng.standard_normal(n) for n in orders]
     xs, per, rep = sai.solve_batched([to_dev(A) for A in As], [torch.as_tensor(b, device="cuda") for b in bs],
                                      eps=1e-10, maxit=60, **kw)
