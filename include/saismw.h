@@ -328,7 +328,7 @@ sai_status sai_krylov_solve(sai_split h, sai_precond P, int32_t k, const double*
  * Y: n x (s+1) row-major, column 0 = yhat, columns 1..s = What.
  * x: n. c_out (host, may be NULL): c = ||(I + V^T What)^{-1} V^T yhat||.
  * Gaussian elimination with partial pivoting on the s x s matrix (the
- * largest |pivot|, the first row on ties): one thread block for s <= 256, a
+ * largest |pivot|, the first row on ties): one thread block for s <= 160, a
  * blocked right-looking LU (panels of 16 columns, FP64 tiles for the
  * trailing update) for larger s. SAI_SINGULAR on a zero pivot, after which
  * x is not valid.

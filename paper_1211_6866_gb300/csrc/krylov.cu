@@ -13,8 +13,9 @@
 // last block to arrive rebuilding the list); data-parallel kernels loop over the
 // items (system in the list) x (row tile or row chunk), so converged systems
 // cost nothing and the host never needs to know which systems are active.
-// Inner products are formed per (system, row chunk) by one warp and summed
-// in a fixed order, so results do not depend on scheduling.
+// Inner products are formed per (system, row chunk) by one block and summed
+// in a fixed order, so results do not depend on scheduling. Small orders run
+// in one thread-block cluster per system (bicg_cluster.cuh, gmres_cluster.cuh).
 //
 // BiCGStab: van der Vorst's recurrence on A~ M z = b with y = M z updated
 // directly; stop tests after the half step (s) and the full step (r).
