@@ -2258,6 +2258,9 @@ __global__ void __launch_bounds__(STEP_THREADS) k_dc_step(int k, int nch, const 
         }
         __syncthreads();
         const double al = sh[0], d = sh[1], ial = sh[2];
+        static_assert(STEP_THREADS >= 32 + GM_MAXM + 1, "a row of Hbar s per thread past the first warp");
+        const int row = tid - 32;
+        T hs = 0;
         for (int i = tid; i < j; i += blockDim.x) rsT[i] = (T)red[2 * i];
         if (j >= 1) {
             // column j-1: first-pass coefficients + s, subdiagonal alpha
@@ -2268,6 +2271,22 @@ __global__ void __launch_bounds__(STEP_THREADS) k_dc_step(int k, int nch, const 
                 rc[i] = (T)v;
             }
             __syncthreads();
+            // (Hbar s)_i = sum_{q >= max(i-1,0)} Hbar(i,q) s_q over the final columns q < j
+            // (in shared memory, in T), one thread per row i, q ascending, the column
+            // loads in batches of 8 ahead of their FMAs; beside the rotations of thread 0,
+            // in other warps (after them: 37^3 in FP64 20.5 ms against 20.2, 64^3 refined 47.9
+            // against 47.6)
+            if (row >= 0 && row <= j) {
+                int q = row > 0 ? row - 1 : 0;
+                for (; q + 8 <= j; q += 8) {
+                    T hv[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) hv[u] = hsmT[(size_t)(q + u) * (m + 1) + row];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) hs = fma(hv[u], rsT[q + u], hs);
+                }
+                for (; q < j; ++q) hs = fma(hsmT[(size_t)q * (m + 1) + row], rsT[q], hs);
+            }
             if (tid == 0) {
                 T ri = rc[0];
                 for (int i = 0; i < j - 1; ++i) {
@@ -2308,24 +2327,8 @@ __global__ void __launch_bounds__(STEP_THREADS) k_dc_step(int k, int nch, const 
         }
         __syncthreads();
         if (!stop) {
-            // first-pass coefficients of column j and the update coefficients;
-            // (Hbar s)_i = sum_{q >= max(i-1,0)} Hbar(i,q) s_q over the final columns q < j
-            // (in shared memory, in T), one thread per row i, q ascending, the column
-            // loads in batches of 8 ahead of their FMAs
-            for (int i = tid; i <= j; i += blockDim.x) {
-                T hs = 0;
-                int q = i > 0 ? i - 1 : 0;
-                for (; q + 8 <= j; q += 8) {
-                    T hv[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) hv[u] = hsmT[(size_t)(q + u) * (m + 1) + i];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) hs = fma(hv[u], rsT[q + u], hs);
-                }
-                for (; q < j; ++q) hs = fma(hsmT[(size_t)q * (m + 1) + i], rsT[q], hs);
-                const double cz = i < j ? red[2 * i + 1] : d;
-                hpc[i] = (cz - (double)hs) * ial;
-            }
+            // first-pass coefficients of column j and the update coefficients
+            if (row >= 0 && row <= j) hpc[row] = ((row < j ? red[2 * row + 1] : d) - (double)hs) * ial;
             for (int i = tid; i < j; i += blockDim.x) {
                 G.sco[(size_t)c * (m + 1) + i] = red[2 * i];
                 G.cco[(size_t)c * (m + 1) + i] = red[2 * i + 1];
