@@ -7,7 +7,9 @@
 // blocks keeps all nine vectors of its system in shared memory (block b the
 // rows [b R, (b + 1) R)), reads the matrices through L1, gathers x across the
 // cluster by distributed-shared-memory loads and runs every iteration without
-// leaving the kernel; a phase costs a cluster barrier.
+// leaving the kernel; a phase costs a cluster barrier. A 45 x 45 grid with four
+// systems, 80 iterations: 11.5 ms per call at first, 2.5 ms here, 22 us per
+// iteration (six barriers, four products, three scalar chains).
 //
 // A system's bits do not depend on the cluster size or on the other systems:
 // row sums run over the row's entries in order, and an inner product is a
