@@ -202,14 +202,11 @@ sai_status sai_split_create(const sai_csc_view* A, const sai_split_params* prm, 
     *out = nullptr;
     if (prm && prm->zero_diag != 0) return SAI_INVALID_ARG;  // the repair belongs to sai_solve
     sai_pool_init_once();
-    sai_split_s* h = new (std::nothrow) sai_split_s();
+    std::unique_ptr<sai_split_s> h(new (std::nothrow) sai_split_s());
     if (!h) return SAI_OOM;
-    sai_status st = sai_split_build(A, prm, S(stream), false, h);
-    if (st != SAI_OK) {
-        delete h;
-        return st;
-    }
-    *out = h;
+    HandleUse use{h.get(), nullptr, S(stream)};
+    SAI_TRY(sai_split_build(A, prm, S(stream), false, h.get()));
+    *out = h.release();
     return SAI_OK;
 }
 
@@ -233,6 +230,7 @@ sai_status sai_split_copy_out(sai_split h, int64_t* At_col_ptr, int32_t* At_row_
 {
     if (!h) return SAI_INVALID_ARG;
     cudaStream_t st = S(stream);
+    HandleUse use{h, nullptr, st};
     const cudaMemcpyKind D = cudaMemcpyDeviceToDevice;
     if (At_col_ptr) SAI_CUDA(cudaMemcpyAsync(At_col_ptr, h->At_cp.p, sizeof(int64_t) * (h->n + 1), D, st));
     if (At_row_idx && h->nnz_At) SAI_CUDA(cudaMemcpyAsync(At_row_idx, h->At_ri.p, sizeof(int32_t) * h->nnz_At, D, st));
@@ -250,6 +248,7 @@ sai_status sai_build_autotune(sai_split h, int32_t sai, const sai_spai_params* s
                               sai_stream_t stream, sai_build_tuning* out)
 {
     sai_pool_init_once();
+    HandleUse use{h, nullptr, S(stream)};
     return sai_build_autotune_run(h, sai, spai, psai, S(stream), out);
 }
 
@@ -260,14 +259,11 @@ sai_status sai_build_spai(sai_split h, const sai_spai_params* prm, sai_stream_t 
     if (!out) return SAI_INVALID_ARG;
     *out = nullptr;
     sai_pool_init_once();
-    sai_precond_s* P = new (std::nothrow) sai_precond_s();
+    std::unique_ptr<sai_precond_s> P(new (std::nothrow) sai_precond_s());
     if (!P) return SAI_OOM;
-    sai_status st = sai_spai_build(h, prm, S(stream), false, P);
-    if (st != SAI_OK) {
-        delete P;
-        return st;
-    }
-    *out = P;
+    HandleUse use{h, P.get(), S(stream)};
+    SAI_TRY(sai_spai_build(h, prm, S(stream), false, P.get()));
+    *out = P.release();
     return SAI_OK;
 }
 
@@ -276,14 +272,11 @@ sai_status sai_build_psai(sai_split h, const sai_psai_params* prm, sai_stream_t 
     if (!out) return SAI_INVALID_ARG;
     *out = nullptr;
     sai_pool_init_once();
-    sai_precond_s* P = new (std::nothrow) sai_precond_s();
+    std::unique_ptr<sai_precond_s> P(new (std::nothrow) sai_precond_s());
     if (!P) return SAI_OOM;
-    sai_status st = sai_psai_build(h, prm, S(stream), false, P);
-    if (st != SAI_OK) {
-        delete P;
-        return st;
-    }
-    *out = P;
+    HandleUse use{h, P.get(), S(stream)};
+    SAI_TRY(sai_psai_build(h, prm, S(stream), false, P.get()));
+    *out = P.release();
     return SAI_OK;
 }
 
@@ -300,6 +293,7 @@ sai_status sai_precond_create(const sai_csc_view* M, sai_stream_t stream, sai_pr
     SAI_TRY(sai_validate_csc(n, n, nnz, M->col_ptr, M->row_idx, st));
     std::unique_ptr<sai_precond_s> P(new (std::nothrow) sai_precond_s());
     if (!P) return SAI_OOM;
+    HandleUse use{nullptr, P.get(), st};
     P->n = n;
     P->nnz = nnz;
     const size_t nn = (size_t)(n > 0 ? n : 1), nz = (size_t)(nnz > 0 ? nnz : 1);
@@ -342,6 +336,7 @@ sai_status sai_precond_copy_out(sai_precond P, int64_t* col_ptr, int32_t* row_id
 {
     if (!P) return SAI_INVALID_ARG;
     cudaStream_t st = S(stream);
+    HandleUse use{nullptr, P, st};
     const cudaMemcpyKind D = cudaMemcpyDeviceToDevice;
     if (col_ptr) SAI_CUDA(cudaMemcpyAsync(col_ptr, P->M_cp.p, sizeof(int64_t) * (P->n + 1), D, st));
     if (row_idx && P->nnz) SAI_CUDA(cudaMemcpyAsync(row_idx, P->M_ri.p, sizeof(int32_t) * P->nnz, D, st));
@@ -359,12 +354,14 @@ sai_status sai_krylov_solve(sai_split h, sai_precond P, int32_t k, const double*
                             sai_stream_t stream)
 {
     sai_pool_init_once();
+    HandleUse use{h, P, S(stream)};
     return sai_krylov_run(h, P, k, B, thr, prm, X, iters, status, S(stream));
 }
 
 sai_status sai_smw_recover(sai_split h, const double* Y, double* x, double* c_out, sai_stream_t stream)
 {
     sai_pool_init_once();
+    HandleUse use{h, nullptr, S(stream)};
     return sai_smw_run(h, Y, x, c_out, S(stream));
 }
 
@@ -796,6 +793,7 @@ extern "C" sai_status sai_solve_with(const sai_csc_view* A, sai_split h, sai_pre
                                      sai_solve_report* rep, sai_stream_t stream)
 {
     sai_pool_init_once();
+    HandleUse use{h, P, S(stream)};
     return solve_with_impl(A, h, P, b, prm, x, iters, iters_cap, rep, S(stream));
 }
 
@@ -804,6 +802,7 @@ extern "C" sai_status sai_backward(const sai_csc_view* A, sai_split h, sai_preco
                                    int32_t* iters, int32_t iters_cap, sai_solve_report* rep, sai_stream_t stream)
 {
     sai_pool_init_once();
+    HandleUse use{h, P, S(stream)};
     return backward_impl(A, h, P, x, g, prm, lambda, grad_vals, iters, iters_cap, rep, S(stream));
 }
 

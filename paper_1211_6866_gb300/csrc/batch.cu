@@ -1283,15 +1283,12 @@ extern "C" sai_status sai_build_batched(int32_t nmat, const sai_csc_view* A, con
     std::vector<std::unique_ptr<sai_split_s>> hs;
     sai_split_s bd;
     SAI_TRY(split_and_stack(nmat, A, prm, hs, bd, st));
-    sai_precond_s* P = new (std::nothrow) sai_precond_s();
+    std::unique_ptr<sai_precond_s> P(new (std::nothrow) sai_precond_s());
     if (!P) return SAI_OOM;
-    const sai_status r = prm->sai == 0 ? sai_spai_build(&bd, &prm->spai, st, false, P)
-                                       : sai_psai_build(&bd, &prm->psai, st, false, P);
-    if (r != SAI_OK) {
-        delete P;
-        return r;
-    }
-    *out = P;
+    HandleUse use{nullptr, P.get(), st};
+    SAI_TRY(prm->sai == 0 ? sai_spai_build(&bd, &prm->spai, st, false, P.get())
+                          : sai_psai_build(&bd, &prm->psai, st, false, P.get()));
+    *out = P.release();
     return SAI_OK;
 }
 

@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "common.cuh"
 #include "saismw.h"
 
@@ -12,9 +14,9 @@
 // handle has ten to twelve buffers, and cudaMalloc / cudaFree of them took a
 // third of a small split or build), larger ones from cudaMalloc, so that a
 // large handle's memory goes back to the driver when it is destroyed. A
-// handle's creation synchronises its stream before it returns, and its
-// destruction waits for the device (as cudaFree does) before it frees: its
-// buffers may be used on any stream meanwhile.
+// handle's creation synchronises its stream before it returns; its pooled
+// buffers are freed on a stream of their own (sai_free_stream) after the work
+// of every stream that has used the handle (HandleUses).
 constexpr size_t HANDLE_POOL_MAX = size_t(32) << 20;
 struct Buf {
     void* p = nullptr;
@@ -55,12 +57,36 @@ sai_status sai_csc_residual_norms(int32_t n, const int64_t* cp, const int32_t* r
                                   const double* b, const double* x, double* out2_host, cudaStream_t st);
 
 // Handle internals --------------------------------------------------------
-// Waits for the device of a handle's pooled buffer.
-void sai_quiesce(const Buf& b);
+// Library-owned non-blocking stream of the current device on which handles'
+// pooled buffers are freed (nothing else runs on it, and it is never captured),
+// or nullptr.
+cudaStream_t sai_free_stream();
+
+// The streams that have used a handle, each with an event behind its last use.
+// A handle's destruction makes the free stream wait for these events. It does
+// not synchronise the device: that is not permitted while another thread
+// captures a stream (every GMRES call of a large order does) and would break
+// that capture.
+class HandleUses {
+  public:
+    // The work enqueued on st so far may use the handle. A stream in capture
+    // runs nothing: whoever replays its graph keeps the handle alive.
+    void record(cudaStream_t st);
+    // Orders the free stream after every recorded use.
+    void before_free();
+
+  private:
+    static constexpr int MAX = 16;  // further streams share the last event
+    std::mutex mu;
+    int cnt = 0, dev = -1;
+    cudaStream_t st[MAX];
+    cudaEvent_t ev[MAX];
+};
 
 struct sai_split_s {
     sai_split_s() = default;
-    ~sai_split_s() { sai_quiesce(J); }
+    ~sai_split_s() { uses.before_free(); }
+    mutable HandleUses uses;
     int32_t n = 0, s = 0, p = 0, p_keep = 0;
     double tau = 0.0, norm1 = 0.0;
     int64_t nnz_At = 0, nnz_U = 0;
@@ -74,7 +100,8 @@ struct sai_split_s {
 
 struct sai_precond_s {
     sai_precond_s() = default;
-    ~sai_precond_s() { sai_quiesce(loops); }
+    ~sai_precond_s() { uses.before_free(); }
+    mutable HandleUses uses;
     int32_t n = 0;
     int64_t nnz = 0;
     int32_t n_c = 0, l_m = 0;
@@ -83,6 +110,19 @@ struct sai_precond_s {
     Buf M_cp, M_ri, M_v;     // CSC
     Buf Mr_rp, Mr_ci, Mr_v;  // CSR
     Buf loops, res, res_post;
+};
+
+// Records the use of handles (nullptr: none) by a call on st when it ends,
+// with whatever status: an error may leave work in flight.
+struct HandleUse {
+    const sai_split_s* h;
+    const sai_precond_s* P;
+    cudaStream_t st;
+    ~HandleUse()
+    {
+        if (h) h->uses.record(st);
+        if (P) P->uses.record(st);
+    }
 };
 
 sai_status sai_split_build(const sai_csc_view* A, const sai_split_params* prm, cudaStream_t st, bool async,

@@ -13,7 +13,7 @@ sai_status Buf::alloc(size_t nbytes, cudaStream_t s, bool use_async)
     bytes = nbytes;
     dev = -1;
     if (nbytes == 0) return SAI_OK;
-    const bool pool = use_async || nbytes <= HANDLE_POOL_MAX;
+    const bool pool = use_async || (nbytes <= HANDLE_POOL_MAX && sai_free_stream());
     int d = -1;
     if (pool && !use_async && cudaGetDevice(&d) != cudaSuccess) return SAI_CUDA_ERROR;
     cudaError_t e = pool ? cudaMallocAsync(&p, nbytes, s) : cudaMalloc(&p, nbytes);
@@ -31,10 +31,9 @@ void Buf::release()
     if (p && async) {
         cudaFreeAsync(p, st);
     } else if (p && dev >= 0) {
-        // the creating stream may be gone: the device's legacy stream orders the free
         int cur = -1;
         const bool other = cudaGetDevice(&cur) == cudaSuccess && cur != dev && cudaSetDevice(dev) == cudaSuccess;
-        cudaFreeAsync(p, nullptr);
+        cudaFreeAsync(p, sai_free_stream());
         if (other) cudaSetDevice(cur);
     } else if (p) {
         cudaFree(p);
@@ -44,12 +43,65 @@ void Buf::release()
     dev = -1;
 }
 
-void sai_quiesce(const Buf& b)
+cudaStream_t sai_free_stream()
 {
-    if (!b.p || b.async || b.dev < 0) return;
+    static std::mutex mu;
+    static cudaStream_t streams[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!streams[dev] && cudaStreamCreateWithFlags(&streams[dev], cudaStreamNonBlocking) != cudaSuccess) {
+        (void)cudaGetLastError();
+        streams[dev] = nullptr;
+    }
+    return streams[dev];
+}
+
+void HandleUses::record(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cs;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return;
+    }
+    if (cs != cudaStreamCaptureStatusNone) return;
+    std::lock_guard<std::mutex> lk(mu);
+    int q = 0;
+    while (q < cnt && st[q] != s) ++q;
+    bool ok = true;
+    if (q == cnt && cnt < MAX) {
+        ok = (dev >= 0 || cudaGetDevice(&dev) == cudaSuccess) &&
+             cudaEventCreateWithFlags(&ev[q], cudaEventDisableTiming) == cudaSuccess;
+        if (ok) ++cnt;
+    } else {
+        // the event moves on to this use and stays behind its earlier ones: of
+        // another stream (the table is full, or a new stream has an old one's
+        // handle) or of this one, for which the wait is nothing
+        if (q == cnt) q = MAX - 1;
+        ok = cudaStreamWaitEvent(s, ev[q], 0) == cudaSuccess;
+    }
+    if (ok) {
+        st[q] = s;
+        ok = cudaEventRecord(ev[q], s) == cudaSuccess;
+    }
+    if (!ok) {
+        (void)cudaGetLastError();
+        cudaStreamSynchronize(s);
+    }
+}
+
+void HandleUses::before_free()
+{
+    if (cnt == 0) return;
     int cur = -1;
-    const bool other = cudaGetDevice(&cur) == cudaSuccess && cur != b.dev && cudaSetDevice(b.dev) == cudaSuccess;
-    cudaDeviceSynchronize();
+    const bool other = cudaGetDevice(&cur) == cudaSuccess && cur != dev && cudaSetDevice(dev) == cudaSuccess;
+    cudaStream_t f = sai_free_stream();
+    for (int q = 0; q < cnt; ++q) {
+        if (!f || cudaStreamWaitEvent(f, ev[q], 0) != cudaSuccess) cudaEventSynchronize(ev[q]);
+        cudaEventDestroy(ev[q]);
+    }
+    (void)cudaGetLastError();
+    cnt = 0;
     if (other) cudaSetDevice(cur);
 }
 
