@@ -958,7 +958,7 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     const bool stA = some && bd.nnz_At > SB_ROW * N, stM = some && P.nnz > SB_ROW * N;
     const size_t sm0 = sizeof(double) * SB, sm1 = sm0 + sizeof(double) * (size_t)nst;
     for (auto kern : {k_b_spmv<0, true>, k_b_spmv<1, true>, k_b_spmv<2, true>})
-        SAI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
+        SAI_CUDA(sai_smem_limit(kern, sizeof(double) * (SB + SB_CAP)));
     const unsigned gw = grid_for(sai_div_up(nit, BR / 32), cap);  // vector kernels: one warp per item
     const unsigned gs = sai_div_up((int64_t)nsys * 32, 256);
     double* pt = part.as<double>();
@@ -1141,8 +1141,8 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
     W.c = cvec;
     W.err = errv;
     const size_t smw_smem = sizeof(double) * ((size_t)smax * smax + smax);
-    if (smw_smem > 48 * 1024)
-        SAI_CUDA(cudaFuncSetAttribute(k_b_smw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw_smem));
+    constexpr size_t smw_limit = 220 * 1024;  // larger systems are refused here
+    if (smw_smem > 48 * 1024) SAI_CUDA(sai_smem_limit(k_b_smw, smw_smem > smw_limit ? smw_smem : smw_limit));
     auto smw_all = [&]() -> sai_status {
         SAI_CUDA(cudaMemsetAsync(cvec, 0, sizeof(double) * nmat, st));
         SAI_CUDA(cudaMemsetAsync(errv, 0, sizeof(int) * nmat, st));

@@ -25,6 +25,7 @@ constexpr int CL_MAXN = CL_MAXR * CL_MAXC;
 constexpr int CL_UNIT = 64;      // rows per reduction unit
 constexpr int CL_VECS = 9;
 constexpr int CL_SLOTS = 6;      // partial sums: rhat^T v; ||s||; t^T s, t^T t; ||r||, rhat^T r
+constexpr size_t CL_SMEM = sizeof(double) * ((size_t)CL_VECS * CL_MAXR + (size_t)CL_SLOTS * (CL_MAXN / CL_UNIT));  // at most
 
 // A matrix in slices of 32 rows, entries column-major within a slice (slice q
 // at sp[q] .. sp[q + 1]). With ord, the rows of each block are sorted by
@@ -481,9 +482,10 @@ inline int cl_blocks(int k, int n)
     return C;
 }
 
-// true when the GPU holds k clusters of 16 blocks of kern at once
+// true when the GPU holds k clusters of 16 blocks of kern at once; limit: the
+// most dynamic shared memory of kern's launches
 template <class... Params>
-bool cl_fits16(void (*kern)(Params...), int k, int threads, size_t smem)
+bool cl_fits16(void (*kern)(Params...), int k, int threads, size_t limit, size_t smem)
 {
     if (16 * (int64_t)k > g_sms) return false;
     cudaLaunchConfig_t cfg = {};
@@ -498,7 +500,7 @@ bool cl_fits16(void (*kern)(Params...), int k, int threads, size_t smem)
     cfg.numAttrs = 1;
     int most = 0;
     const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+                    sai_smem_limit(kern, limit) == cudaSuccess &&
                     cudaOccupancyMaxActiveClusters(&most, kern, &cfg) == cudaSuccess;
     if (!ok) (void)cudaGetLastError();
     return ok && most >= k;
@@ -506,9 +508,9 @@ bool cl_fits16(void (*kern)(Params...), int k, int threads, size_t smem)
 
 // Launches kern with k clusters of C blocks; false when the device refuses the shape.
 template <class... Params, class... Args>
-bool cl_run(void (*kern)(Params...), int k, int C, int threads, size_t smem, cudaStream_t st, Args... args)
+bool cl_run(void (*kern)(Params...), int k, int C, int threads, size_t limit, size_t smem, cudaStream_t st, Args... args)
 {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (sai_smem_limit(kern, limit) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
     }
@@ -548,14 +550,14 @@ inline sai_status cl_bicgstab(const Ops<double>& A, int k, int n, int64_t ld, co
     // from 512 rows per block on the FP64 pipe outweighs the barriers
     if (C == CL_MAXC && rmax >= 512) {
         shape(16);
-        if (!cl_fits16(k_bicg_cluster<true>, k, CL_T, smem)) shape(CL_MAXC);
+        if (!cl_fits16(k_bicg_cluster<true>, k, CL_T, CL_SMEM, smem)) shape(CL_MAXC);
     }
     ClMat<double> a, m;
     Buf ab[4], mb[4];
     *ran = false;
     if (cl_matrix(A.A, n, rmax, C, ab, a, st) != SAI_OK || cl_matrix(A.M, n, rmax, C, mb, m, st) != SAI_OK)
         return SAI_OK;  // no memory for the sorted forms: the kernels below need none
-    *ran = cl_run(C > 1 ? k_bicg_cluster<true> : k_bicg_cluster<false>, k, C, CL_T, smem, st, a, m, n, ld, rmax, umax,
-                  B, X, thr, maxit, iters, status);
+    *ran = cl_run(C > 1 ? k_bicg_cluster<true> : k_bicg_cluster<false>, k, C, CL_T, CL_SMEM, smem, st, a, m, n, ld, rmax,
+                  umax, B, X, thr, maxit, iters, status);
     return SAI_OK;
 }

@@ -26,6 +26,15 @@
 
 void sai_internal_note_cuda_error(cudaError_t e, const char* what, const char* file, int line);
 
+// Opts a kernel in to `bytes` of dynamic shared memory: the most that any of
+// its launches takes, never what one launch takes. The limit belongs to the
+// function, so every host thread shares it, and a launch above it is refused.
+template <class K>
+static inline cudaError_t sai_smem_limit(K* kern, size_t bytes)
+{
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 static inline unsigned sai_div_up(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 
 // ---------------------------------------------------------------- warp tools

@@ -24,6 +24,7 @@ constexpr int GC_SUB = 2048;   // rows per partial sum
 constexpr int GC_MAXR = 6144;  // rows per block
 // orders up to which the form is used: FP32 vectors fill the shared memory
 // there; in FP64 the eight SMs' FP64 pipes are slower than all SMs' above
+constexpr size_t GC_SMEM = 220 * 1024;  // shared memory of a block, at most
 constexpr int GC_MAXN32 = GC_MAXR * CL_MAXC, GC_MAXN64 = 10240;
 
 // Shared-memory layout of one block (bytes from the start).
@@ -442,11 +443,11 @@ sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* 
     auto rows = [&](int blocks) { return ((n + blocks - 1) / blocks + CL_UNIT - 1) / CL_UNIT * CL_UNIT; };
     // from 512 rows per block on the work outweighs the barriers
     if (C == CL_MAXC && rows(C) >= 512 &&
-        cl_fits16(k_gmres_cluster<T, true>, k, GC_T, GcLayout<T>(rows(16), m, 16).bytes))
+        cl_fits16(k_gmres_cluster<T, true>, k, GC_T, GC_SMEM, GcLayout<T>(rows(16), m, 16).bytes))
         C = 16;
     const int R = rows(C);
     const GcLayout<T> L(R, m, C);
-    if (L.bytes > 220 * 1024) return SAI_OK;
+    if (L.bytes > GC_SMEM) return SAI_OK;
     GcArgs P;
     P.n = n;
     P.m = m;
@@ -476,7 +477,7 @@ sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* 
     ClMat<T> a, mm;
     Buf ab[4], mb[4];
     if (cl_matrix(A.A, n, R, C, ab, a, st) != SAI_OK || cl_matrix(A.M, n, R, C, mb, mm, st) != SAI_OK) return SAI_OK;
-    *ran = cl_run(C > 1 ? k_gmres_cluster<T, true> : k_gmres_cluster<T, false>, k, C, GC_T, L.bytes, st, a, mm, P, Wk.B, Bs,
-                  Xs, (const double*)S.thr, cap, S.iters, S.status, D);
+    *ran = cl_run(C > 1 ? k_gmres_cluster<T, true> : k_gmres_cluster<T, false>, k, C, GC_T, GC_SMEM, L.bytes, st, a, mm, P,
+                  Wk.B, Bs, Xs, (const double*)S.thr, cap, S.iters, S.status, D);
     return SAI_OK;
 }

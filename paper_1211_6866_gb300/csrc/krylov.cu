@@ -2981,9 +2981,10 @@ sai_status gmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs,
     }
     // dynamic shared memory of the two kernels that stage Hbar / R (their
     // static shared memory counts against the same per-block limit)
-    const size_t tri_smem = sizeof(double) * ((size_t)m * (m + 1) + m);
-    SAI_CUDA(cudaFuncSetAttribute(k_dc_trisolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem));
-    SAI_CUDA(cudaFuncSetAttribute(k_dc_step<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step_smem(m)));
+    auto tri = [](int r) { return sizeof(double) * ((size_t)r * (r + 1) + r); };
+    const size_t tri_smem = tri(m);
+    SAI_CUDA(sai_smem_limit(k_dc_trisolve, tri(GM_MAXM - 1)));
+    SAI_CUDA(sai_smem_limit(k_dc_step<T>, step_smem(GM_MAXM - 1)));
     int hflag = 0;
     T* r = Wk.r;
     T* w = Wk.w;
@@ -3806,7 +3807,7 @@ sai_status bgmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs
     const int64_t ld = I.ld;
     const int ib = item_blocks(n > 0 ? n : 1, k);
     const unsigned gg = bg_rows_grid(n, 256) * 4;
-    SAI_CUDA(cudaFuncSetAttribute(k_bg_lsq<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bg_lsq_smem(k)));
+    SAI_CUDA(sai_smem_limit(k_bg_lsq<T>, bg_lsq_smem(BG_KMAX)));
     VKT(I, k_gm_init, T)<<<SAI_GRID(ib), VT, 0, st>>>(I, k, Bs, Xs, R, S.lall, pt2, S.acnt, S.hn);
     SAI_CUDA(cudaMemsetAsync(B.flags, 0, sizeof(int) * 4, st));
     int h[3] = {0, 0, 0};

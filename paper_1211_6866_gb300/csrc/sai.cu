@@ -1831,7 +1831,8 @@ sai_status launch_tier(const SaiMat& A, const SpaiArgs& sa, const PsaiArgs& pa, 
     const size_t smem = WS == WS_GLOBAL ? 0 : (WS == WS_HYBRID ? T::OFF_Q : T::STRIDE) * groups;
     int per_sm = cfg.blocks_per_sm_t12;
     if (WS != WS_GLOBAL) {
-        SAI_CUDA(cudaFuncSetAttribute(k_sai<T, G, WS, PSAI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        constexpr int most = WS == WS_SHARED && T::LCAP <= 64 ? 8 : 1;  // warps per block
+        SAI_CUDA(sai_smem_limit(k_sai<T, G, WS, PSAI>, (WS == WS_HYBRID ? T::OFF_Q : T::STRIDE) * (32 / G) * most));
         SAI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sai<T, G, WS, PSAI>, threads, smem));
         if (per_sm < 1) per_sm = 1;
     }
@@ -1860,7 +1861,7 @@ sai_status launch_lane(const SaiMat& A, const SpaiArgs& sa, const PsaiArgs& pa, 
 {
     if (nwork <= 0) return SAI_OK;
     const size_t smem = LaneLayout<TQ>::WARP_BYTES;
-    SAI_CUDA(cudaFuncSetAttribute(k_sai_lane<TQ, PSAI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SAI_CUDA(sai_smem_limit(k_sai_lane<TQ, PSAI>, smem));
     int per_sm = 0;
     SAI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sai_lane<TQ, PSAI>, 32, smem));
     if (per_sm < 1) per_sm = 1;

@@ -190,8 +190,7 @@ __global__ void __launch_bounds__(LU_T) k_lu_solve(int32_t s, double* C, double*
 sai_status lu_small(int32_t s, double* C, double* g, double* z, double* c_out, int* err, cudaStream_t st)
 {
     if (s <= LU_SMEM) {
-        SAI_CUDA(cudaFuncSetAttribute(k_lu_solve<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)lu_smem(LU_SMEM)));
+        SAI_CUDA(sai_smem_limit(k_lu_solve<true>, lu_smem(LU_SMEM)));
         k_lu_solve<true><<<SAI_GRID(1), LU_T, lu_smem(s), st>>>(s, C, g, z, c_out, err);
     } else {
         k_lu_solve<false><<<SAI_GRID(1), LU_T, 0, st>>>(s, C, g, z, c_out, err);
@@ -237,6 +236,9 @@ constexpr int LU_PLD = LU_NB + 1;
 constexpr int LU_CL = 8;        // blocks per cluster
 constexpr int LU_CT = 256;      // threads per block
 constexpr int LU_PROWS = 1600;  // rows per block (218 KB)
+constexpr size_t LU_PANEL_SMEM = sizeof(double) * LU_PROWS * LU_PLD;
+// of the triangular solves, a value per row of a block: s up to 8 * 24576, whose matrix would take 309 GB
+constexpr size_t LU_TRSV_SMEM = sizeof(double) * 24576;
 
 __device__ __forceinline__ uint32_t smw_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t smw_map(uint32_t a, uint32_t rank)
@@ -603,11 +605,11 @@ __global__ void __launch_bounds__(LU_CT) k_lu_trsv(int32_t s, int R, const doubl
     }
 }
 
-// a launch of one cluster of LU_CL blocks
+// a launch of one cluster of LU_CL blocks; limit: the most dynamic shared memory of kern's launches
 template <class... Args>
-sai_status lu_cluster(void (*kern)(Args...), size_t smem, cudaStream_t st, Args... args)
+sai_status lu_cluster(void (*kern)(Args...), size_t limit, size_t smem, cudaStream_t st, Args... args)
 {
-    SAI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SAI_CUDA(sai_smem_limit(kern, limit));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(SAI_GRID(LU_CL));
     cfg.blockDim = dim3(LU_CT);
@@ -686,7 +688,8 @@ sai_status lu_big(int32_t s, double* C, double* g, double* z, double* c_out, int
         const int kb = s - k0 < LU_NB ? s - k0 : LU_NB;
         const int rows = (s - k0 + LU_CL - 1) / LU_CL;
         if (rows <= LU_PROWS)
-            SAI_TRY(lu_cluster(k_lu_panel_cluster, sizeof(double) * rows * LU_PLD, st, s, k0, kb, rows, C, piv, err));
+            SAI_TRY(lu_cluster(k_lu_panel_cluster, LU_PANEL_SMEM, sizeof(double) * rows * LU_PLD, st, s, k0, kb, rows, C,
+                               piv, err));
         else
             k_lu_panel<<<SAI_GRID(1), 1024, 0, st>>>(s, k0, kb, C, piv, err);
         k_lu_swap<<<SAI_GRID(sai_div_up((int64_t)s + 1, 256)), 256, 0, st>>>(s, k0, kb, C, g, piv, err);
@@ -699,8 +702,8 @@ sai_status lu_big(int32_t s, double* C, double* g, double* z, double* c_out, int
         }
     }
     const int R = (((int)s + LU_CL - 1) / LU_CL + 31) / 32 * 32;
-    SAI_TRY(lu_cluster(k_lu_trsv, sizeof(double) * R, st, s, R, (const double*)C, (const double*)g, z, c_out,
-                       (const int*)err));
+    SAI_TRY(lu_cluster(k_lu_trsv, LU_TRSV_SMEM, sizeof(double) * R, st, s, R, (const double*)C, (const double*)g, z,
+                       c_out, (const int*)err));
     SAI_CUDA(cudaGetLastError());
     return SAI_OK;
 }
