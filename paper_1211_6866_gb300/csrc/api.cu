@@ -64,16 +64,38 @@ void sai_pool_init_once()
 
 static inline cudaStream_t S(sai_stream_t s) { return (cudaStream_t)s; }
 
-cudaStream_t sai_aux_stream()
+// idle streams by device; more than AUX_IDLE calls at once create and destroy theirs
+static constexpr int AUX_IDLE = 8;
+static std::mutex g_aux_mu;
+static cudaStream_t g_aux[64][AUX_IDLE];
+static int g_aux_n[64];
+
+void AuxStream::lease()
 {
-    static std::mutex mu;
-    static cudaStream_t streams[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    std::lock_guard<std::mutex> lk(mu);
-    if (!streams[dev] && cudaStreamCreateWithFlags(&streams[dev], cudaStreamNonBlocking) != cudaSuccess)
-        streams[dev] = nullptr;
-    return streams[dev];
+    int d = 0;
+    if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return;
+    {
+        std::lock_guard<std::mutex> lk(g_aux_mu);
+        if (g_aux_n[d] > 0) s = g_aux[d][--g_aux_n[d]];
+    }
+    if (!s && cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) {
+        (void)cudaGetLastError();
+        s = nullptr;
+    }
+    dev = d;
+}
+
+AuxStream::~AuxStream()
+{
+    if (!s) return;
+    {
+        std::lock_guard<std::mutex> lk(g_aux_mu);
+        if (g_aux_n[dev] < AUX_IDLE) {
+            g_aux[dev][g_aux_n[dev]++] = s;
+            return;
+        }
+    }
+    cudaStreamDestroy(s);  // after its work
 }
 
 // Every launch of a profiled site is counted; the first k_prof_all launches

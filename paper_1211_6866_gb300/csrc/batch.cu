@@ -1037,9 +1037,11 @@ sai_status batched_impl(int32_t nmat, const sai_csc_view* A, const double* const
         cudaEvent_t ev_in = nullptr, ev_out = nullptr;
         cudaGraphExec_t gexec = nullptr;
         bool whole = false;  // gexec is the whole loop
+        AuxStream lease;
         const int max_body = (maxit + ITERS_PER_CHECK - 1) / ITERS_PER_CHECK;
         if (!sai_prof_on()) {
-            cudaStream_t aux = sai_aux_stream();
+            lease.lease();
+            cudaStream_t aux = lease.s;
             if (aux) {
                 SAI_CUDA(cudaEventCreateWithFlags(&ev_in, cudaEventDisableTiming));
                 SAI_CUDA(cudaEventCreateWithFlags(&ev_out, cudaEventDisableTiming));

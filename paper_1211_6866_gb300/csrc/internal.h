@@ -149,8 +149,19 @@ sai_status sai_permute_rows_run(const sai_csc_view* A, const int32_t* p, int64_t
 sai_status sai_gather_vec(int32_t n, const int32_t* p, const double* x, double* y, cudaStream_t st);
 
 void sai_pool_init_once();
-// Library-owned non-blocking stream of the current device (for graph capture), or nullptr.
-cudaStream_t sai_aux_stream();
+// A library-owned non-blocking stream of the current device for graph capture
+// and replay, held by one call at a time (of two calls that capture on one
+// stream the second would join, or end, the first one's capture) and given back
+// at the end of the scope. s is nullptr when no stream can be had.
+struct AuxStream {
+    cudaStream_t s = nullptr;
+    int dev = -1;
+    void lease();
+    AuxStream() = default;
+    AuxStream(const AuxStream&) = delete;
+    AuxStream& operator=(const AuxStream&) = delete;
+    ~AuxStream();
+};
 
 // Device-side algorithmic work per profiled site ([site][0] bytes, [1] flops),
 // one accumulator per translation unit.

@@ -2993,8 +2993,10 @@ sai_status gmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs,
     const bool use_graph = !sai_prof_on();
     cudaStream_t caller = st;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+    AuxStream lease;
     if (use_graph) {
-        cudaStream_t aux = sai_aux_stream();
+        lease.lease();
+        cudaStream_t aux = lease.s;
         if (aux) {
             SAI_CUDA(cudaEventCreateWithFlags(&ev_in, cudaEventDisableTiming));
             SAI_CUDA(cudaEventCreateWithFlags(&ev_out, cudaEventDisableTiming));

@@ -1,7 +1,7 @@
 """Calls from two host threads at once, each on a stream of its own.
 
 The kernels with dynamic shared memory take as much as their problem needs; two threads with problems of different size
-must not see each other's limits. Every call must succeed and give, bit for bit, what it gives alone: no sum of these
+must not see each other's limits, and calls that capture graphs must not capture on one stream. Every call must succeed and give, bit for bit, what it gives alone: no sum of these
 solvers depends on what else runs.
 """
 import threading
@@ -39,17 +39,32 @@ def _krylov(sai, n, k, **kw):
     return lambda: sai.krylov_solve(h, P, Bd, thr, **kw)[0]
 
 
+def _batch(sai, orders):
+    rng = np.random.default_rng(sum(orders))
+    As, bs = [], []
+    for n in orders:
+        d = [np.full(n - abs(o), 0.1) for o in (-7, -3, 3, 7)]
+        A = sp.diags([np.full(n - 1, -1.5), np.full(n, 5.5), -np.ones(n - 1)] + d, (-1, 0, 1, -7, -3, 3, 7))
+        As.append(to_dev(sp.csc_matrix(A)))
+        bs.append(torch.as_tensor(rng.standard_normal(n), device="cuda"))
+    return lambda: torch.cat(sai.solve_batched(As, bs, eps=1e-10)[0])
+
+
 def _pair(kind):
     sai = lib()
     if kind == "recovery":
         return _recovery(sai, 700), _recovery(sai, 2000)
     if kind == "bicgstab":
         return _krylov(sai, 2000, 4), _krylov(sai, 20000, 4)
+    if kind == "batch":
+        return _batch(sai, (700, 900)), _batch(sai, (12000, 12100))
     kw = dict(method=sai.GMRES, restart=20)
+    if kind == "gmres_graphs":  # beyond the cluster form: both capture their steps
+        return _krylov(sai, 50000, 3, **kw), _krylov(sai, 20000, 5, **kw)
     return _krylov(sai, 500, 3, **kw), _krylov(sai, 10000, 3, **kw)
 
 
-@pytest.mark.parametrize("kind", ["recovery", "bicgstab", "gmres"])
+@pytest.mark.parametrize("kind", ["recovery", "bicgstab", "gmres", "gmres_graphs", "batch"])
 def test_two_threads_with_problems_of_different_size(kind):
     need_gpu()
     calls = _pair(kind)
