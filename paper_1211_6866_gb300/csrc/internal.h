@@ -10,14 +10,17 @@
 
 // Ownership mode of a device buffer. CALL: lives inside one call, from the
 // stream-ordered pool, freed on the call's stream. HANDLE: part of a handle
-// returned to the user; up to HANDLE_POOL_MAX bytes from the same pool (a
-// handle has ten to twelve buffers, and cudaMalloc / cudaFree of them took a
-// third of a small split or build), larger ones from cudaMalloc, so that a
-// large handle's memory goes back to the driver when it is destroyed. A
+// returned to the user; up to HANDLE_POOL_MAX bytes from a pool of the
+// handles' own (a handle has ten to twelve buffers, and cudaMalloc / cudaFree
+// of them took a third of a small split or build), larger ones from
+// cudaMalloc. What is free in that pool above HANDLE_POOL_KEEP bytes goes back
+// to the driver at the next synchronisation, as destroyed handles' memory
+// should; the call pool keeps all of its scratch. A
 // handle's creation synchronises its stream before it returns; its pooled
 // buffers are freed on a stream of their own (sai_free_stream) after the work
 // of every stream that has used the handle (HandleUses).
 constexpr size_t HANDLE_POOL_MAX = size_t(32) << 20;
+constexpr size_t HANDLE_POOL_KEEP = size_t(256) << 20;  // two handles of 262144 rows
 struct Buf {
     void* p = nullptr;
     size_t bytes = 0;
@@ -59,8 +62,9 @@ sai_status sai_csc_residual_norms(int32_t n, const int64_t* cp, const int32_t* r
 // Handle internals --------------------------------------------------------
 // Library-owned non-blocking stream of the current device on which handles'
 // pooled buffers are freed (nothing else runs on it, and it is never captured),
-// or nullptr.
+// or nullptr; and the pool they come from, nullptr without either.
 cudaStream_t sai_free_stream();
+cudaMemPool_t sai_handle_pool();
 
 // The streams that have used a handle, each with an event behind its last use.
 // A handle's destruction makes the free stream wait for these events. It does

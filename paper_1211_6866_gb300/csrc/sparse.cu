@@ -13,10 +13,12 @@ sai_status Buf::alloc(size_t nbytes, cudaStream_t s, bool use_async)
     bytes = nbytes;
     dev = -1;
     if (nbytes == 0) return SAI_OK;
-    const bool pool = use_async || (nbytes <= HANDLE_POOL_MAX && sai_free_stream());
+    const cudaMemPool_t pool = !use_async && nbytes <= HANDLE_POOL_MAX ? sai_handle_pool() : nullptr;
     int d = -1;
-    if (pool && !use_async && cudaGetDevice(&d) != cudaSuccess) return SAI_CUDA_ERROR;
-    cudaError_t e = pool ? cudaMallocAsync(&p, nbytes, s) : cudaMalloc(&p, nbytes);
+    if (pool && cudaGetDevice(&d) != cudaSuccess) return SAI_CUDA_ERROR;
+    cudaError_t e = use_async ? cudaMallocAsync(&p, nbytes, s)
+                    : pool    ? cudaMallocFromPoolAsync(&p, nbytes, pool, s)
+                              : cudaMalloc(&p, nbytes);
     if (e == cudaSuccess) dev = d;
     if (e != cudaSuccess) {
         p = nullptr;
@@ -55,6 +57,31 @@ cudaStream_t sai_free_stream()
         streams[dev] = nullptr;
     }
     return streams[dev];
+}
+
+cudaMemPool_t sai_handle_pool()
+{
+    static std::mutex mu;
+    static cudaMemPool_t pools[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || !sai_free_stream()) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!pools[dev]) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        uint64_t keep = HANDLE_POOL_KEEP;
+        cudaMemPool_t pool = nullptr;
+        if (cudaMemPoolCreate(&pool, &props) == cudaSuccess &&
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+            pools[dev] = pool;
+        else if (pool)
+            cudaMemPoolDestroy(pool);
+        (void)cudaGetLastError();
+    }
+    return pools[dev];
 }
 
 void HandleUses::record(cudaStream_t s)

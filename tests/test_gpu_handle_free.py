@@ -93,3 +93,21 @@ def test_split_destroyed_behind_a_solve_on_another_stream():
         s.synchronize()
         assert rep["status"] == sai.SAI_OK
         assert np.linalg.norm(b - A @ x.cpu().numpy()) <= (1e-10 + 1e-12) * np.linalg.norm(b)
+
+
+def test_memory_of_destroyed_handles_goes_back():
+    """Sixteen handles of 120 MB in buffers of at most 32 MB: all but what the handles' pool keeps (256 MB; 512 MB allow
+    for its granularity) is free again after a synchronisation."""
+    need_gpu()
+    sai = lib()
+    n = 2000000
+    M = to_dev(sp.identity(n, format="csc"))
+    sai.precond_from_csc(M)  # the calls' own scratch
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    handles = [sai.precond_from_csc(M) for _ in range(16)]
+    held = before - torch.cuda.mem_get_info()[0]
+    assert held > 1500 << 20
+    del handles
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] < 512 << 20
