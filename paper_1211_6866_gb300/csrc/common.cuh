@@ -75,6 +75,16 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
     return v;
 }
 
+// x / d by the reciprocal rd = 1 / d formed ahead of the chain that x waits
+// for; by a division where rd is no normal number (|d| below 5.6e-309, where it
+// overflows, or above 4.5e307)
+inline __device__ __noinline__ double div_slow(double x, double d) { return x / d; }
+__device__ __forceinline__ double div_by(double x, double d, double rd)
+{
+    const unsigned e = ((unsigned)__double2hiint(rd) >> 20) & 0x7ffu;
+    return e - 1u < 2046u ? x * rd : div_slow(x, d);
+}
+
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
 // ---------------------------------------------------------------- accounting

@@ -373,7 +373,7 @@ k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restri
 #pragma unroll
                 for (int e = 0; e < RPL; ++e)
                     if (q / 32 == e) {
-                        if (lane == q % 32) w[e] *= rd[e];
+                        if (lane == q % 32) w[e] = div_by(w[e], (double)Rm[(size_t)q * (q + 1) / 2 + q], rd[e]);
                         yq = __shfl_sync(SAI_FULL, w[e], q % 32);
                     }
 #pragma unroll

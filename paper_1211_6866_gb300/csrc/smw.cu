@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(LU_T) k_lu_solve(int32_t s, double* C, double*
 #pragma unroll
             for (int q = 0; q < RPL; ++q)
                 if (j / 32 == q) {
-                    if (lane == j % 32) t[q] *= rd[q];
+                    if (lane == j % 32) t[q] = div_by(t[q], A[(size_t)j * ld + j], rd[q]);
                     zj = __shfl_sync(SAI_FULL, t[q], j % 32);
                 }
 #pragma unroll
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(LU_CT) k_lu_panel_cluster(int32_t s, int32_t k
         for (int r = tid; r < nr; r += LU_CT) {
             if (b0 + r <= j) continue;
             double* x = P + r * LU_PLD;
-            const double l = x[j] * inv;
+            const double l = div_by(x[j], uj[j], inv);
             x[j] = l;
 #pragma unroll
             for (int c = 1; c < LU_NB; ++c)
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(LU_CT) k_lu_trsv(int32_t s, int R, const doubl
                     } else {
                         const double rd = lane < jb ? 1.0 / D[lane][lane] : 0.0;
                         for (int jj = jb - 1; jj >= 0; --jj) {
-                            if (lane == jj) v *= rd;
+                            if (lane == jj) v = div_by(v, D[jj][jj], rd);
                             const double zj = __shfl_sync(SAI_FULL, v, jj);
                             if (lane < jj) v = fma(-D[jj][lane], zj, v);
                         }
