@@ -263,7 +263,9 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n, int64_t ld, int rmax, in
                int* __restrict__ iters, int* __restrict__ status)
 {
     extern __shared__ __align__(16) double sm[];
-    __shared__ double sc[5];  // alpha, omega, beta, alpha / (omega rho), rho of the running iteration
+    // alpha, omega, beta, alpha / (omega rho f), rho of the running iteration, f = the power of two that
+    // takes rho near 1 (the quotient must not overflow where rho is small, as it is when b is)
+    __shared__ double sc[6];
     __shared__ int flag;      // 0 go on (first iteration), 1 half step, then stop, 2 stop, 3 go on
     uint32_t rank = 0, nranks = 1;
     if (MULTI) {
@@ -314,7 +316,7 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n, int64_t ld, int rmax, in
             return 2;
         }
         // beta = (rho / rho_old) (alpha / omega), the quotient without rho formed earlier
-        if (lane == 0) sc[2] = it == 1 ? 0.0 : rho * sc[3];
+        if (lane == 0) sc[2] = it == 1 ? 0.0 : rho * sc[5] * sc[3];
         return 0;
     };
     if (wid == 0) {
@@ -415,7 +417,12 @@ k_bicg_cluster(ClMat<double> A, ClMat<double> M, int n, int64_t ld, int rmax, in
         {
             const double al = sc[0], om = sc[1];
             // beside the update, in the warp that has the fewest units
-            if (wid == NW - 1 && lane == 0) sc[3] = al / (om * sc[4]);
+            if (wid == NW - 1 && lane == 0) {
+                const int e = ((__double2hiint(sc[4]) >> 20) & 0x7ff) - 1023;
+                const double f = __hiloint2double((1023 - min(max(e, -1022), 1022)) << 20, 0);
+                sc[5] = f;
+                sc[3] = al / (om * (sc[4] * f));
+            }
             for (int u = wid; u < W.units; u += NW) {
                 const int i = u * CL_UNIT + lane;
                 double rv[2];
