@@ -3187,9 +3187,6 @@ constexpr int BG_KMAX = 32;  // largest block (systems per block)
 constexpr int BG_CR = 512;   // rows per chunk of the Gram kernel
 constexpr int BG_GV = 8;     // warps per Gram block
 constexpr int BG_UT = 128;   // threads (rows) per block of the triangular solve
-constexpr int BG_UR = 64;    // rows per block of the update kernel
-constexpr int BG_UP = 4;     // its parts: each takes a quarter of the basis vectors
-constexpr int BG_HB = 16;    // rows of H staged at a time and part
 constexpr int BG_LT = 256;   // threads of the least-squares kernel
 
 template <class T>
@@ -3298,36 +3295,52 @@ __global__ void k_bg_reduce(int nch, int nv, int kb, const double* __restrict__ 
 }
 
 // W -= V H (overwrite = 0) or W = V H (overwrite = 1); H: nv x kb, ld ldhh.
-// A block takes BG_UR rows; its BG_UP parts each sum a quarter of the basis
-// vectors (eight loads in flight per thread), then add up in a fixed order:
-// four times the warps of a thread per row, which the row count alone cannot
-// give (27000 rows, 275 vectors on average: 23 us, 40 us with one part).
-template <class T, int KB>
-__global__ void __launch_bounds__(BG_UR * BG_UP)
-k_bg_update(int32_t n, int64_t ld, const T* __restrict__ V, int nv, const double* __restrict__ H, int ldhh,
-            int kb, T* __restrict__ W, int overwrite)
+// A block takes BG_UH / UP rows; its UP parts each sum a share of the basis
+// vectors (eight loads in flight per thread), then add up in a fixed order; HB
+// rows of H per part are staged at a time.
+// Four parts give a small order four times the warps of a thread per row; with
+// one, H is staged a quarter as often. Times of one update, 30 steps, four
+// parts and one (27000, 64000, 110592, 262144 rows; 11 columns): FP32 17 and 21,
+// 31 and 26, 47 and 38, 114 and 76 us; FP64 121 and 147, 269 and 280, 453 and
+// 419, 1048 and 951 us (the first form, one part of 256 rows with plain loads:
+// 20, 25, 36, 75 and 157, 302, 451, 1032 us). One part is taken from one block
+// per SM on in FP32; in FP64, whose pipe four parts keep busier, from 2.5, or 1.5
+// where at most four columns leave it idle (64000 rows, 2 columns: 30 and 25 us).
+constexpr int BG_UH = 256;
+inline bool bg_one_part(int32_t n, int kb, size_t esz)
 {
-    __shared__ T hs[BG_UP][BG_HB * KB];
-    __shared__ T sums[BG_UR][KB + 1];
-    const int row = threadIdx.x % BG_UR, part = threadIdx.x / BG_UR;
-    const int per = (nv + BG_UP - 1) / BG_UP;  // basis vectors per part
+    const double blocks = (double)n / BG_UH / g_sms;
+    return blocks >= (esz == 4 ? 1.0 : kb <= 4 ? 1.5 : 2.5);
+}
+
+template <class T, int KB, int UP, int HB>
+__device__ __forceinline__ void bg_update_rows(int32_t n, int64_t ld, const T* __restrict__ V, int nv,
+                                               const double* __restrict__ H, int ldhh, int kb, T* __restrict__ W,
+                                               int overwrite)
+{
+    constexpr int UR = BG_UH / UP;
+    __shared__ T hs[UP][HB * KB];
+    __shared__ T sums[UP > 1 ? UR : 1][KB + 1];
+    const int row = threadIdx.x % UR, part = threadIdx.x / UR;
+    const int per = (nv + UP - 1) / UP;  // basis vectors per part
     const int v0 = part * per, v1 = v0 + per < nv ? v0 + per : nv;
-    for (int64_t base = (int64_t)blockIdx.x * BG_UR; base < n; base += (int64_t)gridDim.x * BG_UR) {
+    for (int64_t base = (int64_t)blockIdx.x * UR; base < n; base += (int64_t)gridDim.x * UR) {
         const int64_t r = base + row;
         const bool ok = r < n;
         T acc[KB];
 #pragma unroll
         for (int c = 0; c < KB; ++c) acc[c] = 0;
-        for (int q0 = 0; q0 < per; q0 += BG_HB) {
+        for (int q0 = 0; q0 < per; q0 += HB) {
             __syncthreads();
-            for (int e = threadIdx.x; e < BG_UP * BG_HB * KB; e += BG_UR * BG_UP) {
-                const int p = e / (BG_HB * KB), t = e / KB % BG_HB, c = e % KB;
+            for (int e = threadIdx.x; e < UP * HB * KB; e += BG_UH) {
+                const int p = e / (HB * KB), t = e / KB % HB, c = e % KB;
                 const int b = p * per + q0 + t;
                 hs[p][t * KB + c] = (c < kb && q0 + t < per && b < nv) ? (T)H[(int64_t)c * ldhh + b] : T(0);
             }
             __syncthreads();
-#pragma unroll
-            for (int t0 = 0; t0 < BG_HB; t0 += 8) {
+            const int tl = per - q0 < HB ? per - q0 : HB;
+#pragma unroll 1
+            for (int t0 = 0; t0 < tl; t0 += 8) {
                 T x[8];
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {
@@ -3340,21 +3353,37 @@ k_bg_update(int32_t n, int64_t ld, const T* __restrict__ V, int nv, const double
                     for (int c = 0; c < KB; ++c) acc[c] = fma(x[t], hs[part][(t0 + t) * KB + c], acc[c]);
             }
         }
-        for (int p = BG_UP - 1; p > 0; --p) {
+        for (int p = UP - 1; p > 0; --p) {
             if (part == p)
 #pragma unroll
-                for (int c = 0; c < KB; ++c) sums[row][c] = p == BG_UP - 1 ? acc[c] : acc[c] + sums[row][c];
+                for (int c = 0; c < KB; ++c) sums[row][c] = p == UP - 1 ? acc[c] : acc[c] + sums[row][c];
             __syncthreads();
         }
         if (part == 0 && ok)
 #pragma unroll
             for (int c = 0; c < KB; ++c)
                 if (c < kb) {
-                    const T v = acc[c] + sums[row][c];
+                    const T v = UP > 1 ? acc[c] + sums[row][c] : acc[c];
                     T* w = W + (int64_t)c * ld + r;
                     *w = overwrite ? v : *w - v;
                 }
     }
+}
+
+template <class T, int KB>
+__global__ void __launch_bounds__(BG_UH) k_bg_update(int32_t n, int64_t ld, const T* __restrict__ V, int nv,
+                                                     const double* __restrict__ H, int ldhh, int kb,
+                                                     T* __restrict__ W, int overwrite)
+{
+    bg_update_rows<T, KB, 4, 16>(n, ld, V, nv, H, ldhh, kb, W, overwrite);
+}
+
+template <class T, int KB>
+__global__ void __launch_bounds__(BG_UH) k_bg_update1(int32_t n, int64_t ld, const T* __restrict__ V, int nv,
+                                                      const double* __restrict__ H, int ldhh, int kb,
+                                                      T* __restrict__ W, int overwrite)
+{
+    bg_update_rows<T, KB, 1, 64>(n, ld, V, nv, H, ldhh, kb, W, overwrite);
 }
 
 // one QR pass's Cholesky factor: Gm (+ shift on the first pass) = Rp^T Rp,
@@ -3789,9 +3818,11 @@ template <class T>
 void bg_update(int32_t n, int64_t ld, const T* V, int nv, const double* H, int ldhh, int kb, T* W, int overwrite,
                cudaStream_t st)
 {
-    const unsigned g = bg_rows_grid(n, BG_UR);
+    const bool one = bg_one_part(n, kb, sizeof(T));
+    const unsigned g = bg_rows_grid(n, one ? BG_UH : BG_UH / 4);
     sai_count_grid(g);
-    BG_DISPATCH(kb, k_bg_update, T, <<<g, BG_UR * BG_UP, 0, st>>>(n, ld, V, nv, H, ldhh, kb, W, overwrite));
+    if (one) BG_DISPATCH(kb, k_bg_update1, T, <<<g, BG_UH, 0, st>>>(n, ld, V, nv, H, ldhh, kb, W, overwrite));
+    else BG_DISPATCH(kb, k_bg_update, T, <<<g, BG_UH, 0, st>>>(n, ld, V, nv, H, ldhh, kb, W, overwrite));
 }
 
 // W = Q R: shifted Cholesky QR in three passes, R accumulated in B.Rt. The
