@@ -9,32 +9,38 @@
 // b of the cluster owns rows [b R, (b + 1) R): the candidate u, t = M u, z =
 // A~ t and x live in its shared memory, its rows of the basis in global
 // memory (read by this block only, so from L1 while they fit). Products
-// gather u, t and x across the cluster; a step has four cluster barriers.
+// gather u, t and x across the cluster; a step has three cluster barriers.
 // Every block keeps the small Hessenberg problem itself and runs the same
 // control arithmetic on the same sums, so no value has to be sent back.
 //
-// Sums: products accumulate in T along 16 rows per lane and component and up
-// a shuffle tree per GC_SUB rows, the rest in FP64 in a fixed order, as in
-// k_dc_dots. The Hessenberg columns are kept in T, the type k_dc_step uses
-// them in (its rotated columns are T values stored as FP64).
+// A system's bits depend on n, m, T and the matrices, not on the systems that
+// run with it: the number of blocks follows k, but a sum is a tree per unit of
+// rows (GcUnits, gc_dots) and the units' sums added pairwise in FP64, each block
+// holding whole units. With sums per block instead, this form took 2.94, 4.02
+// and 11.7 ms where it takes 2.98, 4.4 and 12.9 (35937 rows in FP32, 6, 11 and 40
+// systems, 101 steps), and 6.3 where it takes 6.8 (1728 rows in FP64, 256
+// systems, 60 steps). The Hessenberg columns are kept in T, the type k_dc_step
+// uses them in (its rotated columns are T values stored as FP64).
 
 constexpr int GC_T = 512;      // threads per block
 constexpr int GC_UT = GC_T - 32;  // of them in the update; the last warp runs the Givens rotations meanwhile
-constexpr int GC_SUB = 2048;   // rows per partial sum
+constexpr int GC_MAXU = 16;    // units of a system
 constexpr int GC_MAXR = 6144;  // rows per block
-// orders up to which the form is used: FP32 vectors fill the shared memory
-// there; in FP64 the eight SMs' FP64 pipes are slower than all SMs' above
+// orders up to which the form is used, by n alone. FP32: the multi-kernel form
+// takes as long at 35937 rows with 153 systems (46.0 and 42.7 ms) and longer with
+// up to 40 (4.4 and 6.0 ms with 11, 12.9 and 13.1 with 40); at 46656 rows it is
+// the faster one from 16 systems on (31.6 and 26.0 ms with 77). FP64: above, the
+// FP64 pipes of eight SMs are slower than those of all.
 constexpr size_t GC_SMEM = 220 * 1024;  // shared memory of a block, at most
-constexpr int GC_MAXN32 = GC_MAXR * CL_MAXC, GC_MAXN64 = 10240;
+constexpr int GC_MAXN32 = 36864, GC_MAXN64 = 10240;
 
 // Shared-memory layout of one block (bytes from the start).
 template <class T>
 struct GcLayout {
     size_t u, t, z, x, hb, r, cs, sn, rc, s, c, parts, red, hp, g, y, bytes;
-    int nsub, ns;  // partial sums per block and slot; slots
-    GcLayout(int R, int m, int C)
+    int ns;  // slots of a unit's partial sums
+    GcLayout(int R, int m, int units)
     {
-        nsub = (R + GC_SUB - 1) / GC_SUB;
         ns = 2 * m + 4;
         size_t o = 0;
         auto take = [&](size_t b) {
@@ -53,7 +59,7 @@ struct GcLayout {
         rc = take(sizeof(T) * (m + 2));
         s = take(sizeof(T) * (m + 1));
         c = take(sizeof(T) * (m + 1));
-        parts = take(sizeof(double) * (size_t)C * nsub * ns);
+        parts = take(sizeof(double) * (size_t)units * ns);
         red = take(sizeof(double) * ns);
         hp = take(sizeof(double) * (m + 2));
         g = take(sizeof(double) * (m + 2));
@@ -66,7 +72,7 @@ struct GcArgs {
     int n, m, R, k;
     int64_t ld, vs;
     double tiny;
-    int nsub, ns;
+    int units, U, ns;  // GcUnits; ns as in GcLayout
     uint32_t u, t, z, x, hb, r, cs, sn, rc, s, c, parts, red, hp, g, y;  // offsets of GcLayout
 };
 
@@ -80,6 +86,22 @@ __device__ __forceinline__ T gc_sum2(T a, T b)
     for (int o = 8; o > 0; o >>= 1) w += __shfl_xor_sync(SAI_FULL, w, o);
     return w;
 }
+
+// The units of a system: a power of two of them, of U rows (the last ones
+// fewer, or none). A block of the cluster holds units / C of them, so the order
+// of every sum depends on n alone: a tree per unit (gc_dots), and the units'
+// sums added pairwise.
+struct GcUnits {
+    int units, U;
+    explicit GcUnits(int n)
+    {
+        // at least 128 rows per unit; sixteen from 512 rows per eighth on, where the work outweighs the barriers
+        units = 1;
+        while (units < 8 && n / (2 * units) >= 2 * CL_UNIT) units *= 2;
+        if (units == 8 && n > 8 * (512 - CL_UNIT)) units = GC_MAXU;
+        U = ((n + units - 1) / units + 31) / 32 * 32;
+    }
+};
 
 template <class T>
 struct Comp;  // the components of a Vec<T>
@@ -103,6 +125,110 @@ struct Comp<double> {
     }
     __device__ static double sum(const double2& a) { return a.x + a.y; }
 };
+
+// v^T u and v^T z over rows [at, at + U) below nrow by one warp, in FP32: plain
+// sums over at most eight row pieces per lane and component and, for more than
+// 512 rows, those and the tree over the lanes with their rounding errors carried
+// along. (A plain tree over 2048 rows has twice the error of the multi-kernel
+// form's four over 512 rows each, added in FP64.) Lane 0 returns v^T u, lane 16
+// v^T z. Two basis vectors at a time, sharing the loads of u and z, were no
+// faster.
+__device__ __noinline__ double gc_dots(const float* v, const float* u, const float* z, int at, int U, int nrow, int)
+{
+    __builtin_assume(__isShared(u));
+    __builtin_assume(__isShared(z));
+    const int lane = threadIdx.x & 31, r1 = min(nrow, at + U);
+    auto add = [](float& h, float& l, float x) {  // (h, l) += x (Knuth's two-sum)
+        const float s = h + x, t = s - h;
+        l += (h - (s - t)) + (x - t);
+        h = s;
+    };
+    float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
+#pragma unroll 1
+    for (int r0 = at + 4 * lane; r0 - 4 * lane < r1;) {
+        float4 as = {}, ac = {};
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half, r0 += 512) {
+            float4 x[4];
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                if (r0 + 128 * s < r1) x[s] = *reinterpret_cast<const float4*>(v + r0 + 128 * s);
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                if (r0 + 128 * s < r1) {
+                    Comp<float>::fma4(x[s], *reinterpret_cast<const float4*>(u + r0 + 128 * s), as);
+                    Comp<float>::fma4(x[s], *reinterpret_cast<const float4*>(z + r0 + 128 * s), ac);
+                }
+        }
+        const float a = Comp<float>::sum(as), c = Comp<float>::sum(ac);
+        if (U <= 512) return (double)gc_sum2(a, c);
+        add(h0, l0, a);
+        add(h1, l1, c);
+    }
+    const bool up = (lane & 16) != 0;
+    float h = up ? h1 : h0, l = up ? l1 : l0;
+    const float hx = __shfl_xor_sync(SAI_FULL, up ? h0 : h1, 16), lx = __shfl_xor_sync(SAI_FULL, up ? l0 : l1, 16);
+    add(h, l, hx);
+    l += lx;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+        const float hy = __shfl_xor_sync(SAI_FULL, h, o), ly = __shfl_xor_sync(SAI_FULL, l, o);
+        add(h, l, hy);
+        l += ly;
+    }
+    return (double)h + (double)l;
+}
+
+// Sums a[0..7] over the warp, each with the additions of gc_sum2's tree: lanes
+// 4 i to 4 i + 3 get the sum of a[i].
+__device__ __forceinline__ double gc_sum8(double (&a)[8])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 2; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < o / 4; ++i) {
+            const double keep = up ? a[i + o / 4] : a[i], send = up ? a[i] : a[i + o / 4];
+            a[i] = keep + __shfl_xor_sync(SAI_FULL, send, o);
+        }
+    }
+    double w = a[0];
+    w += __shfl_xor_sync(SAI_FULL, w, 2);
+    return w + __shfl_xor_sync(SAI_FULL, w, 1);
+}
+
+// The same in FP64 for uw <= 4 units of U rows at a time, whose trees share
+// their additions (9 for four units, 5 for one). Unit e's sums: lanes 8 e and
+// 8 e + 4, or lanes 0 and 16 for one unit.
+__device__ __noinline__ double gc_dots(const double* v, const double* u, const double* z, int at, int U, int nrow, int uw)
+{
+    __builtin_assume(__isShared(u));
+    __builtin_assume(__isShared(z));
+    const int lane = threadIdx.x & 31;
+    double sums[8];
+#pragma unroll
+    for (int e = 0; e < 4; ++e, at += U) {
+        const int r1 = e < uw ? min(nrow, at + U) : 0;
+        double a = 0.0, b = 0.0;
+#pragma unroll 1
+        for (int r0 = at + 2 * lane; r0 - 2 * lane < r1; r0 += 256) {
+            double2 x[4];
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                if (r0 + 64 * s < r1) x[s] = *reinterpret_cast<const double2*>(v + r0 + 64 * s);
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                if (r0 + 64 * s < r1) {
+                    a = Vec<double>::dot(x[s], *reinterpret_cast<const double2*>(u + r0 + 64 * s), a);
+                    b = Vec<double>::dot(x[s], *reinterpret_cast<const double2*>(z + r0 + 64 * s), b);
+                }
+        }
+        sums[2 * e] = a;
+        sums[2 * e + 1] = b;
+    }
+    return uw > 1 ? gc_sum8(sums) : gc_sum2(sums[0], sums[1]);
+}
 
 // v_j = ia (u - V s), u <- ia (z - V c - dd v_j) on the block's rows: a thread
 // per row (W = 1) or per 16-byte piece
@@ -189,40 +315,44 @@ k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restri
     const int most = cap[c];
     int it = 0, stat = ST_OK;         // the same in every thread of the cluster
     double wsteps = 0.0, wj = 0.0;    // work: steps, and basis vectors over the steps
-    // a partial sum (lane 0: a, lane 16: b, from gc_sum2) to slots sl, sl + 1 of every block
-    auto put2 = [&](T w, int sl, int sub) {
-        const double v = (double)w;
-        double* p = parts + ((size_t)rank * P.nsub + sub) * P.ns + sl;
-        const double a = __shfl_sync(SAI_FULL, v, 0), b = __shfl_sync(SAI_FULL, v, 16);
-        if (MULTI) {
-            // lanes 0..7 send the first value, lanes 16..23 the second
-            const int to = lane & 15;
-            if (to < (int)nranks) cl_st(cl_map(smem_u32(p + (lane >> 4)), (uint32_t)to), lane < 16 ? a : b);
-        } else if (lane == 0) {
-            p[0] = a;
-            p[1] = b;
+    const int lr = 31 - __clz((int)nranks), ub = P.units >> lr;  // ub: units of this block
+    // v^T u and v^T zz on units g w to g w + w - 1 of the block, stored in slots sl, sl + 1 of every block (one warp; the
+    // sums do not depend on w)
+    auto dots = [&](const T* v, const T* zz, int g, int w, int sl) {
+        const double d = gc_dots(v, u, zz, g * w * P.U, P.U, W.nrow, w);
+        // a store per lane: (unit, part, block)
+        const int vi = lane >> lr, to = lane & ((int)nranks - 1);
+        const int e = vi >> 1, b = vi & 1;
+        const double val = __shfl_sync(SAI_FULL, d, (w > 1 ? 8 * e + 4 * b : 16 * b) & 31);
+        if (vi < 2 * w) {
+            double* p = parts + (size_t)((int)rank * ub + g * w + e) * P.ns + sl + b;
+            if (MULTI) cl_st(cl_map(smem_u32(p), (uint32_t)to), val);
+            else *p = val;
         }
     };
-    // red[t] = the sum of slot t over the blocks and their parts, t < cnt
+    // red[t] = the sum of slot t over the units, t < cnt
     auto total = [&](int cnt) {
         for (int q = tid; q < cnt; q += GC_T) {
-            double a = 0.0;
-            for (int e = 0; e < (int)nranks * P.nsub; ++e) a += parts[(size_t)e * P.ns + q];
+            auto eight = [&](int e0) {  // of units e0 to e0 + 7
+                double a[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) a[e] = e0 + e < P.units ? parts[(size_t)(e0 + e) * P.ns + q] : 0.0;
+#pragma unroll
+                for (int w = 1; w < 8; w *= 2)
+                    if (w < P.units)
+#pragma unroll
+                        for (int e = 0; e < 8; e += 2 * w) a[e] += a[e + w];
+                return a[0];
+            };
+            double a = eight(0);
+            if (P.units > 8) a += eight(8);
             red[q] = a;
         }
         __syncthreads();
     };
-    // the block's rows of u = r: ||r||^2 into slot 0 (slot 1: 0)
+    // the block's rows of u = r: ||r||^2 into slot 0 (and 1)
     auto norm = [&]() {
-        for (int sub = wid; sub < P.nsub; sub += NW) {
-            VT acc = Vec<T>::zero();
-            const int r1 = min(W.nrow, (sub + 1) * GC_SUB);
-            for (int r = sub * GC_SUB + lane * VW; r < r1; r += 32 * VW) {
-                const VT a = *reinterpret_cast<const VT*>(u + r);
-                Comp<T>::fma4(a, a, acc);
-            }
-            put2(gc_sum2(Comp<T>::sum(acc), T(0)), 0, sub);
-        }
+        for (int g = wid; g < ub; g += NW) dots(u, u, g, 1, 0);
     };
     for (int i = tid; i < P.R; i += GC_T) {
         u[i] = i < W.nrow ? B[o + i] : T(0);
@@ -254,18 +384,12 @@ k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restri
                 __syncthreads();
             }
             // s = V^T u, c = V^T z (slots 2 i, 2 i + 1), u^T u, u^T z (2 j, 2 j + 1)
-            for (int q = wid; q < (j + 1) * P.nsub; q += NW) {
-                const int i = q / P.nsub, sub = q - i * P.nsub;
-                const int r1 = min(W.nrow, (sub + 1) * GC_SUB);
-                VT as = Vec<T>::zero(), ac = Vec<T>::zero();
-                const T* v = i < j ? V + (int64_t)i * P.vs : u;
-#pragma unroll 4
-                for (int r = sub * GC_SUB + lane * VW; r < r1; r += 32 * VW) {
-                    const VT vv = *reinterpret_cast<const VT*>(v + r);
-                    Comp<T>::fma4(vv, *reinterpret_cast<const VT*>(u + r), as);
-                    Comp<T>::fma4(vv, *reinterpret_cast<const VT*>(z + r), ac);
-                }
-                put2(gc_sum2(Comp<T>::sum(as), Comp<T>::sum(ac)), 2 * i, sub);
+            int w = sizeof(T) == 4 ? 1 : min(4, ub);  // units a warp takes at a time: fewer while warps would idle
+            while (w > 1 && (j + 1) * (ub / w) < NW) w >>= 1;
+            const int lu = 31 - __clz(ub / w);
+            for (int q = wid; q < (j + 1) << lu; q += NW) {
+                const int i = q >> lu;
+                dots(i < j ? V + (int64_t)i * P.vs : u, z, q - (i << lu), w, 2 * i);
             }
             cl_barrier<MULTI>();
             total(2 * j + 2);
@@ -436,18 +560,21 @@ sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* 
 {
     *ran = false;
     if (n < 1 || n > (sizeof(T) == 4 ? GC_MAXN32 : GC_MAXN64)) return SAI_OK;
+    // whether the form is used depends on n and m alone, as the sums do: a
+    // system's bits do not depend on the systems that run with it
+    const GcUnits N(n);
+    auto rows = [&](int blocks) { return N.U * (N.units / blocks); };
+    const int most = N.units < CL_MAXC ? N.units : CL_MAXC;
     int C = 1;
-    while (C < CL_MAXC && (int64_t)C * GC_MAXR < n) C *= 2;
-    if ((int64_t)k * C > 4 * (int64_t)g_sms) return SAI_OK;  // more systems: the multi-kernel form fills the GPU
-    while (C < CL_MAXC && (int64_t)2 * C * k <= (int64_t)g_sms * 7 / 8 && n / (2 * C) >= 2 * CL_UNIT) C *= 2;
-    auto rows = [&](int blocks) { return ((n + blocks - 1) / blocks + CL_UNIT - 1) / CL_UNIT * CL_UNIT; };
-    // from 512 rows per block on the work outweighs the barriers
-    if (C == CL_MAXC && rows(C) >= 512 &&
-        cl_fits16(k_gmres_cluster<T, true>, k, GC_T, GC_SMEM, GcLayout<T>(rows(16), m, 16).bytes))
+    while (C < most && (rows(C) > GC_MAXR || GcLayout<T>(rows(C), m, N.units).bytes > GC_SMEM)) C *= 2;
+    if (rows(C) > GC_MAXR || GcLayout<T>(rows(C), m, N.units).bytes > GC_SMEM) return SAI_OK;
+    // then as many blocks as leave every system on the GPU at once
+    while (C < most && (int64_t)2 * C * k <= (int64_t)g_sms * 7 / 8) C *= 2;
+    if (C == CL_MAXC && N.units == GC_MAXU &&
+        cl_fits16(k_gmres_cluster<T, true>, k, GC_T, GC_SMEM, GcLayout<T>(rows(16), m, N.units).bytes))
         C = 16;
     const int R = rows(C);
-    const GcLayout<T> L(R, m, C);
-    if (L.bytes > GC_SMEM) return SAI_OK;
+    const GcLayout<T> L(R, m, N.units);
     GcArgs P;
     P.n = n;
     P.m = m;
@@ -456,7 +583,8 @@ sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* 
     P.ld = ld;
     P.vs = Wk.B.vs;
     P.tiny = tiny;
-    P.nsub = L.nsub;
+    P.units = N.units;
+    P.U = N.U;
     P.ns = L.ns;
     P.u = (uint32_t)L.u;
     P.t = (uint32_t)L.t;
