@@ -478,35 +478,28 @@ __global__ void k_cl_work(int k, const int* iters, Dims D)
     kwork_add(PROF_BICG_VEC, 8.0 * D.n * 19 * sum, D.n * 23.0 * sum);
 }
 
-// blocks per cluster for k systems of order at most n: enough for the rows,
-// then as many as leave every system on the GPU at once with two units of
-// rows per block (the reductions' cost does not shrink with more)
-inline int cl_blocks(int k, int n)
-{
-    int C = 1;
-    while (C < CL_MAXC && (int64_t)C * CL_MAXR < n) C *= 2;
-    while (C < CL_MAXC && (int64_t)2 * C * k <= (int64_t)g_sms * 7 / 8 && n / (2 * C) >= 2 * CL_UNIT) C *= 2;
-    return C;
-}
-
-// true when the GPU holds k clusters of 16 blocks of kern at once; limit: the
-// most dynamic shared memory of kern's launches
+// true when the GPU holds k clusters of C blocks of kern at once (fewer than its
+// SMs suggest: a cluster stays within one group of them, and sixteen clusters of
+// eight blocks take two rounds on 152 SMs); limit: the most dynamic shared memory
+// of kern's launches
 template <class... Params>
-bool cl_fits16(void (*kern)(Params...), int k, int threads, size_t limit, size_t smem)
+bool cl_fits(void (*kern)(Params...), int k, int C, int threads, size_t limit, size_t smem)
 {
-    if (16 * (int64_t)k > g_sms) return false;
+    if ((int64_t)C * k > g_sms) return false;
+    if (C <= CL_MAXC && (int64_t)2 * C * k <= g_sms) return true;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(16u * (unsigned)k);
+    cfg.gridDim = dim3((unsigned)C * (unsigned)k);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = 16;
+    at.val.clusterDim.x = (unsigned)C;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int most = 0;
-    const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+    const bool ok = (C <= CL_MAXC ||
+                     cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
                     sai_smem_limit(kern, limit) == cudaSuccess &&
                     cudaOccupancyMaxActiveClusters(&most, kern, &cfg) == cudaSuccess;
     if (!ok) (void)cudaGetLastError();
@@ -544,21 +537,22 @@ bool cl_run(void (*kern)(Params...), int k, int C, int threads, size_t limit, si
 inline sai_status cl_bicgstab(const Ops<double>& A, int k, int n, int64_t ld, const double* B, double* X,
                               const double* thr, int maxit, int* iters, int* status, cudaStream_t st, bool* ran)
 {
-    int C = cl_blocks(k, n);
     const int umax = (n + CL_UNIT - 1) / CL_UNIT;
-    int rmax = 0;
-    size_t smem = 0;
-    auto shape = [&](int blocks) {
-        C = blocks;
-        rmax = ((n + C - 1) / C + CL_UNIT - 1) / CL_UNIT * CL_UNIT;
-        smem = sizeof(double) * ((size_t)CL_VECS * rmax + (size_t)CL_SLOTS * umax);
+    auto rows = [&](int blocks) { return ((n + blocks - 1) / blocks + CL_UNIT - 1) / CL_UNIT * CL_UNIT; };
+    auto bytes = [&](int blocks) {
+        return sizeof(double) * ((size_t)CL_VECS * rows(blocks) + (size_t)CL_SLOTS * umax);
     };
-    shape(C);
-    // from 512 rows per block on the FP64 pipe outweighs the barriers
-    if (C == CL_MAXC && rmax >= 512) {
-        shape(16);
-        if (!cl_fits16(k_bicg_cluster<true>, k, CL_T, CL_SMEM, smem)) shape(CL_MAXC);
-    }
+    auto fits = [&](int blocks) { return cl_fits(k_bicg_cluster<true>, k, blocks, CL_T, CL_SMEM, bytes(blocks)); };
+    // enough blocks for the rows, then as many as leave every system on the GPU
+    // at once with two units of rows per block (the reductions' cost does not
+    // shrink with more); sixteen where the FP64 pipe outweighs the barriers, from
+    // 512 rows per block on
+    int C = 1;
+    while (C < CL_MAXC && (int64_t)C * CL_MAXR < n) C *= 2;
+    while (C < CL_MAXC && n / (2 * C) >= 2 * CL_UNIT && fits(2 * C)) C *= 2;
+    if (C == CL_MAXC && rows(C) >= 512 && fits(16)) C = 16;
+    const int rmax = rows(C);
+    const size_t smem = bytes(C);
     ClMat<double> a, m;
     Buf ab[4], mb[4];
     *ran = false;

@@ -569,10 +569,11 @@ sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* 
     while (C < most && (rows(C) > GC_MAXR || GcLayout<T>(rows(C), m, N.units).bytes > GC_SMEM)) C *= 2;
     if (rows(C) > GC_MAXR || GcLayout<T>(rows(C), m, N.units).bytes > GC_SMEM) return SAI_OK;
     // then as many blocks as leave every system on the GPU at once
-    while (C < most && (int64_t)2 * C * k <= (int64_t)g_sms * 7 / 8) C *= 2;
-    if (C == CL_MAXC && N.units == GC_MAXU &&
-        cl_fits16(k_gmres_cluster<T, true>, k, GC_T, GC_SMEM, GcLayout<T>(rows(16), m, N.units).bytes))
-        C = 16;
+    auto fits = [&](int blocks) {
+        return cl_fits(k_gmres_cluster<T, true>, k, blocks, GC_T, GC_SMEM, GcLayout<T>(rows(blocks), m, N.units).bytes);
+    };
+    while (C < most && fits(2 * C)) C *= 2;
+    if (C == CL_MAXC && N.units == GC_MAXU && fits(16)) C = 16;
     const int R = rows(C);
     const GcLayout<T> L(R, m, N.units);
     GcArgs P;
