@@ -22,6 +22,24 @@ constexpr int CL_T = 512;        // threads per block
 constexpr int CL_MAXR = 2560;    // rows per block: nine vectors of 20 KB
 constexpr int CL_MAXC = 8;       // blocks per cluster (the portable limit; 16 where all systems run at once)
 constexpr int CL_MAXN = CL_MAXR * CL_MAXC;
+// Limits of the form, against the multi-kernel form (40 iterations unless
+// stated, in ms):
+// - systems: at 10000 rows of a power-law matrix 52 against 56 with 511, 101
+//   against 33 with 1020, for which the other form goes over to panels of
+//   systems;
+constexpr int CL_MAXK = 256;
+// - a scattered matrix, most of whose gathers cross the cluster, up to this
+//   order only (in GMRES too): with 8, 32 and 128 systems 4.9, 7.0 and 27
+//   against 5.0, 9.3 and 28 at 10000 rows, 6.6, 20 and 29 (of half the
+//   iterations) against 5.4, 11 and 17 at 14500;
+constexpr int CL_FAR_N = 10240;
+// - above this order only so many systems (60 iterations on a grid): 8, 64 and
+//   256 systems 3.0, 14.0 and 49.7 against 5.8, 15.0 and 50.2 at 12167 rows, 3.6,
+//   17.0 and 60.6 against 5.7, 15.4 and 53.3 at 15625, 4.1, 19.8 and 70.5 against
+//   6.4, 16.1 and 53.5 at 19683. (From 17 on, which take two rounds, the other
+//   form is up to a fifth faster; the line lies higher so that a system keeps its
+//   bits among a few dozen others.)
+constexpr int CL_MANY_N = 14336, CL_MANY_K = 64;
 constexpr int CL_UNIT = 64;      // rows per reduction unit
 constexpr int CL_VECS = 9;
 constexpr int CL_SLOTS = 6;      // partial sums: rhat^T v; ||s||; t^T s, t^T t; ||r||, rhat^T r
@@ -533,10 +551,13 @@ bool cl_run(void (*kern)(Params...), int k, int C, int threads, size_t limit, si
     return true;
 }
 
-// BiCGStab of k systems in clusters; *ran is false when the device refuses the shape.
+// BiCGStab of k systems in clusters; *ran is false when the form does not take
+// them or the device refuses the shape.
 inline sai_status cl_bicgstab(const Ops<double>& A, int k, int n, int64_t ld, const double* B, double* X,
                               const double* thr, int maxit, int* iters, int* status, cudaStream_t st, bool* ran)
 {
+    *ran = false;
+    if (n > CL_MAXN || k > (n > CL_MANY_N ? CL_MANY_K : CL_MAXK) || (n > CL_FAR_N && A.scattered)) return SAI_OK;
     const int umax = (n + CL_UNIT - 1) / CL_UNIT;
     auto rows = [&](int blocks) { return ((n + blocks - 1) / blocks + CL_UNIT - 1) / CL_UNIT * CL_UNIT; };
     auto bytes = [&](int blocks) {
@@ -555,7 +576,6 @@ inline sai_status cl_bicgstab(const Ops<double>& A, int k, int n, int64_t ld, co
     const size_t smem = bytes(C);
     ClMat<double> a, m;
     Buf ab[4], mb[4];
-    *ran = false;
     if (cl_matrix(A.A, n, rmax, C, ab, a, st) != SAI_OK || cl_matrix(A.M, n, rmax, C, mb, m, st) != SAI_OK)
         return SAI_OK;  // no memory for the sorted forms: the kernels below need none
     *ran = cl_run(C > 1 ? k_bicg_cluster<true> : k_bicg_cluster<false>, k, C, CL_T, CL_SMEM, smem, st, a, m, n, ld, rmax,

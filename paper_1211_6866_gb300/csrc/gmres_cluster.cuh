@@ -33,6 +33,10 @@ constexpr int GC_MAXR = 6144;  // rows per block
 // FP64 pipes of eight SMs are slower than those of all.
 constexpr size_t GC_SMEM = 220 * 1024;  // shared memory of a block, at most
 constexpr int GC_MAXN32 = 36864, GC_MAXN64 = 10240;
+// of a scattered matrix in FP32 (8, 16, 19 and 76 systems of 12000 rows: 2.95,
+// 4.0, 4.1 and 5.2 ms against 3.1, 4.0, 4.4 and 12.0; 4, 16 and 76 systems of 20000
+// rows 3.0, 7.6 and 16 against 2.7, 4.4 and 13.8)
+constexpr int GC_FAR_N32 = 12288;
 
 // Shared-memory layout of one block (bytes from the start).
 template <class T>
@@ -559,7 +563,8 @@ sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* 
                const int* cap, const Dims& D, double tiny, cudaStream_t st, bool* ran)
 {
     *ran = false;
-    if (n < 1 || n > (sizeof(T) == 4 ? GC_MAXN32 : GC_MAXN64)) return SAI_OK;
+    if (n < 1 || n > (sizeof(T) == 4 ? GC_MAXN32 : GC_MAXN64) || (n > (sizeof(T) == 4 ? GC_FAR_N32 : CL_FAR_N) && A.scattered))
+        return SAI_OK;
     // whether the form is used depends on n and m alone, as the sums do: a
     // system's bits do not depend on the systems that run with it
     const GcUnits N(n);

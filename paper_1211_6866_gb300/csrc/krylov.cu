@@ -269,6 +269,7 @@ struct Mat {
     const int32_t* sci = nullptr;
     const T* sv = nullptr;
     int64_t nslices = 0;
+    int64_t far = 0;  // entries outside the diagonal blocks that build_sell was asked to look at
 };
 
 // Sliced-ELL SpMV: one warp per slice (lane = row of the slice). A slice of
@@ -606,24 +607,48 @@ void spmv(int32_t n, int64_t ld, const Mat<T>& A, int k, const T* X, T* Y, const
     else k_spmv<T, MODE, false><<<SAI_GRID(g), TILE, 0, st>>>(n, ld, A.rp, A.ci, A.v, X, Y, B, list, jstop, jmax);
 }
 
+// far += the entries whose row and column lie in different blocks of `rows` rows, a warp per row
+__global__ void __launch_bounds__(256) k_far_entries(int32_t n, int32_t rows, const int64_t* __restrict__ rp,
+                                                     const int32_t* __restrict__ ci, unsigned long long* far)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned cnt = 0;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n;
+         i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int32_t b = (int32_t)i / rows;
+        for (int64_t q = rp[i] + lane; q < rp[i + 1]; q += 32) cnt += ci[q] / rows != b;
+    }
+    cnt = __reduce_add_sync(SAI_FULL, cnt);
+    if (lane == 0 && cnt) atomicAdd(far, (unsigned long long)cnt);
+}
+
 // Adds a sliced-ELL copy (values converted to T) of the CSR matrix (rp, ci,
 // v64) to m, unless slice padding would exceed half of nnz (then m keeps
-// only its CSR form). Synchronises the stream once to read the size.
+// only its CSR form). Synchronises the stream once to read the size, and, with
+// far_rows > 0, the count of entries between blocks of far_rows rows.
 template <class T>
-sai_status build_sell(int32_t n, int64_t nnz, const int64_t* rp, const int32_t* ci, const double* v64, Buf& spb,
-                      Buf& cib, Buf& vb, Mat<T>& m, cudaStream_t st)
+sai_status build_sell(int32_t n, int64_t nnz, const int64_t* rp, const int32_t* ci, const double* v64, int32_t far_rows,
+                      Buf& spb, Buf& cib, Buf& vb, Mat<T>& m, cudaStream_t st)
 {
     if (n <= 0) return SAI_OK;
     const int64_t ns = ((int64_t)n + SELL_C - 1) / SELL_C;
     Buf cnt;
     SAI_TRY(cnt.alloc(sizeof(int64_t) * (size_t)ns, st, true));
-    SAI_TRY(spb.alloc(sizeof(int64_t) * (size_t)(ns + 1), st, true));
+    SAI_TRY(spb.alloc(sizeof(int64_t) * (size_t)(ns + 2), st, true));  // the last value: far
     const unsigned g = sai_div_up(ns * 32, 256);
+    SAI_CUDA(cudaMemsetAsync(spb.as<int64_t>() + ns + 1, 0, sizeof(int64_t), st));
+    if (far_rows > 0) {
+        const unsigned gf = sai_div_up((int64_t)n * 32, 256), cap = (unsigned)g_sms * 8;
+        k_far_entries<<<SAI_GRID(gf < cap ? gf : cap), 256, 0, st>>>(
+            n, far_rows, rp, ci, reinterpret_cast<unsigned long long*>(spb.as<int64_t>() + ns + 1));
+    }
     k_sell_width<<<SAI_GRID(g), 256, 0, st>>>(n, rp, ns, cnt.as<int64_t>());
     SAI_TRY(sai_scan_counts_i64(cnt.as<int64_t>(), spb.as<int64_t>(), ns, st));
-    int64_t total = 0;
-    SAI_CUDA(cudaMemcpyAsync(&total, spb.as<int64_t>() + ns, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    int64_t sizes[2] = {0, 0};
+    SAI_CUDA(cudaMemcpyAsync(sizes, spb.as<int64_t>() + ns, sizeof(sizes), cudaMemcpyDeviceToHost, st));
     SAI_CUDA(cudaStreamSynchronize(st));
+    const int64_t total = sizes[0];
+    m.far = sizes[1];
     if ((double)total > 1.5 * (double)nnz + (double)SELL_C * ns) return SAI_OK;  // too much padding: CSR
     SAI_TRY(cib.alloc(sizeof(int32_t) * (size_t)(total > 0 ? total : 1), st, true));
     SAI_TRY(vb.alloc(sizeof(T) * (size_t)(total > 0 ? total : 1), st, true));
@@ -639,6 +664,7 @@ sai_status build_sell(int32_t n, int64_t nnz, const int64_t* rp, const int32_t* 
 template <class T>
 struct Ops {  // A~ (or A~^T) and M (or M^T) with values of type T
     Mat<T> A, M;
+    bool scattered = false;  // most entries lie far from the diagonal (far_rows)
 };
 
 // ---------------------------------------------------------------- item kernels
@@ -1284,10 +1310,6 @@ void pnl_apply2(int32_t n, int64_t ld, int k, const Ops<double>& A, const double
 #include "sorted_rows.cuh"
 #include "bicg_cluster.cuh"
 
-// Up to this many systems of order CL_MAXN or less run in clusters; with more
-// the multi-kernel form fills the GPU and reads the matrices once for all.
-constexpr int CL_MAXK = CTRL;
-
 sai_status bicgstab_run(const Items& I, int k, const Ops<double>& A, const double* Bsd, double* Xsd, Sys& S,
                         double* pt, int* fl, int maxit, const Dims& D, cudaStream_t st)
 {
@@ -1297,7 +1319,7 @@ sai_status bicgstab_run(const Items& I, int k, const Ops<double>& A, const doubl
     const int ib = item_blocks(n > 0 ? n : 1, k);
     const int check_every = 4;
     int hflag = 0;
-    if (n > 0 && n <= CL_MAXN && k <= CL_MAXK) {
+    if (n > 0) {
         bool ran;
         {
             ProfScope ps(PROF_SPMM, st);
@@ -4120,12 +4142,20 @@ sai_status sai_krylov_run(const sai_split_s* h, const sai_precond_s* P, int32_t 
     k_fill_int<<<SAI_GRID(1), 256, 0, st>>>(k, cap, prm->maxit);
     SAI_CUDA(cudaGetLastError());
 
+    // sixteenths of the rows, the blocks that the cluster forms' choice between
+    // local and scattered matrices looks at (0: no choice)
+    const bool cluster = (prm->method == SAI_BICGSTAB && n <= CL_MAXN) || (prm->method == SAI_GMRES && n <= GC_MAXN32);
+    const int32_t far_rows = cluster && n > CL_FAR_N ? (n + 15) / 16 : 0;
+    auto scattered = [&](int64_t far) { return (double)far > 0.55 * (double)(h->nnz_At + P->nnz); };
     // sliced-ELL copies for the FP64 solvers; the refined forms build FP32
     // ones in the same buffers and keep the CSR arrays for the FP64 residual
     if (prm->precision == SAI_FP64) {
         Ops<double> S64 = A64;
-        SAI_TRY(build_sell<double>(n, h->nnz_At, A64.A.rp, A64.A.ci, A64.A.v, sell[0], sell[1], sell[2], S64.A, st));
-        SAI_TRY(build_sell<double>(n, P->nnz, A64.M.rp, A64.M.ci, A64.M.v, sell[3], sell[4], sell[5], S64.M, st));
+        SAI_TRY(build_sell<double>(n, h->nnz_At, A64.A.rp, A64.A.ci, A64.A.v, far_rows, sell[0], sell[1], sell[2], S64.A,
+                                   st));
+        SAI_TRY(build_sell<double>(n, P->nnz, A64.M.rp, A64.M.ci, A64.M.v, far_rows, sell[3], sell[4], sell[5], S64.M,
+                                   st));
+        S64.scattered = scattered(S64.A.far + S64.M.far);
         A64 = S64;
     }
     if (prm->method == SAI_BICGSTAB) {
@@ -4198,8 +4228,11 @@ sai_status sai_krylov_run(const sai_split_s* h, const sai_precond_s* P, int32_t 
         A32.M.rp = A64.M.rp;
         A32.M.ci = A64.M.ci;
         A32.M.v = m32.as<float>();
-        SAI_TRY(build_sell<float>(n, h->nnz_At, A64.A.rp, A64.A.ci, A64.A.v, sell[0], sell[1], sell[2], A32.A, st));
-        SAI_TRY(build_sell<float>(n, P->nnz, A64.M.rp, A64.M.ci, A64.M.v, sell[3], sell[4], sell[5], A32.M, st));
+        SAI_TRY(build_sell<float>(n, h->nnz_At, A64.A.rp, A64.A.ci, A64.A.v, far_rows, sell[0], sell[1], sell[2], A32.A,
+                                  st));
+        SAI_TRY(build_sell<float>(n, P->nnz, A64.M.rp, A64.M.ci, A64.M.v, far_rows, sell[3], sell[4], sell[5], A32.M,
+                                  st));
+        A32.scattered = scattered(A32.A.far + A32.M.far);
         double* r64 = r64b.as<double>();
         float* r32 = v32b.as<float>();
         float* d32 = r32 + blk;
