@@ -223,6 +223,24 @@ sai_status cl_matrix(const Mat<T>& X, int n, int R, int C, Buf (&buf)[4], ClMat<
     return SAI_OK;
 }
 
+// The two matrices of a cluster kernel, formed once per call of the solver (a
+// refined solve runs GMRES once per outer step; the blocks stay the same).
+template <class T>
+struct ClPair {
+    ClMat<T> A, M;
+    Buf ab[4], mb[4];
+    bool ready = false;
+    // SAI_OOM: no memory for the sorted forms, of which the multi-kernel form needs none
+    sai_status form(const Mat<T>& a, const Mat<T>& m, int n, int R, int C, cudaStream_t st)
+    {
+        if (ready) return SAI_OK;
+        SAI_TRY(cl_matrix(a, n, R, C, ab, A, st));
+        SAI_TRY(cl_matrix(m, n, R, C, mb, M, st));
+        ready = true;
+        return SAI_OK;
+    }
+};
+
 // Stores a unit's partial sum in slot `slot` of every block of the cluster.
 template <bool MULTI>
 __device__ __noinline__ void cl_put(double v, int slot, int unit, double* parts, int pstride, int nranks)
@@ -574,11 +592,11 @@ inline sai_status cl_bicgstab(const Ops<double>& A, int k, int n, int64_t ld, co
     if (C == CL_MAXC && rows(C) >= 512 && fits(16)) C = 16;
     const int rmax = rows(C);
     const size_t smem = bytes(C);
-    ClMat<double> a, m;
-    Buf ab[4], mb[4];
-    if (cl_matrix(A.A, n, rmax, C, ab, a, st) != SAI_OK || cl_matrix(A.M, n, rmax, C, mb, m, st) != SAI_OK)
-        return SAI_OK;  // no memory for the sorted forms: the kernels below need none
-    *ran = cl_run(C > 1 ? k_bicg_cluster<true> : k_bicg_cluster<false>, k, C, CL_T, CL_SMEM, smem, st, a, m, n, ld, rmax,
+    ClPair<double> F;
+    const sai_status fs = F.form(A.A, A.M, n, rmax, C, st);
+    if (fs == SAI_OOM) return SAI_OK;
+    SAI_TRY(fs);
+    *ran = cl_run(C > 1 ? k_bicg_cluster<true> : k_bicg_cluster<false>, k, C, CL_T, CL_SMEM, smem, st, F.A, F.M, n, ld, rmax,
                   umax, B, X, thr, maxit, iters, status);
     return SAI_OK;
 }

@@ -559,8 +559,8 @@ k_gmres_cluster(ClMat<T> A, ClMat<T> M, GcArgs P, Basis<T> Bv, const T* __restri
 
 // Runs the k systems in clusters when they fit (*ran).
 template <class T>
-sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* Bs, T* Xs, const GmWork<T>& Wk, Sys& S,
-               const int* cap, const Dims& D, double tiny, cudaStream_t st, bool* ran)
+sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, ClPair<T>& F, const T* Bs, T* Xs,
+                     const GmWork<T>& Wk, Sys& S, const int* cap, const Dims& D, double tiny, cudaStream_t st, bool* ran)
 {
     *ran = false;
     if (n < 1 || n > (sizeof(T) == 4 ? GC_MAXN32 : GC_MAXN64) || (n > (sizeof(T) == 4 ? GC_FAR_N32 : CL_FAR_N) && A.scattered))
@@ -608,10 +608,10 @@ sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, const T* 
     P.hp = (uint32_t)L.hp;
     P.g = (uint32_t)L.g;
     P.y = (uint32_t)L.y;
-    ClMat<T> a, mm;
-    Buf ab[4], mb[4];
-    if (cl_matrix(A.A, n, R, C, ab, a, st) != SAI_OK || cl_matrix(A.M, n, R, C, mb, mm, st) != SAI_OK) return SAI_OK;
-    *ran = cl_run(C > 1 ? k_gmres_cluster<T, true> : k_gmres_cluster<T, false>, k, C, GC_T, GC_SMEM, L.bytes, st, a, mm, P,
+    const sai_status fs = F.form(A.A, A.M, n, R, C, st);
+    if (fs == SAI_OOM) return SAI_OK;
+    SAI_TRY(fs);
+    *ran = cl_run(C > 1 ? k_gmres_cluster<T, true> : k_gmres_cluster<T, false>, k, C, GC_T, GC_SMEM, L.bytes, st, F.A, F.M, P,
                   Wk.B, Bs, Xs, (const double*)S.thr, cap, S.iters, S.status, D);
     return SAI_OK;
 }

@@ -2998,8 +2998,8 @@ constexpr int GM_LAUNCHES_PER_STEP = 5;
 // Unless a profile is open, each group of GM_STEPS_PER_CHECK Arnoldi steps
 // runs as one captured CUDA graph.
 template <class T>
-sai_status gmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs, T* Xs, const GmWork<T>& Wk, Sys& S,
-                     Gm& G, const int* cap, double* pt, double* pt2, int* fl, const Dims& D, cudaStream_t st)
+sai_status gmres_run(const Items& I, int k, int m, const Ops<T>& A, ClPair<T>& F, const T* Bs, T* Xs,
+                     const GmWork<T>& Wk, Sys& S, Gm& G, const int* cap, double* pt, double* pt2, int* fl, const Dims& D, cudaStream_t st)
 {
     const int32_t n = I.n;
     const int64_t ld = I.ld;
@@ -3011,7 +3011,7 @@ sai_status gmres_run(const Items& I, int k, int m, const Ops<T>& A, const T* Bs,
     {
         bool ran;
         ProfScope ps(D.site_dots, st);
-        SAI_TRY(gc_launch<T>(n, ld, k, m, A, Bs, Xs, Wk, S, cap, D, tiny, st, &ran));
+        SAI_TRY(gc_launch<T>(n, ld, k, m, A, F, Bs, Xs, Wk, S, cap, D, tiny, st, &ran));
         if (ran) return SAI_OK;
     }
     // dynamic shared memory of the two kernels that stage Hbar / R (their
@@ -4193,7 +4193,8 @@ sai_status sai_krylov_run(const sai_split_s* h, const sai_precond_s* P, int32_t 
         GmWork<double> Wk;
         SAI_TRY(gm_alloc(k, prm->restart, hb, ibuf, G, st));
         SAI_TRY(gm_work_alloc<double>(blk, prm->restart, vb, wb, Wk, st));
-        SAI_TRY(gmres_run<double>(I, k, prm->restart, A64, Bsd, Xsd, Wk, S, G, cap, pt, pt2, fl, D, st));
+        ClPair<double> F;
+        SAI_TRY(gmres_run<double>(I, k, prm->restart, A64, F, Bsd, Xsd, Wk, S, G, cap, pt, pt2, fl, D, st));
     } else {
         // GMRES with iterative refinement: FP64 residual, correction and stop
         // tests outside; the inner solves run entirely in FP32.
@@ -4201,6 +4202,7 @@ sai_status sai_krylov_run(const sai_split_s* h, const sai_precond_s* P, int32_t 
         Gm G;
         Buf hb, ibuf, vb, wb, a32, m32, r64b, v32b, irb, ird;
         GmWork<float> Wk;
+        ClPair<float> F;
         Bg<float> Bgm;  // block GMRES inner solver
         if (prm->method == SAI_BGMRES) {
             SAI_TRY(bg_alloc<float>(k, prm->restart, n, ld, vb, hb, ibuf, Bgm, st));
@@ -4262,7 +4264,7 @@ sai_status sai_krylov_run(const sai_split_s* h, const sai_precond_s* P, int32_t 
             if (prm->method == SAI_BGMRES)
                 SAI_TRY(bgmres_run<float>(I, k, prm->restart, A32, r32, d32, Bgm.R, Bgm, S, cap, pt2, D32, st));
             else
-                SAI_TRY(gmres_run<float>(I, k, prm->restart, A32, r32, d32, Wk, S, G, cap, pt, pt2, fl, D32, st));
+                SAI_TRY(gmres_run<float>(I, k, prm->restart, A32, F, r32, d32, Wk, S, G, cap, pt, pt2, fl, D32, st));
             VK(I, k_ir_update)<<<SAI_GRID(ib), VT, 0, st>>>(I, Xsd, d32, beta, lir);
             k_ir_total<<<SAI_GRID(1), 32, 0, st>>>(k, lir, S.iters, tot);
             spmv<double, 1>(n, ld, A64.A, k, Xsd, r64, Bsd, lir, st);

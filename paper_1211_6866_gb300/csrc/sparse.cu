@@ -22,6 +22,7 @@ sai_status Buf::alloc(size_t nbytes, cudaStream_t s, bool use_async)
     if (e == cudaSuccess) dev = d;
     if (e != cudaSuccess) {
         p = nullptr;
+        (void)cudaGetLastError();  // the status carries it: a caller may go on without the buffer
         sai_internal_note_cuda_error(e, "device allocation", __FILE__, __LINE__);
         return e == cudaErrorMemoryAllocation ? SAI_OOM : SAI_CUDA_ERROR;
     }
