@@ -2092,20 +2092,30 @@ sai_status build_common(const sai_split_s* h, const SpaiArgs& sa, const PsaiArgs
         // Up to two columns per SM a column's latency counts: the workspace in
         // shared memory (12 columns of the 255^2 anisotropic operator 4.2 -> 3.4
         // ms); up to 64 per SM the longest columns' latency still does: the
-        // hybrid form, nine columns per SM (tiers 1 and 2 of the Zipf matrix of
-        // order 20000, 7037 and 651 columns: build 48 -> 42 ms). With more, the
-        // number in flight counts: 260095 columns of the 512^2 operator took 461
-        // ms in the hybrid form, 282 ms in the global one (sixteen per SM).
-        const auto tier1 = hc[1] <= 2 * g_num_sms    ? launch_tier<T1, 32, WS_SHARED, PSAI>
-                           : hc[1] <= 64 * g_num_sms ? launch_tier<T1, 32, WS_HYBRID, PSAI>
-                                                     : launch_tier<T1, 32, WS_GLOBAL, PSAI>;
+        // hybrid form, nine columns per SM (7827 columns of the Zipf matrix of
+        // order 20000: build 36 -> 26 ms). With more, the number in flight counts
+        // (sixteen per SM in the global form): 260095 columns of the 512^2
+        // operator took 461 ms in the hybrid form, 282 ms in the global one. It
+        // counts too where SPAI's patterns may outgrow the tier, which keeps its
+        // columns long and full: delta 0.1, 20 augmentations, 3491 columns of the
+        // 60^2 operator 71 and 66 ms.
+        const bool grows = !PSAI && smax > T1::SCAP;
+        const auto tier1 = hc[1] <= 2 * g_num_sms              ? launch_tier<T1, 32, WS_SHARED, PSAI>
+                           : hc[1] <= 64 * g_num_sms && !grows ? launch_tier<T1, 32, WS_HYBRID, PSAI>
+                                                               : launch_tier<T1, 32, WS_GLOBAL, PSAI>;
         SAI_TRY(tier1(A, sa, pa, ovf0.as<int32_t>(), hc[1], c + 0, out, ovf1.as<int32_t>(), c + 2, c + 3, 1, cfg, st));
         SAI_CUDA(cudaMemcpyAsync(hc, c, sizeof(hc), cudaMemcpyDeviceToHost, st));
         SAI_CUDA(cudaStreamSynchronize(st));
         if (hc[2] > 0) {
-            // tier 2 queues its overflows in ovf0 (tier 1's input, no longer read)
-            const auto tier2 = hc[2] <= 8 * g_num_sms ? launch_tier<T2, 32, WS_HYBRID, PSAI>
-                                                      : launch_tier<T2, 32, WS_GLOBAL, PSAI>;
+            // tier 2 queues its overflows in ovf0 (tier 1's input, no longer
+            // read). Hybrid, two columns per SM, up to that number: 6 columns of the
+            // 60^2 operator 18.2 -> 15.1 ms, 192 of the Zipf matrix of order 8000
+            // 9.5 -> 8.6, but 1164 of order 4000 30 -> 40. PSAI's columns of this
+            // tier have several hundred rows, whose factors fill L1, which the
+            // workspaces would take: 17 columns of order 4000 in FP32 19.2 ms hybrid,
+            // 7.4 global.
+            const auto tier2 = !PSAI && hc[2] <= 2 * g_num_sms ? launch_tier<T2, 32, WS_HYBRID, PSAI>
+                                                               : launch_tier<T2, 32, WS_GLOBAL, PSAI>;
             SAI_TRY(tier2(A, sa, pa, ovf1.as<int32_t>(), hc[2], c + 0, out, ovf0.as<int32_t>(), c + 12, c + 3, 2, cfg,
                           st));
             int h3 = 0;
