@@ -2518,6 +2518,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t par)
     return false;
 }
 
+// orders this thread's accesses to shared memory before those of later bulk copies
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 // bytes (a multiple of 16) from src (16-byte aligned) to dst (16-byte aligned shared memory)
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* b)
 {
@@ -2652,8 +2655,6 @@ __global__ void __launch_bounds__((UP_CWARPS + 1) * 32) k_dc_update_ring(Items I
 #pragma unroll
                 for (int p = 0; p < UP_PT; ++p)
                     if (t < nv) v[t][p] = reinterpret_cast<const VT*>(ring + st * STB + t * SEGB)[tid + p * NC];
-            __syncwarp();
-            if (lane == 0 && !dead) mbar_arrive(&empty[st]);
 #pragma unroll
             for (int t = 0; t < UP_VPS; ++t) {
                 const int sg = v0 + t;
@@ -2669,6 +2670,12 @@ __global__ void __launch_bounds__((UP_CWARPS + 1) * 32) k_dc_update_ring(Items I
                     }
                 }
             }
+            // the loads above come before the copies that refill the stage: a
+            // barrier alone orders them for the generic proxy only (beside other
+            // kernels one warp in some ten thousand read the next contents)
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0 && !dead) mbar_arrive(&empty[st]);
         }
         if (!dead) {
             const T ia = coef[0], dd = coef[1];

@@ -77,7 +77,8 @@ def test_two_threads_with_problems_of_different_size(kind):
         try:
             with torch.cuda.stream(torch.cuda.Stream()):
                 start.wait()
-                for _ in range(60):
+                # the update's copy ring has more chances beside another thread's kernels
+                for _ in range(1000 if kind == "gmres_graphs" else 60):
                     got = f()
                     if not torch.equal(got, want):
                         failed.append("other bits")
