@@ -227,7 +227,7 @@ sai_status sai_split_create(const sai_csc_view* A, const sai_split_params* prm, 
     std::unique_ptr<sai_split_s> h(new (std::nothrow) sai_split_s());
     if (!h) return SAI_OOM;
     HandleUse use{h.get(), nullptr, S(stream)};
-    SAI_TRY(sai_split_build(A, prm, S(stream), false, h.get()));
+    SAI_TRY(use.synced(sai_split_build(A, prm, S(stream), false, h.get())));
     *out = h.release();
     return SAI_OK;
 }
@@ -284,7 +284,7 @@ sai_status sai_build_spai(sai_split h, const sai_spai_params* prm, sai_stream_t 
     std::unique_ptr<sai_precond_s> P(new (std::nothrow) sai_precond_s());
     if (!P) return SAI_OOM;
     HandleUse use{h, P.get(), S(stream)};
-    SAI_TRY(sai_spai_build(h, prm, S(stream), false, P.get()));
+    SAI_TRY(use.synced(sai_spai_build(h, prm, S(stream), false, P.get())));
     *out = P.release();
     return SAI_OK;
 }
@@ -297,7 +297,7 @@ sai_status sai_build_psai(sai_split h, const sai_psai_params* prm, sai_stream_t 
     std::unique_ptr<sai_precond_s> P(new (std::nothrow) sai_precond_s());
     if (!P) return SAI_OOM;
     HandleUse use{h, P.get(), S(stream)};
-    SAI_TRY(sai_psai_build(h, prm, S(stream), false, P.get()));
+    SAI_TRY(use.synced(sai_psai_build(h, prm, S(stream), false, P.get())));
     *out = P.release();
     return SAI_OK;
 }
@@ -337,6 +337,7 @@ sai_status sai_precond_create(const sai_csc_view* M, sai_stream_t stream, sai_pr
     SAI_TRY(sai_csc_to_csr(n, n, nnz, P->M_cp.as<int64_t>(), P->M_ri.as<int32_t>(), P->M_v.as<double>(), P->Mr_rp,
                            P->Mr_ci, P->Mr_v, st, false));
     SAI_CUDA(cudaStreamSynchronize(st));
+    use.synced(SAI_OK);
     *out = P.release();
     return SAI_OK;
 }
@@ -377,7 +378,7 @@ sai_status sai_krylov_solve(sai_split h, sai_precond P, int32_t k, const double*
 {
     sai_pool_init_once();
     HandleUse use{h, P, S(stream)};
-    return sai_krylov_run(h, P, k, B, thr, prm, X, iters, status, S(stream));
+    return use.synced(sai_krylov_run(h, P, k, B, thr, prm, X, iters, status, S(stream)));
 }
 
 sai_status sai_smw_recover(sai_split h, const double* Y, double* x, double* c_out, sai_stream_t stream)
@@ -816,7 +817,7 @@ extern "C" sai_status sai_solve_with(const sai_csc_view* A, sai_split h, sai_pre
 {
     sai_pool_init_once();
     HandleUse use{h, P, S(stream)};
-    return solve_with_impl(A, h, P, b, prm, x, iters, iters_cap, rep, S(stream));
+    return use.synced(solve_with_impl(A, h, P, b, prm, x, iters, iters_cap, rep, S(stream)));
 }
 
 extern "C" sai_status sai_backward(const sai_csc_view* A, sai_split h, sai_precond P, const double* x,
@@ -825,7 +826,7 @@ extern "C" sai_status sai_backward(const sai_csc_view* A, sai_split h, sai_preco
 {
     sai_pool_init_once();
     HandleUse use{h, P, S(stream)};
-    return backward_impl(A, h, P, x, g, prm, lambda, grad_vals, iters, iters_cap, rep, S(stream));
+    return use.synced(backward_impl(A, h, P, x, g, prm, lambda, grad_vals, iters, iters_cap, rep, S(stream)));
 }
 
 extern "C" sai_status sai_dmperm(const sai_csc_view* A, int32_t* p, int32_t* rank_out, int32_t* moved_out,

@@ -1299,8 +1299,8 @@ extern "C" sai_status sai_build_batched(int32_t nmat, const sai_csc_view* A, con
     std::unique_ptr<sai_precond_s> P(new (std::nothrow) sai_precond_s());
     if (!P) return SAI_OOM;
     HandleUse use{nullptr, P.get(), st};
-    SAI_TRY(prm->sai == 0 ? sai_spai_build(&bd, &prm->spai, st, false, P.get())
-                          : sai_psai_build(&bd, &prm->psai, st, false, P.get()));
+    SAI_TRY(use.synced(prm->sai == 0 ? sai_spai_build(&bd, &prm->spai, st, false, P.get())
+                                     : sai_psai_build(&bd, &prm->psai, st, false, P.get())));
     *out = P.release();
     return SAI_OK;
 }

@@ -116,16 +116,23 @@ struct sai_precond_s {
     Buf loops, res, res_post;
 };
 
-// Records the use of handles (nullptr: none) by a call on st when it ends,
-// with whatever status: an error may leave work in flight.
+// Records the use of handles (nullptr: none) by a call on st when it ends, unless
+// it ended synchronised: an error may leave work in flight.
 struct HandleUse {
     const sai_split_s* h;
     const sai_precond_s* P;
     cudaStream_t st;
+    bool idle = false;
+    // passes on the status of a call that synchronises st before it returns without an error
+    sai_status synced(sai_status r)
+    {
+        idle = r == SAI_OK || r == SAI_MAXITER || r == SAI_BREAKDOWN;
+        return r;
+    }
     ~HandleUse()
     {
-        if (h) h->uses.record(st);
-        if (P) P->uses.record(st);
+        if (h && !idle) h->uses.record(st);
+        if (P && !idle) P->uses.record(st);
     }
 };
 
