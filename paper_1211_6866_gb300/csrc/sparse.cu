@@ -36,7 +36,7 @@ void Buf::release()
     } else if (p && dev >= 0) {
         int cur = -1;
         const bool other = cudaGetDevice(&cur) == cudaSuccess && cur != dev && cudaSetDevice(dev) == cudaSuccess;
-        cudaFreeAsync(p, sai_free_stream());
+        cudaFreeAsync(p, st);  // chosen by free_on
         if (other) cudaSetDevice(cur);
     } else if (p) {
         cudaFree(p);
@@ -118,19 +118,26 @@ void HandleUses::record(cudaStream_t s)
     }
 }
 
-void HandleUses::before_free()
+cudaStream_t HandleUses::before_free(const Buf& b)
 {
-    if (cnt == 0) return;
+    if (b.async) return nullptr;  // no handle: a call's own buffers
+    const int d = b.dev >= 0 ? b.dev : dev;
     int cur = -1;
-    const bool other = cudaGetDevice(&cur) == cudaSuccess && cur != dev && cudaSetDevice(dev) == cudaSuccess;
-    cudaStream_t f = sai_free_stream();
+    const bool other = d >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != d && cudaSetDevice(d) == cudaSuccess;
+    cudaStream_t f = nullptr;
+    // not the legacy stream while one that it would wait for captures
+    cudaStreamCaptureStatus cs;
+    if ((b.st != nullptr && b.st != cudaStreamLegacy) || cudaStreamIsCapturing(nullptr, &cs) != cudaSuccess ||
+        cs != cudaStreamCaptureStatusNone)
+        f = sai_free_stream();
     for (int q = 0; q < cnt; ++q) {
-        if (!f || cudaStreamWaitEvent(f, ev[q], 0) != cudaSuccess) cudaEventSynchronize(ev[q]);
+        if (cudaStreamWaitEvent(f, ev[q], 0) != cudaSuccess) cudaEventSynchronize(ev[q]);
         cudaEventDestroy(ev[q]);
     }
     (void)cudaGetLastError();
     cnt = 0;
     if (other) cudaSetDevice(cur);
+    return f;
 }
 
 // ------------------------------------------------------------------ scan

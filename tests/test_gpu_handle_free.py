@@ -28,8 +28,14 @@ def _copy_out(sai, P, v, stream):
 
 @pytest.mark.parametrize("nstreams", [1, 3, 20])  # 20: more streams than a handle keeps events for
 @pytest.mark.parametrize("capture", [False, True])
-def test_destroyed_with_copies_in_flight(nstreams, capture):
+@pytest.mark.parametrize("own", [False, True])  # created on the legacy stream, or on one of the caller's
+def test_destroyed_with_copies_in_flight(nstreams, capture, own):
     need_gpu()
+    with torch.cuda.stream(torch.cuda.Stream() if own else torch.cuda.default_stream()):
+        _destroyed_with_copies_in_flight(nstreams, capture)
+
+
+def _destroyed_with_copies_in_flight(nstreams, capture):
     sai = lib()
     n = 100000
     streams = [torch.cuda.Stream() for _ in range(nstreams)]
