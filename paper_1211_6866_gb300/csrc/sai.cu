@@ -1707,11 +1707,11 @@ __global__ void __launch_bounds__(256) k_sai(SaiMat A, SpaiArgs sa, PsaiArgs pa,
                     oval[t] = w.m[t];
                 }
                 if (big && g.l == 0) out.big_slot[k] = item;
-                int cb = 0;  // in 4-byte words
+                long long cb = 0;  // in 4-byte words: the rows of a column may hold more than 2^31 of them
 #pragma unroll 1
-                for (int t = g.l; t < nS; t += G) cb += 3 * (int)(A.cp[w.S[t] + 1] - A.cp[w.S[t]]) + 3;
+                for (int t = g.l; t < nS; t += G) cb += 3 * (A.cp[w.S[t] + 1] - A.cp[w.S[t]]) + 3;
 #pragma unroll 1
-                for (int t = g.l; t < nL; t += G) cb += (int)(A.rp[w.Lrow[t] + 1] - A.rp[w.Lrow[t]]);
+                for (int t = g.l; t < nL; t += G) cb += A.rp[w.Lrow[t] + 1] - A.rp[w.Lrow[t]];
                 work_bytes += 4LL * g.sum(cb);
                 work_flops += cfl;
                 work_flops_q += cfq;
