@@ -3,15 +3,17 @@
 // namespace).
 //
 // At these orders an iteration of the multi-kernel form is nine launches of a
-// few microseconds each, whatever the work. Here a cluster of 1, 2, 4 or 8
+// few microseconds each, whatever the work. Here a cluster of 1, 2, 4, 8 or 16
 // blocks keeps all nine vectors of its system in shared memory (block b the
 // rows [b R, (b + 1) R)), reads the matrices through L1, gathers x across the
 // cluster by distributed-shared-memory loads and runs every iteration without
 // leaving the kernel; a phase costs a cluster barrier. A 45 x 45 grid with four
 // systems, 80 iterations: 11.5 ms per call at first, 2.5 ms here, 22 us per
-// iteration (six barriers, four products, three scalar chains).
+// iteration (seven barriers, four products, three scalar chains).
 //
-// A system's bits do not depend on the cluster size or on the other systems:
+// A system's bits do not depend on the cluster size, nor on the systems that
+// run with it as long as their number leaves the form in use (the limits below;
+// the multi-kernel form adds in another order):
 // row sums run over the row's entries in order, and an inner product is a
 // fixed tree per unit of 64 rows (two rows per lane, five shuffle levels)
 // followed by the units' sums in a fixed order (lane l takes units l, l + 32,
