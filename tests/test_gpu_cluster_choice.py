@@ -41,3 +41,27 @@ def test_around_the_limits(n, k, method, scattered):
         assert st == sai.SAI_OK and stt == [0] * k
         R = np.linalg.norm(B - Aop @ X.cpu().numpy(), axis=0)
         assert np.all(R <= np.asarray(thr) + 1e-12 * norms), (R, thr)
+
+
+@pytest.mark.parametrize("n", [1, 2, 511, 512, 513, 1537, 16383, 16384, 16385])
+def test_vector_kernels_of_many_systems(n):
+    """More systems than the cluster form takes: BiCGStab's vector kernels at the edges of their chunks of 512 rows (2048
+    from 16384 on). 257 and 300 systems give the same bits: a system's sums depend on n alone."""
+    need_gpu()
+    sai = lib()
+    rng = np.random.default_rng(n)
+    A = sp.csc_matrix(sp.diags([-1.0 - 0.5 * rng.random(max(n - 1, 0)), np.full(n, 4.5), -np.ones(max(n - 1, 0))],
+                               (-1, 0, 1), shape=(n, n)))
+    h = sai.split(to_dev(A), abs_tau=float("inf"))
+    P = sai.precond_from_csc(to_dev(sp.csc_matrix(sp.diags(1.0 / A.diagonal()))))
+    B = rng.standard_normal((n, 300))
+    norms = np.linalg.norm(B, axis=0)
+    thr = list(norms * 10.0 ** -np.linspace(2, 10, 300))
+    thr[3] = 2.0 * norms[3]
+    Bd = torch.as_tensor(B, device="cuda")
+    X, it, stt, st = sai.krylov_solve(h, P, Bd, thr, maxit=60)
+    assert st == sai.SAI_OK and stt == [0] * 300 and it[3] == 0
+    R = np.linalg.norm(B - A @ X.cpu().numpy(), axis=0)
+    assert np.all(R <= np.asarray(thr) + 1e-12 * norms), (R, thr)
+    x, i, _, _ = sai.krylov_solve(h, P, Bd[:, :257].contiguous(), thr[:257], maxit=60)
+    assert i == it[:257] and torch.equal(x, X[:, :257])
