@@ -516,19 +516,28 @@ __global__ void k_cl_work(int k, const int* iters, Dims D)
     kwork_add(PROF_BICG_VEC, 8.0 * D.n * 19 * sum, D.n * 23.0 * sum);
 }
 
+// Clusters of C blocks of kern that the GPU holds at once, by log2 C (0: not
+// asked yet). A block's registers leave room for no second one on its SM
+// whatever its shared memory, so the answer depends on the GPU and C alone and is
+// kept: asking takes 20 to 30 us, 2% of a small solve.
+using ClHeld = std::atomic<int>[5];
+
 // true when the GPU holds k clusters of C blocks of kern at once (fewer than its
 // SMs suggest: a cluster stays within one group of them, and sixteen clusters of
 // eight blocks take two rounds on 152 SMs); limit: the most dynamic shared memory
 // of kern's launches
 template <class... Params>
-bool cl_fits(void (*kern)(Params...), int k, int C, int threads, size_t limit, size_t smem)
+bool cl_fits(void (*kern)(Params...), int k, int C, int threads, size_t limit, ClHeld& held)
 {
     if ((int64_t)C * k > g_sms) return false;
     if (C <= CL_MAXC && (int64_t)2 * C * k <= g_sms) return true;
+    int lg = 0;
+    while ((1 << lg) < C) ++lg;
+    if (held[lg].load(std::memory_order_relaxed) > 0) return held[lg].load(std::memory_order_relaxed) >= k;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)C * (unsigned)k);
     cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = limit;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = (unsigned)C;
@@ -541,6 +550,7 @@ bool cl_fits(void (*kern)(Params...), int k, int C, int threads, size_t limit, s
                     sai_smem_limit(kern, limit) == cudaSuccess &&
                     cudaOccupancyMaxActiveClusters(&most, kern, &cfg) == cudaSuccess;
     if (!ok) (void)cudaGetLastError();
+    if (ok && most > 0) held[lg].store(most, std::memory_order_relaxed);
     return ok && most >= k;
 }
 
@@ -548,7 +558,8 @@ bool cl_fits(void (*kern)(Params...), int k, int C, int threads, size_t limit, s
 template <class... Params, class... Args>
 bool cl_run(void (*kern)(Params...), int k, int C, int threads, size_t limit, size_t smem, cudaStream_t st, Args... args)
 {
-    if (sai_smem_limit(kern, limit) != cudaSuccess) {
+    if (sai_smem_limit(kern, limit) != cudaSuccess ||
+        (C > CL_MAXC && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
         (void)cudaGetLastError();
         return false;
     }
@@ -583,7 +594,8 @@ inline sai_status cl_bicgstab(const Ops<double>& A, int k, int n, int64_t ld, co
     auto bytes = [&](int blocks) {
         return sizeof(double) * ((size_t)CL_VECS * rows(blocks) + (size_t)CL_SLOTS * umax);
     };
-    auto fits = [&](int blocks) { return cl_fits(k_bicg_cluster<true>, k, blocks, CL_T, CL_SMEM, bytes(blocks)); };
+    static ClHeld held;
+    auto fits = [&](int blocks) { return cl_fits(k_bicg_cluster<true>, k, blocks, CL_T, CL_SMEM, held); };
     // enough blocks for the rows, then as many as leave every system on the GPU
     // at once with two units of rows per block (the reductions' cost does not
     // shrink with more); sixteen where the FP64 pipe outweighs the barriers, from

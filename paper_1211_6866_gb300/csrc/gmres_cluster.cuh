@@ -574,9 +574,8 @@ sai_status gc_launch(int n, int64_t ld, int k, int m, const Ops<T>& A, ClPair<T>
     while (C < most && (rows(C) > GC_MAXR || GcLayout<T>(rows(C), m, N.units).bytes > GC_SMEM)) C *= 2;
     if (rows(C) > GC_MAXR || GcLayout<T>(rows(C), m, N.units).bytes > GC_SMEM) return SAI_OK;
     // then as many blocks as leave every system on the GPU at once
-    auto fits = [&](int blocks) {
-        return cl_fits(k_gmres_cluster<T, true>, k, blocks, GC_T, GC_SMEM, GcLayout<T>(rows(blocks), m, N.units).bytes);
-    };
+    static ClHeld held;
+    auto fits = [&](int blocks) { return cl_fits(k_gmres_cluster<T, true>, k, blocks, GC_T, GC_SMEM, held); };
     while (C < most && fits(2 * C)) C *= 2;
     if (C == CL_MAXC && N.units == GC_MAXU && fits(16)) C = 16;
     const int R = rows(C);

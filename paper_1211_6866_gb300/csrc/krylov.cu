@@ -24,6 +24,7 @@
 // reduction and one update pass over the basis per step); Givens rotations;
 // stop on the rotated residual |g_{j+1}|; restart from the true residual
 // b - A~ y.
+#include <atomic>
 #include <math.h>
 
 #include "internal.h"
