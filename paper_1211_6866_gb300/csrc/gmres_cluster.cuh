@@ -17,7 +17,7 @@
 // run with it: the number of blocks follows k, but a sum is a tree per unit of
 // rows (GcUnits, gc_dots) and the units' sums added pairwise in FP64, each block
 // holding whole units. With sums per block instead, this form took 2.94, 4.02
-// and 11.7 ms where it takes 2.98, 4.4 and 12.9 (35937 rows in FP32, 6, 11 and 40
+// and 11.7 ms where it takes 2.90, 4.2 and 12.2 (35937 rows in FP32, 6, 11 and 40
 // systems, 101 steps), and 6.3 where it takes 6.8 (1728 rows in FP64, 256
 // systems, 60 steps). The Hessenberg columns are kept in T, the type k_dc_step
 // uses them in (its rotated columns are T values stored as FP64).
@@ -27,8 +27,8 @@ constexpr int GC_UT = GC_T - 32;  // of them in the update; the last warp runs t
 constexpr int GC_MAXU = 16;    // units of a system
 constexpr int GC_MAXR = 6144;  // rows per block
 // orders up to which the form is used, by n alone. FP32: the multi-kernel form
-// takes as long at 35937 rows with 153 systems (46.0 and 42.7 ms) and longer with
-// up to 40 (4.4 and 6.0 ms with 11, 12.9 and 13.1 with 40); at 46656 rows it is
+// takes as long at 35937 rows with 153 systems (43.4 and 42.7 ms) and longer with
+// up to 40 (4.2 and 6.0 ms with 11, 12.2 and 13.1 with 40); at 46656 rows it is
 // the faster one from 16 systems on (31.6 and 26.0 ms with 77). FP64: above, the
 // FP64 pipes of eight SMs are slower than those of all.
 constexpr size_t GC_SMEM = 220 * 1024;  // shared memory of a block, at most
@@ -136,8 +136,9 @@ struct Comp<double> {
 // along. (A plain tree over 2048 rows has twice the error of the multi-kernel
 // form's four over 512 rows each, added in FP64.) Lane 0 returns v^T u, lane 16
 // v^T z. Two basis vectors at a time, sharing the loads of u and z, were no
-// faster.
-__device__ __noinline__ double gc_dots(const float* v, const float* u, const float* z, int at, int U, int nrow, int)
+// faster; as a call it is slower (13.8 against 13.1 us a step at 2500 rows, 23.7
+// against 22.6 at 27000) by the registers saved around it.
+__device__ __forceinline__ double gc_dots(const float* v, const float* u, const float* z, int at, int U, int nrow, int)
 {
     __builtin_assume(__isShared(u));
     __builtin_assume(__isShared(z));
@@ -202,10 +203,9 @@ __device__ __forceinline__ double gc_sum8(double (&a)[8])
     return w + __shfl_xor_sync(SAI_FULL, w, 1);
 }
 
-// The same in FP64 for uw <= 4 units of U rows at a time, whose trees share
-// their additions (9 for four units, 5 for one). Unit e's sums: lanes 8 e and
-// 8 e + 4, or lanes 0 and 16 for one unit.
-__device__ __noinline__ double gc_dots(const double* v, const double* u, const double* z, int at, int U, int nrow, int uw)
+// The same in FP64 for 2 or 4 units of U rows at a time, whose trees share their
+// additions (9 for four units, 5 for one). Unit e's sums: lanes 8 e and 8 e + 4.
+__device__ __noinline__ double gc_dots_units(const double* v, const double* u, const double* z, int at, int U, int nrow, int uw)
 {
     __builtin_assume(__isShared(u));
     __builtin_assume(__isShared(z));
@@ -231,7 +231,22 @@ __device__ __noinline__ double gc_dots(const double* v, const double* u, const d
         sums[2 * e] = a;
         sums[2 * e + 1] = b;
     }
-    return uw > 1 ? gc_sum8(sums) : gc_sum2(sums[0], sums[1]);
+    return gc_sum8(sums);
+}
+
+// uw units in FP64; one alone in line (2401 rows: a step 26.9 -> 24.1 us)
+__device__ __forceinline__ double gc_dots(const double* v, const double* u, const double* z, int at, int U, int nrow, int uw)
+{
+    if (uw > 1) return gc_dots_units(v, u, z, at, U, nrow, uw);
+    const int r1 = min(nrow, at + U);
+    double a = 0.0, b = 0.0;
+#pragma unroll 4
+    for (int r = at + 2 * (threadIdx.x & 31); r < r1; r += 64) {
+        const double2 x = *reinterpret_cast<const double2*>(v + r);
+        a = Vec<double>::dot(x, *reinterpret_cast<const double2*>(u + r), a);
+        b = Vec<double>::dot(x, *reinterpret_cast<const double2*>(z + r), b);
+    }
+    return gc_sum2(a, b);
 }
 
 // v_j = ia (u - V s), u <- ia (z - V c - dd v_j) on the block's rows: a thread
