@@ -26,15 +26,17 @@ constexpr int GC_T = 512;      // threads per block
 constexpr int GC_UT = GC_T - 32;  // of them in the update; the last warp runs the Givens rotations meanwhile
 constexpr int GC_MAXU = 16;    // units of a system
 constexpr int GC_MAXR = 6144;  // rows per block
-// orders up to which the form is used, by n alone. FP32: the multi-kernel form
-// takes as long at 35937 rows with 153 systems (43.4 and 42.7 ms) and longer with
-// up to 40 (4.2 and 6.0 ms with 11, 12.2 and 13.1 with 40); at 46656 rows it is
-// the faster one from 16 systems on (31.6 and 26.0 ms with 77). FP64: above, the
+// orders up to which the form is used, by n alone. FP32: at 46656 rows a few
+// systems take 3.08, 3.10 and 4.93 ms (2, 6 and 11) against 4.37, 5.05 and 6.11 in
+// the multi-kernel form, which is the faster one there from 16 systems on (9.7 and
+// 7.6 ms, 15.2 and 14.6 with 40, 29.8 and 25.7 with 77); at 35937 rows the two
+// meet at 153 systems (43.4 and 42.7; 12.2 and 13.1 with 40). A split's systems are
+// its dense columns and one, so the few decide. FP64: above, the
 // FP64 pipes of eight SMs are slower than those of all.
 constexpr size_t GC_SMEM = 220 * 1024;  // shared memory of a block, at most
-constexpr int GC_MAXN32 = 36864, GC_MAXN64 = 10240;
-// of a scattered matrix in FP32 (8, 16, 19 and 76 systems of 12000 rows: 2.95,
-// 4.0, 4.1 and 5.2 ms against 3.1, 4.0, 4.4 and 12.0; 4, 16 and 76 systems of 20000
+constexpr int GC_MAXN32 = 49152, GC_MAXN64 = 10240;
+// of a scattered matrix in FP32 (8, 16, 19 and 76 systems of 12000 rows: 2.88,
+// 3.9, 4.0 and 4.9 ms against 3.1, 4.0, 4.4 and 12.0; 4, 16 and 76 systems of 20000
 // rows 3.0, 7.6 and 16 against 2.7, 4.4 and 13.8)
 constexpr int GC_FAR_N32 = 12288;
 

@@ -1,6 +1,6 @@
 """Orders around the limits at which the cluster forms are left: 10240 rows (12288 in refined GMRES) where most entries lie
 far from the diagonal (a random permutation of a tridiagonal matrix), 14336 rows for more than 64 systems, 20480
-(BiCGStab) and 36864 rows (refined GMRES) for a banded matrix; and the vector kernels of more than 256 systems at the
+(BiCGStab) and 49152 rows (refined GMRES) for a banded matrix; and the vector kernels of more than 256 systems at the
 edges of their row chunks. Each against its true residual, and transposed.
 
 Tolerance: the solvers stop on the recursive (BiCGStab) residual or on the true one (refined GMRES); with ||A|| <= 6 and
@@ -19,7 +19,8 @@ pytestmark = pytest.mark.gpu
     (10240, 3, "bicgstab"), (10241, 3, "bicgstab"), (14336, 80, "bicgstab"), (14337, 8, "bicgstab"),
     (14337, 64, "bicgstab"), (14337, 65, "bicgstab"), (20480, 257, "bicgstab"), (9000, 257, "bicgstab"), (511, 300, "bicgstab"),
     (1537, 257, "bicgstab"), (16383, 40, "bicgstab"), (16384, 40, "bicgstab"), (12288, 3, "gmres32"),
-    (12289, 3, "gmres32"), (36864, 2, "gmres32"), (36865, 2, "gmres32"), (10240, 5, "gmres"), (10241, 5, "gmres")])
+    (12289, 3, "gmres32"), (36864, 2, "gmres32"), (36865, 2, "gmres32"), (49152, 2, "gmres32"), (49153, 2, "gmres32"),
+    (10240, 5, "gmres"), (10241, 5, "gmres")])
 def test_around_the_limits(n, k, method, scattered):
     need_gpu()
     sai = lib()

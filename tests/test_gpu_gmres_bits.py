@@ -1,6 +1,6 @@
 """A GMRES system gives the same bits and the same step count alone, with a few others and with many: at the edges of the
 units that its sums are formed by (128 rows at least; sixteen units from 3585 rows on), of the blocks per cluster and of
-the cluster form itself (10240 rows in FP64, 36864 in FP32), with short and long restarts, rows of equal length and with
+the cluster form itself (10240 rows in FP64, 49152 in FP32), with short and long restarts, rows of equal length and with
 every 64th row 40 entries longer. Every comparison is exact: no sum may depend on the other systems."""
 import numpy as np
 import pytest
@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
     (1, 3, 5, 0), (33, 40, 7, 1), (255, 200, 10, 0), (256, 200, 10, 1), (513, 200, 20, 0), (1025, 120, 127, 0),
     (2047, 100, 12, 1), (2049, 80, 30, 0), (3584, 40, 30, 0), (3585, 40, 30, 1), (5000, 256, 10, 0), (6145, 70, 30, 0),
     (10240, 70, 20, 0), (10240, 10, 127, 0), (10241, 9, 20, 0), (12289, 60, 30, 1), (24577, 30, 30, 1),
-    (36864, 25, 20, 1), (36864, 3, 127, 1), (36865, 9, 20, 1)])
+    (36864, 25, 20, 1), (36864, 3, 127, 1), (36865, 9, 20, 1), (49152, 25, 20, 1), (49152, 3, 127, 1), (49153, 9, 20, 1)])
 def test_bits_do_not_depend_on_the_other_systems(n, k, m, precision, uneven):
     need_gpu()
     sai = lib()
