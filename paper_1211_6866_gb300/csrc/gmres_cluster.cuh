@@ -5,7 +5,7 @@
 // k_dc_step / k_dc_update, restarts included, without leaving the kernel: at
 // small orders a step of the multi-kernel form is five launches that wait for
 // one another (45 us at 35937 rows and 6 systems, most of it latency; the
-// whole call 10.4 ms, 7.0 ms here). Block
+// whole call 10.4 ms, 6.9 ms here). Block
 // b of the cluster owns rows [b R, (b + 1) R): the candidate u, t = M u, z =
 // A~ t and x live in its shared memory, its rows of the basis in global
 // memory (read by this block only, so from L1 while they fit). Products
